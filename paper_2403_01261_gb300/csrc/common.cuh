@@ -13,13 +13,14 @@ constexpr int ERRBIT_OVERFLOW = 2;  // weighted degree >= 2^31
 constexpr int ERRBIT_TIMEOUT = 4;   // a bounded retry loop ran out
 
 // Degree classes of the sweep.  A vertex of degree d goes to
-//   class 0..5 : d in [1,1], [2,2], [3,4], [5,8], [9,16], [17,32]  (lane groups of 1..32)
+//   class 0..5 : d in [1,1], [2,2], [3,4], [5,8], [9,16], [17,32]  (tile_kernels.cu)
 //   class 6    : 32 < d <= warp_small   (one warp, small shared-memory table)
 //   class 7    : warp_small < d <= warp_max (one warp, large shared-memory table)
 //   class 8    : warp_max < d <= blk_max   (one block, shared-memory table)
 //   class 9    : d > blk_max               (one block, may use global tables)
 // Degree-0 vertices never change label and are not binned.
 constexpr int NCLASS = 10;
+constexpr int CLS_BINNED = 3;   // classes 0..2 are swept in natural order and not binned
 constexpr int CLS_WARP_S = 6;
 constexpr int CLS_WARP_L = 7;
 constexpr int CLS_BLOCK = 8;
@@ -40,6 +41,8 @@ struct Counters {
   unsigned int pad3;
   unsigned int uns_count[NCLASS];          // majority filter: rows left for the table kernels
   unsigned int phase_cls[NCLASS];          // asynchronous sweeps: cls_count of the sweep's first phase
+  unsigned long long tile_active;          // vertices of classes 0..2 swept
+  unsigned long long tile_scanned;         // and their CSR entries
   int err;                      // ERRBIT_* (sticky for the call)
   unsigned any_bad;             // host-buffer overlap: a landed row is not strictly increasing (sticky)
   int pad1;

@@ -233,13 +233,14 @@ int map_err(gsl_ctx* c, int bits, const char* where) {
 // ------------------------------------------------------------- profiling
 enum Slot {
   SL_CLASSIFY = 0, SL_INIT, SL_BIN, SL_SWEEP0, SL_SPLIT = SL_SWEEP0 + NCLASS, SL_COUNT, SL_MOD, SL_IDENT, SL_PRE,
-  SL_FILTER, SL_N
+  SL_FILTER, SL_LANES, SL_N
 };
 const char* slot_name(int k) {
   static const char* names[SL_N] = {"classify", "init_labels", "bin_frontier", "sweep_deg1", "sweep_deg2",
                                     "sweep_deg3_4", "sweep_deg5_8", "sweep_deg9_16", "sweep_deg17_32",
                                     "sweep_warp_small", "sweep_warp_large", "sweep_block", "sweep_hub",
-                                    "split_unionfind", "split_count_renumber", "modularity", "sweep1_stream", "pregather", "majority_filter"};
+                                    "split_unionfind", "split_count_renumber", "modularity", "sweep1_stream", "pregather", "majority_filter",
+                                    "sweep_deg1_4"};
   return names[k];
 }
 
@@ -276,6 +277,13 @@ void prof_resolve(gsl_ctx* c) {
   }
   c->pending.clear();
   c->ev_used = 0;
+}
+
+// Vertices of classes first..last of the prepared graph.
+long long class_vertices(const gsl_ctx* c, int first, int last) {
+  long long v = 0;
+  for (int k = first; k <= last; ++k) v += (long long)c->ctr_h->cls_total[k];
+  return v;
 }
 
 // Resets all counters, classifies every vertex by degree (validating the
@@ -384,6 +392,7 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
   bool converged = resume ? resume->converged : false, marked_prev = resume ? resume->marked_prev : false;
   long long dn_prev = resume ? resume->dn_prev : n;
   long long scanned = resume ? resume->scanned : 0;
+  bool binned_all = false;
   while (t < max_iters && !converged) {
     ++t;
     if (int r = reset_sweep_counters(c, s)) return r;
@@ -454,20 +463,27 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
     const int phases = async_mode ? 2 : 1;
     for (int ph = 0; ph < phases; ++ph) {
       if (ph == 1) CK(launch_phase_reset(c->ctr, nullptr, s));
-      {
+      // classes without a vertex in the graph are not launched
+      if (class_vertices(c, CLS_BINNED, NCLASS - 1) > 0) {
         const int pe = prof_begin(c, s);
-        CK(launch_bin(OFF(g), n, c->flag[t & 1], all_active ? 1 : 0, c->tune, c->work, c->ctr, c->di, s, nullptr,
-                      nullptr, nullptr, async_mode ? ph : -1, (unsigned)t));
+        if (all_active && binned_all) {
+          CK(launch_all_counts(c->ctr, CLS_BINNED, s));
+        } else {
+          CK(launch_bin(OFF(g), n, c->flag[t & 1], all_active ? 1 : 0, c->tune, c->work, c->ctr, c->di, s, nullptr,
+                        nullptr, nullptr, async_mode ? ph : -1, (unsigned)t, CLS_BINNED));
+          binned_all = all_active && !async_mode;   // the worklist now holds every vertex of these classes
+        }
         prof_end(c, pe, SL_BIN, s, 1);
       }
       SweepArgs af = a;   // the filtered classes read the filter's worklist
-      if (filter) {
+      if (filter && class_vertices(c, filter_from, CLS_BLOCK) > 0) {
         const int pe = prof_begin(c, s);
         CK(launch_majority_filter(a, c->work2, weights != nullptr, async_mode, c->di, s, filter_from));
         prof_end(c, pe, SL_FILTER, s, 2);
         af.work = c->work2;
       }
-      for (int k = NCLASS - 1; k >= 0; --k) {   // the longest rows first
+      for (int k = NCLASS - 1; k >= CLS_BINNED; --k) {   // the longest rows first
+        if (class_vertices(c, k, k) == 0) continue;
         const int pe = prof_begin(c, s);
         if (k == CLS_WARP_L || k == CLS_BLOCK || (k == CLS_WARP_S && filter_from == CLS_WARP_S)) {
           CK(launch_sweep_class(af, k, weights != nullptr, async_mode, c->tune, c->di, s));
@@ -483,6 +499,12 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
           CK(launch_sweep_class(a, k, weights != nullptr, async_mode, c->tune, c->di, s));
           prof_end(c, pe, SL_SWEEP0 + k, s, 1);
         }
+      }
+      if (class_vertices(c, 0, CLS_BINNED - 1) > 0) {
+        const int pe = prof_begin(c, s);
+        CK(launch_sweep_lanes(a, weights != nullptr, async_mode, 0, n, c->flag[t & 1], all_active ? 1 : 0, nullptr, ph,
+                             (unsigned)t, c->di, s));
+        prof_end(c, pe, SL_LANES, s, 1);
       }
     }
     CK(cudaMemcpyAsync(c->ctr_h, c->ctr, offsetof(Counters, pad1), cudaMemcpyDeviceToHost, s));
@@ -505,10 +527,14 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
         sl.bytes += per_v * (double)v + per_e * (double)e;
         act_all += v;
       }
+      auto& sl = c->profile.slot[SL_LANES];   // no worklist entry
+      sl.vertices += (long long)c->ctr_h->tile_active;
+      sl.entries += (long long)c->ctr_h->tile_scanned;
+      sl.bytes += (per_v - 4.0) * (double)c->ctr_h->tile_active + per_e * (double)c->ctr_h->tile_scanned;
       if (filter) {
         // the filter read every row of classes 7 and 8: the settled ones (their
         // entries are in `scanned` but in no class) and those it passed on
-        long long cls_e = 0, rows = (long long)c->ctr_h->fast_active;
+        long long cls_e = (long long)c->ctr_h->tile_scanned, rows = (long long)c->ctr_h->fast_active;
         for (int k = 0; k < NCLASS; ++k) cls_e += (long long)c->ctr_h->cls_scanned[k];
         long long fe = (long long)c->ctr_h->scanned - cls_e;
         for (int k = CLS_WARP_L; k <= CLS_BLOCK; ++k) {
@@ -528,7 +554,7 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
     if (int r = map_err(c, c->ctr_h->err, "lpa")) return r;
     c->hub_dirty = false;   // every hub's final pass reset the slots its pieces claimed
     const long long dn = (long long)c->ctr_h->dn;
-    long long act = (long long)c->ctr_h->fast_active;
+    long long act = (long long)(c->ctr_h->fast_active + c->ctr_h->tile_active);
     for (int k = 0; k < NCLASS; ++k) act += (long long)(c->ctr_h->cls_count[k] + c->ctr_h->phase_cls[k]);
     scanned += (long long)c->ctr_h->scanned;
     if (st && t <= GSL_STATS_SWEEPS) {
@@ -861,22 +887,31 @@ cudaError_t enqueue_batch_sweeps(gsl_ctx* c, const gsl_csr* g, int num_graphs, c
     const int phases = async_mode ? 2 : 1;   // asynchronous sweeps in two phases, as in run_lpa
     for (int ph = 0; ph < phases; ++ph) {
       if (ph == 1) ck(launch_phase_reset(c->ctr, c->stop, cs));
-      pe = prof ? prof_begin(c, cs) : -1;
-      ck(launch_bin(OFF(g), n, c->flag[t & 1], t <= 2 ? 1 : 0, c->tune, c->work, c->ctr, c->di, cs, c->gid, c->done,
-                    c->stop, async_mode ? ph : -1, (unsigned)t));
-      if (prof) prof_end(c, pe, SL_BIN, cs, 1);
+      if (class_vertices(c, CLS_BINNED, NCLASS - 1) > 0) {
+        pe = prof ? prof_begin(c, cs) : -1;
+        ck(launch_bin(OFF(g), n, c->flag[t & 1], t <= 2 ? 1 : 0, c->tune, c->work, c->ctr, c->di, cs, c->gid, c->done,
+                      c->stop, async_mode ? ph : -1, (unsigned)t, CLS_BINNED));
+        if (prof) prof_end(c, pe, SL_BIN, cs, 1);
+      }
       SweepArgs af = a;
-      if (filter) {
+      if (filter && class_vertices(c, filter_from, CLS_BLOCK) > 0) {
         pe = prof ? prof_begin(c, cs) : -1;
         ck(launch_majority_filter(a, c->work2, weights != nullptr, async_mode, c->di, cs, filter_from));
         if (prof) prof_end(c, pe, SL_FILTER, cs, 2);
         af.work = c->work2;
       }
-      for (int k = 0; k < NCLASS; ++k) {
+      for (int k = CLS_BINNED; k < NCLASS; ++k) {
+        if (class_vertices(c, k, k) == 0) continue;
         pe = prof ? prof_begin(c, cs) : -1;
         const bool filtered = k == CLS_WARP_L || k == CLS_BLOCK || (k == CLS_WARP_S && filter_from == CLS_WARP_S);
         ck(launch_sweep_class(filtered ? af : a, k, weights != nullptr, async_mode, c->tune, c->di, cs));
         if (prof) prof_end(c, pe, SL_SWEEP0 + k, cs, 1);
+      }
+      if (class_vertices(c, 0, CLS_BINNED - 1) > 0) {
+        pe = prof ? prof_begin(c, cs) : -1;
+        ck(launch_sweep_lanes(a, weights != nullptr, async_mode, 0, n, c->flag[t & 1], t <= 2 ? 1 : 0, c->done, ph,
+                             (unsigned)t, c->di, cs));
+        if (prof) prof_end(c, pe, SL_LANES, cs, 1);
       }
     }
     ck(launch_graph_update(t, tol, max_iters, c->vptr, num_graphs, c->dn_graph, c->iters, c->done, c->stop, cs));
@@ -1506,7 +1541,12 @@ int gsl_gsllpa_batch(gsl_ctx* c, const gsl_csr* g, int32_t num_graphs, const int
   CK(launch_graph_update(0, tol, max_iters, c->vptr, num_graphs, c->dn_graph, c->iters, c->done, c->stop, s));
   // The sweep loop, unrolled over max_iters and captured once as a CUDA
   // graph; sweeps after the last graph stops return at once.
-  const std::vector<long long> key = {(long long)OFF(g), (long long)g->cols, (long long)weights, n, g->nnz,
+  // The launches depend on which classes the graph populates: part of the
+  // key, since other offsets may come in the same buffers.
+  long long populated = 0;
+  for (int k = 0; k < NCLASS; ++k)
+    if (n > 0 && class_vertices(c, k, k) > 0) populated |= 1ll << k;
+  const std::vector<long long> key = {populated, (long long)OFF(g), (long long)g->cols, (long long)weights, n, g->nnz,
                                       num_graphs, max_iters, mode, (long long)(tol * 1e12), c->ctr_h->max_degree,
                                       (long long)c->lab[0], (long long)c->wtab, (long long)c->btab,
                                       c->tune.warp_max, c->tune.blk_max, (long long)c->work2,
@@ -1709,13 +1749,16 @@ int gsllpa_host_overlapped(gsl_ctx* c, int64_t n, int64_t nnz, const int64_t* of
                           s));
     if (stop1) continue;
     if (k > 0) CK(launch_phase_reset(c->ctr, nullptr, s));
-    CK(launch_bin_range(OFF(&g), vb[k], vb[k + 1], c->tune, c->work, c->ctr, c->di, s));
+    CK(launch_sweep_lanes(a, false, false, vb[k], vb[k + 1], nullptr, 1, nullptr, 0, 2u, c->di, s));
+    if (class_vertices(c, CLS_BINNED, NCLASS - 1) == 0) continue;
+    CK(launch_bin_range(OFF(&g), vb[k], vb[k + 1], c->tune, c->work, c->ctr, c->di, s, CLS_BINNED));
     SweepArgs af = a;
     if (filter) {
       CK(launch_majority_filter(a, c->work2, false, false, c->di, s));
       af.work = c->work2;
     }
-    for (int cls = NCLASS - 1; cls >= 0; --cls) {
+    for (int cls = NCLASS - 1; cls >= CLS_BINNED; --cls) {
+      if (class_vertices(c, cls, cls) == 0) continue;
       if (cls == CLS_WARP_L || cls == CLS_BLOCK) {
         CK(launch_sweep_class(af, cls, false, false, c->tune, c->di, s));
       } else if (cls == CLS_HUB && c->hub_ready) {
@@ -1752,7 +1795,7 @@ int gsllpa_host_overlapped(gsl_ctx* c, int64_t n, int64_t nnz, const int64_t* of
   }
   if (!stop1) {
     const long long dn2 = (long long)c->ctr_h->dn;
-    long long act2 = (long long)c->ctr_h->fast_active;
+    long long act2 = (long long)(c->ctr_h->fast_active + c->ctr_h->tile_active);
     for (int k = 0; k < NCLASS; ++k) act2 += (long long)(c->ctr_h->cls_count[k] + c->ctr_h->phase_cls[k]);
     rs.done = 2;
     rs.converged = (double)dn2 / (double)n <= tol;

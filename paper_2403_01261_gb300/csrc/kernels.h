@@ -42,7 +42,6 @@ struct Tuning {
   int blk_max = 32768;       // class 7 upper degree bound (one block per vertex; above: class 8)
   int warp_slots = 1024;     // shared-memory table slots per warp of class 7 (8 bytes each)
   int blk_slots = 12288;     // shared-memory table slots per block
-  int group_block = 256;     // threads per block of the lane-group kernels
   int warp_block = 256;      // threads per block of the warp kernel
   int blk_block = 512;       // threads per block of the block kernel
   int pregather = 0;         // two-phase sweeps: 0 never, 1 when the frontier is large, 2 always
@@ -68,15 +67,24 @@ struct DeviceInfo {
 cudaError_t launch_class_histogram(const long long* off, long long n, long long nnz, const Tuning& t,
                                    Counters* ctr, const DeviceInfo& di, cudaStream_t s);
 // phase >= 0: only the frontier vertices of that phase of an asynchronous
-// sweep (a hash of the vertex id and `seed`); the others keep their flags.
+// sweep (a hash of the vertex id and `seed`); the others keep their flags,
+// as do the vertices of the classes below first_cls.
 cudaError_t launch_bin(const long long* off, long long n, unsigned char* fcur, int all_active,
                        const Tuning& t, int* work, Counters* ctr, const DeviceInfo& di, cudaStream_t s,
                        const int* gid = nullptr, const unsigned char* done = nullptr, const int* stop = nullptr,
-                       int phase = -1, unsigned seed = 0);
+                       int phase = -1, unsigned seed = 0, int first_cls = 0);
+// The class counts of an all-active binning whose worklist is still in place.
+cudaError_t launch_all_counts(Counters* ctr, int first_cls, cudaStream_t s);
+// tile_kernels.cu: the rows of 1..4 entries among the vertices [v0, v1) (all
+// of them, or those flagged in fcur, whose flags are cleared), and the rows
+// of classes 3..5 on the worklist.
+cudaError_t launch_sweep_lanes(const SweepArgs& a, bool weighted, bool async_mode, long long v0, long long v1,
+                               unsigned char* fcur, int all_active, const unsigned char* done, int phase,
+                               unsigned seed, const DeviceInfo& di, cudaStream_t s);
+cudaError_t launch_sweep_tile(const SweepArgs& a, int cls, bool weighted, bool async_mode, const DeviceInfo& di,
+                              cudaStream_t s);
 // Between the two phases of an asynchronous sweep (see Counters::phase_cls).
 cudaError_t launch_phase_reset(Counters* ctr, const int* stop, cudaStream_t s);
-cudaError_t launch_sweep(const SweepArgs& a, bool weighted, bool async_mode, const Tuning& t,
-                         const DeviceInfo& di, cudaStream_t s);
 cudaError_t launch_sweep_class(const SweepArgs& a, int cls, bool weighted, bool async_mode, const Tuning& t,
                                const DeviceInfo& di, cudaStream_t s);
 void count_launches(long long k);   // process-wide tally of kernels this library launched
@@ -120,7 +128,7 @@ cudaError_t launch_chunk_check(const long long* off, long long n, const int* col
                                long long e1, const unsigned* bits, unsigned char* bad, unsigned* any_bad,
                                Counters* ctr, const DeviceInfo& di, cudaStream_t s);
 cudaError_t launch_bin_range(const long long* off, long long v0, long long v1, const Tuning& t, int* work,
-                             Counters* ctr, const DeviceInfo& di, cudaStream_t s);
+                             Counters* ctr, const DeviceInfo& di, cudaStream_t s, int first_cls = 0);
 // Streaming sweep 1 with float weights: for strictly increasing rows the
 // label is the neighbour of largest weight (smallest id among equals).
 cudaError_t launch_ident_stream_f32(const long long* off, long long n, const int* col, const float* wf,

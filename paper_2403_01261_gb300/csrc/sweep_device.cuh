@@ -80,6 +80,20 @@ __device__ __forceinline__ void count_graph_change(const SweepArgs& a, int v) {
 
 __device__ __forceinline__ bool stopped(const SweepArgs& a) { return a.stop && *(volatile const int*)a.stop; }
 
+// Phase of vertex v in the asynchronous sweep with seed `seed` (the sweep
+// number): the top bit of a mixed hash, so that two neighbours fall in the
+// same phase of a sweep with probability 1/2, independently from sweep to
+// sweep.
+__device__ __forceinline__ int sweep_phase(long long v, unsigned seed) {
+  unsigned h = (unsigned)v * 0x9E3779B1u + seed * 0x85EBCA6Bu;
+  h ^= h >> 16;
+  h *= 0x7FEB352Du;
+  h ^= h >> 15;
+  h *= 0x846CA68Bu;
+  h ^= h >> 16;
+  return (int)(h >> 31);
+}
+
 template <bool ASYNC>
 __device__ __forceinline__ int gather_label(const SweepArgs& a, int j, const Pol& pol) {
   if (a.ident) return j;
@@ -185,6 +199,30 @@ __device__ __forceinline__ unsigned label_group(int l, int spread) {
   if (spread) return 1u << (threadIdx.x & 31);
   return __match_any_sync(FULL, l);
 }
+
+// ---------------------------------------------------------------------------
+// Counting labels without a match and without probing.  A row's entries add
+// their weights to slots picked by a hash of their label and leave the label
+// in the slot (the last store wins).  A slot whose entries all read their own
+// label back is pure: its sum is exactly that label's sum.  A slot shared by
+// several labels bounds each of them by its sum less one (every weight is at
+// least 1), so only the labels of shared slots that could still beat the best
+// pure label (larger sum, then smaller label) go into another round with
+// another hash.  All entries of a label share its slot and decide alike, so
+// every round is exact for the labels it settles.  Per 32 entries that is one
+// shared add (2.6 cycles of an SM, measured), two stores and two loads;
+// __match_any_sync costs 64 cycles there when the labels are distinct (two a
+// value) and 8 when there are four.
+struct SketchBest {
+  unsigned sum, inv;   // largest label sum so far and ~label (0: none)
+};
+
+__device__ __forceinline__ unsigned sketch_hash(unsigned x, int round) {
+  x ^= x >> 15;
+  return (x + (unsigned)round) * (0x9E3779B1u + 0x3C6EF372u * (unsigned)round);   // the multiplier stays odd
+}
+
+constexpr int SKETCH_ROUNDS = 8;   // shared slots left after these many hashes are settled by a match
 
 // Row loops specialised for sweep 2 from the identity labelling (SPREAD):
 // the labels of sweep 1 are nearly all distinct and the vertex's own label
