@@ -789,10 +789,12 @@ int run_modularity(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const i
   CK(cudaMemsetAsync(c->sigma, 0, sizeof(unsigned long long) * (size_t)n, s));
   CK(cudaMemsetAsync(c->sums, 0, sizeof(ModSums), s));
   if (int r = reset_sweep_counters(c, s)) return r;
-  CK(launch_bin(OFF(g), n, nullptr, 1, c->tune, c->work, c->ctr, c->di, s));
+  if (class_vertices(c, CLS_BINNED, NCLASS - 1) > 0)
+    CK(launch_bin(OFF(g), n, nullptr, 1, c->tune, c->work, c->ctr, c->di, s, nullptr, nullptr, nullptr, -1, 0u,
+                  CLS_BINNED));
   const int pe = prof_begin(c, s);
-  CK(launch_modularity(OFF(g), g->cols, weights, n, labels, c->work, c->ctr, c->sigma, c->partials, np, c->sums,
-                       c->tune, c->di, s));
+  CK(launch_modularity(OFF(g), g->cols, weights, n, labels, c->work, c->ctr, c->ctr_h->cls_total, c->sigma,
+                       c->partials, np, c->sums, c->di, s));
   prof_end(c, pe, SL_MOD, s, 13);
   // per vertex: offsets, label, Sigma update (read+write) and square pass;
   // per entry: column, neighbour label and weight

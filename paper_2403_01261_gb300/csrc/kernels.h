@@ -222,10 +222,12 @@ struct ModSums {
   unsigned long long s1;
   unsigned long long s2_lo, s2_hi;
 };
+// `work` holds the binning of classes CLS_BINNED.. of every vertex, totals
+// the host's copy of the class totals.
 cudaError_t launch_modularity(const long long* off, const int* col, const int* w, long long n,
-                              const int* labels, const int* work, Counters* ctr,
+                              const int* labels, const int* work, Counters* ctr, const unsigned long long* totals,
                               unsigned long long* sigma, unsigned long long* partials, long long nparts,
-                              ModSums* out, const Tuning& t, const DeviceInfo& di, cudaStream_t s);
+                              ModSums* out, const DeviceInfo& di, cudaStream_t s);
 long long modularity_partials(const DeviceInfo& di);
 
 }  // namespace gsl

@@ -5,10 +5,20 @@
 //   S1            = sum_c sigma_c = weights of entries (i, j) with C_i == C_j,
 //   Sigma_c       = sum of K_i over the vertices of c,
 //   S2            = sum_c Sigma_c^2 (128-bit).
-// Pass 1 (per vertex, by degree class) accumulates K_i into Sigma[C_i] and
-// the block sums of 2m and S1; pass 2 squares and sums Sigma in 128 bits;
-// the host forms Q once in double.  All sums are integers, so the result is
-// independent of summation order.
+// Pass 1 accumulates K_i into Sigma[C_i] and the block sums of 2m and S1:
+// rows of 1..4 entries one lane each in natural order, longer ones from the
+// worklist by degree class.  Unit-weight K_i are degrees, so every vertex's
+// K_i is added by the natural-order kernel and the class kernels only count
+// S1.  Pass 2 squares and sums Sigma in 128 bits; the host forms Q once in
+// double.  All sums are integers, so the result is independent of summation
+// order.
+//
+// A partition that sweeps leave on a skewed graph holds one community of
+// nearly every vertex: adding each lane's part to Sigma directly made 52 of
+// 52.5 ms of an R-MAT scale 23 call wait on atomics to one address.  Equal
+// communities of a warp are added up first, then in a per-block table of
+// MOD_CACHE communities, which reaches Sigma once per block.  What is left
+// is bound by the gathers of the neighbours' labels.
 #include "kernels.h"
 
 namespace gsl {
@@ -50,50 +60,160 @@ __device__ __forceinline__ void flush_sums(ModSums* out, unsigned long long k, u
   }
 }
 
-// One row slice: returns (sum of weights, sum of weights inside C_u).
-template <bool WEIGHTED>
-__device__ __forceinline__ void mod_entry(const int* col, const int* w, const int* labels, long long n, int cu,
-                                          long long e, unsigned long long& k, unsigned long long& s1, int* err) {
-  const int j = ld_stream(col + e);
-  const unsigned long long we = WEIGHTED ? (unsigned long long)(unsigned)ld_stream(w + e) : 1ull;
-  if ((unsigned)j >= (unsigned)n) {
-    raise_err(err, ERRBIT_INVALID);
-    return;
+// Per-block table of community sums (direct mapped, first come): what does
+// not fit goes to Sigma at once.
+constexpr int MOD_CACHE = 256;
+struct SigmaCache {
+  int key[MOD_CACHE];   // -1: free
+  unsigned long long sum[MOD_CACHE];
+};
+
+__device__ __forceinline__ void cache_clear(SigmaCache& sc) {
+  for (int k = threadIdx.x; k < MOD_CACHE; k += blockDim.x) {
+    sc.key[k] = -1;
+    sc.sum[k] = 0;
   }
-  k += we;
-  if (ld_label_ro(labels + j) == cu) s1 += we;
+  __syncthreads();
 }
+
+__device__ __forceinline__ void cache_add(SigmaCache& sc, unsigned long long* sigma, int c, unsigned long long k) {
+  const int slot = (int)(hash32((unsigned)c) >> 24);
+  const int old = atomicCAS(&sc.key[slot], -1, c);
+  if (old == -1 || old == c) atomicAdd(&sc.sum[slot], k);
+  else atomicAdd(sigma + c, k);
+}
+
+// Every lane of the warp with its community c and sum k (k = 0: nothing):
+// the lanes that share the first such lane's community are added up first.
+__device__ __forceinline__ void warp_add_sigma(SigmaCache& sc, unsigned long long* sigma, int c,
+                                               unsigned long long k) {
+  const unsigned has = __ballot_sync(FULL, k != 0);
+  if (!has) return;
+  const int first = __ffs((int)has) - 1;
+  const int cf = __shfl_sync(FULL, c, first);   // every lane takes part
+  const bool same = k != 0 && c == cf;
+  const unsigned long long total = warp_sum_u64(same ? k : 0ull);
+  if ((int)(threadIdx.x & 31) == first) cache_add(sc, sigma, c, total);
+  else if (k && !same) cache_add(sc, sigma, c, k);
+}
+
+__device__ __forceinline__ void cache_flush(SigmaCache& sc, unsigned long long* sigma) {
+  __syncthreads();
+  for (int k = threadIdx.x; k < MOD_CACHE; k += blockDim.x)
+    if (sc.key[k] >= 0 && sc.sum[k]) atomicAdd(sigma + sc.key[k], sc.sum[k]);
+}
+
+// U entries e, e + step, .. of a row of u's community cu, the loads of all
+// in flight together: adds their weights to k and, inside cu, to s1.
+template <bool WEIGHTED, int U>
+__device__ __forceinline__ void mod_entries(const int* col, const int* w, const int* labels, long long n, int cu,
+                                            long long e, long long end, int step, unsigned long long& k,
+                                            unsigned long long& s1, int* err) {
+  int j[U], x[U];
+#pragma unroll
+  for (int q = 0; q < U; ++q) {
+    const bool in = e + (long long)q * step < end;
+    j[q] = in ? ld_stream(col + e + (long long)q * step) : -1;
+    x[q] = 1;
+    if (WEIGHTED && in) x[q] = ld_stream(w + e + (long long)q * step);
+    if (in && (unsigned)j[q] >= (unsigned)n) {
+      raise_err(err, ERRBIT_INVALID);
+      j[q] = -1;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < U; ++q) {
+    if (j[q] >= 0) {
+      const unsigned long long we = (unsigned long long)(unsigned)x[q];
+      if (WEIGHTED) k += we;
+      if (ld_label_ro(labels + j[q]) == cu) s1 += we;
+    }
+  }
+}
+
+constexpr int MOD_LANE_ROW = 4;   // longest row of one lane (classes 0..2)
 
 }  // namespace
 
+// Every vertex in natural order, one lane each: label range, unit-weight
+// K_i, and the rows of 1..4 entries.
+template <bool WEIGHTED>
+__global__ void __launch_bounds__(256) mod_lane_kernel(const long long* __restrict__ off, const int* __restrict__ col,
+                                                        const int* __restrict__ w, const int* __restrict__ labels,
+                                                        long long n, Counters* ctr, unsigned long long* sigma,
+                                                        ModSums* out) {
+  __shared__ SigmaCache sc;
+  cache_clear(sc);
+  unsigned long long tk = 0, ts1 = 0;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  const long long v0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
+  for (long long wv = v0; wv < n; wv += stride) {   // warp-uniform
+    const long long v = wv + (threadIdx.x & 31);
+    unsigned long long k = 0;
+    int cu = 0;
+    if (v < n) {
+      const long long s = off[v], e = off[v + 1];
+      cu = labels[v];
+      if ((unsigned)cu >= (unsigned)n) {
+        raise_err(&ctr->err, ERRBIT_INVALID);
+        cu = 0;
+      } else {
+        if (e - s <= MOD_LANE_ROW) mod_entries<WEIGHTED, MOD_LANE_ROW>(col, w, labels, n, cu, s, e, 1, k, ts1, &ctr->err);
+        if (!WEIGHTED) k = (unsigned long long)(e - s);
+      }
+    }
+    tk += k;
+    warp_add_sigma(sc, sigma, cu, k);
+  }
+  cache_flush(sc, sigma);
+  flush_sums(out, tk, ts1);
+}
+
+// Classes 3..7 from the worklist: G lanes per row, four entries of a lane in
+// flight on rows longer than G.
 template <int G, bool WEIGHTED>
 __global__ void __launch_bounds__(256) mod_group_kernel(const long long* __restrict__ off, const int* __restrict__ col,
                                                          const int* __restrict__ w, const int* __restrict__ labels,
                                                          long long n, const int* __restrict__ work, Counters* ctr,
                                                          int cls, unsigned long long* sigma, ModSums* out) {
+  __shared__ SigmaCache sc;
+  if (WEIGHTED) cache_clear(sc);
   const unsigned cnt = (unsigned)ctr->cls_total[cls];
   const int* wl = work + ctr->cls_start[cls];
-  const int gl = threadIdx.x & (G - 1);
-  const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
-  const long long ng = ((long long)gridDim.x * blockDim.x) / G;
+  constexpr int PER = 32 / G;
+  const int lane = threadIdx.x & 31, gl = lane & (G - 1);
+  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   unsigned long long tk = 0, ts1 = 0;
-  // the loop trip count differs between groups: no warp collectives inside
-  for (long long item = gid; item < (long long)cnt; item += ng) {
-    const int u = wl[item];
-    const long long s = off[u], e = off[u + 1];
-    const int cu = labels[u];
-    if ((unsigned)cu >= (unsigned)n) {
-      raise_err(&ctr->err, ERRBIT_INVALID);
-      continue;
-    }
+  for (long long i0 = warp * PER; i0 < (long long)cnt; i0 += nwarps * PER) {   // warp-uniform
+    const long long item = i0 + lane / G;
     unsigned long long k = 0;
-    for (long long x = s + gl; x < e; x += G) mod_entry<WEIGHTED>(col, w, labels, n, cu, x, k, ts1, &ctr->err);
-    tk += k;
-    if (k) atomicAdd(sigma + cu, k);
+    int cu = 0;
+    if (item < (long long)cnt) {
+      const int u = wl[item];
+      const long long s = off[u], e = off[u + 1];
+      cu = labels[u];
+      if ((unsigned)cu >= (unsigned)n) {
+        cu = 0;   // reported by the natural-order kernel
+      } else if (G < 32 || e - s <= 32) {
+        mod_entries<WEIGHTED, 1>(col, w, labels, n, cu, s + gl, e, G, k, ts1, &ctr->err);
+      } else {
+        for (long long x = s + gl; x < e; x += 4 * G)
+          mod_entries<WEIGHTED, 4>(col, w, labels, n, cu, x, e, G, k, ts1, &ctr->err);
+      }
+    }
+    if (WEIGHTED) {
+      tk += k;
+#pragma unroll
+      for (int o = G / 2; o; o >>= 1) k += __shfl_xor_sync(FULL, k, o);
+      warp_add_sigma(sc, sigma, cu, gl == 0 ? k : 0ull);
+    }
   }
+  if (WEIGHTED) cache_flush(sc, sigma);
   flush_sums(out, tk, ts1);
 }
 
+// Classes 8 and 9: one block per row, four entries of a thread in flight.
 template <bool WEIGHTED>
 __global__ void __launch_bounds__(512) mod_block_kernel(const long long* __restrict__ off, const int* __restrict__ col,
                                                          const int* __restrict__ w, const int* __restrict__ labels,
@@ -106,23 +226,17 @@ __global__ void __launch_bounds__(512) mod_block_kernel(const long long* __restr
     const int u = wl[item];
     const long long s = off[u], e = off[u + 1];
     const int cu = labels[u];
-    if ((unsigned)cu >= (unsigned)n) {
-      if (threadIdx.x == 0) raise_err(&ctr->err, ERRBIT_INVALID);
-      continue;
-    }
+    if ((unsigned)cu >= (unsigned)n) continue;   // reported by the natural-order kernel
     unsigned long long k = 0;
-    for (long long x = s + threadIdx.x; x < e; x += blockDim.x) mod_entry<WEIGHTED>(col, w, labels, n, cu, x, k, ts1, &ctr->err);
-    tk += k;
-    if (k) atomicAdd(sigma + cu, k);
+    for (long long x = s + threadIdx.x; x < e; x += 4 * blockDim.x)
+      mod_entries<WEIGHTED, 4>(col, w, labels, n, cu, x, e, (int)blockDim.x, k, ts1, &ctr->err);
+    if (WEIGHTED) {
+      tk += k;
+      k = warp_sum_u64(k);
+      if ((threadIdx.x & 31) == 0 && k) atomicAdd(sigma + cu, k);
+    }
   }
   flush_sums(out, tk, ts1);
-}
-
-// Isolated vertices (degree 0) contribute nothing to 2m, S1 or Sigma; their
-// labels still have to be in range.
-__global__ void mod_check_labels_kernel(const int* __restrict__ labels, long long n, Counters* ctr) {
-  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x)
-    if ((unsigned)labels[v] >= (unsigned)n) raise_err(&ctr->err, ERRBIT_INVALID);
 }
 
 __global__ void __launch_bounds__(256) mod_square_kernel(const unsigned long long* __restrict__ sigma, long long n,
@@ -149,50 +263,68 @@ __global__ void __launch_bounds__(256) mod_square_kernel(const unsigned long lon
   }
 }
 
-__global__ void mod_final_kernel(const unsigned long long* partials, long long nparts, ModSums* out) {
-  if (threadIdx.x != 0) return;
+__global__ void __launch_bounds__(256) mod_final_kernel(const unsigned long long* partials, long long nparts,
+                                                        ModSums* out) {
+  __shared__ unsigned long long lo[256], hi[256];
   U128 acc{0, 0};
-  for (long long b = 0; b < nparts; ++b) acc = add128(acc, U128{partials[2 * b], partials[2 * b + 1]});
-  out->s2_lo = acc.lo;
-  out->s2_hi = acc.hi;
+  for (long long b = threadIdx.x; b < nparts; b += 256) acc = add128(acc, U128{partials[2 * b], partials[2 * b + 1]});
+  lo[threadIdx.x] = acc.lo;
+  hi[threadIdx.x] = acc.hi;
+  __syncthreads();
+  for (int o = 128; o; o >>= 1) {
+    if (threadIdx.x < (unsigned)o) {
+      const U128 r = add128(U128{lo[threadIdx.x], hi[threadIdx.x]}, U128{lo[threadIdx.x + o], hi[threadIdx.x + o]});
+      lo[threadIdx.x] = r.lo;
+      hi[threadIdx.x] = r.hi;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    out->s2_lo = lo[0];
+    out->s2_hi = hi[0];
+  }
 }
+
+namespace {
+template <bool W>
+int launch_mod_rows(const long long* off, const int* col, const int* w, long long n, const int* labels,
+                    const int* work, Counters* ctr, const unsigned long long* totals, unsigned long long* sigma,
+                    ModSums* out, const DeviceInfo& di, cudaStream_t s) {
+  const int g = 8 * di.sm_count;
+  const long long blocks = (n + 255) / 256;
+  mod_lane_kernel<W><<<(int)(blocks < g ? blocks : g), 256, 0, s>>>(off, col, w, labels, n, ctr, sigma, out);
+  int launches = 1;
+  for (int k = NCLASS - 1; k >= CLS_BINNED; --k) {   // the longest rows first; classes without a vertex not at all
+    if (!totals[k]) continue;
+    ++launches;
+    if (k >= CLS_BLOCK)
+      mod_block_kernel<W><<<4 * di.sm_count, 512, 0, s>>>(off, col, w, labels, n, work, ctr, k, sigma, out);
+    else if (k >= 5)
+      mod_group_kernel<32, W><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, k, sigma, out);
+    else if (k == 4)
+      mod_group_kernel<16, W><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, k, sigma, out);
+    else
+      mod_group_kernel<8, W><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, k, sigma, out);
+  }
+  return launches;
+}
+}  // namespace
 
 long long modularity_partials(const DeviceInfo& di) { return 4ll * di.sm_count; }
 
 cudaError_t launch_modularity(const long long* off, const int* col, const int* w, long long n, const int* labels,
-                              const int* work, Counters* ctr, unsigned long long* sigma, unsigned long long* partials,
-                              long long nparts, ModSums* out, const Tuning& t, const DeviceInfo& di, cudaStream_t s) {
-  (void)t;
+                              const int* work, Counters* ctr, const unsigned long long* totals,
+                              unsigned long long* sigma, unsigned long long* partials, long long nparts, ModSums* out,
+                              const DeviceInfo& di, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int g = 8 * di.sm_count;
-  mod_check_labels_kernel<<<g, 256, 0, s>>>(labels, n, ctr);
-  if (w) {
-    mod_group_kernel<1, true><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, 0, sigma, out);
-    mod_group_kernel<2, true><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, 1, sigma, out);
-    mod_group_kernel<4, true><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, 2, sigma, out);
-    mod_group_kernel<8, true><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, 3, sigma, out);
-    mod_group_kernel<16, true><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, 4, sigma, out);
-    mod_group_kernel<32, true><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, 5, sigma, out);
-    mod_group_kernel<32, true><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, CLS_WARP_S, sigma, out);
-    mod_group_kernel<32, true><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, CLS_WARP_L, sigma, out);
-    mod_block_kernel<true><<<4 * di.sm_count, 512, 0, s>>>(off, col, w, labels, n, work, ctr, CLS_BLOCK, sigma, out);
-    mod_block_kernel<true><<<4 * di.sm_count, 512, 0, s>>>(off, col, w, labels, n, work, ctr, CLS_HUB, sigma, out);
-  } else {
-    mod_group_kernel<1, false><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, 0, sigma, out);
-    mod_group_kernel<2, false><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, 1, sigma, out);
-    mod_group_kernel<4, false><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, 2, sigma, out);
-    mod_group_kernel<8, false><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, 3, sigma, out);
-    mod_group_kernel<16, false><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, 4, sigma, out);
-    mod_group_kernel<32, false><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, 5, sigma, out);
-    mod_group_kernel<32, false><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, CLS_WARP_S, sigma, out);
-    mod_group_kernel<32, false><<<g, 256, 0, s>>>(off, col, w, labels, n, work, ctr, CLS_WARP_L, sigma, out);
-    mod_block_kernel<false><<<4 * di.sm_count, 512, 0, s>>>(off, col, w, labels, n, work, ctr, CLS_BLOCK, sigma, out);
-    mod_block_kernel<false><<<4 * di.sm_count, 512, 0, s>>>(off, col, w, labels, n, work, ctr, CLS_HUB, sigma, out);
-  }
-  const long long np = nparts < modularity_partials(di) ? nparts : modularity_partials(di);
+  static_assert(CLS_BINNED == 3 && MOD_LANE_ROW == 4, "classes 0..2 are the rows of one lane");
+  int launches = w ? launch_mod_rows<true>(off, col, w, n, labels, work, ctr, totals, sigma, out, di, s)
+                   : launch_mod_rows<false>(off, col, w, n, labels, work, ctr, totals, sigma, out, di, s);
+  long long np = nparts < modularity_partials(di) ? nparts : modularity_partials(di);
+  if (np > (n + 255) / 256) np = (n + 255) / 256;
   mod_square_kernel<<<(int)np, 256, 0, s>>>(sigma, n, partials);
-  mod_final_kernel<<<1, 32, 0, s>>>(partials, np, out);
-  count_launches(13);
+  mod_final_kernel<<<1, 256, 0, s>>>(partials, np, out);
+  count_launches(launches + 2);
   return cudaGetLastError();
 }
 
