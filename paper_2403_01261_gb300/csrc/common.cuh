@@ -14,10 +14,10 @@ constexpr int ERRBIT_TIMEOUT = 4;   // a bounded retry loop ran out
 
 // Degree classes of the sweep.  A vertex of degree d goes to
 //   class 0..5 : d in [1,1], [2,2], [3,4], [5,8], [9,16], [17,32]  (tile_kernels.cu)
-//   class 6    : 32 < d <= warp_small   (one warp, small shared-memory table)
-//   class 7    : warp_small < d <= warp_max (one warp, large shared-memory table)
-//   class 8    : warp_max < d <= blk_max   (one block, shared-memory table)
-//   class 9    : d > blk_max               (one block, may use global tables)
+//   class 6    : 32 < d <= warp_small   (one warp per row)
+//   class 7    : warp_small < d <= warp_max (a small block per row)
+//   class 8    : warp_max < d <= blk_max   (one block per row)
+//   class 9    : d > blk_max               (thread-block clusters, or pieces)
 // Degree-0 vertices never change label and are not binned.
 constexpr int NCLASS = 10;
 constexpr int CLS_BINNED = 3;   // classes 0..2 are swept in natural order and not binned
@@ -41,6 +41,7 @@ struct Counters {
   unsigned int pad3;
   unsigned int uns_count[NCLASS];          // majority filter: rows left for the table kernels
   unsigned int phase_cls[NCLASS];          // asynchronous sweeps: cls_count of the sweep's first phase
+  unsigned int row_next[NCLASS];           // rows of a class taken so far by the blocks that share them
   unsigned long long tile_active;          // vertices of classes 0..2 swept
   unsigned long long tile_scanned;         // and their CSR entries
   int err;                      // ERRBIT_* (sticky for the call)

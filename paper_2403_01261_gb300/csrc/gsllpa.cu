@@ -47,10 +47,8 @@ struct gsl_ctx {
   long long cap_work2 = 0;
   int* lg = nullptr;                    // labels gathered per CSR entry (two-phase sweeps)
   long long cap_lg = 0;
-  unsigned long long* wtab = nullptr;   // warp-kernel fallback tables
-  long long cap_wtab = 0;
-  unsigned long long* btab = nullptr;   // block-kernel fallback tables
-  long long cap_btab = 0;
+  int* scratch = nullptr;               // label lists of rows longer than a block's registers
+  long long cap_scratch = 0;
   // class 9 in pieces (hub_kernels.cu)
   int* hub_piece_start = nullptr;
   long long* hub_ustart = nullptr;
@@ -300,15 +298,6 @@ int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s) {
   prof_resolve(c);
   if (int r = map_err(c, c->ctr_h->err, "offsets")) return r;
   const long long maxd = c->ctr_h->max_degree;
-  if (maxd > c->tune.warp_slots / 2 && maxd > 32) {
-    // a class-6 vertex may overflow its shared table: 2 * warp_max slots per warp
-    const long long need = warp_grid_warps(c->tune, c->di) * 2ll * c->tune.warp_max;
-    if (int r = grow(c, c->wtab, c->cap_wtab, need)) return r;
-  }
-  if (maxd > c->tune.warp_max) {
-    const long long need = block_grid_size(c->tune, c->di) * 2ll * maxd;
-    if (int r = grow(c, c->btab, c->cap_btab, need)) return r;
-  }
   // class 9 (hubs) in pieces: per-hub plan arrays and table regions
   const long long hubs = (long long)c->ctr_h->cls_total[CLS_HUB];
   const long long hub_e = (long long)c->ctr_h->hub_entries;
@@ -338,6 +327,22 @@ int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s) {
   return GSL_OK;
 }
 
+
+// Label lists for the rows of up to `longest` entries that one block sweeps.
+int ensure_scratch(gsl_ctx* c, long long longest, SweepArgs* a) {
+  a->scratch_region = longest > sketch_register_row() ? longest : 0;
+  if (a->scratch_region)
+    if (int r = grow(c, c->scratch, c->cap_scratch, sketch_blocks(c->di) * a->scratch_region)) return r;
+  a->scratch = c->scratch;
+  return GSL_OK;
+}
+
+// Longest row the block kernel sweeps: hubs go to their own kernels when the
+// plan for them is ready.
+long long longest_block_row(const gsl_ctx* c) {
+  const long long maxd = c->ctr_h->max_degree;
+  return c->hub_ready && maxd > c->tune.blk_max ? c->tune.blk_max : maxd;
+}
 
 int reset_sweep_counters(gsl_ctx* c, cudaStream_t s) {
   CK(cudaMemsetAsync(c->ctr, 0, offsetof(Counters, err), s));
@@ -379,10 +384,7 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
   a.ctr = c->ctr;
   a.probe_cap = c->tune.probe_cap;
   a.work = c->work;
-  a.wtab = c->wtab;
-  a.wtab_region = 2ll * c->tune.warp_max;
-  a.btab = c->btab;
-  a.btab_region = 2ll * c->ctr_h->max_degree;
+  if (int r = ensure_scratch(c, longest_block_row(c), &a)) return r;
   a.n = n;
   if (weights) {   // weighted degrees, written by sweep 1 for the early stops of later sweeps
     if (int r = grow(c, c->kw, c->cap_kw, n)) return r;
@@ -393,6 +395,7 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
   long long dn_prev = resume ? resume->dn_prev : n;
   long long scanned = resume ? resume->scanned : 0;
   bool binned_all = false;
+  const int maxd = (int)c->ctr_h->max_degree;
   while (t < max_iters && !converged) {
     ++t;
     if (int r = reset_sweep_counters(c, s)) return r;
@@ -438,9 +441,7 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
     }
     a.check = t == 1 ? 1 : 0;
     // the first sweep that gathers labels after the identity sweep sees
-    // almost as many distinct labels as neighbours (about 0.3 d on R-MAT
-    // hubs): hubs beyond three shared tables' worth go to global tables
-    a.gthresh = (t == 2 && !async_mode && !labels_init) ? 3 * c->tune.blk_slots : 0;
+    // almost as many distinct labels as neighbours (about 0.3 d on R-MAT hubs)
     a.spread = (t == 2 && !async_mode && !labels_init) ? 1 : 0;
     // Sweep 1 changes every vertex that has a neighbour, and a sweep after
     // one that changed more than half of the vertices is run on all
@@ -486,7 +487,7 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
         if (class_vertices(c, k, k) == 0) continue;
         const int pe = prof_begin(c, s);
         if (k == CLS_WARP_L || k == CLS_BLOCK || (k == CLS_WARP_S && filter_from == CLS_WARP_S)) {
-          CK(launch_sweep_class(af, k, weights != nullptr, async_mode, c->tune, c->di, s));
+          CK(launch_sweep_class(af, k, weights != nullptr, async_mode, c->tune, maxd, c->di, s));
           prof_end(c, pe, SL_SWEEP0 + k, s, 1);
         } else if (k == CLS_HUB && c->hub_ready) {
           HubPlan hp{c->hub_piece_start, c->hub_ustart, c->hub_best, c->hub_own,
@@ -496,7 +497,7 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
           CK(launch_hub_pieces(a, hp, weights != nullptr, async_mode, filter, c->tune, c->di, s, &kernels));
           prof_end(c, pe, SL_SWEEP0 + k, s, kernels);
         } else {
-          CK(launch_sweep_class(a, k, weights != nullptr, async_mode, c->tune, c->di, s));
+          CK(launch_sweep_class(a, k, weights != nullptr, async_mode, c->tune, maxd, c->di, s));
           prof_end(c, pe, SL_SWEEP0 + k, s, 1);
         }
       }
@@ -861,10 +862,8 @@ cudaError_t enqueue_batch_sweeps(gsl_ctx* c, const gsl_csr* g, int num_graphs, c
   a.ctr = c->ctr;
   a.probe_cap = c->tune.probe_cap;
   a.work = c->work;
-  a.wtab = c->wtab;
-  a.wtab_region = 2ll * c->tune.warp_max;
-  a.btab = c->btab;
-  a.btab_region = 2ll * c->ctr_h->max_degree;
+  a.scratch = c->scratch;   // allocated before the capture
+  a.scratch_region = c->ctr_h->max_degree;
   a.n = n;
   a.gid = c->gid;
   a.vptr = c->vptr;
@@ -884,7 +883,6 @@ cudaError_t enqueue_batch_sweeps(gsl_ctx* c, const gsl_csr* g, int num_graphs, c
     a.mark = t >= 2 ? 1 : 0;   // sweep 2 runs on all vertices, later ones on the marked frontier
     const bool filter = !a.ident && !a.check && (c->tune.majority == 2 || (c->tune.majority == 1 && t >= 3));
     const int filter_from = (filter && t >= BATCH_FILTER6_FROM) ? CLS_WARP_S : CLS_WARP_L;
-    a.gthresh = (t == 2 && !async_mode) ? 3 * c->tune.blk_slots : 0;
     a.spread = (t == 2 && !async_mode) ? 1 : 0;
     const int phases = async_mode ? 2 : 1;   // asynchronous sweeps in two phases, as in run_lpa
     for (int ph = 0; ph < phases; ++ph) {
@@ -906,7 +904,8 @@ cudaError_t enqueue_batch_sweeps(gsl_ctx* c, const gsl_csr* g, int num_graphs, c
         if (class_vertices(c, k, k) == 0) continue;
         pe = prof ? prof_begin(c, cs) : -1;
         const bool filtered = k == CLS_WARP_L || k == CLS_BLOCK || (k == CLS_WARP_S && filter_from == CLS_WARP_S);
-        ck(launch_sweep_class(filtered ? af : a, k, weights != nullptr, async_mode, c->tune, c->di, cs));
+        ck(launch_sweep_class(filtered ? af : a, k, weights != nullptr, async_mode, c->tune,
+                              (int)c->ctr_h->max_degree, c->di, cs));
         if (prof) prof_end(c, pe, SL_SWEEP0 + k, cs, 1);
       }
       if (class_vertices(c, 0, CLS_BINNED - 1) > 0) {
@@ -979,7 +978,7 @@ int gsl_ctx_destroy(gsl_ctx* c) {
   if (!c) return GSL_OK;
   DeviceGuard dg(c->device);
   void* dptrs[] = {c->lab[0], c->lab[1], c->flag[0], c->flag[1], c->work, c->parent, c->rank, c->sigma,
-                   c->block_sums, c->partials, c->wtab, c->btab, c->rowbits, c->lg, c->work2, c->fkeys, c->fvals, c->hub_piece_start,
+                   c->block_sums, c->partials, c->scratch, c->rowbits, c->lg, c->work2, c->fkeys, c->fvals, c->hub_piece_start,
                    c->hub_ustart, c->hub_best, c->hub_own, c->hub_wsum, c->hub_used_cnt, c->hub_clu, c->hub_used, c->hub_tab,
                    c->ctr, c->sums, c->k_dev,
                    c->st_off, c->st_col, c->st_w, c->st_lab, c->fix_w, c->fix_dev, c->kw};
@@ -1537,6 +1536,10 @@ int gsl_gsllpa_batch(gsl_ctx* c, const gsl_csr* g, int32_t num_graphs, const int
   CK(launch_fill_gid(c->vptr, num_graphs, n, c->gid, c->di, s));
   if (n > 0)
     if (int r = prepare_graph(c, g, s)) return r;
+  if (n > 0) {
+    SweepArgs lists{};
+    if (int r = ensure_scratch(c, c->ctr_h->max_degree, &lists)) return r;
+  }
   CK(cudaMemsetAsync(c->done, 0, (size_t)num_graphs, s));
   CK(cudaMemsetAsync(c->iters, 0, sizeof(int) * (size_t)num_graphs, s));
   CK(cudaMemsetAsync(c->stop, 0, sizeof(int), s));
@@ -1550,7 +1553,7 @@ int gsl_gsllpa_batch(gsl_ctx* c, const gsl_csr* g, int32_t num_graphs, const int
     if (n > 0 && class_vertices(c, k, k) > 0) populated |= 1ll << k;
   const std::vector<long long> key = {populated, (long long)OFF(g), (long long)g->cols, (long long)weights, n, g->nnz,
                                       num_graphs, max_iters, mode, (long long)(tol * 1e12), c->ctr_h->max_degree,
-                                      (long long)c->lab[0], (long long)c->wtab, (long long)c->btab,
+                                      (long long)c->lab[0], (long long)c->scratch,
                                       c->tune.warp_max, c->tune.blk_max, (long long)c->work2,
                                       c->tune.majority, c->tune.blk_block, c->tune.blk_slots, c->tune.probe_cap,
                                       c->tune.uf_cap};
@@ -1729,16 +1732,12 @@ int gsllpa_host_overlapped(gsl_ctx* c, int64_t n, int64_t nnz, const int64_t* of
   a.ctr = c->ctr;
   a.probe_cap = c->tune.probe_cap;
   a.work = c->work;
-  a.wtab = c->wtab;
-  a.wtab_region = 2ll * c->tune.warp_max;
-  a.btab = c->btab;
-  a.btab_region = 2ll * c->ctr_h->max_degree;
+  if (int r = ensure_scratch(c, longest_block_row(c), &a)) return r;
   a.n = n;
   a.prev = c->lab[1];
   a.next = c->lab[0];
   a.fnext = c->flag[1];
-  a.gthresh = 3 * c->tune.blk_slots;   // as run_lpa's sweep 2
-  a.spread = 1;
+  a.spread = 1;   // as run_lpa's sweep 2
   a.mark = 2 * dn1 <= n ? 1 : 0;
   const bool filter = c->tune.majority == 2;
   if (filter)
@@ -1762,14 +1761,14 @@ int gsllpa_host_overlapped(gsl_ctx* c, int64_t n, int64_t nnz, const int64_t* of
     for (int cls = NCLASS - 1; cls >= CLS_BINNED; --cls) {
       if (class_vertices(c, cls, cls) == 0) continue;
       if (cls == CLS_WARP_L || cls == CLS_BLOCK) {
-        CK(launch_sweep_class(af, cls, false, false, c->tune, c->di, s));
+        CK(launch_sweep_class(af, cls, false, false, c->tune, (int)c->ctr_h->max_degree, c->di, s));
       } else if (cls == CLS_HUB && c->hub_ready) {
         HubPlan hp{c->hub_piece_start, c->hub_ustart, c->hub_best, c->hub_own,
                    c->hub_wsum,        c->hub_used_cnt, c->hub_used, c->hub_tab, c->hub_clu};
         int kernels = 0;
         CK(launch_hub_pieces(a, hp, false, false, filter, c->tune, c->di, s, &kernels));
       } else {
-        CK(launch_sweep_class(a, cls, false, false, c->tune, c->di, s));
+        CK(launch_sweep_class(a, cls, false, false, c->tune, (int)c->ctr_h->max_degree, c->di, s));
       }
     }
   }

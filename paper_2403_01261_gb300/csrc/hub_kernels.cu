@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(512, 2) hub_piece_kernel(SweepArgs a, HubPlan 
     const unsigned want = 2u * (unsigned)len;
     const unsigned cap = want < tb ? want : tb;
     const SlotTable st = make_table(smem_h64, tb);
-    block_row<WEIGHTED, ASYNC, false>(a, v, own, cp, wp, lp, len, st, cap, 0xFFFFFFFFu, pol, sh, par);
+    block_row<WEIGHTED, ASYNC>(a, v, own, cp, wp, lp, len, st, cap, pol, sh, par);
     // the piece's (label, sum) pairs into the hub's global table
     unsigned long long* tab = hp.tab + 2 * hp.ustart[i];
     const unsigned gcap = (unsigned)(2 * d);
@@ -595,7 +595,7 @@ cudaError_t launch_hub_t(const SweepArgs& a, const HubPlan& hp, bool maj, const 
     if (e != cudaSuccess) return e;
     ++launches;
   }
-  hub_piece_kernel<W, A><<<(int)block_grid_size(t, di), t.blk_block, smem, s>>>(a, hp, (unsigned)t.blk_slots);
+  hub_piece_kernel<W, A><<<2 * di.sm_count, t.blk_block, smem, s>>>(a, hp, (unsigned)t.blk_slots);
   hub_final_kernel<A><<<2 * di.sm_count, 256, 0, s>>>(a, hp, W ? 1 : 0);
   count_launches(launches);
   *kernels = launches;

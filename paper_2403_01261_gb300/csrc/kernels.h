@@ -16,12 +16,9 @@ struct SweepArgs {
   unsigned char* fnext;      // frontier flags of the next sweep (set, never cleared here)
   const int* work;           // worklist (class regions at Counters::cls_start)
   Counters* ctr;
-  unsigned long long* wtab;  // global fallback tables of the warp kernel, one region per warp
-  long long wtab_region;     // slots per warp region (2 * warp_max)
-  unsigned long long* btab;  // global fallback tables of the block kernel, one region per block
-  long long btab_region;     // slots per block region (2 * largest degree of classes 7-8)
+  int* scratch;              // label lists of rows longer than a block's registers, one region per block
+  long long scratch_region;  // ints per region
   long long n;
-  int gthresh;               // hub degree above which the block kernel goes straight to global tables (0: never)
   // batched mode (many graphs packed in one CSR); all null for one graph
   const int* gid;            // graph of every vertex
   const long long* vptr;     // vertex range of every graph [vptr[g], vptr[g+1])
@@ -38,12 +35,10 @@ struct SweepArgs {
 };
 
 struct Tuning {
-  int warp_max = 1024;       // class 6 upper degree bound (one warp per vertex)
-  int blk_max = 32768;       // class 7 upper degree bound (one block per vertex; above: class 8)
-  int warp_slots = 1024;     // shared-memory table slots per warp of class 7 (8 bytes each)
-  int blk_slots = 12288;     // shared-memory table slots per block
-  int warp_block = 256;      // threads per block of the warp kernel
-  int blk_block = 512;       // threads per block of the block kernel
+  int warp_max = 1024;       // class 7 upper degree bound (a small block per row)
+  int blk_max = 32768;       // class 8 upper degree bound (a block per row; above: class 9)
+  int blk_slots = 12288;     // shared-memory table slots per block of the hub kernels
+  int blk_block = 512;       // threads per block of the hub-piece kernel
   int pregather = 0;         // two-phase sweeps: 0 never, 1 when the frontier is large, 2 always
   int majority = 1;          // own-label majority pass: 0 never, 1 once labels settle, 2 always
   int hub_cluster_max = 1 << 30;  // hubs up to this degree go to one thread-block cluster each (0: never)
@@ -85,8 +80,17 @@ cudaError_t launch_sweep_tile(const SweepArgs& a, int cls, bool weighted, bool a
                               cudaStream_t s);
 // Between the two phases of an asynchronous sweep (see Counters::phase_cls).
 cudaError_t launch_phase_reset(Counters* ctr, const int* stop, cudaStream_t s);
+// sketch_kernels.cu: the rows of class cls on the worklist, none longer than
+// `longest`.  Rows longer than
+// sketch_register_row() need SweepArgs::scratch, sketch_blocks() regions of
+// the longest row's length.  weights: 0 unit, 1 int32.
+long long sketch_blocks(const DeviceInfo& di);
+long long sketch_register_row();
+cudaError_t launch_sketch(const SweepArgs& a, int cls, int longest, int weights, bool async_mode,
+                          const DeviceInfo& di, cudaStream_t s);
+// Classes 3..9 on the worklist (class 9 as the block rows it then is).
 cudaError_t launch_sweep_class(const SweepArgs& a, int cls, bool weighted, bool async_mode, const Tuning& t,
-                               const DeviceInfo& di, cudaStream_t s);
+                               int longest, const DeviceInfo& di, cudaStream_t s);
 void count_launches(long long k);   // process-wide tally of kernels this library launched
 // Raises kernel fn's dynamic shared-memory limit to at least `bytes` (never
 // lowers it, so launches of other host threads with smaller tables stay
@@ -136,8 +140,6 @@ cudaError_t launch_ident_stream_f32(const long long* off, long long n, const int
                                     const DeviceInfo& di, cudaStream_t s);
 cudaError_t launch_init_labels(const int* init, int* a, int* b, long long n, Counters* ctr,
                                const DeviceInfo& di, cudaStream_t s);
-long long block_grid_size(const Tuning& t, const DeviceInfo& di);   // blocks of the class 8/9 kernel
-long long warp_grid_warps(const Tuning& t, const DeviceInfo& di);   // warps of the class 7 kernel
 ClassBounds class_bounds(const Tuning& t);
 
 // batch_kernels.cu

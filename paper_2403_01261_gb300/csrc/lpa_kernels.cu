@@ -9,15 +9,10 @@
 //
 // Work is split by degree class (binning pass below):
 //   d <= 32          one lane, half a warp or a warp per row (tile_kernels.cu).
-//   d <= warp_small  one warp per vertex, 4 KB shared table (never overflows).
-//   d <= warp_max    one warp per vertex, 8 KB shared table, global spill.
-//   d <= blk_max     one block per vertex, 96 KB shared table, global spill.
-//   larger           one block per vertex, straight to global tables when
-//                    labels are known to be mostly distinct.
-// The hash kernels never scan their table: every insert returns the new sum
-// of its label, each thread keeps the largest packed key it has produced,
-// and the final sum of every label is produced by the thread that added
-// last, so the maximum of those keys is the argmax.
+//   d <= warp_small  one warp per row      (sketch_kernels.cu)
+//   d <= warp_max    128 threads per row   (the same)
+//   d <= blk_max     256 threads per row   (the same)
+//   larger           thread-block clusters or pieces (hub_kernels.cu)
 //
 // Pruning (lpaMove(): a processed vertex is re-marked when a neighbour
 // changes): a vertex whose label changes sets the next-frontier flag of each
@@ -175,454 +170,6 @@ __global__ void init_labels_kernel(const int* __restrict__ init, int* __restrict
     a[v] = x;
     if (b) b[v] = x;
   }
-}
-
-// ---------------------------------------------------------------------------
-// Sweep 1 from the identity labelling on a row whose columns are strictly
-// increasing: every neighbour id is its own label and occurs once, so the
-// sum of label j is w_ij and the argmax is the max of (w_ij, ~j).  Returns
-// false if the row is not strictly increasing (the caller then hashes).
-// `best` is the per-thread partial key; `wsum` the per-thread weight sum.
-template <bool WEIGHTED>
-__device__ __forceinline__ bool ident_sorted_pass(const SweepArgs& a, int v, long long s, int d, int tid, int nthreads,
-                                                  const Pol& pol, unsigned long long& best, unsigned long long& wsum) {
-  bool sorted = true;
-  const int* cp = a.col + s;
-  const int* wp = a.w + s;
-  const int lane = tid & 31, wid = tid >> 5, nw = nthreads >> 5;
-  // each warp takes 128-entry rounds: four chunks in flight per lane
-  for (int e0 = wid * 128; e0 < d; e0 += nw * 128) {
-    int j[4], w[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) load_entry<WEIGHTED>(a, cp, wp, d, e0 + 32 * u + lane, pol, j[u], w[u]);
-    const int tail = (lane == 31 && e0 + 128 < d) ? ld_stream(cp + e0 + 128, pol.stream) : 0x7FFFFFFF;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int e = e0 + 32 * u + lane;
-      int nxt = __shfl_down_sync(FULL, j[u], 1);
-      const int head = u < 3 ? __shfl_sync(FULL, j[u < 3 ? u + 1 : u], 0) : tail;
-      if (lane == 31) nxt = head;
-      check_same_graph(a, v, j[u]);
-      if (j[u] >= 0 && e + 1 < d && !(j[u] < nxt)) sorted = false;
-      if (j[u] < 0 && e < d) sorted = false;      // invalid entry: let the hash path handle it
-      if (j[u] >= 0) {
-        wsum += (unsigned long long)w[u];
-        if (j[u] != v) {
-          const unsigned long long k = pack_key((unsigned)w[u], j[u]);
-          best = k > best ? k : best;
-        }
-      }
-    }
-  }
-  return sorted;
-}
-
-// ---------------------------------------------------------------------------
-
-// Rows of 33..SORT_MAX entries, unit weights: one warp sorts the row's
-// labels in registers instead of hashing them.  Lane l holds entries
-// r * 32 + l (r < SORT_K); a bitonic network (shuffles for partners in other
-// lanes, in-register steps for partners r ^ (j / 32)) sorts the keys
-// ascending, with absent entries (past the row end, out of range, the vertex
-// itself) as 0xFFFFFFFF at the end.  Equal labels then form runs: a run's
-// length is the label's count, and the largest packed key (count, ~label)
-// over the run starts is Eq. 2's argmax with ties to the smallest label, the
-// same as the table's.  No shared memory, no atomics.  Returns the lane's
-// partial key (0: none).
-constexpr int SORT_K = 2;
-constexpr int SORT_MAX = 32 * SORT_K;
-
-template <bool ASYNC>
-__device__ __forceinline__ unsigned long long warp_sort_row(const SweepArgs& a, int v, const int* cp, const int* lp,
-                                                            int d, const Pol& pol) {
-  constexpr int N = 32 * SORT_K;
-  const int lane = threadIdx.x & 31;
-  unsigned x[SORT_K];
-#pragma unroll
-  for (int r = 0; r < SORT_K; ++r) {
-    int j, wt;
-    load_entry<false>(a, cp, nullptr, d, r * 32 + lane, pol, j, wt);
-    check_same_graph(a, v, j);
-    const int l = entry_label<ASYNC>(a, lp, r * 32 + lane, j, v, pol);
-    x[r] = l >= 0 ? (unsigned)l : 0xFFFFFFFFu;
-  }
-#pragma unroll
-  for (int k = 2; k <= N; k <<= 1) {
-#pragma unroll
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      if (j >= 32) {   // partner r ^ (j / 32): the same lane's other keys
-#pragma unroll
-        for (int r = 0; r < SORT_K; ++r) {
-          const int h = r ^ (j >> 5);
-          if (r < h) {
-            const bool ascending = (((r * 32 + lane) & k) == 0);
-            const unsigned lo = min(x[r], x[h]), hi = max(x[r], x[h]);
-            x[r] = ascending ? lo : hi;
-            x[h] = ascending ? hi : lo;
-          }
-        }
-      } else {
-#pragma unroll
-        for (int r = 0; r < SORT_K; ++r) {
-          const unsigned y = __shfl_xor_sync(FULL, x[r], j);
-          const bool ascending = (((r * 32 + lane) & k) == 0);
-          const bool keep_min = ((lane & j) == 0) == ascending;
-          x[r] = keep_min ? min(x[r], y) : max(x[r], y);
-        }
-      }
-    }
-  }
-  // run starts: key i differs from key i - 1
-  unsigned w[SORT_K];
-  bool st[SORT_K];
-#pragma unroll
-  for (int r = 0; r < SORT_K; ++r) {
-    unsigned p = __shfl_up_sync(FULL, x[r], 1);
-    const unsigned last = __shfl_sync(FULL, x[r > 0 ? r - 1 : 0], 31);
-    if (lane == 0 && r > 0) p = last;
-    st[r] = (lane == 0 && r == 0) || x[r] != p;
-    w[r] = __ballot_sync(FULL, st[r]);
-  }
-  unsigned long long best = 0;
-#pragma unroll
-  for (int r = 0; r < SORT_K; ++r) {
-    if (st[r] && x[r] != 0xFFFFFFFFu) {
-      const unsigned above = lane < 31 ? w[r] & ~((2u << lane) - 1u) : 0u;
-      int next = N;
-      if (above) {
-        next = r * 32 + __ffs((int)above) - 1;
-      } else {
-#pragma unroll
-        for (int q = SORT_K - 1; q > r; --q)
-          if (w[q]) next = q * 32 + __ffs((int)w[q]) - 1;
-      }
-      const unsigned long long key = pack_key((unsigned)(next - (r * 32 + lane)), (int)x[r]);
-      best = key > best ? key : best;
-    }
-  }
-  return best;
-}
-
-// One warp aggregates the row (cp, wp, d) of vertex v into `tab` (cap
-// slots).  Four 32-entry chunks are loaded (columns, then labels) before any
-// is hashed, so each lane keeps eight loads in flight.  Within a chunk equal
-// labels are merged with __match_any_sync (label_group) and only the lowest
-// lane of each group inserts.  Returns true (warp-uniform) once more than `limit`
-// distinct labels have been inserted: the table is then abandoned.
-template <bool WEIGHTED, bool ASYNC, bool GLOBAL, bool SPREAD = false, bool LEAN_OK = false>
-__device__ __forceinline__ bool warp_row(const SweepArgs& a, int v, int own, const int* cp, const int* wp,
-                                         const int* lp, int d,
-                                         SlotTable tab, unsigned cap, unsigned limit, const Pol& pol,
-                                         unsigned long long& best, unsigned long long& wsum, unsigned& own_sum) {
-  const int lane = threadIdx.x & 31;
-  // three rounds in flight: labels of round r+1 and columns of round r+2
-  // are requested before round r is hashed
-  int jn[4], wn[4], ln[4], lw[4];
-  // sweep 2's lean loads (sweep_device.cuh) in classes 6 and 7 (class 6:
-  // 9.1 -> 8.5 ms per step on R-MAT 25); the compare-and-swap-first insert
-  // in class 7 only (on class 6's short rows it measured 9.2 -> 9.5 ms)
-  constexpr bool LEAN = SPREAD && !WEIGHTED;
-  constexpr bool LEAN_CAS = LEAN && LEAN_OK;
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    if (LEAN) {
-      jn[u] = spread_col(a, cp, d, 32 * u + lane, pol);
-      wn[u] = 1;
-    } else {
-      load_entry<WEIGHTED>(a, cp, wp, d, 32 * u + lane, pol, jn[u], wn[u]);
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    if (!LEAN) check_same_graph(a, v, jn[u]);
-    if (jn[u] >= 0) wsum += (unsigned long long)wn[u];
-    ln[u] = LEAN ? spread_label(a, jn[u], v, pol) : entry_label<ASYNC>(a, lp, 32 * u + lane, jn[u], v, pol);
-    lw[u] = wn[u];
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    if (LEAN) {
-      jn[u] = spread_col(a, cp, d, 128 + 32 * u + lane, pol);
-      wn[u] = 1;
-    } else {
-      load_entry<WEIGHTED>(a, cp, wp, d, 128 + 32 * u + lane, pol, jn[u], wn[u]);
-    }
-  }
-  for (unsigned k = lane; k < cap; k += 32) {
-    tab.keys[k] = EMPTY32;
-    tab.sums[k] = 0;
-  }
-  __syncwarp();
-  unsigned used = 0;
-  for (int e0 = 0; e0 < d; e0 += 128) {
-    int l[4], w[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      l[u] = ln[u];
-      w[u] = lw[u];
-    }
-    if (e0 + 128 < d) {   // warp-uniform
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (!LEAN) check_same_graph(a, v, jn[u]);
-        if (jn[u] >= 0) wsum += (unsigned long long)wn[u];
-        ln[u] = LEAN ? spread_label(a, jn[u], v, pol)
-                     : entry_label<ASYNC>(a, lp, e0 + 128 + 32 * u + lane, jn[u], v, pol);
-        lw[u] = wn[u];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (LEAN) {
-          jn[u] = spread_col(a, cp, d, e0 + 256 + 32 * u + lane, pol);
-          wn[u] = 1;
-        } else {
-          load_entry<WEIGHTED>(a, cp, wp, d, e0 + 256 + 32 * u + lane, pol, jn[u], wn[u]);
-        }
-      }
-    }
-    if (!WEIGHTED && !SPREAD) {
-      // entries carrying the vertex's own label are counted in registers,
-      // the round's four chunks first: once they are more than half of the
-      // row's d entries no other label can reach their count, and the rest
-      // of the row is not needed (after sweep 1, which reads every entry)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (e0 + 32 * u < d) {   // warp-uniform: skip empty chunks of short rows
-          const bool mine = l[u] == own;
-          own_sum += (unsigned)__popc(__ballot_sync(FULL, mine));
-          if (mine) l[u] = -1;
-        }
-      }
-      if (!a.check && 2u * own_sum > (unsigned)d) return false;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (e0 + 32 * u < d) {   // warp-uniform: skip empty chunks of short rows
-        if (WEIGHTED && !SPREAD) {   // own-label weights summed in registers
-          const bool mine = l[u] == own;
-          own_sum += __reduce_add_sync(FULL, mine ? (unsigned)w[u] : 0u);
-          if (mine) l[u] = -1;
-        }
-        if (__ballot_sync(FULL, l[u] >= 0) == 0) continue;
-        const unsigned m = SPREAD ? 1u << lane : label_group(l[u], a.spread);
-        const unsigned c = SPREAD ? (WEIGHTED ? (unsigned)w[u] : 1u)
-                                  : (WEIGHTED ? __reduce_add_sync(m, (unsigned)w[u]) : (unsigned)__popc(m));
-        bool created = false;
-        if (l[u] >= 0 && (SPREAD || (m & lanemask_lt()) == 0)) {
-          const unsigned sum = (LEAN_CAS && !GLOBAL)
-                                   ? slot_add_cas(tab, cap, (unsigned)l[u], c, created, &a.ctr->err, a.probe_cap)
-                                   : slot_add<GLOBAL>(tab, cap, (unsigned)l[u], c, created, &a.ctr->err, a.probe_cap);
-          const unsigned long long k = pack_key(sum, l[u]);
-          best = k > best ? k : best;
-        }
-        if (limit != 0xFFFFFFFFu) used += __popc(__ballot_sync(FULL, created));
-      }
-    }
-    if (used > limit) return true;   // at most 128 slots past the limit
-  }
-  return false;
-}
-
-// Classes 6 and 7: one warp per vertex, TW slots of shared memory per warp
-// (class 6: four 256-thread blocks per SM, registers capped to fit; class
-// 7's 8 KB tables allow three).
-// With SPILL, a vertex whose labels overflow the shared table is redone in
-// the warp's region of the global fallback tables (2 * warp_max slots);
-// without it the class bound guarantees 2 d <= TW.  The worklist entry of
-// the row after next and the offsets of the next row are loaded while the
-// current one is processed.
-template <bool WEIGHTED, bool ASYNC, int TW, bool SPILL, bool SPREAD = false>
-__global__ void __launch_bounds__(256, TW <= 512 ? 4 : 3) sweep_warp_kernel(SweepArgs a, int cls) {
-  if (stopped(a)) return;
-  extern __shared__ unsigned long long smem_w64[];
-  const int lane = threadIdx.x & 31;
-  const SlotTable tab = make_table(smem_w64 + (size_t)(threadIdx.x >> 5) * TW, TW);
-  const long long warp_id = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  const SlotTable gtab = SPILL ? make_table(a.wtab + warp_id * a.wtab_region, a.wtab_region) : SlotTable{nullptr, nullptr};
-  const unsigned cnt = a.ctr->cls_count[cls];
-  const int* __restrict__ work = a.work + a.ctr->cls_start[cls];
-  const Pol pol = make_pol();
-  unsigned long long my_dn = 0, my_scan = 0;
-  long long item = warp_id;
-  int vn = 0, vnn = 0;
-  long long sn = 0, en = 0;
-  if (item < (long long)cnt) {
-    vn = work[item];
-    sn = a.off[vn];
-    en = a.off[vn + 1];
-  }
-  if (item + nwarps < (long long)cnt) vnn = work[item + nwarps];
-  while (item < (long long)cnt) {
-    const int v = vn;
-    const long long s = sn;
-    const int d = (int)(en - sn);
-    const long long next_item = item + nwarps;
-    if (next_item < (long long)cnt) {   // its worklist entry came one row earlier
-      vn = vnn;
-      sn = a.off[vn];
-      en = a.off[vn + 1];
-    }
-    if (next_item + nwarps < (long long)cnt) vnn = work[next_item + nwarps];
-    const int old = own_label<ASYNC>(a, v);
-    const int* cp = a.col + s;
-    const int* wp = a.w + s;
-    unsigned long long best = 0, wsum = 0;
-    bool done = false;
-    if (a.ident && !ASYNC) done = __all_sync(FULL, ident_sorted_pass<WEIGHTED>(a, v, s, d, lane, 32, pol, best, wsum));
-    if (!done && !WEIGHTED && d <= SORT_MAX) {   // warp-uniform
-      best = warp_sort_row<ASYNC>(a, v, cp, a.lg ? a.lg + s : nullptr, d, pol);
-      done = true;
-    }
-    if (!done) {
-      best = 0;
-      wsum = 0;
-      const unsigned want = 2u * (unsigned)d;
-      const unsigned cap = want < (unsigned)TW ? want : (unsigned)TW;
-      const unsigned limit = (!SPILL || cap >= want) ? 0xFFFFFFFFu : cap / 4 * 3 - 128;
-      unsigned own_sum = 0;
-      const int* lp = a.lg ? a.lg + s : nullptr;
-      if (warp_row<WEIGHTED, ASYNC, false, SPREAD, SPILL>(a, v, old, cp, wp, lp, d, tab, cap, limit, pol, best, wsum,
-                                                          own_sum) &&
-          SPILL) {
-        best = 0;
-        wsum = 0;
-        own_sum = 0;
-        warp_row<WEIGHTED, ASYNC, true, SPREAD, SPILL>(a, v, old, cp, wp, lp, d, gtab, want, 0xFFFFFFFFu, pol, best,
-                                                       wsum, own_sum);
-      }
-      __syncwarp();
-      if (own_sum) {   // own_sum is warp-uniform
-        const unsigned long long k = pack_key(own_sum, old);
-        best = k > best ? k : best;
-      }
-    }
-    best = warp_max_u64(best);
-    if (WEIGHTED && a.check) {
-      wsum = warp_sum_u64(wsum);
-      if (lane == 0 && wsum >= (1ull << 31)) raise_err(&a.ctr->err, ERRBIT_OVERFLOW);
-      if (lane == 0 && a.kw) a.kw[v] = wsum < (1ull << 32) ? (unsigned)wsum : ~0u;
-    }
-    const int nl = best ? (int)~(unsigned)best : old;
-    const bool changed = nl != old;
-    if (lane == 0) {
-      store_label<ASYNC>(a, v, nl, changed);
-      if (changed) count_graph_change(a, v);
-      my_scan += (unsigned long long)d;
-      my_dn += changed ? 1ull : 0ull;
-    }
-    if (changed && a.mark) {
-      for (int e = lane; e < d; e += 32) {
-        const int j = ld_stream(cp + e, pol.stream);
-        if ((unsigned)j < (unsigned)a.n) a.fnext[j] = 1;
-      }
-      if (!ASYNC && lane == 0) a.fnext[v] = 1;
-    }
-    item = next_item;
-  }
-  flush_counters(a.ctr, cls, my_dn, my_scan);
-}
-
-// Classes 8 and 9: one block per vertex, `tb` slots of shared memory; a
-// vertex whose labels overflow it (or, when gthresh > 0, whose degree
-// exceeds gthresh) is aggregated in the block's region of the global
-// fallback tables instead (a.btab_region slots).  Two barriers per row: one
-// after the table is cleared, one after the partial results are published.
-// The worklist entry of the row after next and the offsets and own label
-// of the next row are loaded while the current row is processed.
-template <bool WEIGHTED, bool ASYNC, bool SPREAD = false>
-__global__ void __launch_bounds__(512, 2) sweep_block_kernel(SweepArgs a, int cls, unsigned tb, int gthresh) {
-  if (stopped(a)) return;
-  extern __shared__ unsigned long long smem_b64[];
-  __shared__ BlockRowShared sh;
-  const SlotTable gtab = make_table(a.btab + (long long)blockIdx.x * a.btab_region, a.btab_region);
-  const SlotTable stab = make_table(smem_b64, tb);
-  const unsigned cnt = a.ctr->cls_count[cls];
-  const int* __restrict__ work = a.work + a.ctr->cls_start[cls];
-  const Pol pol = make_pol();
-  const long long G = gridDim.x;
-  unsigned long long my_dn = 0, my_scan = 0;
-  long long item = blockIdx.x;
-  int v = 0, old = 0, v1 = 0;
-  long long s = 0, e = 0;
-  if (item < (long long)cnt) {
-    v = work[item];
-    s = a.off[v];
-    e = a.off[v + 1];
-    old = own_label<ASYNC>(a, v);
-  }
-  if (item + G < (long long)cnt) v1 = work[item + G];
-  for (int par = 0; item < (long long)cnt; item += G, par ^= 1) {
-    long long s1 = 0, e1 = 0;
-    int old1 = 0, v2 = 0;
-    if (item + G < (long long)cnt) {
-      s1 = a.off[v1];
-      e1 = a.off[v1 + 1];
-      old1 = own_label<ASYNC>(a, v1);
-    }
-    if (item + 2 * G < (long long)cnt) v2 = work[item + 2 * G];
-    const int d = (int)(e - s);
-    const int* cp = a.col + s;
-    const int* wp = a.w + s;
-    const int* lp = a.lg ? a.lg + s : nullptr;
-    int sorted = 0;
-    if (a.ident && !ASYNC) {
-      unsigned long long best = 0, wsum = 0;
-      if (threadIdx.x == 0) {
-        sh.best[par] = 0;
-        sh.wsum[par] = 0;
-        sh.own[par] = 0;
-      }
-      sorted = __syncthreads_and(ident_sorted_pass<WEIGHTED>(a, v, s, d, threadIdx.x, blockDim.x, pol, best, wsum));
-      if (sorted) {
-        block_publish<WEIGHTED>(a, sh, par, best, wsum, 0u);
-        __syncthreads();
-      }
-    }
-    if (!sorted) {
-      const unsigned want = 2u * (unsigned)d;
-      int ovf = 1;
-      if (!(gthresh > 0 && d > gthresh)) {
-        const unsigned cap = want < tb ? want : tb;
-        // each warp may add up to 128 new slots (one round) after the flag is
-        // raised: at most 4 * threads, within the last quarter of a table of
-        // at least 16 * threads slots
-        const unsigned limit = cap >= want ? 0xFFFFFFFFu : cap / 4 * 3;
-        ovf = block_row<WEIGHTED, ASYNC, false, SPREAD>(a, v, old, cp, wp, lp, d, stab, cap, limit, pol, sh, par);
-      }
-      if (ovf)
-        block_row<WEIGHTED, ASYNC, true, SPREAD>(a, v, old, cp, wp, lp, d, gtab, want, 0xFFFFFFFFu, pol, sh, par);
-    }
-    unsigned long long b = sh.best[par];
-    const unsigned own_sum = sh.own[par];
-    if (own_sum) {
-      const unsigned long long k = pack_key(own_sum, old);
-      b = k > b ? k : b;
-    }
-    const int nl = b ? (int)~(unsigned)b : old;
-    const bool changed = nl != old;
-    if (threadIdx.x == 0) {
-      if (WEIGHTED && a.check && sh.wsum[par] >= (1ull << 31)) raise_err(&a.ctr->err, ERRBIT_OVERFLOW);
-      if (WEIGHTED && a.check && a.kw) a.kw[v] = sh.wsum[par] < (1ull << 32) ? (unsigned)sh.wsum[par] : ~0u;
-      store_label<ASYNC>(a, v, nl, changed);
-      if (changed) count_graph_change(a, v);
-      my_scan += (unsigned long long)d;
-      my_dn += changed ? 1ull : 0ull;
-    }
-    if (changed && a.mark) {   // block-uniform
-      for (int x = threadIdx.x; x < d; x += blockDim.x) {
-        const int j = ld_stream(cp + x, pol.stream);
-        if ((unsigned)j < (unsigned)a.n) a.fnext[j] = 1;
-      }
-      if (!ASYNC && threadIdx.x == 0) a.fnext[v] = 1;
-    }
-    v = v1;
-    s = s1;
-    e = e1;
-    old = old1;
-    v1 = v2;
-  }
-  flush_counters(a.ctr, cls, my_dn, my_scan);
 }
 
 // ---------------------------------------------------------------------------
@@ -1051,73 +598,16 @@ cudaError_t launch_bin_range(const long long* off, long long v0, long long v1, c
 namespace {
 std::atomic<long long> g_launches{0};
 
-template <typename K>
-int occupancy_grid(K kernel, int block, size_t smem, const DeviceInfo& di) {
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem);
-  cudaGetLastError();
-  if (per_sm < 1) per_sm = 1;
-  return per_sm * di.sm_count;
-}
-
-constexpr int TW_SMALL = 512;    // slots per warp, class 6 (2 d <= 512)
-constexpr int TW_LARGE = 1024;   // slots per warp, class 7
-
-// One warp per row (classes 6 and 7); the grid is sized once per host
-// thread and instantiation from the kernel's occupancy.  With SPILL every
-// warp owns one region of the global fallback tables, which are sized for
-// warp_grid_warps warps: the grid never exceeds that.
-template <bool W, bool A, int TW, bool SPILL, bool SPREAD>
-void launch_warp_class(const SweepArgs& a, int cls, const Tuning& t, const DeviceInfo& di, cudaStream_t s) {
-  const size_t smem = (size_t)(t.warp_block / 32) * TW * sizeof(unsigned long long);
-  thread_local int grid = 0;
-  if (!grid) {
-    raise_smem_limit((const void*)sweep_warp_kernel<W, A, TW, SPILL, SPREAD>, smem);
-    grid = occupancy_grid(sweep_warp_kernel<W, A, TW, SPILL, SPREAD>, t.warp_block, smem, di);
-    if (SPILL) {
-      const long long cap = warp_grid_warps(t, di) / (t.warp_block / 32);
-      if (grid > cap) grid = (int)(cap > 0 ? cap : 1);
-    }
-  }
-  sweep_warp_kernel<W, A, TW, SPILL, SPREAD><<<grid, t.warp_block, smem, s>>>(a, cls);
-}
-
-template <bool W, bool A>
-cudaError_t launch_sweep_t(const SweepArgs& a, int cls, const Tuning& t, const DeviceInfo& di, cudaStream_t s) {
-  switch (cls) {
-    case 3:
-    case 4:
-    case 5:
-      return launch_sweep_tile(a, cls, W, A, di, s);
-    case CLS_WARP_S:
-      if (!A && a.spread && !a.lg) launch_warp_class<W, A, TW_SMALL, false, true>(a, CLS_WARP_S, t, di, s);
-      else launch_warp_class<W, A, TW_SMALL, false, false>(a, CLS_WARP_S, t, di, s);
-      break;
-    case CLS_WARP_L:
-      if (!A && a.spread && !a.lg) launch_warp_class<W, A, TW_LARGE, true, true>(a, CLS_WARP_L, t, di, s);
-      else launch_warp_class<W, A, TW_LARGE, true, false>(a, CLS_WARP_L, t, di, s);
-      break;
-    case CLS_BLOCK:
-    case CLS_HUB: {
-      const size_t smem = (size_t)t.blk_slots * sizeof(unsigned long long);
-      const int grid = (int)block_grid_size(t, di);
-      const int gth = cls == CLS_HUB ? a.gthresh : 0;
-      if (!A && a.spread && !a.lg) {
-        raise_smem_limit((const void*)sweep_block_kernel<W, A, true>, smem);
-        sweep_block_kernel<W, A, true><<<grid, t.blk_block, smem, s>>>(a, cls, (unsigned)t.blk_slots, gth);
-      } else {
-        raise_smem_limit((const void*)sweep_block_kernel<W, A, false>, smem);
-        sweep_block_kernel<W, A, false><<<grid, t.blk_block, smem, s>>>(a, cls, (unsigned)t.blk_slots, gth);
-      }
-      break;
-    }
-    default:
-      return cudaErrorInvalidValue;
-  }
-  count_launches(1);
-  return cudaGetLastError();
-}
+constexpr int WARP_SMALL = 256;   // longest row of one warp (class 6)
 }  // namespace
+
+cudaError_t launch_sweep_class(const SweepArgs& a, int cls, bool weighted, bool async_mode, const Tuning& t,
+                               int longest, const DeviceInfo& di, cudaStream_t s) {
+  if (cls < CLS_WARP_S) return launch_sweep_tile(a, cls, weighted, async_mode, di, s);
+  const ClassBounds cb = class_bounds(t);
+  const int bound = cls == CLS_WARP_S ? cb.warp_small : (cls == CLS_WARP_L ? cb.warp_max : (cls == CLS_BLOCK ? cb.blk_max : longest));
+  return launch_sketch(a, cls, bound < longest ? bound : longest, weighted ? 1 : 0, async_mode, di, s);
+}
 
 void count_launches(long long k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 
@@ -1133,38 +623,10 @@ cudaError_t raise_smem_limit(const void* fn, size_t bytes) {
 }
 long long launches_total() { return g_launches.load(std::memory_order_relaxed); }
 
-long long block_grid_size(const Tuning& t, const DeviceInfo& di) {
-  // per host thread: contexts with different block shapes may run on several threads at once
-  thread_local long long cached = 0;
-  thread_local int cached_slots = 0, cached_block = 0;
-  if (cached && cached_slots == t.blk_slots && cached_block == t.blk_block) return cached;
-  int per_sm = 0;
-  const size_t smem = (size_t)t.blk_slots * sizeof(unsigned long long);
-  raise_smem_limit((const void*)sweep_block_kernel<false, false>, smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_block_kernel<false, false>, t.blk_block, smem);
-  cudaGetLastError();
-  if (per_sm < 1) per_sm = 1;
-  cached = (long long)per_sm * di.sm_count;
-  cached_slots = t.blk_slots;
-  cached_block = t.blk_block;
-  return cached;
-}
-
-long long warp_grid_warps(const Tuning& t, const DeviceInfo& di) {
-  int per_sm = 0;
-  const size_t smem = (size_t)(t.warp_block / 32) * TW_LARGE * sizeof(unsigned long long);
-  raise_smem_limit((const void*)sweep_warp_kernel<false, false, TW_LARGE, true>, smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_warp_kernel<false, false, TW_LARGE, true>,
-                                                t.warp_block, smem);
-  cudaGetLastError();
-  if (per_sm < 1) per_sm = 1;
-  return (long long)per_sm * di.sm_count * (t.warp_block / 32);
-}
-
 ClassBounds class_bounds(const Tuning& t) {
   ClassBounds cb;
   cb.warp_max = t.warp_max;
-  cb.warp_small = TW_SMALL / 2 < t.warp_max ? TW_SMALL / 2 : t.warp_max;
+  cb.warp_small = WARP_SMALL < t.warp_max ? WARP_SMALL : t.warp_max;
   cb.blk_max = t.blk_max;
   return cb;
 }
@@ -1220,6 +682,7 @@ __global__ void phase_reset_kernel(Counters* ctr, const int* stop) {
     ctr->phase_cls[k] += ctr->cls_count[k];
     ctr->cls_count[k] = 0;
     ctr->uns_count[k] = 0;
+    ctr->row_next[k] = 0;
   }
   ctr->hub_pieces = 0;
   ctr->hub_clusters = 0;
@@ -1240,13 +703,6 @@ cudaError_t launch_init_labels(const int* init, int* a, int* b, long long n, Cou
   init_labels_kernel<<<(int)(blocks < cap ? blocks : cap), 256, 0, s>>>(init, a, b, n, ctr);
   count_launches(1);
   return cudaGetLastError();
-}
-
-cudaError_t launch_sweep_class(const SweepArgs& a, int cls, bool weighted, bool async_mode, const Tuning& t,
-                               const DeviceInfo& di, cudaStream_t s) {
-  if (weighted)
-    return async_mode ? launch_sweep_t<true, true>(a, cls, t, di, s) : launch_sweep_t<true, false>(a, cls, t, di, s);
-  return async_mode ? launch_sweep_t<false, true>(a, cls, t, di, s) : launch_sweep_t<false, false>(a, cls, t, di, s);
 }
 
 }  // namespace gsl

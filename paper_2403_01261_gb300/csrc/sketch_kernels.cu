@@ -1,0 +1,610 @@
+// sketch_kernels.cu -- the sweep for rows of more than 32 entries (classes
+// 6..8, and class 9 where the hub kernels do not take it).
+//
+// A team (one warp, or a block of 128 or 256 threads) takes a row, keeps its
+// neighbours' labels in registers and adds every entry's weight to the
+// counter its label hashes to.  The adds return running sums, so the largest
+// (sum, smallest label) over the team names the fullest counter and a label
+// in it.  When no other label of the row lies in that counter, its sum is
+// that label's and no other label can reach it (its own counter is no fuller,
+// and a counter as full gives a larger label or is shared): one round, no
+// probing, no compare-and-swap, no match.  Otherwise the named label is summed
+// exactly, labels whose counters cannot beat it drop out, and the rest is
+// settled in rounds that also leave a label per slot (sketch_rounds): slots
+// that end up with one label hold its exact sum.
+//
+// Rows longer than the registers hold (4096 entries) keep their labels in a
+// scratch list of the block; if more of them stay open than the table has
+// slots, the list is counted in parts by a second hash.
+//
+// Bound by instruction issue and the label gathers: the hash tables before
+// spent 150 to 210 warp instructions per 32 entries (compare-and-swap 5
+// cycles of an SM, match up to 64, a counter add 2.6).
+#include "sweep_device.cuh"
+
+namespace gsl {
+
+namespace {
+
+constexpr unsigned SETTLED = 0x80000000u;   // label bit: no longer in question (absent entries are -1)
+
+template <int WT>
+struct SumOf { using T = unsigned; };
+template <>
+struct SumOf<2> { using T = unsigned long long; };
+
+// Best label so far: largest sum, then smallest label (inv = ~label).
+template <typename S>
+struct Best {
+  S sum;
+  unsigned inv;
+};
+
+template <typename S>
+__device__ __forceinline__ bool beats(S s, unsigned inv, const Best<S>& b) {
+  return s > b.sum || (s == b.sum && inv > b.inv);
+}
+
+__device__ __forceinline__ Best<unsigned> warp_best(Best<unsigned> b) {
+  const unsigned m = __reduce_max_sync(FULL, b.sum);
+  return {m, __reduce_max_sync(FULL, b.sum == m ? b.inv : 0u)};
+}
+__device__ __forceinline__ Best<unsigned long long> warp_best(Best<unsigned long long> b) {
+  const unsigned hi = __reduce_max_sync(FULL, (unsigned)(b.sum >> 32));
+  const bool h = (unsigned)(b.sum >> 32) == hi;
+  const unsigned lo = __reduce_max_sync(FULL, h ? (unsigned)b.sum : 0u);
+  const unsigned inv = __reduce_max_sync(FULL, (h && (unsigned)b.sum == lo) ? b.inv : 0u);
+  return {((unsigned long long)hi << 32) | lo, inv};
+}
+
+__device__ __forceinline__ unsigned ceil_log2(unsigned x) { return x <= 1 ? 0u : 32u - (unsigned)__clz((int)(x - 1)); }
+
+template <int T>
+__device__ __forceinline__ void team_sync() {
+  if (T == 32) __syncwarp();
+  else __syncthreads();
+}
+template <int T>
+__device__ __forceinline__ bool team_any(bool p) {
+  if (T != 32) return __syncthreads_or(p) != 0;
+  __syncwarp();
+  return __any_sync(FULL, p);
+}
+
+// What a team shares besides its table.
+template <int T, typename S>
+struct TeamShared {
+  S sum[T / 32];
+  unsigned inv[T / 32];
+  unsigned long long wsum;
+  unsigned cnt;
+  long long next;
+};
+
+template <int T, typename S>
+__device__ __forceinline__ Best<S> team_best(Best<S> b, TeamShared<T, S>* sh) {
+  b = warp_best(b);
+  if (T == 32) return b;
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) {
+    sh->sum[threadIdx.x >> 5] = b.sum;
+    sh->inv[threadIdx.x >> 5] = b.inv;
+  }
+  __syncthreads();
+  b = {0, 0u};
+  if (lane < T / 32) b = {sh->sum[lane], sh->inv[lane]};
+  return warp_best(b);   // the next barrier comes before sh is written again
+}
+
+// The table's memory holds 1 << lg counters of the counting round, or half
+// as many slots of (sum, label) in the rounds after it.
+template <typename S>
+struct Sketch {
+  S* sum;
+  unsigned lg;
+  __device__ __forceinline__ unsigned slot(unsigned label) const { return sketch_hash(label, 0) >> (32u - lg); }
+};
+template <typename S>
+struct Slots {
+  S* sum;
+  unsigned* lab;
+  unsigned lg;
+  __device__ __forceinline__ explicit Slots(const Sketch<S>& t)
+      : sum(t.sum), lab(reinterpret_cast<unsigned*>(t.sum + (1u << (t.lg - 1)))), lg(t.lg - 1) {}
+  __device__ __forceinline__ unsigned slot(unsigned label, int round) const {
+    return sketch_hash(label, round) >> (32u - lg);
+  }
+};
+
+template <int T, typename S>
+__device__ __forceinline__ void sketch_clear(S* sum, unsigned lg, int tid) {
+  constexpr unsigned PER = 16 / sizeof(S);   // at least 64 counters: whole 16-byte words
+  int4* p = reinterpret_cast<int4*>(sum);
+#pragma unroll 4
+  for (unsigned k = tid; k < (1u << lg) / PER; k += T) p[k] = make_int4(0, 0, 0, 0);
+}
+
+// Labels of a row in registers: entry k * T + tid in l[k].
+template <int T, int K>
+struct RegItems {
+  int (&l)[K];
+  int d, tid;
+  template <typename F>
+  __device__ __forceinline__ void each(F&& f) {
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (k * T < d) f(l[k], k * T + tid);   // team-uniform; absent entries are -1
+  }
+};
+
+// Labels of a row in the block's scratch list.
+template <int T>
+struct MemItems {
+  int* list;
+  int d, tid;
+  template <typename F>
+  __device__ __forceinline__ void each(F&& f) {
+#pragma unroll 4
+    for (int e = tid; e < d; e += T) {
+      const int was = list[e];
+      int l = was;
+      f(l, e);
+      if (l != was) list[e] = l;
+    }
+  }
+};
+
+// Sum of label x over the items not settled, for the whole team.
+template <int T, int WT, typename S, typename Items>
+__device__ __forceinline__ S team_sum_of(Items& items, const int* wp, unsigned x, TeamShared<T, S>* sh) {
+  unsigned long long mine = 0;
+  items.each([&](int& l, int e) {
+    if ((unsigned)l == x) mine += WT ? (unsigned long long)(unsigned)__ldg(wp + e) : 1ull;
+  });
+  mine = warp_sum_u64(mine);
+  if (T == 32) return (S)mine;
+  __syncthreads();
+  if (threadIdx.x == 0) sh->wsum = 0;
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&sh->wsum, mine);
+  __syncthreads();
+  return (S)sh->wsum;
+}
+
+// The counting round's outcome: `mine` is each thread's largest (running
+// sum, label) over its adds, counters hold the final sums.  Returns whether
+// `best` is the row's argmax; if not, the labels that could still beat it
+// are left open, `open_items` of them.
+template <int T, int WT, typename S, typename Items>
+__device__ __forceinline__ bool sketch_top(Items& items, const int* wp, const Sketch<S>& t, Best<S> mine,
+                                           Best<S>& best, unsigned& open_items, TeamShared<T, S>* sh) {
+  best = team_best<T, S>(mine, sh);   // with the barrier that ends the adds
+  open_items = 0;
+  if (best.sum == 0) return true;   // no neighbour but the vertex itself (team-uniform)
+  const unsigned x = ~best.inv, hx = t.slot(x);
+  bool other = false;
+  items.each([&](int& l, int) { other = other || (l >= 0 && (unsigned)l != x && t.slot((unsigned)l) == hx); });
+  if (!team_any<T>(other)) return true;
+  const S full = best.sum, sum = team_sum_of<T, WT, S>(items, wp, x, sh);
+  best.sum = sum;
+  unsigned left = 0;
+  items.each([&](int& l, int) {
+    if (l >= 0) {
+      const unsigned h = t.slot((unsigned)l);
+      const S c = h == hx ? full - sum : t.sum[h];   // a bound of every other label in the slot
+      if ((unsigned)l != x && beats<S>(c, ~(unsigned)l, best)) ++left;
+      else l = (int)((unsigned)l | SETTLED);
+    }
+  });
+  left = __reduce_add_sync(FULL, left);
+  if (T == 32) {
+    __syncwarp();
+  } else {
+    __syncthreads();
+    if (threadIdx.x == 0) sh->cnt = 0;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0 && left) atomicAdd(&sh->cnt, left);
+    __syncthreads();
+    left = sh->cnt;
+  }
+  open_items = left;
+  return left == 0;
+}
+
+// Rounds first_round.. over the items whose label is not settled (and lies
+// in part `part` of `parts` by the second hash): on return all of those are
+// settled and `best` covers them.  Starts and ends with the team in step.
+template <int T, int WT, typename S, typename Items>
+__device__ __forceinline__ void sketch_rounds(Items& items, const int* wp, const Slots<S> t, int first_round,
+                                              int rounds, unsigned part, unsigned parts, Best<S>& best,
+                                              TeamShared<T, S>* sh, int* err) {
+  const int tid = T == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  auto open = [&](int l) {
+    return l >= 0 && (parts <= 1 || __umulhi((unsigned)l * 0x7FEB352Du, parts) == part);
+  };
+  for (int r = first_round;; ++r) {
+    sketch_clear<T, S>(t.sum, t.lg, tid);
+    team_sync<T>();
+    items.each([&](int& l, int e) {
+      if (open(l)) {
+        const unsigned h = t.slot((unsigned)l, r);
+        atomicAdd(t.sum + h, WT ? (S)(unsigned)__ldg(wp + e) : (S)1);
+        *(volatile unsigned*)(t.lab + h) = (unsigned)l;
+      }
+    });
+    team_sync<T>();
+    items.each([&](int& l, int) {   // a label that lost its slot marks it shared
+      if (open(l)) {
+        volatile unsigned* p = t.lab + t.slot((unsigned)l, r);
+        if (*p != (unsigned)l) *p = EMPTY32;
+      }
+    });
+    team_sync<T>();
+    Best<S> mine{0, 0u};
+    items.each([&](int& l, int) {
+      if (open(l)) {
+        const unsigned h = t.slot((unsigned)l, r);
+        const S c = t.sum[h];
+        if (t.lab[h] != EMPTY32 && beats<S>(c, ~(unsigned)l, mine)) mine = {c, ~(unsigned)l};
+      }
+    });
+    mine = team_best<T, S>(mine, sh);
+    if (beats<S>(mine.sum, mine.inv, best)) best = mine;
+    bool left = false;
+    items.each([&](int& l, int) {
+      if (open(l)) {
+        const unsigned h = t.slot((unsigned)l, r);
+        // every weight is at least 1, so a label of a shared slot has at most the slot's sum less one
+        if (t.lab[h] == EMPTY32 && beats<S>(t.sum[h] - 1, ~(unsigned)l, best)) left = true;
+        else l = (int)((unsigned)l | SETTLED);
+      }
+    });
+    if (!team_any<T>(left)) return;
+    if (r + 1 - first_round >= rounds) break;
+  }
+  if (rounds < SKETCH_ROUNDS) raise_err(err, ERRBIT_TIMEOUT);   // a lowered retry bound
+  // labels that met another one in every round: one by one, the smallest first
+  for (;;) {
+    unsigned x = EMPTY32;
+    items.each([&](int& l, int) {
+      if (open(l) && (unsigned)l < x) x = (unsigned)l;
+    });
+    const Best<unsigned> lowest = warp_best(Best<unsigned>{~x, 0u});
+    x = ~lowest.sum;
+    if (T != 32) {
+      __syncthreads();
+      if (threadIdx.x == 0) sh->cnt = EMPTY32;
+      __syncthreads();
+      if ((threadIdx.x & 31) == 0) atomicMin(&sh->cnt, x);
+      __syncthreads();
+      x = sh->cnt;
+    }
+    if (x == EMPTY32) return;
+    const S c = team_sum_of<T, WT, S>(items, wp, x, sh);
+    if (beats<S>(c, ~x, best)) best = {c, ~x};
+    items.each([&](int& l, int) {
+      if ((unsigned)l == x) l = (int)((unsigned)l | SETTLED);
+    });
+    team_sync<T>();
+  }
+}
+
+// One row in registers, K entries per thread (d <= T * K), LG counters (log2).
+// GENERAL: first-sweep checks, identity labels, pre-gathered labels.
+template <int T, int K, int LG, int WT, bool ASYNC, bool GENERAL, typename S>
+__device__ __forceinline__ void sketch_row(const SweepArgs& a, int v, int old, const int* cp, const int* wp,
+                                           const int* lp, int d, int tid, S* mem, int rounds, const Pol& pol,
+                                           Best<S>& best, unsigned long long& ws, TeamShared<T, S>* sh) {
+  int l[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    l[k] = -1;
+    if (k * T < d) {   // team-uniform
+      int w;
+      if (GENERAL) load_entry<WT != 0>(a, cp, wp, d, k * T + tid, pol, l[k], w);
+      else l[k] = later_col(a, cp, d, k * T + tid, pol);
+      if (GENERAL && WT && l[k] >= 0) ws += (unsigned long long)(unsigned)w;
+    }
+  }
+  const Sketch<S> t{mem, LG};
+  sketch_clear<T, S>(t.sum, LG, tid);   // under the column loads
+  if (GENERAL && a.ident) {
+    // strictly increasing: every label (its id) occurs once
+    bool inc = true;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int e = k * T + tid;
+      if (e < d && (l[k] < 0 || (e + 1 < d && __ldg(cp + e + 1) <= l[k]))) inc = false;
+      check_same_graph(a, v, l[k]);
+      if (l[k] >= 0 && l[k] != v) {
+        const S c = WT ? (S)(unsigned)__ldg(wp + e) : (S)1;
+        if (beats<S>(c, ~(unsigned)l[k], best)) best = {c, ~(unsigned)l[k]};
+      }
+    }
+    if (!team_any<T>(!inc)) {
+      best = team_best<T, S>(best, sh);
+      return;
+    }
+    best = {0, 0u};
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    if (k * T < d) {
+      if (GENERAL) {
+        check_same_graph(a, v, l[k]);
+        l[k] = entry_label<ASYNC>(a, lp, k * T + tid, l[k], v, pol);
+      } else if (l[k] >= 0) {
+        l[k] = l[k] == v ? -1 : (ASYNC ? ld_label_rw(a.prev + l[k]) : ld_label_ro(a.prev + l[k], pol.label));
+      }
+    }
+  }
+  if (T == 32 && !GENERAL && WT != 2 && !a.spread) {
+    // a strict majority of the own label needs no table
+    unsigned own = 0;
+    const unsigned long long bound = WT ? (a.kw ? (unsigned long long)a.kw[v] : ~0ull) : (unsigned long long)d;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      if (k * T < d) {
+        const bool mine = l[k] == old;
+        if (WT) own += __reduce_add_sync(FULL, mine ? (unsigned)__ldg(wp + k * T + tid) : 0u);
+        else own += (unsigned)__popc(__ballot_sync(FULL, mine));
+      }
+    }
+    if (2ull * own > bound) {
+      best = {(S)own, ~(unsigned)old};
+      return;
+    }
+  }
+  team_sync<T>();   // the counters are clear
+  RegItems<T, K> items{l, d, tid};
+  Best<S> mine{0, 0u};
+  items.each([&](int& x, int e) {
+    if (x >= 0) {
+      const S w = WT ? (S)(unsigned)__ldg(wp + e) : (S)1;
+      const S c = atomicAdd(t.sum + t.slot((unsigned)x), w) + w;
+      if (beats<S>(c, ~(unsigned)x, mine)) mine = {c, ~(unsigned)x};
+    }
+  });
+  unsigned left;
+  if (!sketch_top<T, WT, S>(items, wp, t, mine, best, left, sh))
+    sketch_rounds<T, WT, S>(items, wp, Slots<S>(t), 1, rounds, 0u, 1u, best, sh, &a.ctr->err);
+}
+
+// One row through the block's scratch list.
+template <int T, int LG, int WT, bool ASYNC, bool GENERAL, typename S>
+__device__ __forceinline__ void sketch_long_row(const SweepArgs& a, int v, const int* cp, const int* wp,
+                                                const int* lp, int d, int tid, S* mem, int rounds, const Pol& pol,
+                                                Best<S>& best, unsigned long long& ws, TeamShared<T, S>* sh) {
+  if (GENERAL && a.ident) {
+    // strictly increasing: every label (its id) occurs once
+    bool inc = true;
+    unsigned long long sum = 0;
+#pragma unroll 4
+    for (int e = tid; e < d; e += T) {
+      int j, w;
+      load_entry<WT != 0>(a, cp, wp, d, e, pol, j, w);
+      if (j < 0 || (e + 1 < d && __ldg(cp + e + 1) <= j)) inc = false;
+      check_same_graph(a, v, j);
+      if (WT && j >= 0) sum += (unsigned long long)(unsigned)w;
+      if (j >= 0 && j != v && beats<S>((S)(unsigned)w, ~(unsigned)j, best)) best = {(S)(unsigned)w, ~(unsigned)j};
+    }
+    if (!team_any<T>(!inc)) {
+      best = team_best<T, S>(best, sh);
+      ws = sum;
+      return;
+    }
+    best = {0, 0u};
+  }
+  int* list = a.scratch + (long long)blockIdx.x * a.scratch_region;
+  const Sketch<S> t{mem, LG};
+  sketch_clear<T, S>(t.sum, LG, tid);
+  team_sync<T>();
+  Best<S> mine{0, 0u};
+  // gather and count; eight entries of a thread in flight
+  for (int e0 = 0; e0 < d; e0 += 8 * T) {
+    int l[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      int w;
+      const int e = e0 + u * T + tid;
+      if (GENERAL) load_entry<WT != 0>(a, cp, wp, d, e, pol, l[u], w);
+      else l[u] = later_col(a, cp, d, e, pol);
+      if (GENERAL && WT && l[u] >= 0) ws += (unsigned long long)(unsigned)w;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (GENERAL) check_same_graph(a, v, l[u]);
+      l[u] = entry_label<ASYNC>(a, lp, e0 + u * T + tid, l[u], v, pol);
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int e = e0 + u * T + tid;
+      if (e < d) list[e] = l[u];
+      if (l[u] >= 0) {
+        const S w = WT ? (S)(unsigned)__ldg(wp + e) : (S)1;
+        const S c = atomicAdd(t.sum + t.slot((unsigned)l[u]), w) + w;
+        if (beats<S>(c, ~(unsigned)l[u], mine)) mine = {c, ~(unsigned)l[u]};
+      }
+    }
+  }
+  MemItems<T> items{list, d, tid};
+  unsigned left;
+  if (!sketch_top<T, WT, S>(items, wp, t, mine, best, left, sh)) {
+    const Slots<S> slots(t);
+    const unsigned parts = (left >> slots.lg) + 1;
+    for (unsigned p = 0; p < parts; ++p)
+      sketch_rounds<T, WT, S>(items, wp, slots, 1, rounds, p, parts, best, sh, &a.ctr->err);
+  }
+}
+
+constexpr int K_WARP = 8, K_SMALL = 8, K_BLOCK = 16;               // entries per thread
+constexpr int T_SMALL = 128, T_BLOCK = 256;                         // threads per row (class 6: a warp)
+constexpr int LG_WARP = 10, LG_SMALL = 11, LG_BLOCK = 13;           // counters per row (log2)
+constexpr int BLOCKS_PER_SM = 4;                                    // of T_BLOCK threads
+
+template <int T>
+constexpr int team_lg() { return T == 32 ? LG_WARP : (T == T_SMALL ? LG_SMALL : LG_BLOCK); }
+
+}  // namespace
+
+// Rows of class cls by teams of T threads: up to T * K entries in registers
+// (fewer per thread on shorter rows), longer ones (T_BLOCK only) through the
+// block's scratch region.  Blocks take rows from a counter, warps in strides.
+template <int T, int WT, bool ASYNC, bool GENERAL>
+__global__ void __launch_bounds__(T == 32 ? 256 : T, T == 32 ? 4 : (T == T_SMALL ? 8 : BLOCKS_PER_SM))
+    sketch_kernel(SweepArgs a, int cls) {
+  using S = typename SumOf<WT>::T;
+  if (stopped(a)) return;
+  extern __shared__ int4 smem_sketch[];
+  __shared__ TeamShared<T, S> sh;
+  const int tid = T == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  S* mem = reinterpret_cast<S*>(smem_sketch) + (T == 32 ? (size_t)(threadIdx.x >> 5) << team_lg<T>() : 0);
+  const unsigned cnt = a.ctr->cls_count[cls];
+  const int* __restrict__ work = a.work + a.ctr->cls_start[cls];
+  const Pol pol = make_pol();
+  const int rounds = a.probe_cap < SKETCH_ROUNDS ? a.probe_cap : SKETCH_ROUNDS;
+  unsigned long long my_dn = 0, my_scan = 0;
+  const long long nteams = ((long long)gridDim.x * blockDim.x) / T;
+  long long item = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / T;
+  int vn = 0;
+  long long sn = 0, en = 0;
+  if (item < (long long)cnt) {
+    vn = work[item];
+    sn = a.off[vn];
+    en = a.off[vn + 1];
+  }
+  while (item < (long long)cnt) {
+    const int v = vn;
+    const long long s = sn;
+    const int d = (int)(en - sn);
+    // the next row: blocks take those beyond the first nteams in order
+    long long next = item + nteams;
+    if (T != 32) {
+      __syncthreads();   // the previous row's last reads of sh and the table
+      if (threadIdx.x == 0) sh.next = nteams + (long long)atomicAdd(&a.ctr->row_next[cls], 1u);
+      __syncthreads();
+      next = sh.next;
+    }
+    if (next < (long long)cnt) {
+      vn = work[next];
+      sn = a.off[vn];
+      en = a.off[vn + 1];
+    }
+    const int old = own_label<ASYNC>(a, v);
+    const int* cp = a.col + s;
+    const int* wp = a.w + s;
+    const int* lp = a.lg ? a.lg + s : nullptr;
+    Best<S> best{0, 0u};
+    unsigned long long ws = 0;
+    if (T == 32) {
+      if (d <= 64)
+        sketch_row<T, 2, 8, WT, ASYNC, GENERAL, S>(a, v, old, cp, wp, lp, d, tid, mem, rounds, pol, best, ws, &sh);
+      else if (d <= 128)
+        sketch_row<T, 4, 9, WT, ASYNC, GENERAL, S>(a, v, old, cp, wp, lp, d, tid, mem, rounds, pol, best, ws, &sh);
+      else
+        sketch_row<T, K_WARP, LG_WARP, WT, ASYNC, GENERAL, S>(a, v, old, cp, wp, lp, d, tid, mem, rounds, pol, best,
+                                                              ws, &sh);
+    } else if (T == T_SMALL) {
+      if (d <= T * K_SMALL / 2)
+        sketch_row<T, K_SMALL / 2, LG_SMALL, WT, ASYNC, GENERAL, S>(a, v, old, cp, wp, lp, d, tid, mem, rounds, pol,
+                                                                    best, ws, &sh);
+      else
+        sketch_row<T, K_SMALL, LG_SMALL, WT, ASYNC, GENERAL, S>(a, v, old, cp, wp, lp, d, tid, mem, rounds, pol, best,
+                                                                ws, &sh);
+    } else {
+      if (d <= T * K_BLOCK / 2)
+        sketch_row<T, K_BLOCK / 2, LG_BLOCK - 1, WT, ASYNC, GENERAL, S>(a, v, old, cp, wp, lp, d, tid, mem, rounds,
+                                                                        pol, best, ws, &sh);
+      else if (d <= T * K_BLOCK)
+        sketch_row<T, K_BLOCK, LG_BLOCK, WT, ASYNC, GENERAL, S>(a, v, old, cp, wp, lp, d, tid, mem, rounds, pol, best,
+                                                                ws, &sh);
+      else
+        sketch_long_row<T, LG_BLOCK, WT, ASYNC, GENERAL, S>(a, v, cp, wp, lp, d, tid, mem, rounds, pol, best, ws,
+                                                            &sh);
+    }
+    if (WT == 1 && GENERAL && a.check) {
+      ws = warp_sum_u64(ws);
+      if (T != 32) {
+        __syncthreads();
+        if (threadIdx.x == 0) sh.wsum = 0;
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0 && ws) atomicAdd(&sh.wsum, ws);
+        __syncthreads();
+        ws = sh.wsum;
+      }
+      if (tid == 0) {
+        if (ws >= (1ull << 31)) raise_err(&a.ctr->err, ERRBIT_OVERFLOW);
+        if (a.kw) a.kw[v] = ws < (1ull << 32) ? (unsigned)ws : ~0u;
+      }
+    }
+    const int nl = best.sum ? (int)~best.inv : old;
+    const bool changed = nl != old;   // team-uniform
+    if (tid == 0) {
+      store_label<ASYNC>(a, v, nl, changed);
+      if (changed) count_graph_change(a, v);
+      my_scan += (unsigned long long)d;
+      my_dn += changed ? 1ull : 0ull;
+    }
+    if (changed && a.mark) {
+      for (int e = tid; e < d; e += T) {
+        const int j = ld_stream(cp + e, pol.stream);
+        if ((unsigned)j < (unsigned)a.n) a.fnext[j] = 1;
+      }
+      if (!ASYNC && tid == 0) a.fnext[v] = 1;
+    }
+    item = next;
+    if (T == 32) __syncwarp();   // the table's last reads before it is cleared
+  }
+  flush_counters(a.ctr, cls, my_dn, my_scan);
+}
+
+namespace {
+template <int T, int WT, bool A, bool G>
+cudaError_t launch_sketch_g(const SweepArgs& a, int cls, const DeviceInfo& di, cudaStream_t s) {
+  using S = typename SumOf<WT>::T;
+  constexpr int block = T == 32 ? 256 : T;
+  const size_t smem = (sizeof(S) << team_lg<T>()) * (size_t)(block / T);
+  thread_local int grid = 0;
+  if (!grid) {
+    if (cudaError_t e = raise_smem_limit((const void*)sketch_kernel<T, WT, A, G>, smem)) return e;
+    int per_sm = 0;
+    if (cudaError_t e =
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sketch_kernel<T, WT, A, G>, block, smem))
+      return e;
+    grid = (per_sm < 1 ? 1 : per_sm) * di.sm_count;
+    if (T == T_BLOCK && grid > sketch_blocks(di)) grid = (int)sketch_blocks(di);   // one scratch region each
+  }
+  sketch_kernel<T, WT, A, G><<<grid, block, smem, s>>>(a, cls);
+  count_launches(1);
+  return cudaGetLastError();
+}
+
+template <int T, int WT>
+cudaError_t launch_sketch_t(const SweepArgs& a, int cls, bool async_mode, const DeviceInfo& di, cudaStream_t s) {
+  const bool general = a.check || a.ident || a.lg;
+  if (async_mode)
+    return general ? launch_sketch_g<T, WT, true, true>(a, cls, di, s)
+                   : launch_sketch_g<T, WT, true, false>(a, cls, di, s);
+  return general ? launch_sketch_g<T, WT, false, true>(a, cls, di, s)
+                 : launch_sketch_g<T, WT, false, false>(a, cls, di, s);
+}
+
+template <int WT>
+cudaError_t launch_sketch_w(const SweepArgs& a, int cls, int longest, bool async_mode, const DeviceInfo& di,
+                            cudaStream_t s) {
+  if (longest <= 32 * K_WARP) return launch_sketch_t<32, WT>(a, cls, async_mode, di, s);
+  if (longest <= T_SMALL * K_SMALL) return launch_sketch_t<T_SMALL, WT>(a, cls, async_mode, di, s);
+  return launch_sketch_t<T_BLOCK, WT>(a, cls, async_mode, di, s);
+}
+}  // namespace
+
+long long sketch_blocks(const DeviceInfo& di) { return (long long)BLOCKS_PER_SM * di.sm_count; }
+long long sketch_register_row() { return (long long)T_BLOCK * K_BLOCK; }
+
+cudaError_t launch_sketch(const SweepArgs& a, int cls, int longest, int weights, bool async_mode,
+                          const DeviceInfo& di, cudaStream_t s) {
+  if (weights == 0) return launch_sketch_w<0>(a, cls, longest, async_mode, di, s);
+  return launch_sketch_w<1>(a, cls, longest, async_mode, di, s);
+}
+
+}  // namespace gsl

@@ -132,7 +132,7 @@ __device__ __forceinline__ void tile_entry(const SweepArgs& a, const int* cp, co
   if (FIRST) {
     load_entry<WEIGHTED>(a, cp, wp, d, e, pol, j, wt);
   } else {
-    j = spread_col(a, cp, d, e, pol);
+    j = later_col(a, cp, d, e, pol);
     wt = WEIGHTED && e < d ? ld_stream(wp + e, pol.stream) : (e < d ? 1 : 0);
   }
 }
