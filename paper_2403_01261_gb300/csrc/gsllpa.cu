@@ -330,7 +330,7 @@ int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s) {
 
 // Label lists for the rows of up to `longest` entries that one block sweeps.
 int ensure_scratch(gsl_ctx* c, long long longest, SweepArgs* a) {
-  a->scratch_region = longest > sketch_register_row() ? longest : 0;
+  a->scratch_region = longest > sketch_register_row() ? 3 * longest : 0;   // labels, parts, their weights
   if (a->scratch_region)
     if (int r = grow(c, c->scratch, c->cap_scratch, sketch_blocks(c->di) * a->scratch_region)) return r;
   a->scratch = c->scratch;
@@ -365,8 +365,9 @@ struct LpaResume {
 // the labels.  prepare_graph must have run.
 int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t* labels_init, double tol,
             int32_t max_iters, int32_t mode, gsl_stats* st, cudaStream_t s, int** final,
-            const LpaResume* resume = nullptr) {
+            const LpaResume* resume = nullptr, bool wide = false) {
   const long long n = g->n;
+  const int wt = !weights ? 0 : (wide ? 2 : 1);
   const bool async_mode = mode == GSL_MODE_ASYNC;
   if (!resume) {
     CK(cudaMemsetAsync(c->flag[0], 0, (size_t)n, s));
@@ -384,9 +385,11 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
   a.ctr = c->ctr;
   a.probe_cap = c->tune.probe_cap;
   a.work = c->work;
-  if (int r = ensure_scratch(c, longest_block_row(c), &a)) return r;
+  // the hub kernels sum in 32 bits: with 64-bit sums their rows are block rows
+  const bool hub_kernels = c->hub_ready && !wide;
+  if (int r = ensure_scratch(c, wide ? (long long)c->ctr_h->max_degree : longest_block_row(c), &a)) return r;
   a.n = n;
-  if (weights) {   // weighted degrees, written by sweep 1 for the early stops of later sweeps
+  if (wt == 1) {   // weighted degrees, written by sweep 1 for the early stops of later sweeps
     if (int r = grow(c, c->kw, c->cap_kw, n)) return r;
     a.kw = c->kw;
   }
@@ -479,7 +482,7 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
       SweepArgs af = a;   // the filtered classes read the filter's worklist
       if (filter && class_vertices(c, filter_from, CLS_BLOCK) > 0) {
         const int pe = prof_begin(c, s);
-        CK(launch_majority_filter(a, c->work2, weights != nullptr, async_mode, c->di, s, filter_from));
+        CK(launch_majority_filter(a, c->work2, wt, async_mode, c->di, s, filter_from));
         prof_end(c, pe, SL_FILTER, s, 2);
         af.work = c->work2;
       }
@@ -487,23 +490,23 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
         if (class_vertices(c, k, k) == 0) continue;
         const int pe = prof_begin(c, s);
         if (k == CLS_WARP_L || k == CLS_BLOCK || (k == CLS_WARP_S && filter_from == CLS_WARP_S)) {
-          CK(launch_sweep_class(af, k, weights != nullptr, async_mode, c->tune, maxd, c->di, s));
+          CK(launch_sweep_class(af, k, wt, async_mode, c->tune, maxd, c->di, s));
           prof_end(c, pe, SL_SWEEP0 + k, s, 1);
-        } else if (k == CLS_HUB && c->hub_ready) {
+        } else if (k == CLS_HUB && hub_kernels) {
           HubPlan hp{c->hub_piece_start, c->hub_ustart, c->hub_best, c->hub_own,
                      c->hub_wsum,        c->hub_used_cnt, c->hub_used, c->hub_tab, c->hub_clu};
           c->hub_dirty = true;   // until this sweep is known to have finished cleanly
           int kernels = 0;
-          CK(launch_hub_pieces(a, hp, weights != nullptr, async_mode, filter, c->tune, c->di, s, &kernels));
+          CK(launch_hub_pieces(a, hp, wt != 0, async_mode, filter, c->tune, c->di, s, &kernels));
           prof_end(c, pe, SL_SWEEP0 + k, s, kernels);
         } else {
-          CK(launch_sweep_class(a, k, weights != nullptr, async_mode, c->tune, maxd, c->di, s));
+          CK(launch_sweep_class(a, k, wt, async_mode, c->tune, maxd, c->di, s));
           prof_end(c, pe, SL_SWEEP0 + k, s, 1);
         }
       }
       if (class_vertices(c, 0, CLS_BINNED - 1) > 0) {
         const int pe = prof_begin(c, s);
-        CK(launch_sweep_lanes(a, weights != nullptr, async_mode, 0, n, c->flag[t & 1], all_active ? 1 : 0, nullptr, ph,
+        CK(launch_sweep_lanes(a, wt, async_mode, 0, n, c->flag[t & 1], all_active ? 1 : 0, nullptr, ph,
                              (unsigned)t, c->di, s));
         prof_end(c, pe, SL_LANES, s, 1);
       }
@@ -721,9 +724,12 @@ int run_lpa_f32(gsl_ctx* c, const gsl_csr* g, const float* wf, const int32_t* la
 // its labels.  Sets *wi to the converted weights, or leaves it NULL (float
 // path) when the weights do not qualify or the context's mode is 0; invalid
 // weights are left to the float path, which reports them.  After
-// prepare_graph(g).
-int f32_fixed_point(gsl_ctx* c, const gsl_csr* g, const float* w, cudaStream_t s, int** wi) {
+// prepare_graph(g).  *wide: the weights fit int32 but a row total needs up to
+// 53 bits, so the sweeps sum in 64 bits; the float64 sums are exact there too
+// (multiples of 2^-S below 2^(53-S)).
+int f32_fixed_point(gsl_ctx* c, const gsl_csr* g, const float* w, cudaStream_t s, int** wi, bool* wide) {
   *wi = nullptr;
+  *wide = false;
   if (c->f32_fixed == 0 || g->nnz == 0) return GSL_OK;
   CK(launch_f32_exact_scan(w, g->nnz, c->fix_dev, c->di, s));
   CK(cudaMemcpyAsync(c->fix_h, c->fix_dev, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -734,7 +740,8 @@ int f32_fixed_point(gsl_ctx* c, const gsl_csr* g, const float* w, cudaStream_t s
   int dbits = 0;   // ceil(log2(largest degree))
   while ((1ll << dbits) < c->ctr_h->max_degree) ++dbits;
   // a weight is below 2^(hi+1), so a row total times 2^shift is below 2^(hi+1+shift+dbits)
-  if (shift > 30 || hi + 1 + shift + dbits > 31) return GSL_OK;
+  if (shift > 30 || hi + 1 + shift > 31 || hi + 1 + shift + dbits > 53) return GSL_OK;
+  *wide = hi + 1 + shift + dbits > 31;
   if (int r = grow(c, c->fix_w, c->cap_fix_w, g->nnz)) return r;
   CK(launch_f32_to_fixed(w, g->nnz, shift, c->fix_w, c->di, s));
   *wi = c->fix_w;
@@ -863,7 +870,7 @@ cudaError_t enqueue_batch_sweeps(gsl_ctx* c, const gsl_csr* g, int num_graphs, c
   a.probe_cap = c->tune.probe_cap;
   a.work = c->work;
   a.scratch = c->scratch;   // allocated before the capture
-  a.scratch_region = c->ctr_h->max_degree;
+  a.scratch_region = 3 * c->ctr_h->max_degree;
   a.n = n;
   a.gid = c->gid;
   a.vptr = c->vptr;
@@ -896,7 +903,7 @@ cudaError_t enqueue_batch_sweeps(gsl_ctx* c, const gsl_csr* g, int num_graphs, c
       SweepArgs af = a;
       if (filter && class_vertices(c, filter_from, CLS_BLOCK) > 0) {
         pe = prof ? prof_begin(c, cs) : -1;
-        ck(launch_majority_filter(a, c->work2, weights != nullptr, async_mode, c->di, cs, filter_from));
+        ck(launch_majority_filter(a, c->work2, weights ? 1 : 0, async_mode, c->di, cs, filter_from));
         if (prof) prof_end(c, pe, SL_FILTER, cs, 2);
         af.work = c->work2;
       }
@@ -904,13 +911,13 @@ cudaError_t enqueue_batch_sweeps(gsl_ctx* c, const gsl_csr* g, int num_graphs, c
         if (class_vertices(c, k, k) == 0) continue;
         pe = prof ? prof_begin(c, cs) : -1;
         const bool filtered = k == CLS_WARP_L || k == CLS_BLOCK || (k == CLS_WARP_S && filter_from == CLS_WARP_S);
-        ck(launch_sweep_class(filtered ? af : a, k, weights != nullptr, async_mode, c->tune,
+        ck(launch_sweep_class(filtered ? af : a, k, weights ? 1 : 0, async_mode, c->tune,
                               (int)c->ctr_h->max_degree, c->di, cs));
         if (prof) prof_end(c, pe, SL_SWEEP0 + k, cs, 1);
       }
       if (class_vertices(c, 0, CLS_BINNED - 1) > 0) {
         pe = prof ? prof_begin(c, cs) : -1;
-        ck(launch_sweep_lanes(a, weights != nullptr, async_mode, 0, n, c->flag[t & 1], t <= 2 ? 1 : 0, c->done, ph,
+        ck(launch_sweep_lanes(a, weights ? 1 : 0, async_mode, 0, n, c->flag[t & 1], t <= 2 ? 1 : 0, c->done, ph,
                              (unsigned)t, c->di, cs));
         if (prof) prof_end(c, pe, SL_LANES, cs, 1);
       }
@@ -1305,10 +1312,11 @@ int gsl_lpa_f32(gsl_ctx* c, const gsl_csr* g, const float* weights, const int32_
   CK(cudaEventRecord(c->ev[0], s));
   if (int r = prepare_graph(c, g, s)) return r;
   int* wi = nullptr;
-  if (int r = f32_fixed_point(c, g, weights, s, &wi)) return r;
+  bool wide = false;
+  if (int r = f32_fixed_point(c, g, weights, s, &wi, &wide)) return r;
   int* fin = nullptr;
   if (wi) {
-    if (int r = run_lpa(c, g, wi, labels_init, tol, max_iters, mode, st, s, &fin)) return r;
+    if (int r = run_lpa(c, g, wi, labels_init, tol, max_iters, mode, st, s, &fin, nullptr, wide)) return r;
   } else {
     if (int r = run_lpa_f32(c, g, weights, labels_init, tol, max_iters, mode, st, s, &fin)) return r;
   }
@@ -1333,10 +1341,11 @@ int gsl_gsllpa_f32(gsl_ctx* c, const gsl_csr* g, const float* weights, double to
   CK(cudaEventRecord(c->ev[0], s));
   if (int r = prepare_graph(c, g, s)) return r;
   int* wi = nullptr;
-  if (int r = f32_fixed_point(c, g, weights, s, &wi)) return r;
+  bool wide = false;
+  if (int r = f32_fixed_point(c, g, weights, s, &wi, &wide)) return r;
   int* fin = nullptr;
   if (wi) {
-    if (int r = run_lpa(c, g, wi, nullptr, tol, max_iters, mode, st, s, &fin)) return r;
+    if (int r = run_lpa(c, g, wi, nullptr, tol, max_iters, mode, st, s, &fin, nullptr, wide)) return r;
   } else {
     if (int r = run_lpa_f32(c, g, weights, nullptr, tol, max_iters, mode, st, s, &fin)) return r;
   }
@@ -1750,25 +1759,25 @@ int gsllpa_host_overlapped(gsl_ctx* c, int64_t n, int64_t nnz, const int64_t* of
                           s));
     if (stop1) continue;
     if (k > 0) CK(launch_phase_reset(c->ctr, nullptr, s));
-    CK(launch_sweep_lanes(a, false, false, vb[k], vb[k + 1], nullptr, 1, nullptr, 0, 2u, c->di, s));
+    CK(launch_sweep_lanes(a, 0, false, vb[k], vb[k + 1], nullptr, 1, nullptr, 0, 2u, c->di, s));
     if (class_vertices(c, CLS_BINNED, NCLASS - 1) == 0) continue;
     CK(launch_bin_range(OFF(&g), vb[k], vb[k + 1], c->tune, c->work, c->ctr, c->di, s, CLS_BINNED));
     SweepArgs af = a;
     if (filter) {
-      CK(launch_majority_filter(a, c->work2, false, false, c->di, s));
+      CK(launch_majority_filter(a, c->work2, 0, false, c->di, s));
       af.work = c->work2;
     }
     for (int cls = NCLASS - 1; cls >= CLS_BINNED; --cls) {
       if (class_vertices(c, cls, cls) == 0) continue;
       if (cls == CLS_WARP_L || cls == CLS_BLOCK) {
-        CK(launch_sweep_class(af, cls, false, false, c->tune, (int)c->ctr_h->max_degree, c->di, s));
+        CK(launch_sweep_class(af, cls, 0, false, c->tune, (int)c->ctr_h->max_degree, c->di, s));
       } else if (cls == CLS_HUB && c->hub_ready) {
         HubPlan hp{c->hub_piece_start, c->hub_ustart, c->hub_best, c->hub_own,
                    c->hub_wsum,        c->hub_used_cnt, c->hub_used, c->hub_tab, c->hub_clu};
         int kernels = 0;
         CK(launch_hub_pieces(a, hp, false, false, filter, c->tune, c->di, s, &kernels));
       } else {
-        CK(launch_sweep_class(a, cls, false, false, c->tune, (int)c->ctr_h->max_degree, c->di, s));
+        CK(launch_sweep_class(a, cls, 0, false, c->tune, (int)c->ctr_h->max_degree, c->di, s));
       }
     }
   }

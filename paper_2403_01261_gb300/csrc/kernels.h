@@ -17,7 +17,7 @@ struct SweepArgs {
   const int* work;           // worklist (class regions at Counters::cls_start)
   Counters* ctr;
   int* scratch;              // label lists of rows longer than a block's registers, one region per block
-  long long scratch_region;  // ints per region
+  long long scratch_region;  // ints per region (three lists of the longest row)
   long long n;
   // batched mode (many graphs packed in one CSR); all null for one graph
   const int* gid;            // graph of every vertex
@@ -73,23 +73,24 @@ cudaError_t launch_all_counts(Counters* ctr, int first_cls, cudaStream_t s);
 // tile_kernels.cu: the rows of 1..4 entries among the vertices [v0, v1) (all
 // of them, or those flagged in fcur, whose flags are cleared), and the rows
 // of classes 3..5 on the worklist.
-cudaError_t launch_sweep_lanes(const SweepArgs& a, bool weighted, bool async_mode, long long v0, long long v1,
+cudaError_t launch_sweep_lanes(const SweepArgs& a, int weights, bool async_mode, long long v0, long long v1,
                                unsigned char* fcur, int all_active, const unsigned char* done, int phase,
                                unsigned seed, const DeviceInfo& di, cudaStream_t s);
-cudaError_t launch_sweep_tile(const SweepArgs& a, int cls, bool weighted, bool async_mode, const DeviceInfo& di,
+cudaError_t launch_sweep_tile(const SweepArgs& a, int cls, int weights, bool async_mode, const DeviceInfo& di,
                               cudaStream_t s);
 // Between the two phases of an asynchronous sweep (see Counters::phase_cls).
 cudaError_t launch_phase_reset(Counters* ctr, const int* stop, cudaStream_t s);
 // sketch_kernels.cu: the rows of class cls on the worklist, none longer than
 // `longest`.  Rows longer than
 // sketch_register_row() need SweepArgs::scratch, sketch_blocks() regions of
-// the longest row's length.  weights: 0 unit, 1 int32.
+// three times the longest row's length.  weights: 0 unit, 1 int32, 2 int32 with 64-bit
+// sums (so in the other sweep launchers).
 long long sketch_blocks(const DeviceInfo& di);
 long long sketch_register_row();
 cudaError_t launch_sketch(const SweepArgs& a, int cls, int longest, int weights, bool async_mode,
                           const DeviceInfo& di, cudaStream_t s);
 // Classes 3..9 on the worklist (class 9 as the block rows it then is).
-cudaError_t launch_sweep_class(const SweepArgs& a, int cls, bool weighted, bool async_mode, const Tuning& t,
+cudaError_t launch_sweep_class(const SweepArgs& a, int cls, int weights, bool async_mode, const Tuning& t,
                                int longest, const DeviceInfo& di, cudaStream_t s);
 void count_launches(long long k);   // process-wide tally of kernels this library launched
 // Raises kernel fn's dynamic shared-memory limit to at least `bytes` (never
@@ -103,7 +104,7 @@ long long launches_total();
 // block kernels, which must then read `out` as their worklist.
 // The class counts of classes first_cls..8 become the rows a filter passed on.
 cudaError_t launch_filter_counts(Counters* ctr, const int* stop, cudaStream_t s, int first_cls = CLS_WARP_L);
-cudaError_t launch_majority_filter(const SweepArgs& a, int* out, bool weighted, bool async_mode,
+cudaError_t launch_majority_filter(const SweepArgs& a, int* out, int weights, bool async_mode,
                                    const DeviceInfo& di, cudaStream_t s, int first_cls = CLS_WARP_L);
 // Edge-parallel label gather for a synchronous sweep: lg[e] = prev[col[e]]
 // for every CSR entry (-1 for an out-of-range column).

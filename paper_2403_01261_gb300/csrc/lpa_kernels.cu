@@ -178,15 +178,15 @@ __global__ void init_labels_kernel(const int* __restrict__ init, int* __restrict
 // row's total (d entries, or the weighted degree from sweep 1), since it
 // then holds a strict majority of the whole row whatever the rest carries
 // (`early`).  Returns the entries read.
-template <bool WEIGHTED, bool ASYNC>
+template <int WT, bool ASYNC>
 __device__ __forceinline__ int filter_row(const SweepArgs& a, int v, int own, const int* cp, const int* wp,
-                                          const int* lp, int d, const Pol& pol, unsigned& own_w, unsigned& tot_w,
-                                          bool& early) {
+                                          const int* lp, int d, const Pol& pol, typename SumOf<WT>::T& own_w,
+                                          typename SumOf<WT>::T& tot_w, bool& early) {
   const int lane = threadIdx.x & 31;
-  const unsigned long long bound = !WEIGHTED ? (unsigned long long)d : (a.kw ? (unsigned long long)a.kw[v] : ~0ull);
+  const unsigned long long bound = !WT ? (unsigned long long)d : (WT == 1 && a.kw ? (unsigned long long)a.kw[v] : ~0ull);
   int jn[4], wn[4];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) load_entry<WEIGHTED>(a, cp, wp, d, lane + 32 * u, pol, jn[u], wn[u]);
+  for (int u = 0; u < 4; ++u) load_entry<WT != 0>(a, cp, wp, d, lane + 32 * u, pol, jn[u], wn[u]);
   for (int r0 = 0; r0 < d; r0 += 128) {
     int l[4], w[4];
 #pragma unroll
@@ -197,7 +197,7 @@ __device__ __forceinline__ int filter_row(const SweepArgs& a, int v, int own, co
     const bool more = r0 + 128 < d;   // warp-uniform
     if (more) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) load_entry<WEIGHTED>(a, cp, wp, d, r0 + 128 + lane + 32 * u, pol, jn[u], wn[u]);
+      for (int u = 0; u < 4; ++u) load_entry<WT != 0>(a, cp, wp, d, r0 + 128 + lane + 32 * u, pol, jn[u], wn[u]);
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -206,7 +206,7 @@ __device__ __forceinline__ int filter_row(const SweepArgs& a, int v, int own, co
         if (l[u] == own) own_w += (unsigned)w[u];
       }
     }
-    if (more && 2ull * __reduce_add_sync(FULL, own_w) > bound) {
+    if (WT != 2 && more && 2ull * __reduce_add_sync(FULL, (unsigned)own_w) > bound) {
       early = true;
       return r0 + 128;
     }
@@ -224,7 +224,7 @@ __device__ __forceinline__ int filter_row(const SweepArgs& a, int v, int own, co
 // Other rows are appended to `out` at their class's region and counted in
 // Counters::uns_count; filter_counts_kernel then makes those the class
 // counts for the table kernels.
-template <bool WEIGHTED, bool ASYNC>
+template <int WT, bool ASYNC>
 __global__ void __launch_bounds__(256, 6) majority_filter_kernel(SweepArgs a, int* __restrict__ out, int first_cls) {
   if (stopped(a)) return;
   const int lane = threadIdx.x & 31;
@@ -242,9 +242,9 @@ __global__ void __launch_bounds__(256, 6) majority_filter_kernel(SweepArgs a, in
     const long long s = a.off[v];
     const int d = (int)(a.off[v + 1] - s);
     const int old = own_label<ASYNC>(a, v);
-    unsigned ow = 0, tw = 0;
+    typename SumOf<WT>::T ow = 0, tw = 0;
     bool early = false;
-    const int read = filter_row<WEIGHTED, ASYNC>(a, v, old, a.col + s, a.w + s, a.lg ? a.lg + s : nullptr, d, pol, ow,
+    const int read = filter_row<WT, ASYNC>(a, v, old, a.col + s, a.w + s, a.lg ? a.lg + s : nullptr, d, pol, ow,
                                                  tw, early);
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
@@ -280,15 +280,16 @@ cudaError_t launch_filter_counts(Counters* ctr, const int* stop, cudaStream_t s,
   return cudaGetLastError();
 }
 
-cudaError_t launch_majority_filter(const SweepArgs& a, int* out, bool weighted, bool async_mode,
+cudaError_t launch_majority_filter(const SweepArgs& a, int* out, int weights, bool async_mode,
                                    const DeviceInfo& di, cudaStream_t s, int first_cls) {
   const int grid = 16 * di.sm_count;
-  if (weighted) {
-    if (async_mode) majority_filter_kernel<true, true><<<grid, 256, 0, s>>>(a, out, first_cls);
-    else majority_filter_kernel<true, false><<<grid, 256, 0, s>>>(a, out, first_cls);
-  } else {
-    if (async_mode) majority_filter_kernel<false, true><<<grid, 256, 0, s>>>(a, out, first_cls);
-    else majority_filter_kernel<false, false><<<grid, 256, 0, s>>>(a, out, first_cls);
+  switch (2 * weights + (async_mode ? 1 : 0)) {
+    case 0: majority_filter_kernel<0, false><<<grid, 256, 0, s>>>(a, out, first_cls); break;
+    case 1: majority_filter_kernel<0, true><<<grid, 256, 0, s>>>(a, out, first_cls); break;
+    case 2: majority_filter_kernel<1, false><<<grid, 256, 0, s>>>(a, out, first_cls); break;
+    case 3: majority_filter_kernel<1, true><<<grid, 256, 0, s>>>(a, out, first_cls); break;
+    case 4: majority_filter_kernel<2, false><<<grid, 256, 0, s>>>(a, out, first_cls); break;
+    default: majority_filter_kernel<2, true><<<grid, 256, 0, s>>>(a, out, first_cls); break;
   }
   filter_counts_kernel<<<1, 1, 0, s>>>(a.ctr, a.stop, first_cls);
   count_launches(2);
@@ -601,12 +602,12 @@ std::atomic<long long> g_launches{0};
 constexpr int WARP_SMALL = 256;   // longest row of one warp (class 6)
 }  // namespace
 
-cudaError_t launch_sweep_class(const SweepArgs& a, int cls, bool weighted, bool async_mode, const Tuning& t,
+cudaError_t launch_sweep_class(const SweepArgs& a, int cls, int weights, bool async_mode, const Tuning& t,
                                int longest, const DeviceInfo& di, cudaStream_t s) {
-  if (cls < CLS_WARP_S) return launch_sweep_tile(a, cls, weighted, async_mode, di, s);
+  if (cls < CLS_WARP_S) return launch_sweep_tile(a, cls, weights, async_mode, di, s);
   const ClassBounds cb = class_bounds(t);
   const int bound = cls == CLS_WARP_S ? cb.warp_small : (cls == CLS_WARP_L ? cb.warp_max : (cls == CLS_BLOCK ? cb.blk_max : longest));
-  return launch_sketch(a, cls, bound < longest ? bound : longest, weighted ? 1 : 0, async_mode, di, s);
+  return launch_sketch(a, cls, bound < longest ? bound : longest, weights, async_mode, di, s);
 }
 
 void count_launches(long long k) { g_launches.fetch_add(k, std::memory_order_relaxed); }

@@ -14,8 +14,9 @@
 // that end up with one label hold its exact sum.
 //
 // Rows longer than the registers hold (4096 entries) keep their labels in a
-// scratch list of the block; if more of them stay open than the table has
-// slots, the list is counted in parts by a second hash.
+// scratch list of the block; if many of them stay open (labels of about the
+// same weight, as in the early sweeps over weighted graphs), those are moved
+// into parts by a second hash and counted part by part.
 //
 // Bound by instruction issue and the label gathers: the hash tables before
 // spent 150 to 210 warp instructions per 32 entries (compare-and-swap 5
@@ -27,23 +28,6 @@ namespace gsl {
 namespace {
 
 constexpr unsigned SETTLED = 0x80000000u;   // label bit: no longer in question (absent entries are -1)
-
-template <int WT>
-struct SumOf { using T = unsigned; };
-template <>
-struct SumOf<2> { using T = unsigned long long; };
-
-// Best label so far: largest sum, then smallest label (inv = ~label).
-template <typename S>
-struct Best {
-  S sum;
-  unsigned inv;
-};
-
-template <typename S>
-__device__ __forceinline__ bool beats(S s, unsigned inv, const Best<S>& b) {
-  return s > b.sum || (s == b.sum && inv > b.inv);
-}
 
 __device__ __forceinline__ Best<unsigned> warp_best(Best<unsigned> b) {
   const unsigned m = __reduce_max_sync(FULL, b.sum);
@@ -79,29 +63,37 @@ struct TeamShared {
   unsigned long long wsum;
   unsigned cnt;
   long long next;
+  unsigned part[T == 32 ? 1 : 64 + 1];   // long rows: first entry of every part
+  unsigned fill[T == 32 ? 1 : 64];
 };
 
-template <int T, typename S>
-__device__ __forceinline__ Best<S> team_best(Best<S> b, TeamShared<T, S>* sh) {
+template <int T, typename B, typename S>
+__device__ __forceinline__ Best<B> team_best(Best<B> b, TeamShared<T, S>* sh) {
   b = warp_best(b);
   if (T == 32) return b;
   const int lane = threadIdx.x & 31;
   if (lane == 0) {
-    sh->sum[threadIdx.x >> 5] = b.sum;
+    sh->sum[threadIdx.x >> 5] = (S)b.sum;
     sh->inv[threadIdx.x >> 5] = b.inv;
   }
   __syncthreads();
   b = {0, 0u};
-  if (lane < T / 32) b = {sh->sum[lane], sh->inv[lane]};
+  if (lane < T / 32) b = {(B)sh->sum[lane], sh->inv[lane]};
   return warp_best(b);   // the next barrier comes before sh is written again
 }
 
-// The table's memory holds 1 << lg counters of the counting round, or half
-// as many slots of (sum, label) in the rounds after it.
-template <typename S>
+// The table's memory holds 1 << lg counters of the counting round, or half as
+// many slots of (sum, label) in the rounds after it (a quarter with 64-bit
+// sums).
+//
+// Counters are 32-bit: shared 64-bit adds take eight times as long and far
+// longer still on one hot counter (a 98,000-entry row with a common label
+// took 0.9 ms).  With 64-bit sums they hold bounds instead, (w >> q) + 1 per
+// entry, so that sum < counter << q; the named label's sum is exact anyway.
 struct Sketch {
-  S* sum;
+  unsigned* cnt;
   unsigned lg;
+  unsigned q;   // 64-bit sums: shift of the bounds
   __device__ __forceinline__ unsigned slot(unsigned label) const { return sketch_hash(label, 0) >> (32u - lg); }
 };
 template <typename S>
@@ -109,8 +101,10 @@ struct Slots {
   S* sum;
   unsigned* lab;
   unsigned lg;
-  __device__ __forceinline__ explicit Slots(const Sketch<S>& t)
-      : sum(t.sum), lab(reinterpret_cast<unsigned*>(t.sum + (1u << (t.lg - 1)))), lg(t.lg - 1) {}
+  __device__ __forceinline__ explicit Slots(const Sketch& t)
+      : sum(reinterpret_cast<S*>(t.cnt)), lg(t.lg - (sizeof(S) == 8 ? 2 : 1)) {
+    lab = reinterpret_cast<unsigned*>(sum + (1u << lg));
+  }
   __device__ __forceinline__ unsigned slot(unsigned label, int round) const {
     return sketch_hash(label, round) >> (32u - lg);
   }
@@ -122,6 +116,14 @@ __device__ __forceinline__ void sketch_clear(S* sum, unsigned lg, int tid) {
   int4* p = reinterpret_cast<int4*>(sum);
 #pragma unroll 4
   for (unsigned k = tid; k < (1u << lg) / PER; k += T) p[k] = make_int4(0, 0, 0, 0);
+}
+
+// A counter's step for an entry of weight w.
+template <int WT>
+__device__ __forceinline__ unsigned counter_step(const Sketch& t, const int* wp, int e) {
+  if (WT == 0) return 1u;
+  const unsigned w = (unsigned)wp[e];
+  return WT == 1 ? w : (w >> t.q) + 1u;
 }
 
 // Labels of a row in registers: entry k * T + tid in l[k].
@@ -144,55 +146,71 @@ struct MemItems {
   int d, tid;
   template <typename F>
   __device__ __forceinline__ void each(F&& f) {
-#pragma unroll 4
-    for (int e = tid; e < d; e += T) {
-      const int was = list[e];
-      int l = was;
-      f(l, e);
-      if (l != was) list[e] = l;
+    // eight loads of a thread in flight: a store may alias the next load
+    for (int e0 = tid; e0 < d; e0 += 8 * T) {
+      int was[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) was[u] = e0 + u * T < d ? list[e0 + u * T] : -1;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        int l = was[u];
+        f(l, e0 + u * T);
+        if (l != was[u]) list[e0 + u * T] = l;
+      }
     }
   }
 };
 
-// Sum of label x over the items not settled, for the whole team.
-template <int T, int WT, typename S, typename Items>
-__device__ __forceinline__ S team_sum_of(Items& items, const int* wp, unsigned x, TeamShared<T, S>* sh) {
-  unsigned long long mine = 0;
-  items.each([&](int& l, int e) {
-    if ((unsigned)l == x) mine += WT ? (unsigned long long)(unsigned)__ldg(wp + e) : 1ull;
-  });
-  mine = warp_sum_u64(mine);
-  if (T == 32) return (S)mine;
+// Sum of x over the team's threads.
+template <int T, typename S>
+__device__ __forceinline__ S team_total(unsigned long long x, TeamShared<T, S>* sh) {
+  x = warp_sum_u64(x);
+  if (T == 32) return (S)x;
   __syncthreads();
   if (threadIdx.x == 0) sh->wsum = 0;
   __syncthreads();
-  if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&sh->wsum, mine);
+  if ((threadIdx.x & 31) == 0 && x) atomicAdd(&sh->wsum, x);
   __syncthreads();
   return (S)sh->wsum;
 }
 
 // The counting round's outcome: `mine` is each thread's largest (running
-// sum, label) over its adds, counters hold the final sums.  Returns whether
-// `best` is the row's argmax; if not, the labels that could still beat it
-// are left open, `open_items` of them.
+// sum, label) over its adds, counters hold the final sums; `best` covers the
+// labels counted before (none: sum 0).  Returns whether it now covers these
+// too; if not, the labels that could still beat it are left open,
+// `open_items` of them.
 template <int T, int WT, typename S, typename Items>
-__device__ __forceinline__ bool sketch_top(Items& items, const int* wp, const Sketch<S>& t, Best<S> mine,
+__device__ __forceinline__ bool sketch_top(Items& items, const int* wp, const Sketch& t, Best<unsigned> mine,
                                            Best<S>& best, unsigned& open_items, TeamShared<T, S>* sh) {
-  best = team_best<T, S>(mine, sh);   // with the barrier that ends the adds
+  const Best<unsigned> top = team_best<T>(mine, sh);   // with the barrier that ends the adds
   open_items = 0;
-  if (best.sum == 0) return true;   // no neighbour but the vertex itself (team-uniform)
-  const unsigned x = ~best.inv, hx = t.slot(x);
-  bool other = false;
-  items.each([&](int& l, int) { other = other || (l >= 0 && (unsigned)l != x && t.slot((unsigned)l) == hx); });
-  if (!team_any<T>(other)) return true;
-  const S full = best.sum, sum = team_sum_of<T, WT, S>(items, wp, x, sh);
-  best.sum = sum;
+  // whether a label bounded by counter value c can beat `best`
+  auto can_beat = [&](unsigned c, unsigned inv) {
+    return WT == 2 ? ((unsigned long long)c << t.q) > (unsigned long long)best.sum : beats<S>((S)c, inv, best);
+  };
+  if (top.sum == 0 || !can_beat(top.sum, top.inv)) return true;   // team-uniform
+  const unsigned x = ~top.inv, hx = t.slot(x);
+  bool other = WT == 2;   // bounds always need the comparison with the exact sum
+  unsigned long long mine_x = 0;
+  items.each([&](int& l, int e) {
+    if (l >= 0) {
+      if ((unsigned)l == x) mine_x += WT ? (unsigned long long)(unsigned)wp[e] : 1ull;
+      else if (WT != 2) other = other || t.slot((unsigned)l) == hx;
+    }
+  });
+  if (WT != 2 && !team_any<T>(other)) {
+    best = {(S)top.sum, top.inv};
+    return true;
+  }
+  const S sum = team_total<T, S>(mine_x, sh);
+  const unsigned full = top.sum - (unsigned)(WT == 2 ? (unsigned long long)sum >> t.q : (unsigned long long)sum);
+  if (beats<S>(sum, top.inv, best)) best = {sum, top.inv};
   unsigned left = 0;
   items.each([&](int& l, int) {
     if (l >= 0) {
       const unsigned h = t.slot((unsigned)l);
-      const S c = h == hx ? full - sum : t.sum[h];   // a bound of every other label in the slot
-      if ((unsigned)l != x && beats<S>(c, ~(unsigned)l, best)) ++left;
+      const unsigned c = h == hx ? full : t.cnt[h];   // a bound of every other label in the slot
+      if ((unsigned)l != x && can_beat(c, ~(unsigned)l)) ++left;
       else l = (int)((unsigned)l | SETTLED);
     }
   });
@@ -211,24 +229,20 @@ __device__ __forceinline__ bool sketch_top(Items& items, const int* wp, const Sk
   return left == 0;
 }
 
-// Rounds first_round.. over the items whose label is not settled (and lies
-// in part `part` of `parts` by the second hash): on return all of those are
-// settled and `best` covers them.  Starts and ends with the team in step.
+// Rounds first_round.. over the items whose label is not settled: on return
+// all are, and `best` covers them.  Starts and ends with the team in step.
 template <int T, int WT, typename S, typename Items>
 __device__ __forceinline__ void sketch_rounds(Items& items, const int* wp, const Slots<S> t, int first_round,
-                                              int rounds, unsigned part, unsigned parts, Best<S>& best,
-                                              TeamShared<T, S>* sh, int* err) {
+                                              int rounds, Best<S>& best, TeamShared<T, S>* sh, int* err) {
   const int tid = T == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
-  auto open = [&](int l) {
-    return l >= 0 && (parts <= 1 || __umulhi((unsigned)l * 0x7FEB352Du, parts) == part);
-  };
+  auto open = [](int l) { return l >= 0; };
   for (int r = first_round;; ++r) {
-    sketch_clear<T, S>(t.sum, t.lg, tid);
+    sketch_clear<T>(t.sum, t.lg, tid);
     team_sync<T>();
     items.each([&](int& l, int e) {
       if (open(l)) {
         const unsigned h = t.slot((unsigned)l, r);
-        atomicAdd(t.sum + h, WT ? (S)(unsigned)__ldg(wp + e) : (S)1);
+        atomicAdd(t.sum + h, WT ? (S)(unsigned)wp[e] : (S)1);
         *(volatile unsigned*)(t.lab + h) = (unsigned)l;
       }
     });
@@ -248,7 +262,7 @@ __device__ __forceinline__ void sketch_rounds(Items& items, const int* wp, const
         if (t.lab[h] != EMPTY32 && beats<S>(c, ~(unsigned)l, mine)) mine = {c, ~(unsigned)l};
       }
     });
-    mine = team_best<T, S>(mine, sh);
+    mine = team_best<T>(mine, sh);
     if (beats<S>(mine.sum, mine.inv, best)) best = mine;
     bool left = false;
     items.each([&](int& l, int) {
@@ -280,7 +294,11 @@ __device__ __forceinline__ void sketch_rounds(Items& items, const int* wp, const
       x = sh->cnt;
     }
     if (x == EMPTY32) return;
-    const S c = team_sum_of<T, WT, S>(items, wp, x, sh);
+    unsigned long long of_x = 0;
+    items.each([&](int& l, int e) {
+      if ((unsigned)l == x) of_x += WT ? (unsigned long long)(unsigned)wp[e] : 1ull;
+    });
+    const S c = team_total<T, S>(of_x, sh);
     if (beats<S>(c, ~x, best)) best = {c, ~x};
     items.each([&](int& l, int) {
       if ((unsigned)l == x) l = (int)((unsigned)l | SETTLED);
@@ -289,11 +307,28 @@ __device__ __forceinline__ void sketch_rounds(Items& items, const int* wp, const
   }
 }
 
+// Counts the items (counters clear) and leaves `best` covering them.
+template <int T, int WT, typename S, typename Items>
+__device__ __forceinline__ void sketch_count(Items& items, const int* wp, const Sketch& t, int rounds,
+                                             Best<S>& best, TeamShared<T, S>* sh, int* err) {
+  Best<unsigned> mine{0, 0u};
+  items.each([&](int& x, int e) {
+    if (x >= 0) {
+      const unsigned w = counter_step<WT>(t, wp, e);
+      const unsigned c = atomicAdd(t.cnt + t.slot((unsigned)x), w) + w;
+      if (beats<unsigned>(c, ~(unsigned)x, mine)) mine = {c, ~(unsigned)x};
+    }
+  });
+  unsigned left;
+  if (!sketch_top<T, WT, S>(items, wp, t, mine, best, left, sh))
+    sketch_rounds<T, WT, S>(items, wp, Slots<S>(t), 1, rounds, best, sh, err);
+}
+
 // One row in registers, K entries per thread (d <= T * K), LG counters (log2).
 // GENERAL: first-sweep checks, identity labels, pre-gathered labels.
 template <int T, int K, int LG, int WT, bool ASYNC, bool GENERAL, typename S>
 __device__ __forceinline__ void sketch_row(const SweepArgs& a, int v, int old, const int* cp, const int* wp,
-                                           const int* lp, int d, int tid, S* mem, int rounds, const Pol& pol,
+                                           const int* lp, int d, int tid, unsigned* mem, int rounds, const Pol& pol,
                                            Best<S>& best, unsigned long long& ws, TeamShared<T, S>* sh) {
   int l[K];
 #pragma unroll
@@ -306,8 +341,8 @@ __device__ __forceinline__ void sketch_row(const SweepArgs& a, int v, int old, c
       if (GENERAL && WT && l[k] >= 0) ws += (unsigned long long)(unsigned)w;
     }
   }
-  const Sketch<S> t{mem, LG};
-  sketch_clear<T, S>(t.sum, LG, tid);   // under the column loads
+  const Sketch t{mem, LG, WT == 2 ? ceil_log2((unsigned)d) : 0u};
+  sketch_clear<T>(t.cnt, LG, tid);   // under the column loads
   if (GENERAL && a.ident) {
     // strictly increasing: every label (its id) occurs once
     bool inc = true;
@@ -317,12 +352,12 @@ __device__ __forceinline__ void sketch_row(const SweepArgs& a, int v, int old, c
       if (e < d && (l[k] < 0 || (e + 1 < d && __ldg(cp + e + 1) <= l[k]))) inc = false;
       check_same_graph(a, v, l[k]);
       if (l[k] >= 0 && l[k] != v) {
-        const S c = WT ? (S)(unsigned)__ldg(wp + e) : (S)1;
+        const S c = WT ? (S)(unsigned)wp[e] : (S)1;
         if (beats<S>(c, ~(unsigned)l[k], best)) best = {c, ~(unsigned)l[k]};
       }
     }
     if (!team_any<T>(!inc)) {
-      best = team_best<T, S>(best, sh);
+      best = team_best<T>(best, sh);
       return;
     }
     best = {0, 0u};
@@ -357,23 +392,13 @@ __device__ __forceinline__ void sketch_row(const SweepArgs& a, int v, int old, c
   }
   team_sync<T>();   // the counters are clear
   RegItems<T, K> items{l, d, tid};
-  Best<S> mine{0, 0u};
-  items.each([&](int& x, int e) {
-    if (x >= 0) {
-      const S w = WT ? (S)(unsigned)__ldg(wp + e) : (S)1;
-      const S c = atomicAdd(t.sum + t.slot((unsigned)x), w) + w;
-      if (beats<S>(c, ~(unsigned)x, mine)) mine = {c, ~(unsigned)x};
-    }
-  });
-  unsigned left;
-  if (!sketch_top<T, WT, S>(items, wp, t, mine, best, left, sh))
-    sketch_rounds<T, WT, S>(items, wp, Slots<S>(t), 1, rounds, 0u, 1u, best, sh, &a.ctr->err);
+  sketch_count<T, WT, S>(items, wp, t, rounds, best, sh, &a.ctr->err);
 }
 
 // One row through the block's scratch list.
 template <int T, int LG, int WT, bool ASYNC, bool GENERAL, typename S>
 __device__ __forceinline__ void sketch_long_row(const SweepArgs& a, int v, const int* cp, const int* wp,
-                                                const int* lp, int d, int tid, S* mem, int rounds, const Pol& pol,
+                                                const int* lp, int d, int tid, unsigned* mem, int rounds, const Pol& pol,
                                                 Best<S>& best, unsigned long long& ws, TeamShared<T, S>* sh) {
   if (GENERAL && a.ident) {
     // strictly increasing: every label (its id) occurs once
@@ -389,17 +414,17 @@ __device__ __forceinline__ void sketch_long_row(const SweepArgs& a, int v, const
       if (j >= 0 && j != v && beats<S>((S)(unsigned)w, ~(unsigned)j, best)) best = {(S)(unsigned)w, ~(unsigned)j};
     }
     if (!team_any<T>(!inc)) {
-      best = team_best<T, S>(best, sh);
+      best = team_best<T>(best, sh);
       ws = sum;
       return;
     }
     best = {0, 0u};
   }
   int* list = a.scratch + (long long)blockIdx.x * a.scratch_region;
-  const Sketch<S> t{mem, LG};
-  sketch_clear<T, S>(t.sum, LG, tid);
+  const Sketch t{mem, LG, WT == 2 ? ceil_log2((unsigned)d) : 0u};
+  sketch_clear<T>(t.cnt, LG, tid);
   team_sync<T>();
-  Best<S> mine{0, 0u};
+  Best<unsigned> mine{0, 0u};
   // gather and count; eight entries of a thread in flight
   for (int e0 = 0; e0 < d; e0 += 8 * T) {
     int l[8];
@@ -421,19 +446,69 @@ __device__ __forceinline__ void sketch_long_row(const SweepArgs& a, int v, const
       const int e = e0 + u * T + tid;
       if (e < d) list[e] = l[u];
       if (l[u] >= 0) {
-        const S w = WT ? (S)(unsigned)__ldg(wp + e) : (S)1;
-        const S c = atomicAdd(t.sum + t.slot((unsigned)l[u]), w) + w;
-        if (beats<S>(c, ~(unsigned)l[u], mine)) mine = {c, ~(unsigned)l[u]};
+        const unsigned w = counter_step<WT>(t, wp, e);
+        const unsigned c = atomicAdd(t.cnt + t.slot((unsigned)l[u]), w) + w;
+        if (beats<unsigned>(c, ~(unsigned)l[u], mine)) mine = {c, ~(unsigned)l[u]};
       }
     }
   }
   MemItems<T> items{list, d, tid};
   unsigned left;
-  if (!sketch_top<T, WT, S>(items, wp, t, mine, best, left, sh)) {
-    const Slots<S> slots(t);
-    const unsigned parts = (left >> slots.lg) + 1;
-    for (unsigned p = 0; p < parts; ++p)
-      sketch_rounds<T, WT, S>(items, wp, slots, 1, rounds, p, parts, best, sh, &a.ctr->err);
+  if (sketch_top<T, WT, S>(items, wp, t, mine, best, left, sh)) return;
+  if (left <= (1u << (LG - 2))) {
+    sketch_rounds<T, WT, S>(items, wp, Slots<S>(t), 1, rounds, best, sh, &a.ctr->err);
+    return;
+  }
+  // many labels of about the same weight: the open entries in parts by a
+  // second hash, each counted on its own with the best so far as a bound
+  constexpr int PART = T * 8;   // entries aimed at, half of what the registers hold
+  const unsigned lgp = min(6u, max(1u, ceil_log2(left / PART + 1)));
+  const unsigned np = 1u << lgp;
+  int* out = list + a.scratch_region / 3;
+  int* outw = out + a.scratch_region / 3;
+  auto part_of = [&](int l) { return ((unsigned)l * 0x7FEB352Du) >> (32u - lgp); };
+  __syncthreads();
+  if (tid < 64) sh->fill[tid] = 0;
+  __syncthreads();
+  items.each([&](int& l, int) {
+    if (l >= 0) atomicAdd(&sh->fill[part_of(l)], 1u);
+  });
+  __syncthreads();
+  if (tid == 0) {
+    unsigned run = 0;
+    for (unsigned p = 0; p < np; ++p) {
+      const unsigned n = sh->fill[p];
+      sh->part[p] = run;
+      sh->fill[p] = run;
+      run += n;
+    }
+    sh->part[np] = run;
+  }
+  __syncthreads();
+  items.each([&](int& l, int e) {
+    if (l >= 0) {
+      const unsigned at = atomicAdd(&sh->fill[part_of(l)], 1u);
+      out[at] = l;
+      if (WT) outw[at] = wp[e];
+    }
+  });
+  __syncthreads();
+  for (unsigned p = 0; p < np; ++p) {
+    const int from = (int)sh->part[p], n = (int)sh->part[p + 1] - from;
+    if (n == 0) continue;   // block-uniform
+    sketch_clear<T>(t.cnt, LG, tid);
+    __syncthreads();
+    if (n <= T * 16) {
+      int l[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) l[k] = k * T + tid < n ? out[from + k * T + tid] : -1;
+      RegItems<T, 16> part{l, n, tid};
+      sketch_count<T, WT, S>(part, outw + from, t, rounds, best, sh, &a.ctr->err);
+    } else {
+      MemItems<T> part{out + from, n, tid};
+      sketch_count<T, WT, S>(part, outw + from, t, rounds, best, sh, &a.ctr->err);
+    }
+    __syncthreads();
   }
 }
 
@@ -458,7 +533,7 @@ __global__ void __launch_bounds__(T == 32 ? 256 : T, T == 32 ? 4 : (T == T_SMALL
   extern __shared__ int4 smem_sketch[];
   __shared__ TeamShared<T, S> sh;
   const int tid = T == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
-  S* mem = reinterpret_cast<S*>(smem_sketch) + (T == 32 ? (size_t)(threadIdx.x >> 5) << team_lg<T>() : 0);
+  unsigned* mem = reinterpret_cast<unsigned*>(smem_sketch) + (T == 32 ? (size_t)(threadIdx.x >> 5) << team_lg<T>() : 0);
   const unsigned cnt = a.ctr->cls_count[cls];
   const int* __restrict__ work = a.work + a.ctr->cls_start[cls];
   const Pol pol = make_pol();
@@ -561,9 +636,8 @@ __global__ void __launch_bounds__(T == 32 ? 256 : T, T == 32 ? 4 : (T == T_SMALL
 namespace {
 template <int T, int WT, bool A, bool G>
 cudaError_t launch_sketch_g(const SweepArgs& a, int cls, const DeviceInfo& di, cudaStream_t s) {
-  using S = typename SumOf<WT>::T;
   constexpr int block = T == 32 ? 256 : T;
-  const size_t smem = (sizeof(S) << team_lg<T>()) * (size_t)(block / T);
+  const size_t smem = (sizeof(unsigned) << team_lg<T>()) * (size_t)(block / T);
   thread_local int grid = 0;
   if (!grid) {
     if (cudaError_t e = raise_smem_limit((const void*)sketch_kernel<T, WT, A, G>, smem)) return e;
@@ -604,7 +678,8 @@ long long sketch_register_row() { return (long long)T_BLOCK * K_BLOCK; }
 cudaError_t launch_sketch(const SweepArgs& a, int cls, int longest, int weights, bool async_mode,
                           const DeviceInfo& di, cudaStream_t s) {
   if (weights == 0) return launch_sketch_w<0>(a, cls, longest, async_mode, di, s);
-  return launch_sketch_w<1>(a, cls, longest, async_mode, di, s);
+  if (weights == 1) return launch_sketch_w<1>(a, cls, longest, async_mode, di, s);
+  return launch_sketch_w<2>(a, cls, longest, async_mode, di, s);
 }
 
 }  // namespace gsl

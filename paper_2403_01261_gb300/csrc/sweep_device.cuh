@@ -184,9 +184,25 @@ __device__ __forceinline__ unsigned label_group(int l, int spread) {
 // shared add (2.6 cycles of an SM, measured), two stores and two loads;
 // __match_any_sync costs 64 cycles there when the labels are distinct (two a
 // value) and 8 when there are four.
-struct SketchBest {
-  unsigned sum, inv;   // largest label sum so far and ~label (0: none)
+//
+// Weights WT: 0 unit, 1 int32 with 32-bit sums, 2 int32 with 64-bit sums (the
+// wide fixed-point form of float weights).
+template <int WT>
+struct SumOf { using T = unsigned; };
+template <>
+struct SumOf<2> { using T = unsigned long long; };
+
+// Best label so far: largest sum, then smallest label (inv = ~label).
+template <typename S>
+struct Best {
+  S sum;
+  unsigned inv;
 };
+
+template <typename S>
+__device__ __forceinline__ bool beats(S s, unsigned inv, const Best<S>& b) {
+  return s > b.sum || (s == b.sum && inv > b.inv);
+}
 
 __device__ __forceinline__ unsigned sketch_hash(unsigned x, int round) {
   if (round) x ^= x >> (11 + round);

@@ -33,8 +33,19 @@ constexpr int LANE_ROW = 4;          // longest row of one lane
 
 // Largest (sum, ~label) over the G lanes of gmask; lanes without one pass sum 0.
 template <int G>
-__device__ __forceinline__ SketchBest group_best(unsigned sum, int lbl, unsigned gmask) {
-  SketchBest b;
+__device__ __forceinline__ Best<unsigned long long> group_best(unsigned long long sum, int lbl, unsigned gmask) {
+  Best<unsigned long long> b{sum, sum ? ~(unsigned)lbl : 0u};
+#pragma unroll
+  for (int o = G / 2; o >= 1; o >>= 1) {
+    const unsigned long long s = __shfl_xor_sync(FULL, b.sum, o);
+    const unsigned i = __shfl_xor_sync(FULL, b.inv, o);
+    if (beats<unsigned long long>(s, i, b)) b = {s, i};
+  }
+  return b;
+}
+template <int G>
+__device__ __forceinline__ Best<unsigned> group_best(unsigned sum, int lbl, unsigned gmask) {
+  Best<unsigned> b;
   if (G >= 16) {
     b.sum = __reduce_max_sync(gmask, sum);
     b.inv = __reduce_max_sync(gmask, (sum && sum == b.sum) ? ~(unsigned)lbl : 0u);
@@ -49,48 +60,66 @@ __device__ __forceinline__ SketchBest group_best(unsigned sum, int lbl, unsigned
   return b;
 }
 
-__device__ __forceinline__ void take_better(SketchBest& a, const SketchBest& b) {
-  if (b.sum > a.sum || (b.sum == a.sum && b.inv > a.inv)) a = b;
+template <typename S>
+__device__ __forceinline__ void take_better(Best<S>& a, const Best<S>& b) {
+  if (beats<S>(b.sum, b.inv, a)) a = b;
 }
 
+// Sum of a value over the lanes of mask m (the calling lane's among them).
+__device__ __forceinline__ unsigned mask_sum(unsigned m, unsigned x) { return __reduce_add_sync(m, x); }
+__device__ __forceinline__ unsigned long long mask_sum(unsigned m, unsigned long long x) {   // x below 2^31
+  const unsigned lo = __reduce_add_sync(m, (unsigned)x & 0xFFFFu), hi = __reduce_add_sync(m, (unsigned)x >> 16);
+  return ((unsigned long long)hi << 16) + lo;
+}
+
+// A warp's sketch slots: sums and labels.
+template <typename S>
+struct GroupSlots {
+  S sum[GROUP_SLOTS];
+  unsigned lab[GROUP_SLOTS];
+};
+
 // Eq. 2's argmax of a group of G lanes, one entry each, in the group's 4 G
-// slots (x: sum, all zero on entry and on return; y: label).
+// slots from `base` on (sums all zero on entry and on return).
 // Warp-synchronous; the slots of a warp's groups are disjoint.
-template <int G>
-__device__ __forceinline__ SketchBest group_sketch(uint2* slots, int lbl, unsigned wt, bool valid, unsigned gmask,
-                                                   int rounds, int* err) {
+template <int G, typename S>
+__device__ __forceinline__ Best<S> group_sketch(GroupSlots<S>& slots, int base, int lbl, S wt, bool valid,
+                                                unsigned gmask, int rounds, int* err) {
   constexpr int SHIFT = G == 32 ? 25 : (G == 16 ? 26 : 27);   // 4 G slots
-  SketchBest best{0u, 0u};
+  Best<S> best{0, 0u};
   bool act = valid;
   for (int r = 0;; ++r) {
-    volatile uint2* sl = slots + (sketch_hash((unsigned)lbl, r) >> SHIFT);
+    const int h = base + (int)(sketch_hash((unsigned)lbl, r) >> SHIFT);
+    volatile S* sum = slots.sum + h;
+    volatile unsigned* lab = slots.lab + h;
     if (act) {
-      atomicAdd(const_cast<unsigned*>(&sl->x), wt);
-      sl->y = (unsigned)lbl;
+      atomicAdd(slots.sum + h, wt);
+      *lab = (unsigned)lbl;
     }
     __syncwarp();
-    unsigned c = 0;
+    S c = 0;
     bool shared_slot = false;
     if (act) {
-      c = sl->x;
-      shared_slot = sl->y != (unsigned)lbl;
+      c = *sum;
+      shared_slot = *lab != (unsigned)lbl;
     }
     if (__any_sync(FULL, shared_slot)) {   // the label that won the store learns of the others
       __syncwarp();
-      if (shared_slot) sl->y = EMPTY32;
+      if (shared_slot) *lab = EMPTY32;
       __syncwarp();
-      if (act) shared_slot = sl->y == EMPTY32;
+      if (act) shared_slot = *lab == EMPTY32;
     }
     __syncwarp();
-    if (act) sl->x = 0;
+    if (act) *sum = 0;
     __syncwarp();
-    take_better(best, group_best<G>(act && !shared_slot ? c : 0u, lbl, gmask));
-    act = act && shared_slot && (c - 1 > best.sum || (c - 1 == best.sum && ~(unsigned)lbl > best.inv));
+    take_better(best, group_best<G>(act && !shared_slot ? c : (S)0, lbl, gmask));
+    act = act && shared_slot && beats<S>(c - 1, ~(unsigned)lbl, best);
     if (!__any_sync(FULL, act)) return best;
     if (r + 1 >= rounds) {
       if (rounds < SKETCH_ROUNDS) raise_err(err, ERRBIT_TIMEOUT);   // a lowered retry bound
       const unsigned m = __match_any_sync(FULL, act ? lbl : -1) & gmask;
-      const unsigned e = act ? __reduce_add_sync(m, wt) : 0u;
+      S e = 0;
+      if (act) e = mask_sum(m, wt);   // m: the lanes of this label, all here
       take_better(best, group_best<G>(e, lbl, gmask));
       return best;
     }
@@ -98,8 +127,9 @@ __device__ __forceinline__ SketchBest group_sketch(uint2* slots, int lbl, unsign
 }
 
 // The largest (sum, smallest label) over a lane's labels in registers, -1 for none.
+template <typename S>
 __device__ __forceinline__ int lane_argmax(const int* l, const unsigned* w, int old) {
-  unsigned c[LANE_ROW];
+  S c[LANE_ROW];
 #pragma unroll
   for (int i = 0; i < LANE_ROW; ++i) c[i] = w[i];
 #pragma unroll
@@ -111,7 +141,7 @@ __device__ __forceinline__ int lane_argmax(const int* l, const unsigned* w, int 
       c[k] += same ? w[i] : 0u;
     }
   }
-  unsigned bc = 0;
+  S bc = 0;
   int bl = old;
 #pragma unroll
   for (int i = 0; i < LANE_ROW; ++i) {
@@ -126,14 +156,14 @@ __device__ __forceinline__ int lane_argmax(const int* l, const unsigned* w, int 
 // Neighbour and weight of entry e.  FIRST: with the first sweep's checks;
 // later sweeps only clamp an out-of-range column away (the first sweep, or
 // the streaming check before it, has reported it).
-template <bool WEIGHTED, bool FIRST>
+template <int WT, bool FIRST>
 __device__ __forceinline__ void tile_entry(const SweepArgs& a, const int* cp, const int* wp, int d, int e,
                                            const Pol& pol, int& j, int& wt) {
   if (FIRST) {
-    load_entry<WEIGHTED>(a, cp, wp, d, e, pol, j, wt);
+    load_entry<WT != 0>(a, cp, wp, d, e, pol, j, wt);
   } else {
     j = later_col(a, cp, d, e, pol);
-    wt = WEIGHTED && e < d ? ld_stream(wp + e, pol.stream) : (e < d ? 1 : 0);
+    wt = WT && e < d ? ld_stream(wp + e, pol.stream) : (e < d ? 1 : 0);
   }
 }
 
@@ -150,9 +180,11 @@ __device__ __forceinline__ int tile_label(const SweepArgs& a, int j, int v, cons
 // The tile's rows, one per lane (lanes 0..rows-1: vertex v, row start s,
 // degree d <= G, own label old), counted 32 / G per step by G lanes each.
 // Lane r receives row r's label in `nl`.
-template <bool WEIGHTED, bool ASYNC, bool FIRST, int G>
+template <int WT, bool ASYNC, bool FIRST, int G>
 __device__ __forceinline__ void tile_steps(const SweepArgs& a, int rows, int v, long long s, int d, int old,
-                                           uint2* slots, int rounds, const Pol& pol, int& nl) {
+                                           GroupSlots<typename SumOf<WT>::T>* slots, int rounds, const Pol& pol,
+                                           int& nl) {
+  using S = typename SumOf<WT>::T;
   const int lane = threadIdx.x & 31;
   constexpr int PER = 32 / G;   // rows per step
   const unsigned gmask = G == 32 ? FULL : ((1u << (G & 31)) - 1u) << (lane & ~(G - 1));
@@ -165,7 +197,7 @@ __device__ __forceinline__ void tile_steps(const SweepArgs& a, int rows, int v, 
     const int r = row_at(t);
     const long long rs = __shfl_sync(FULL, s, r & 31);
     const int rd = __shfl_sync(FULL, d, r & 31);
-    tile_entry<WEIGHTED, FIRST>(a, a.col + rs, a.w + rs, r < rows ? rd : 0, e, pol, j, w);
+    tile_entry<WT, FIRST>(a, a.col + rs, a.w + rs, r < rows ? rd : 0, e, pol, j, w);
   };
 #pragma unroll
   for (int u = 0; u < TILE_U; ++u) load(u, jn[u], wn[u]);
@@ -189,7 +221,7 @@ __device__ __forceinline__ void tile_steps(const SweepArgs& a, int rows, int v, 
       const int own = __shfl_sync(FULL, old, r & 31);
       const int lbl = l[u];
       const bool nb = j[u] >= 0, valid = lbl >= 0;
-      if (WEIGHTED && FIRST && a.check) {
+      if (WT == 1 && FIRST && a.check) {
         unsigned long long ws = nb ? (unsigned long long)w[u] : 0ull;
 #pragma unroll
         for (int o = G / 2; o >= 1; o >>= 1) ws += __shfl_xor_sync(FULL, ws, o);
@@ -200,27 +232,27 @@ __device__ __forceinline__ void tile_steps(const SweepArgs& a, int rows, int v, 
       // increasing row, whose labels are all distinct.  The votes are the
       // whole warp's and stand outside every lane's condition.
       bool settled;
-      SketchBest b;
+      Best<S> b;
       if (FIRST && a.ident) {
         const int jp = __shfl_up_sync(FULL, j[u], 1, G);
         const int dd = __shfl_sync(FULL, d, r & 31);
         const unsigned ok = __ballot_sync(FULL, r >= rows || e >= dd || (nb && (e == 0 || jp < j[u])));
         settled = (ok & gmask) == gmask;
-        b = group_best<G>(valid ? (unsigned)w[u] : 0u, lbl, gmask);
+        b = group_best<G>(valid ? (S)(unsigned)w[u] : (S)0, lbl, gmask);
       } else {
         const unsigned all = __ballot_sync(FULL, valid) & gmask;
         const unsigned mine = __ballot_sync(FULL, valid && lbl == own) & gmask;
-        settled = all == 0 || (!WEIGHTED && 2 * __popc(mine) > __popc(all));
-        b = {settled ? (unsigned)__popc(mine) : 0u, ~(unsigned)own};
+        settled = all == 0 || (!WT && 2 * __popc(mine) > __popc(all));
+        b = {settled ? (S)__popc(mine) : (S)0, ~(unsigned)own};
       }
       if (!__all_sync(FULL, settled)) {
-        SketchBest x;
-        if (WEIGHTED) {
-          x = group_sketch<G>(slots + 4 * (lane & ~(G - 1)), lbl, (unsigned)w[u], valid && !settled, gmask, rounds,
-                              &a.ctr->err);
+        Best<S> x;
+        if (WT) {
+          x = group_sketch<G, S>(*slots, 4 * (lane & ~(G - 1)), lbl, (S)(unsigned)w[u], valid && !settled, gmask,
+                                 rounds, &a.ctr->err);
         } else {
           const unsigned m = __match_any_sync(FULL, lbl) & gmask;
-          x = group_best<G>(valid ? (unsigned)__popc(m) : 0u, lbl, gmask);
+          x = group_best<G>(valid ? (S)__popc(m) : (S)0, lbl, gmask);
         }
         if (!settled) b = x;
       }
@@ -271,7 +303,7 @@ __device__ __forceinline__ void count_tile_changes(const SweepArgs& a, int v, bo
 // Classes 0..2 among the vertices [v0, v1): all of them (all_active) or
 // those flagged in fcur, whose flags are cleared; with ASYNC only the
 // vertices of `phase`.
-template <bool WEIGHTED, bool ASYNC, bool FIRST>
+template <int WT, bool ASYNC, bool FIRST>
 __global__ void __launch_bounds__(TILE_BLOCK, LANE_MIN_BLOCKS)
     lane_sweep_kernel(SweepArgs a, long long v0, long long v1, unsigned char* __restrict__ fcur, int all_active,
                       const unsigned char* __restrict__ done, int phase, unsigned seed) {
@@ -312,7 +344,7 @@ __global__ void __launch_bounds__(TILE_BLOCK, LANE_MIN_BLOCKS)
         wt[k] = 1;
         if (k < d) {
           l[k] = __ldg(a.col + s + k);   // neighbouring rows share sectors: through L1
-          if (WEIGHTED) wt[k] = (unsigned)__ldg(a.w + s + k);
+          if (WT) wt[k] = (unsigned)__ldg(a.w + s + k);
         }
       }
       const int old = d ? own_label<ASYNC>(a, (int)v) : 0;
@@ -321,17 +353,17 @@ __global__ void __launch_bounds__(TILE_BLOCK, LANE_MIN_BLOCKS)
       for (int k = 0; k < LANE_ROW; ++k) {
         int j = l[k];
         if (FIRST && k < d) {
-          if ((unsigned)j >= (unsigned)a.n || (WEIGHTED && a.check && (int)wt[k] <= 0)) {
+          if ((unsigned)j >= (unsigned)a.n || (WT && a.check && (int)wt[k] <= 0)) {
             raise_err(&a.ctr->err, ERRBIT_INVALID);
             j = -1;
           }
-          if (WEIGHTED && j >= 0) ws += wt[k];
+          if (WT == 1 && j >= 0) ws += wt[k];
         }
         if (!FIRST && (unsigned)j >= (unsigned)a.n) j = -1;
         l[k] = tile_label<ASYNC, FIRST>(a, j, (int)v, pol);
       }
-      if (WEIGHTED && FIRST && a.check && ws >= (1ull << 31)) raise_err(&a.ctr->err, ERRBIT_OVERFLOW);
-      const int nl = lane_argmax(l, wt, old);
+      if (WT == 1 && FIRST && a.check && ws >= (1ull << 31)) raise_err(&a.ctr->err, ERRBIT_OVERFLOW);
+      const int nl = lane_argmax<typename SumOf<WT>::T>(l, wt, old);
       const bool changed = d > 0 && nl != old;
       if (d) {
         store_label<ASYNC>(a, (int)v, nl, changed);
@@ -357,14 +389,15 @@ __global__ void __launch_bounds__(TILE_BLOCK, LANE_MIN_BLOCKS)
 }
 
 // Class 3, 4 or 5 (G = 8, 16, 32), from the worklist.
-template <bool WEIGHTED, bool ASYNC, bool FIRST, int G>
+template <int WT, bool ASYNC, bool FIRST, int G>
 __global__ void __launch_bounds__(TILE_BLOCK, TILE_MIN_BLOCKS) tile_sweep_kernel(SweepArgs a) {
   if (stopped(a)) return;
   constexpr int cls = G == 8 ? 3 : (G == 16 ? 4 : 5);
-  __shared__ uint2 sketch[TILE_BLOCK / 32][WEIGHTED ? GROUP_SLOTS : 1];
+  using S = typename SumOf<WT>::T;
+  __shared__ GroupSlots<S> sketch[WT ? TILE_BLOCK / 32 : 1];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (WEIGHTED) {
-    for (int k = lane; k < GROUP_SLOTS; k += 32) sketch[wid][k].x = 0;
+  if (WT) {
+    for (int k = lane; k < GROUP_SLOTS; k += 32) sketch[wid].sum[k] = 0;
     __syncwarp();
   }
   const Pol pol = make_pol();
@@ -389,7 +422,7 @@ __global__ void __launch_bounds__(TILE_BLOCK, TILE_MIN_BLOCKS) tile_sweep_kernel
       old = own_label<ASYNC>(a, v);
     }
     int nl = old;
-    tile_steps<WEIGHTED, ASYNC, FIRST, G>(a, rows, v, s, d, old, sketch[wid], rounds, pol, nl);
+    tile_steps<WT, ASYNC, FIRST, G>(a, rows, v, s, d, old, WT ? sketch + wid : sketch, rounds, pol, nl);
     const bool changed = mine && nl != old;
     if (mine) {
       store_label<ASYNC>(a, v, nl, changed);
@@ -417,7 +450,7 @@ __global__ void __launch_bounds__(TILE_BLOCK, TILE_MIN_BLOCKS) tile_sweep_kernel
 }
 
 namespace {
-template <bool W, bool A>
+template <int W, bool A>
 void launch_lane_t(const SweepArgs& a, long long v0, long long v1, unsigned char* fcur, int all_active,
                    const unsigned char* done, int phase, unsigned seed, const DeviceInfo& di, cudaStream_t s) {
   const long long need = (v1 - v0 + TILE_BLOCK - 1) / TILE_BLOCK, most = (long long)LANE_MIN_BLOCKS * di.sm_count;
@@ -428,7 +461,7 @@ void launch_lane_t(const SweepArgs& a, long long v0, long long v1, unsigned char
     lane_sweep_kernel<W, A, false><<<grid, TILE_BLOCK, 0, s>>>(a, v0, v1, fcur, all_active, done, phase, seed);
 }
 
-template <bool W, bool A, bool F>
+template <int W, bool A, bool F>
 void launch_tile_f(const SweepArgs& a, int cls, const DeviceInfo& di, cudaStream_t s) {
   const int grid = TILE_MIN_BLOCKS * di.sm_count;
   if (cls == 3) tile_sweep_kernel<W, A, F, 8><<<grid, TILE_BLOCK, 0, s>>>(a);
@@ -436,37 +469,41 @@ void launch_tile_f(const SweepArgs& a, int cls, const DeviceInfo& di, cudaStream
   else tile_sweep_kernel<W, A, F, 32><<<grid, TILE_BLOCK, 0, s>>>(a);
 }
 
-template <bool W, bool A>
+template <int W, bool A>
 void launch_tile_t(const SweepArgs& a, int cls, const DeviceInfo& di, cudaStream_t s) {
   if (a.check || a.ident) launch_tile_f<W, A, true>(a, cls, di, s);
   else launch_tile_f<W, A, false>(a, cls, di, s);
 }
 }  // namespace
 
-cudaError_t launch_sweep_lanes(const SweepArgs& a, bool weighted, bool async_mode, long long v0, long long v1,
+cudaError_t launch_sweep_lanes(const SweepArgs& a, int weights, bool async_mode, long long v0, long long v1,
                                unsigned char* fcur, int all_active, const unsigned char* done, int phase,
                                unsigned seed, const DeviceInfo& di, cudaStream_t s) {
   if (v1 <= v0) return cudaSuccess;
-  if (weighted) {
-    if (async_mode) launch_lane_t<true, true>(a, v0, v1, fcur, all_active, done, phase, seed, di, s);
-    else launch_lane_t<true, false>(a, v0, v1, fcur, all_active, done, phase, seed, di, s);
-  } else {
-    if (async_mode) launch_lane_t<false, true>(a, v0, v1, fcur, all_active, done, phase, seed, di, s);
-    else launch_lane_t<false, false>(a, v0, v1, fcur, all_active, done, phase, seed, di, s);
+  switch (2 * weights + (async_mode ? 1 : 0)) {
+    case 0: launch_lane_t<0, false>(a, v0, v1, fcur, all_active, done, phase, seed, di, s); break;
+    case 1: launch_lane_t<0, true>(a, v0, v1, fcur, all_active, done, phase, seed, di, s); break;
+    case 2: launch_lane_t<1, false>(a, v0, v1, fcur, all_active, done, phase, seed, di, s); break;
+    case 3: launch_lane_t<1, true>(a, v0, v1, fcur, all_active, done, phase, seed, di, s); break;
+    case 4: launch_lane_t<2, false>(a, v0, v1, fcur, all_active, done, phase, seed, di, s); break;
+    case 5: launch_lane_t<2, true>(a, v0, v1, fcur, all_active, done, phase, seed, di, s); break;
+    default: return cudaErrorInvalidValue;
   }
   count_launches(1);
   return cudaGetLastError();
 }
 
-cudaError_t launch_sweep_tile(const SweepArgs& a, int cls, bool weighted, bool async_mode, const DeviceInfo& di,
+cudaError_t launch_sweep_tile(const SweepArgs& a, int cls, int weights, bool async_mode, const DeviceInfo& di,
                               cudaStream_t s) {
   if (cls < 3 || cls > 5) return cudaErrorInvalidValue;
-  if (weighted) {
-    if (async_mode) launch_tile_t<true, true>(a, cls, di, s);
-    else launch_tile_t<true, false>(a, cls, di, s);
-  } else {
-    if (async_mode) launch_tile_t<false, true>(a, cls, di, s);
-    else launch_tile_t<false, false>(a, cls, di, s);
+  switch (2 * weights + (async_mode ? 1 : 0)) {
+    case 0: launch_tile_t<0, false>(a, cls, di, s); break;
+    case 1: launch_tile_t<0, true>(a, cls, di, s); break;
+    case 2: launch_tile_t<1, false>(a, cls, di, s); break;
+    case 3: launch_tile_t<1, true>(a, cls, di, s); break;
+    case 4: launch_tile_t<2, false>(a, cls, di, s); break;
+    case 5: launch_tile_t<2, true>(a, cls, di, s); break;
+    default: return cudaErrorInvalidValue;
   }
   count_launches(1);
   return cudaGetLastError();
