@@ -483,6 +483,8 @@ __global__ void __launch_bounds__(256) mod_f_square_kernel(const double* __restr
 // (the vertex itself excluded); a strict majority keeps the label (Eq. 2's
 // argmax), other rows go to `out` for the table kernel.  Four 32-entry
 // chunks are loaded before they are summed.
+constexpr int F_FILTER_MAX = 32768;
+
 template <bool ASYNC>
 __global__ void __launch_bounds__(256) majority_filter_f_kernel(SweepArgs a, const float* __restrict__ wf,
                                                                 int* __restrict__ out) {
@@ -501,7 +503,8 @@ __global__ void __launch_bounds__(256) majority_filter_f_kernel(SweepArgs a, con
     const int d = (int)(a.off[v + 1] - s);
     const int old = own_label<ASYNC>(a, v);
     double ow = 0.0, tw = 0.0;
-    for (int e0 = 0; e0 < d; e0 += 128) {
+    const bool read = d <= F_FILTER_MAX;   // a warp takes too long over longer rows
+    for (int e0 = 0; read && e0 < d; e0 += 128) {
       int j[4];
       float w[4];
 #pragma unroll
@@ -576,7 +579,7 @@ cudaError_t launch_majority_filter_f32(const SweepArgs& a, const float* wf, int*
   else majority_filter_f_kernel<false><<<grid, 256, 0, s>>>(a, wf, out);
   count_launches(1);
   if (cudaError_t e = cudaGetLastError()) return e;
-  return launch_filter_counts(a.ctr, a.stop, s);
+  return launch_filter_counts(a.ctr, a.stop, s, CLS_WARP_L, CLS_BLOCK);
 }
 
 cudaError_t launch_sweep_f32(const SweepArgs& a, const float* wf, int cls, bool async_mode, unsigned* gkeys,

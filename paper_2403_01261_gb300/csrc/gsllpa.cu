@@ -43,12 +43,16 @@ struct gsl_ctx {
   unsigned* fkeys = nullptr;            // float-weight sweep: global table regions (keys, sums)
   double* fvals = nullptr;
   long long cap_fkeys = 0, cap_fvals = 0;
+  unsigned* gbits = nullptr;            // majority filter: vertices carrying the giant label
+  long long cap_gbits = 0;
   int* work2 = nullptr;                 // worklist of the rows the majority filter leaves
   long long cap_work2 = 0;
   int* lg = nullptr;                    // labels gathered per CSR entry (two-phase sweeps)
   long long cap_lg = 0;
   int* scratch = nullptr;               // label lists of rows longer than a block's registers
   long long cap_scratch = 0;
+  int* hub_scratch = nullptr;           // the same for class 9 rows
+  long long cap_hub_scratch = 0;
   // class 9 in pieces (hub_kernels.cu)
   int* hub_piece_start = nullptr;
   long long* hub_ustart = nullptr;
@@ -284,6 +288,13 @@ long long class_vertices(const gsl_ctx* c, int first, int last) {
   return v;
 }
 
+// Class 9 rows go to the hub kernels (clusters, pieces) when one is longer than
+// a block should be left with, or when the class starts below its default
+// bound; else to the block kernel.  A block takes about 1 ms per million
+// entries; R-MAT 25's rows of 131,073..864,000 entries beside the shorter ones
+// cost less there than in clusters of their own (2.3 ms a call).
+constexpr long long HUB_BLOCK_MAX = 1ll << 20;
+
 // Resets all counters, classifies every vertex by degree (validating the
 // offsets) and sizes the hub tables.  Synchronises the stream.
 int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s) {
@@ -301,7 +312,8 @@ int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s) {
   // class 9 (hubs) in pieces: per-hub plan arrays and table regions
   const long long hubs = (long long)c->ctr_h->cls_total[CLS_HUB];
   const long long hub_e = (long long)c->ctr_h->hub_entries;
-  c->hub_ready = hubs > 0 && hub_pieces_fit(c->tune) && 2 * hub_e < (1ll << 32);
+  c->hub_ready = hubs > 0 && (maxd > HUB_BLOCK_MAX || c->tune.blk_max < Tuning().blk_max) &&
+                 hub_pieces_fit(c->tune) && 2 * hub_e < (1ll << 32);
   if (c->hub_ready) {
     const long long old_tab = c->cap_hub_tab;
     const unsigned long long* old_ptr = c->hub_tab;
@@ -328,20 +340,26 @@ int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s) {
 }
 
 
-// Label lists for the rows of up to `longest` entries that one block sweeps.
-int ensure_scratch(gsl_ctx* c, long long longest, SweepArgs* a) {
+// Label lists for the rows that one block sweeps.
+int ensure_scratch(gsl_ctx* c, bool hub_kernels, SweepArgs* a) {
+  const long long maxd = c->ctr_h->max_degree;
+  const long long longest = maxd < c->tune.blk_max ? maxd : c->tune.blk_max;
   a->scratch_region = longest > sketch_register_row() ? 3 * longest : 0;   // labels, parts, their weights
   if (a->scratch_region)
     if (int r = grow(c, c->scratch, c->cap_scratch, sketch_blocks(c->di) * a->scratch_region)) return r;
   a->scratch = c->scratch;
+  a->hub_blocks = 0;
+  const long long hubs = (long long)c->ctr_h->cls_total[CLS_HUB];
+  if (hubs > 0 && !hub_kernels) {
+    // one block per SM takes hub rows, fewer when their lists would pass 4 GB
+    a->hub_region = 3 * maxd;
+    long long blocks = (1ll << 30) / a->hub_region;
+    blocks = blocks < 1 ? 1 : (blocks > c->di.sm_count ? c->di.sm_count : blocks);
+    a->hub_blocks = (int)(blocks > hubs ? hubs : blocks);
+    if (int r = grow(c, c->hub_scratch, c->cap_hub_scratch, a->hub_blocks * a->hub_region)) return r;
+    a->hub_scratch = c->hub_scratch;
+  }
   return GSL_OK;
-}
-
-// Longest row the block kernel sweeps: hubs go to their own kernels when the
-// plan for them is ready.
-long long longest_block_row(const gsl_ctx* c) {
-  const long long maxd = c->ctr_h->max_degree;
-  return c->hub_ready && maxd > c->tune.blk_max ? c->tune.blk_max : maxd;
 }
 
 int reset_sweep_counters(gsl_ctx* c, cudaStream_t s) {
@@ -385,11 +403,10 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
   a.ctr = c->ctr;
   a.probe_cap = c->tune.probe_cap;
   a.work = c->work;
-  // the hub kernels sum in 32 bits: with 64-bit sums their rows are block rows
-  const bool hub_kernels = c->hub_ready && !wide;
-  if (int r = ensure_scratch(c, wide ? (long long)c->ctr_h->max_degree : longest_block_row(c), &a)) return r;
+  const bool hub_kernels = c->hub_ready && !wide   /* 32-bit sums */;
+  if (int r = ensure_scratch(c, hub_kernels, &a)) return r;
   a.n = n;
-  if (wt == 1) {   // weighted degrees, written by sweep 1 for the early stops of later sweeps
+  if (wt) {   // weighted degrees, written by sweep 1 for the early stops of later sweeps
     if (int r = grow(c, c->kw, c->cap_kw, n)) return r;
     a.kw = c->kw;
   }
@@ -454,8 +471,10 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
     // (sweep 2 reads the labels of sweep 1, which are nearly all distinct):
     // filter those out before the tables
     const bool filter = !a.ident && !a.check && (c->tune.majority == 2 || (c->tune.majority == 1 && t >= 3));
-    if (filter)
+    if (filter) {
       if (int r = grow(c, c->work2, c->cap_work2, n)) return r;
+      if (int r = grow(c, c->gbits, c->cap_gbits, (n >> 5) + 1)) return r;
+    }
     // from FILTER6_FROM on the filter takes class 6 (rows of 33..warp_small
     // entries) as well
     const int filter_from = (filter && t >= FILTER6_FROM) ? CLS_WARP_S : CLS_WARP_L;
@@ -479,25 +498,26 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
         }
         prof_end(c, pe, SL_BIN, s, 1);
       }
-      SweepArgs af = a;   // the filtered classes read the filter's worklist
-      if (filter && class_vertices(c, filter_from, CLS_BLOCK) > 0) {
+      a.work2 = nullptr;
+      if (filter && class_vertices(c, CLS_WARP_S, CLS_HUB) > 0) {
         const int pe = prof_begin(c, s);
-        CK(launch_majority_filter(a, c->work2, wt, async_mode, c->di, s, filter_from));
-        prof_end(c, pe, SL_FILTER, s, 2);
-        af.work = c->work2;
+        int kernels = 0;
+        CK(launch_majority_filter(a, g->nnz, c->work2, c->gbits, wt, async_mode, filter_from, true, (unsigned)t,
+                                  class_vertices(c, CLS_WARP_S, CLS_WARP_L) > 0,
+                                  class_vertices(c, CLS_BLOCK, CLS_HUB) > 0, c->di, s, &kernels));
+        prof_end(c, pe, SL_FILTER, s, kernels);
+        a.work2 = c->work2;   // the filtered classes read the filter's worklist
       }
       for (int k = NCLASS - 1; k >= CLS_BINNED; --k) {   // the longest rows first
-        if (class_vertices(c, k, k) == 0) continue;
+        if (class_vertices(c, k, k) == 0 && !(k == CLS_BLOCK && a.hub_blocks)) continue;
+        if (k == CLS_HUB && !hub_kernels) continue;   // with class 8
         const int pe = prof_begin(c, s);
-        if (k == CLS_WARP_L || k == CLS_BLOCK || (k == CLS_WARP_S && filter_from == CLS_WARP_S)) {
-          CK(launch_sweep_class(af, k, wt, async_mode, c->tune, maxd, c->di, s));
-          prof_end(c, pe, SL_SWEEP0 + k, s, 1);
-        } else if (k == CLS_HUB && hub_kernels) {
+        if (k == CLS_HUB) {
           HubPlan hp{c->hub_piece_start, c->hub_ustart, c->hub_best, c->hub_own,
                      c->hub_wsum,        c->hub_used_cnt, c->hub_used, c->hub_tab, c->hub_clu};
           c->hub_dirty = true;   // until this sweep is known to have finished cleanly
           int kernels = 0;
-          CK(launch_hub_pieces(a, hp, wt != 0, async_mode, filter, c->tune, c->di, s, &kernels));
+          CK(launch_hub_pieces(a, hp, wt != 0, async_mode, c->tune, c->di, s, &kernels));
           prof_end(c, pe, SL_SWEEP0 + k, s, kernels);
         } else {
           CK(launch_sweep_class(a, k, wt, async_mode, c->tune, maxd, c->di, s));
@@ -535,13 +555,13 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
       sl.vertices += (long long)c->ctr_h->tile_active;
       sl.entries += (long long)c->ctr_h->tile_scanned;
       sl.bytes += (per_v - 4.0) * (double)c->ctr_h->tile_active + per_e * (double)c->ctr_h->tile_scanned;
-      if (filter) {
-        // the filter read every row of classes 7 and 8: the settled ones (their
+      if (a.work2) {
+        // the filter read the rows of its classes: the settled ones (their
         // entries are in `scanned` but in no class) and those it passed on
         long long cls_e = (long long)c->ctr_h->tile_scanned, rows = (long long)c->ctr_h->fast_active;
         for (int k = 0; k < NCLASS; ++k) cls_e += (long long)c->ctr_h->cls_scanned[k];
         long long fe = (long long)c->ctr_h->scanned - cls_e;
-        for (int k = CLS_WARP_L; k <= CLS_BLOCK; ++k) {
+        for (int k = c->ctr_h->filter_from; k <= CLS_HUB; ++k) {
           fe += (long long)c->ctr_h->cls_scanned[k];
           rows += (long long)(c->ctr_h->cls_count[k] + c->ctr_h->phase_cls[k]);
         }
@@ -869,8 +889,7 @@ cudaError_t enqueue_batch_sweeps(gsl_ctx* c, const gsl_csr* g, int num_graphs, c
   a.ctr = c->ctr;
   a.probe_cap = c->tune.probe_cap;
   a.work = c->work;
-  a.scratch = c->scratch;   // allocated before the capture
-  a.scratch_region = 3 * c->ctr_h->max_degree;
+  ck(ensure_scratch(c, false, &a) == GSL_OK ? cudaSuccess : cudaErrorMemoryAllocation);   // in place since before a capture
   a.n = n;
   a.gid = c->gid;
   a.vptr = c->vptr;
@@ -900,19 +919,21 @@ cudaError_t enqueue_batch_sweeps(gsl_ctx* c, const gsl_csr* g, int num_graphs, c
                       c->stop, async_mode ? ph : -1, (unsigned)t, CLS_BINNED));
         if (prof) prof_end(c, pe, SL_BIN, cs, 1);
       }
-      SweepArgs af = a;
-      if (filter && class_vertices(c, filter_from, CLS_BLOCK) > 0) {
+      a.work2 = nullptr;
+      if (filter && class_vertices(c, filter_from, CLS_HUB) > 0) {
         pe = prof ? prof_begin(c, cs) : -1;
-        ck(launch_majority_filter(a, c->work2, weights ? 1 : 0, async_mode, c->di, cs, filter_from));
-        if (prof) prof_end(c, pe, SL_FILTER, cs, 2);
-        af.work = c->work2;
+        int kernels = 0;
+        // no sample: the graphs of a batch share no label
+        ck(launch_majority_filter(a, g->nnz, c->work2, nullptr, weights ? 1 : 0, async_mode, filter_from, false, 0u,
+                                  class_vertices(c, filter_from, CLS_WARP_L) > 0,
+                                  class_vertices(c, CLS_BLOCK, CLS_HUB) > 0, c->di, cs, &kernels));
+        if (prof) prof_end(c, pe, SL_FILTER, cs, kernels);
+        a.work2 = c->work2;
       }
-      for (int k = CLS_BINNED; k < NCLASS; ++k) {
-        if (class_vertices(c, k, k) == 0) continue;
+      for (int k = CLS_BINNED; k < CLS_HUB; ++k) {
+        if (class_vertices(c, k, k) == 0 && !(k == CLS_BLOCK && a.hub_blocks)) continue;
         pe = prof ? prof_begin(c, cs) : -1;
-        const bool filtered = k == CLS_WARP_L || k == CLS_BLOCK || (k == CLS_WARP_S && filter_from == CLS_WARP_S);
-        ck(launch_sweep_class(filtered ? af : a, k, weights ? 1 : 0, async_mode, c->tune,
-                              (int)c->ctr_h->max_degree, c->di, cs));
+        ck(launch_sweep_class(a, k, weights ? 1 : 0, async_mode, c->tune, (int)c->ctr_h->max_degree, c->di, cs));
         if (prof) prof_end(c, pe, SL_SWEEP0 + k, cs, 1);
       }
       if (class_vertices(c, 0, CLS_BINNED - 1) > 0) {
@@ -985,7 +1006,7 @@ int gsl_ctx_destroy(gsl_ctx* c) {
   if (!c) return GSL_OK;
   DeviceGuard dg(c->device);
   void* dptrs[] = {c->lab[0], c->lab[1], c->flag[0], c->flag[1], c->work, c->parent, c->rank, c->sigma,
-                   c->block_sums, c->partials, c->scratch, c->rowbits, c->lg, c->work2, c->fkeys, c->fvals, c->hub_piece_start,
+                   c->block_sums, c->partials, c->scratch, c->hub_scratch, c->rowbits, c->lg, c->work2, c->gbits, c->fkeys, c->fvals, c->hub_piece_start,
                    c->hub_ustart, c->hub_best, c->hub_own, c->hub_wsum, c->hub_used_cnt, c->hub_clu, c->hub_used, c->hub_tab,
                    c->ctr, c->sums, c->k_dev,
                    c->st_off, c->st_col, c->st_w, c->st_lab, c->fix_w, c->fix_dev, c->kw};
@@ -1547,7 +1568,7 @@ int gsl_gsllpa_batch(gsl_ctx* c, const gsl_csr* g, int32_t num_graphs, const int
     if (int r = prepare_graph(c, g, s)) return r;
   if (n > 0) {
     SweepArgs lists{};
-    if (int r = ensure_scratch(c, c->ctr_h->max_degree, &lists)) return r;
+    if (int r = ensure_scratch(c, false, &lists)) return r;
   }
   CK(cudaMemsetAsync(c->done, 0, (size_t)num_graphs, s));
   CK(cudaMemsetAsync(c->iters, 0, sizeof(int) * (size_t)num_graphs, s));
@@ -1562,7 +1583,8 @@ int gsl_gsllpa_batch(gsl_ctx* c, const gsl_csr* g, int32_t num_graphs, const int
     if (n > 0 && class_vertices(c, k, k) > 0) populated |= 1ll << k;
   const std::vector<long long> key = {populated, (long long)OFF(g), (long long)g->cols, (long long)weights, n, g->nnz,
                                       num_graphs, max_iters, mode, (long long)(tol * 1e12), c->ctr_h->max_degree,
-                                      (long long)c->lab[0], (long long)c->scratch,
+                                      (long long)c->lab[0], (long long)c->scratch, (long long)c->hub_scratch,
+                                      (long long)c->ctr_h->cls_total[CLS_HUB],
                                       c->tune.warp_max, c->tune.blk_max, (long long)c->work2,
                                       c->tune.majority, c->tune.blk_block, c->tune.blk_slots, c->tune.probe_cap,
                                       c->tune.uf_cap};
@@ -1741,7 +1763,8 @@ int gsllpa_host_overlapped(gsl_ctx* c, int64_t n, int64_t nnz, const int64_t* of
   a.ctr = c->ctr;
   a.probe_cap = c->tune.probe_cap;
   a.work = c->work;
-  if (int r = ensure_scratch(c, longest_block_row(c), &a)) return r;
+  const bool hub_kernels = c->hub_ready;
+  if (int r = ensure_scratch(c, hub_kernels, &a)) return r;
   a.n = n;
   a.prev = c->lab[1];
   a.next = c->lab[0];
@@ -1762,20 +1785,21 @@ int gsllpa_host_overlapped(gsl_ctx* c, int64_t n, int64_t nnz, const int64_t* of
     CK(launch_sweep_lanes(a, 0, false, vb[k], vb[k + 1], nullptr, 1, nullptr, 0, 2u, c->di, s));
     if (class_vertices(c, CLS_BINNED, NCLASS - 1) == 0) continue;
     CK(launch_bin_range(OFF(&g), vb[k], vb[k + 1], c->tune, c->work, c->ctr, c->di, s, CLS_BINNED));
-    SweepArgs af = a;
-    if (filter) {
-      CK(launch_majority_filter(a, c->work2, 0, false, c->di, s));
-      af.work = c->work2;
+    a.work2 = nullptr;
+    if (filter && class_vertices(c, CLS_WARP_L, CLS_HUB) > 0) {
+      CK(launch_majority_filter(a, nnz, c->work2, nullptr, 0, false, CLS_WARP_L, false, 0u,
+                                class_vertices(c, CLS_WARP_L, CLS_WARP_L) > 0,
+                                class_vertices(c, CLS_BLOCK, CLS_HUB) > 0, c->di, s));
+      a.work2 = c->work2;
     }
     for (int cls = NCLASS - 1; cls >= CLS_BINNED; --cls) {
-      if (class_vertices(c, cls, cls) == 0) continue;
-      if (cls == CLS_WARP_L || cls == CLS_BLOCK) {
-        CK(launch_sweep_class(af, cls, 0, false, c->tune, (int)c->ctr_h->max_degree, c->di, s));
-      } else if (cls == CLS_HUB && c->hub_ready) {
+      if (class_vertices(c, cls, cls) == 0 && !(cls == CLS_BLOCK && a.hub_blocks)) continue;
+      if (cls == CLS_HUB && !hub_kernels) continue;   // with class 8
+      if (cls == CLS_HUB) {
         HubPlan hp{c->hub_piece_start, c->hub_ustart, c->hub_best, c->hub_own,
                    c->hub_wsum,        c->hub_used_cnt, c->hub_used, c->hub_tab, c->hub_clu};
         int kernels = 0;
-        CK(launch_hub_pieces(a, hp, false, false, filter, c->tune, c->di, s, &kernels));
+        CK(launch_hub_pieces(a, hp, false, false, c->tune, c->di, s, &kernels));
       } else {
         CK(launch_sweep_class(a, cls, 0, false, c->tune, (int)c->ctr_h->max_degree, c->di, s));
       }

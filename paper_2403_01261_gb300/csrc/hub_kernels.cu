@@ -103,7 +103,7 @@ __device__ __forceinline__ int piece_hub(const int* piece_start, int cnt, int p)
 // get no pieces; every hub keeps its global table region and used list.
 __global__ void __launch_bounds__(1024) hub_plan_kernel(SweepArgs a, HubPlan hp, long long cmax) {
   const unsigned cnt = a.ctr->cls_count[CLS_HUB];
-  const int* __restrict__ work = a.work + a.ctr->cls_start[CLS_HUB];
+  const int* __restrict__ work = class_work(a, CLS_HUB);
   __shared__ long long s_pieces[1024], s_entries[1024];
   __shared__ int s_clu[1024];
   __shared__ long long base_p, base_e;
@@ -276,54 +276,6 @@ __device__ __forceinline__ void cluster_row(const SweepArgs& a, int v, int own, 
   __syncthreads();
 }
 
-// The cluster's own-label pass over a hub row (own_weight_pass over the
-// cluster's virtual threads).  Each warp adds its round's own-label weight
-// to rank 0's counter `cnt` and stops once the returned total is more than
-// half of `bound` (the row's d entries, or its weighted degree from sweep
-// 1): the own label then holds a strict majority whatever the rest carries.
-template <bool WEIGHTED, bool ASYNC>
-__device__ __forceinline__ void cluster_own_pass(const SweepArgs& a, int v, int own, const int* cp, const int* wp,
-                                                 const int* lp, int d, int tid, int nthr, const Pol& pol,
-                                                 unsigned& own_w, unsigned& tot_w, unsigned* cnt,
-                                                 unsigned long long bound) {
-  const int lane = tid & 31, wid = tid >> 5, nw = nthr >> 5;
-  const int step = nw * 128;
-  const int cb = wid * 32 + lane, cu = nw * 32;
-  int jn[4], wn[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) load_entry<WEIGHTED>(a, cp, wp, d, cb + u * cu, pol, jn[u], wn[u]);
-  for (int r0 = 0; r0 < d; r0 += step) {
-    int l[4], w[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      l[u] = entry_label<ASYNC>(a, lp, r0 + cb + u * cu, jn[u], v, pol);
-      w[u] = wn[u];
-    }
-    const bool more = r0 + step < d;   // cluster-uniform
-    if (more) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) load_entry<WEIGHTED>(a, cp, wp, d, r0 + step + cb + u * cu, pol, jn[u], wn[u]);
-    }
-    unsigned o = 0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (l[u] >= 0) {
-        tot_w += (unsigned)w[u];
-        if (l[u] == own) {
-          own_w += (unsigned)w[u];
-          o += (unsigned)w[u];
-        }
-      }
-    }
-    if (more && bound != ~0ull) {
-      o = __reduce_add_sync(FULL, o);
-      unsigned total = 0;
-      if (lane == 0 && o) total = atomicAdd(cnt, o) + o;
-      if (2ull * __shfl_sync(FULL, total, 0) > bound) return;
-    }
-  }
-}
-
 // Hubs of degree <= cmax (listed by the plan kernel), one thread-block
 // cluster at a time: rank 0 takes the next hub from a counter, the row is
 // aggregated in the CTAs' shared tables (cluster_row), each CTA scans its
@@ -337,25 +289,17 @@ __device__ __forceinline__ void cluster_own_pass(const SweepArgs& a, int v, int 
 // can reach a table before it is empty), B after every insert (all flags
 // final).  Per-hub shared values alternate between two copies (par), so a
 // CTA clears one copy while others may still read the previous hub's.
-// With `maj` (sweeps whose rows mostly keep their label) the cluster first
-// weighs the row's own label (own_weight_pass, barrier C, totals read from
-// all CTAs): a strict majority is Eq. 2's argmax, the label stays and the
-// table pass is skipped.
 // Every branch around a barrier depends only on values all CTAs of the
-// cluster read alike (the hub index from rank 0, the OR of the flags, the
-// majority totals).
+// cluster read alike (the hub index from rank 0, the OR of the flags).
 template <bool WEIGHTED, bool ASYNC>
-__global__ void __launch_bounds__(512, 2) hub_cluster_kernel(SweepArgs a, HubPlan hp, unsigned tb, int maj) {
+__global__ void __launch_bounds__(512, 2) hub_cluster_kernel(SweepArgs a, HubPlan hp, unsigned tb) {
   extern __shared__ unsigned long long smem_c64[];
   __shared__ BlockRowShared sh;
   __shared__ int s_hub[2], s_ovf[2];
-  __shared__ unsigned long long s_mown[2], s_mtot[2];
-  __shared__ unsigned s_mcnt[2];   // rank 0's: own-label entries counted so far (unit weights)
-  __shared__ int s_skip[2];
   cg::cluster_group cl = cg::this_cluster();
   const unsigned rank = cl.block_rank();
   const int nclu = (int)a.ctr->hub_clusters;
-  const int* __restrict__ work = a.work + a.ctr->cls_start[CLS_HUB];
+  const int* __restrict__ work = class_work(a, CLS_HUB);
   const Pol pol = make_pol();
   const SlotTable st = make_table(smem_c64, tb);
   const int tid = (int)(rank * blockDim.x + threadIdx.x), nthr = HUB_CLUSTER * (int)blockDim.x;
@@ -366,9 +310,6 @@ __global__ void __launch_bounds__(512, 2) hub_cluster_kernel(SweepArgs a, HubPla
     }
     if (threadIdx.x == 0) {
       sh.ovf[par] = 0;
-      s_mown[par] = 0;
-      s_mtot[par] = 0;
-      s_mcnt[par] = 0;
       if (rank == 0) s_hub[par] = (int)atomicAdd(&a.ctr->hub_clu_next, 1u);
     }
     cl.sync();   // A
@@ -382,33 +323,6 @@ __global__ void __launch_bounds__(512, 2) hub_cluster_kernel(SweepArgs a, HubPla
     const int* cp = a.col + s;
     const int* wp = a.w + s;
     const int* lp = a.lg ? a.lg + s : nullptr;
-    if (maj) {
-      unsigned own_w = 0, tot_w = 0;
-      const unsigned long long bound =
-          !WEIGHTED ? (unsigned long long)d : (a.kw ? (unsigned long long)a.kw[v] : ~0ull);
-      cluster_own_pass<WEIGHTED, ASYNC>(a, v, own, cp, wp, lp, d, tid, nthr, pol, own_w, tot_w,
-                                        cl.map_shared_rank(&s_mcnt[par], 0), bound);
-      const unsigned long long ow = warp_sum_u64(own_w), tw = warp_sum_u64(tot_w);
-      if ((threadIdx.x & 31) == 0) {
-        if (ow) atomicAdd(&s_mown[par], ow);
-        if (tw) atomicAdd(&s_mtot[par], tw);
-      }
-      cl.sync();   // C
-      if (threadIdx.x < 32) {
-        unsigned long long o = 0, t = 0;
-        if (threadIdx.x < HUB_CLUSTER) {
-          o = *(volatile unsigned long long*)cl.map_shared_rank(&s_mown[par], threadIdx.x);
-          t = *(volatile unsigned long long*)cl.map_shared_rank(&s_mtot[par], threadIdx.x);
-        }
-        o = warp_sum_u64(o);
-        t = warp_sum_u64(t);
-        // a strict majority of the row, or (the pass stopped early) more
-        // than half of its total
-        if (threadIdx.x == 0) s_skip[par] = 2 * o > t || 2 * o > bound;
-      }
-      __syncthreads();
-      if (s_skip[par]) continue;   // the label stays (hp.best 0, hp.own 0)
-    }
     cluster_row<WEIGHTED, ASYNC, false>(a, v, own, cp, wp, lp, d, tid, nthr, st, tb, nullptr, 0, nullptr, nullptr, 0,
                                         pol, sh, par, cl);
     cl.sync();   // B
@@ -450,7 +364,7 @@ __global__ void __launch_bounds__(512, 2) hub_piece_kernel(SweepArgs a, HubPlan 
   __shared__ BlockRowShared sh;
   const unsigned cnt = a.ctr->cls_count[CLS_HUB];
   const unsigned pieces = a.ctr->hub_pieces;
-  const int* __restrict__ work = a.work + a.ctr->cls_start[CLS_HUB];
+  const int* __restrict__ work = class_work(a, CLS_HUB);
   const Pol pol = make_pol();
   int par = 0;
   for (unsigned p = blockIdx.x; p < pieces; p += gridDim.x, par ^= 1) {
@@ -493,7 +407,7 @@ __global__ void __launch_bounds__(512, 2) hub_piece_kernel(SweepArgs a, HubPlan 
 template <bool ASYNC>
 __global__ void __launch_bounds__(256) hub_final_kernel(SweepArgs a, HubPlan hp, int weighted) {
   const unsigned cnt = a.ctr->cls_count[CLS_HUB];
-  const int* __restrict__ work = a.work + a.ctr->cls_start[CLS_HUB];
+  const int* __restrict__ work = class_work(a, CLS_HUB);
   const Pol pol = make_pol();
   unsigned long long my_dn = 0, my_scan = 0;
   for (unsigned i = blockIdx.x; i < cnt; i += gridDim.x) {
@@ -571,7 +485,7 @@ int cluster_slots(size_t smem) {
 }
 
 template <bool W, bool A>
-cudaError_t launch_hub_t(const SweepArgs& a, const HubPlan& hp, bool maj, const Tuning& t, const DeviceInfo& di,
+cudaError_t launch_hub_t(const SweepArgs& a, const HubPlan& hp, const Tuning& t, const DeviceInfo& di,
                          cudaStream_t s, int* kernels) {
   const size_t smem = (size_t)t.blk_slots * sizeof(unsigned long long);
   raise_smem_limit((const void*)hub_piece_kernel<W, A>, smem);
@@ -591,7 +505,7 @@ cudaError_t launch_hub_t(const SweepArgs& a, const HubPlan& hp, bool maj, const 
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, hub_cluster_kernel<W, A>, a, hp, (unsigned)t.blk_slots, maj ? 1 : 0);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, hub_cluster_kernel<W, A>, a, hp, (unsigned)t.blk_slots);
     if (e != cudaSuccess) return e;
     ++launches;
   }
@@ -605,13 +519,13 @@ cudaError_t launch_hub_t(const SweepArgs& a, const HubPlan& hp, bool maj, const 
 
 bool hub_pieces_fit(const Tuning& t) { return HUB_PIECE * 4 <= t.blk_slots * 3 - 4 * 512; }
 
-cudaError_t launch_hub_pieces(const SweepArgs& a, const HubPlan& hp, bool weighted, bool async_mode, bool majority,
+cudaError_t launch_hub_pieces(const SweepArgs& a, const HubPlan& hp, bool weighted, bool async_mode,
                               const Tuning& t, const DeviceInfo& di, cudaStream_t s, int* kernels) {
   if (weighted)
-    return async_mode ? launch_hub_t<true, true>(a, hp, majority, t, di, s, kernels)
-                      : launch_hub_t<true, false>(a, hp, majority, t, di, s, kernels);
-  return async_mode ? launch_hub_t<false, true>(a, hp, majority, t, di, s, kernels)
-                    : launch_hub_t<false, false>(a, hp, majority, t, di, s, kernels);
+    return async_mode ? launch_hub_t<true, true>(a, hp, t, di, s, kernels)
+                      : launch_hub_t<true, false>(a, hp, t, di, s, kernels);
+  return async_mode ? launch_hub_t<false, true>(a, hp, t, di, s, kernels)
+                    : launch_hub_t<false, false>(a, hp, t, di, s, kernels);
 }
 
 }  // namespace gsl

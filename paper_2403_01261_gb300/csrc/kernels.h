@@ -15,9 +15,14 @@ struct SweepArgs {
   int* next;                 // labels written (C^t)
   unsigned char* fnext;      // frontier flags of the next sweep (set, never cleared here)
   const int* work;           // worklist (class regions at Counters::cls_start)
+  const int* work2;          // rows the majority filter left, the same regions (null: no filter this sweep)
+  const unsigned* bits;      // majority filter: one bit per vertex carrying the giant label
   Counters* ctr;
   int* scratch;              // label lists of rows longer than a block's registers, one region per block
   long long scratch_region;  // ints per region (three lists of the longest row)
+  int* hub_scratch;          // the same for class 9, one region for each of the first hub_blocks blocks
+  long long hub_region;
+  int hub_blocks;            // 0: class 9 has its own kernels
   long long n;
   // batched mode (many graphs packed in one CSR); all null for one graph
   const int* gid;            // graph of every vertex
@@ -36,7 +41,7 @@ struct SweepArgs {
 
 struct Tuning {
   int warp_max = 1024;       // class 7 upper degree bound (a small block per row)
-  int blk_max = 32768;       // class 8 upper degree bound (a block per row; above: class 9)
+  int blk_max = 131072;       // class 8 upper degree bound (a block per row; above: class 9)
   int blk_slots = 12288;     // shared-memory table slots per block of the hub kernels
   int blk_block = 512;       // threads per block of the hub-piece kernel
   int pregather = 0;         // two-phase sweeps: 0 never, 1 when the frontier is large, 2 always
@@ -89,7 +94,8 @@ long long sketch_blocks(const DeviceInfo& di);
 long long sketch_register_row();
 cudaError_t launch_sketch(const SweepArgs& a, int cls, int longest, int weights, bool async_mode,
                           const DeviceInfo& di, cudaStream_t s);
-// Classes 3..9 on the worklist (class 9 as the block rows it then is).
+// Classes 3..8 on the worklist; class 8's launch sweeps class 9 as well when
+// SweepArgs::hub_blocks is set.
 cudaError_t launch_sweep_class(const SweepArgs& a, int cls, int weights, bool async_mode, const Tuning& t,
                                int longest, const DeviceInfo& di, cudaStream_t s);
 void count_launches(long long k);   // process-wide tally of kernels this library launched
@@ -98,14 +104,17 @@ void count_launches(long long k);   // process-wide tally of kernels this librar
 // valid); thread-safe.
 cudaError_t raise_smem_limit(const void* fn, size_t bytes);
 long long launches_total();
-// Own-label majority filter over classes first_cls..8 (first_cls 6 or 7):
-// settled rows keep their label; the others go to `out` (n ints, class
-// regions as in the worklist) and become the class counts of the warp and
-// block kernels, which must then read `out` as their worklist.
-// The class counts of classes first_cls..8 become the rows a filter passed on.
-cudaError_t launch_filter_counts(Counters* ctr, const int* stop, cudaStream_t s, int first_cls = CLS_WARP_L);
-cudaError_t launch_majority_filter(const SweepArgs& a, int* out, int weights, bool async_mode,
-                                   const DeviceInfo& di, cudaStream_t s, int first_cls = CLS_WARP_L);
+// filter_kernels.cu: majority filter over the classes from first_cls (or 6,
+// when one label dominates a sample of the entries) to 9.  Settled rows are
+// written; the others go to `out` (n ints, class regions as in the worklist)
+// and become the class counts: the sweep kernels launched next need
+// SweepArgs::work2 = out.  bits: n / 32 + 1 words of scratch.  warps, blocks:
+// whether classes 6-7 and 8-9 hold rows.
+cudaError_t launch_majority_filter(const SweepArgs& a, long long nnz, int* out, unsigned* bits, int weights,
+                                   bool async_mode, int first_cls, bool sample, unsigned seed, bool warps, bool blocks,
+                                   const DeviceInfo& di, cudaStream_t s, int* kernels = nullptr);
+// The class counts of first_cls..last_cls become the rows a filter passed on.
+cudaError_t launch_filter_counts(Counters* ctr, const int* stop, cudaStream_t s, int first_cls, int last_cls);
 // Edge-parallel label gather for a synchronous sweep: lg[e] = prev[col[e]]
 // for every CSR entry (-1 for an out-of-range column).
 cudaError_t launch_pregather(const int* col, long long nnz, const int* prev, long long n, int* lg,
@@ -171,10 +180,9 @@ struct HubPlan {
 };
 // True when a piece always fits the block kernel's shared table.
 bool hub_pieces_fit(const Tuning& t);
-// Class 9: plan, cluster kernel (hubs up to t.hub_cluster_max; with
-// `majority`, rows whose own label holds a strict majority keep it without
-// a table), pieces, final pass.  *kernels = launches made.
-cudaError_t launch_hub_pieces(const SweepArgs& a, const HubPlan& hp, bool weighted, bool async_mode, bool majority,
+// Class 9: plan, cluster kernel (hubs up to t.hub_cluster_max), pieces, final
+// pass.  *kernels = launches made.
+cudaError_t launch_hub_pieces(const SweepArgs& a, const HubPlan& hp, bool weighted, bool async_mode,
                               const Tuning& t, const DeviceInfo& di, cudaStream_t s, int* kernels);
 
 // float_kernels.cu: sweeps with float32 weights and float64 sums.  Classes

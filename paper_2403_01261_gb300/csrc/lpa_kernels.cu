@@ -173,130 +173,6 @@ __global__ void init_labels_kernel(const int* __restrict__ init, int* __restrict
 }
 
 // ---------------------------------------------------------------------------
-// The filter's pass over one row, one warp (own_weight_pass with 32
-// threads): it stops as soon as the own label holds more than half of the
-// row's total (d entries, or the weighted degree from sweep 1), since it
-// then holds a strict majority of the whole row whatever the rest carries
-// (`early`).  Returns the entries read.
-template <int WT, bool ASYNC>
-__device__ __forceinline__ int filter_row(const SweepArgs& a, int v, int own, const int* cp, const int* wp,
-                                          const int* lp, int d, const Pol& pol, typename SumOf<WT>::T& own_w,
-                                          typename SumOf<WT>::T& tot_w, bool& early) {
-  const int lane = threadIdx.x & 31;
-  const unsigned long long bound = !WT ? (unsigned long long)d : (WT == 1 && a.kw ? (unsigned long long)a.kw[v] : ~0ull);
-  int jn[4], wn[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) load_entry<WT != 0>(a, cp, wp, d, lane + 32 * u, pol, jn[u], wn[u]);
-  for (int r0 = 0; r0 < d; r0 += 128) {
-    int l[4], w[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      l[u] = entry_label<ASYNC>(a, lp, r0 + lane + 32 * u, jn[u], v, pol);
-      w[u] = wn[u];
-    }
-    const bool more = r0 + 128 < d;   // warp-uniform
-    if (more) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) load_entry<WT != 0>(a, cp, wp, d, r0 + 128 + lane + 32 * u, pol, jn[u], wn[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (l[u] >= 0) {
-        tot_w += (unsigned)w[u];
-        if (l[u] == own) own_w += (unsigned)w[u];
-      }
-    }
-    if (WT != 2 && more && 2ull * __reduce_add_sync(FULL, (unsigned)own_w) > bound) {
-      early = true;
-      return r0 + 128;
-    }
-  }
-  return d;
-}
-
-// Own-label majority filter for classes 7 and 8 (rows of 257..blk_max
-// entries by default: long enough that one extra lean pass costs less than
-// a table), run before their table kernels once labels have started to
-// settle.  One warp per row, no shared memory and registers capped for six
-// 256-thread blocks per SM (many rows in flight): the weight of the row's entries carrying the vertex's
-// own label is compared with the row's total (the vertex itself excluded).
-// A strict majority is Eq. 2's argmax: the label stays and the row is done.
-// Other rows are appended to `out` at their class's region and counted in
-// Counters::uns_count; filter_counts_kernel then makes those the class
-// counts for the table kernels.
-template <int WT, bool ASYNC>
-__global__ void __launch_bounds__(256, 6) majority_filter_kernel(SweepArgs a, int* __restrict__ out, int first_cls) {
-  if (stopped(a)) return;
-  const int lane = threadIdx.x & 31;
-  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  const Pol pol = make_pol();
-  const long long c6 = first_cls <= CLS_WARP_S ? a.ctr->cls_count[CLS_WARP_S] : 0;
-  const long long c67 = c6 + a.ctr->cls_count[CLS_WARP_L];
-  const long long total = c67 + a.ctr->cls_count[CLS_BLOCK];
-  unsigned long long my_scan = 0, my_settled = 0;
-  for (long long i = warp; i < total; i += nwarps) {
-    const int cls = i < c6 ? CLS_WARP_S : (i < c67 ? CLS_WARP_L : CLS_BLOCK);
-    const long long start = a.ctr->cls_start[cls];
-    const int v = a.work[start + (i - (i < c6 ? 0 : (i < c67 ? c6 : c67)))];
-    const long long s = a.off[v];
-    const int d = (int)(a.off[v + 1] - s);
-    const int old = own_label<ASYNC>(a, v);
-    typename SumOf<WT>::T ow = 0, tw = 0;
-    bool early = false;
-    const int read = filter_row<WT, ASYNC>(a, v, old, a.col + s, a.w + s, a.lg ? a.lg + s : nullptr, d, pol, ow,
-                                                 tw, early);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      ow += __shfl_xor_sync(FULL, ow, o);
-      tw += __shfl_xor_sync(FULL, tw, o);
-    }
-    if (lane == 0) {
-      if (early || 2ull * ow > (unsigned long long)tw) {
-        store_label<ASYNC>(a, v, old, false);
-        my_scan += (unsigned long long)read;
-        my_settled += 1;
-      } else {
-        out[start + atomicAdd(&a.ctr->uns_count[cls], 1u)] = v;
-      }
-    }
-  }
-  my_scan = warp_sum_u64(my_scan);
-  my_settled = warp_sum_u64(my_settled);
-  if (lane == 0) {
-    if (my_scan) atomicAdd(&a.ctr->scanned, my_scan);
-    if (my_settled) atomicAdd(&a.ctr->fast_active, my_settled);
-  }
-}
-
-__global__ void filter_counts_kernel(Counters* ctr, const int* stop, int first_cls) {
-  if (stop && *(volatile const int*)stop) return;
-  for (int k = first_cls; k <= CLS_BLOCK; ++k) ctr->cls_count[k] = ctr->uns_count[k];
-}
-
-cudaError_t launch_filter_counts(Counters* ctr, const int* stop, cudaStream_t s, int first_cls) {
-  filter_counts_kernel<<<1, 1, 0, s>>>(ctr, stop, first_cls);
-  count_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_majority_filter(const SweepArgs& a, int* out, int weights, bool async_mode,
-                                   const DeviceInfo& di, cudaStream_t s, int first_cls) {
-  const int grid = 16 * di.sm_count;
-  switch (2 * weights + (async_mode ? 1 : 0)) {
-    case 0: majority_filter_kernel<0, false><<<grid, 256, 0, s>>>(a, out, first_cls); break;
-    case 1: majority_filter_kernel<0, true><<<grid, 256, 0, s>>>(a, out, first_cls); break;
-    case 2: majority_filter_kernel<1, false><<<grid, 256, 0, s>>>(a, out, first_cls); break;
-    case 3: majority_filter_kernel<1, true><<<grid, 256, 0, s>>>(a, out, first_cls); break;
-    case 4: majority_filter_kernel<2, false><<<grid, 256, 0, s>>>(a, out, first_cls); break;
-    default: majority_filter_kernel<2, true><<<grid, 256, 0, s>>>(a, out, first_cls); break;
-  }
-  filter_counts_kernel<<<1, 1, 0, s>>>(a.ctr, a.stop, first_cls);
-  count_launches(2);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
 // Edge-parallel gather of a synchronous sweep's neighbour labels.  The class
 // kernels hold hash tables in shared memory, which caps their occupancy,
 // and they interleave dependent loads with hashing; this pass has neither:
@@ -606,8 +482,10 @@ cudaError_t launch_sweep_class(const SweepArgs& a, int cls, int weights, bool as
                                int longest, const DeviceInfo& di, cudaStream_t s) {
   if (cls < CLS_WARP_S) return launch_sweep_tile(a, cls, weights, async_mode, di, s);
   const ClassBounds cb = class_bounds(t);
-  const int bound = cls == CLS_WARP_S ? cb.warp_small : (cls == CLS_WARP_L ? cb.warp_max : (cls == CLS_BLOCK ? cb.blk_max : longest));
-  return launch_sketch(a, cls, bound < longest ? bound : longest, weights, async_mode, di, s);
+  // class 8 always takes the block kernel: it sweeps class 9 as well
+  const int bound = cls == CLS_WARP_S ? cb.warp_small : (cls == CLS_WARP_L ? cb.warp_max : cb.blk_max);
+  return launch_sketch(a, cls, cls == CLS_BLOCK ? 1 << 30 : (bound < longest ? bound : longest), weights, async_mode,
+                       di, s);
 }
 
 void count_launches(long long k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
@@ -688,6 +566,7 @@ __global__ void phase_reset_kernel(Counters* ctr, const int* stop) {
   ctr->hub_pieces = 0;
   ctr->hub_clusters = 0;
   ctr->hub_clu_next = 0;
+  ctr->filter_next = 0;
 }
 
 cudaError_t launch_phase_reset(Counters* ctr, const int* stop, cudaStream_t s) {

@@ -398,8 +398,9 @@ __device__ __forceinline__ void sketch_row(const SweepArgs& a, int v, int old, c
 // One row through the block's scratch list.
 template <int T, int LG, int WT, bool ASYNC, bool GENERAL, typename S>
 __device__ __forceinline__ void sketch_long_row(const SweepArgs& a, int v, const int* cp, const int* wp,
-                                                const int* lp, int d, int tid, unsigned* mem, int rounds, const Pol& pol,
-                                                Best<S>& best, unsigned long long& ws, TeamShared<T, S>* sh) {
+                                                const int* lp, int d, int tid, unsigned* mem, int* list,
+                                                long long region, int rounds, const Pol& pol, Best<S>& best,
+                                                unsigned long long& ws, TeamShared<T, S>* sh) {
   if (GENERAL && a.ident) {
     // strictly increasing: every label (its id) occurs once
     bool inc = true;
@@ -420,7 +421,6 @@ __device__ __forceinline__ void sketch_long_row(const SweepArgs& a, int v, const
     }
     best = {0, 0u};
   }
-  int* list = a.scratch + (long long)blockIdx.x * a.scratch_region;
   const Sketch t{mem, LG, WT == 2 ? ceil_log2((unsigned)d) : 0u};
   sketch_clear<T>(t.cnt, LG, tid);
   team_sync<T>();
@@ -464,8 +464,8 @@ __device__ __forceinline__ void sketch_long_row(const SweepArgs& a, int v, const
   constexpr int PART = T * 8;   // entries aimed at, half of what the registers hold
   const unsigned lgp = min(6u, max(1u, ceil_log2(left / PART + 1)));
   const unsigned np = 1u << lgp;
-  int* out = list + a.scratch_region / 3;
-  int* outw = out + a.scratch_region / 3;
+  int* out = list + region / 3;
+  int* outw = out + region / 3;
   auto part_of = [&](int l) { return ((unsigned)l * 0x7FEB352Du) >> (32u - lgp); };
   __syncthreads();
   if (tid < 64) sh->fill[tid] = 0;
@@ -524,7 +524,9 @@ constexpr int team_lg() { return T == 32 ? LG_WARP : (T == T_SMALL ? LG_SMALL : 
 
 // Rows of class cls by teams of T threads: up to T * K entries in registers
 // (fewer per thread on shorter rows), longer ones (T_BLOCK only) through the
-// block's scratch region.  Blocks take rows from a counter, warps in strides.
+// block's scratch region.  Warps take rows in strides, blocks from a counter;
+// the first hub_blocks blocks of T_BLOCK threads take the rows of class 9
+// before those of cls, so that the longest rows run beside the others.
 template <int T, int WT, bool ASYNC, bool GENERAL>
 __global__ void __launch_bounds__(T == 32 ? 256 : T, T == 32 ? 4 : (T == T_SMALL ? 8 : BLOCKS_PER_SM))
     sketch_kernel(SweepArgs a, int cls) {
@@ -534,37 +536,51 @@ __global__ void __launch_bounds__(T == 32 ? 256 : T, T == 32 ? 4 : (T == T_SMALL
   __shared__ TeamShared<T, S> sh;
   const int tid = T == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
   unsigned* mem = reinterpret_cast<unsigned*>(smem_sketch) + (T == 32 ? (size_t)(threadIdx.x >> 5) << team_lg<T>() : 0);
-  const unsigned cnt = a.ctr->cls_count[cls];
-  const int* __restrict__ work = a.work + a.ctr->cls_start[cls];
+  bool hubs = T == T_BLOCK && (int)blockIdx.x < a.hub_blocks;
+  int now = hubs ? CLS_HUB : cls;
+  unsigned cnt = a.ctr->cls_count[now];
+  const int* work = class_work(a, now);
   const Pol pol = make_pol();
   const int rounds = a.probe_cap < SKETCH_ROUNDS ? a.probe_cap : SKETCH_ROUNDS;
-  unsigned long long my_dn = 0, my_scan = 0;
+  unsigned long long my_dn = 0, my_scan = 0, hub_scan = 0;
   const long long nteams = ((long long)gridDim.x * blockDim.x) / T;
   long long item = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / T;
   int vn = 0;
   long long sn = 0, en = 0;
-  if (item < (long long)cnt) {
-    vn = work[item];
-    sn = a.off[vn];
-    en = a.off[vn + 1];
-  }
-  while (item < (long long)cnt) {
-    const int v = vn;
-    const long long s = sn;
-    const int d = (int)(en - sn);
-    // the next row: blocks take those beyond the first nteams in order
-    long long next = item + nteams;
-    if (T != 32) {
-      __syncthreads();   // the previous row's last reads of sh and the table
-      if (threadIdx.x == 0) sh.next = nteams + (long long)atomicAdd(&a.ctr->row_next[cls], 1u);
-      __syncthreads();
-      next = sh.next;
-    }
-    if (next < (long long)cnt) {
-      vn = work[next];
+  auto fetch = [&] {
+    if (item < (long long)cnt) {
+      vn = work[item];
       sn = a.off[vn];
       en = a.off[vn + 1];
     }
+  };
+  auto take = [&] {   // a block's next row, from the class's counter
+    __syncthreads();   // the previous row's last reads of sh and the table
+    if (threadIdx.x == 0) sh.next = (long long)atomicAdd(&a.ctr->row_next[now], 1u);
+    __syncthreads();
+    return sh.next;
+  };
+  if (T != 32) item = take();
+  fetch();
+  for (;;) {
+    if (item >= (long long)cnt) {   // team-uniform
+      if (!hubs) break;
+      hubs = false;
+      hub_scan = my_scan;
+      my_scan = 0;
+      now = cls;
+      cnt = a.ctr->cls_count[now];
+      work = class_work(a, now);
+      item = take();
+      fetch();
+      continue;
+    }
+    const int v = vn;
+    const long long s = sn;
+    const int d = (int)(en - sn);
+    const long long next = T == 32 ? item + nteams : take();
+    item = next;
+    fetch();
     const int old = own_label<ASYNC>(a, v);
     const int* cp = a.col + s;
     const int* wp = a.w + s;
@@ -594,10 +610,13 @@ __global__ void __launch_bounds__(T == 32 ? 256 : T, T == 32 ? 4 : (T == T_SMALL
         sketch_row<T, K_BLOCK, LG_BLOCK, WT, ASYNC, GENERAL, S>(a, v, old, cp, wp, lp, d, tid, mem, rounds, pol, best,
                                                                 ws, &sh);
       else
-        sketch_long_row<T, LG_BLOCK, WT, ASYNC, GENERAL, S>(a, v, cp, wp, lp, d, tid, mem, rounds, pol, best, ws,
-                                                            &sh);
+        sketch_long_row<T, LG_BLOCK, WT, ASYNC, GENERAL, S>(
+            a, v, cp, wp, lp, d, tid, mem,
+            hubs ? a.hub_scratch + (long long)blockIdx.x * a.hub_region
+                 : a.scratch + (long long)blockIdx.x * a.scratch_region,
+            hubs ? a.hub_region : a.scratch_region, rounds, pol, best, ws, &sh);
     }
-    if (WT == 1 && GENERAL && a.check) {
+    if (WT && GENERAL && a.check) {   // the row's total, for the majority filter of later sweeps
       ws = warp_sum_u64(ws);
       if (T != 32) {
         __syncthreads();
@@ -608,8 +627,8 @@ __global__ void __launch_bounds__(T == 32 ? 256 : T, T == 32 ? 4 : (T == T_SMALL
         ws = sh.wsum;
       }
       if (tid == 0) {
-        if (ws >= (1ull << 31)) raise_err(&a.ctr->err, ERRBIT_OVERFLOW);
-        if (a.kw) a.kw[v] = ws < (1ull << 32) ? (unsigned)ws : ~0u;
+        if (WT == 1 && ws >= (1ull << 31)) raise_err(&a.ctr->err, ERRBIT_OVERFLOW);
+        if (a.kw) a.kw[v] = WT == 2 ? (unsigned)(ws >> 22) + 1u : (ws < (1ull << 32) ? (unsigned)ws : ~0u);
       }
     }
     const int nl = best.sum ? (int)~best.inv : old;
@@ -627,10 +646,13 @@ __global__ void __launch_bounds__(T == 32 ? 256 : T, T == 32 ? 4 : (T == T_SMALL
       }
       if (!ASYNC && tid == 0) a.fnext[v] = 1;
     }
-    item = next;
     if (T == 32) __syncwarp();   // the table's last reads before it is cleared
   }
   flush_counters(a.ctr, cls, my_dn, my_scan);
+  if (T == T_BLOCK && a.hub_blocks) {
+    __syncthreads();
+    flush_counters(a.ctr, CLS_HUB, 0, hub_scan);
+  }
 }
 
 namespace {

@@ -78,6 +78,12 @@ __device__ __forceinline__ void count_graph_change(const SweepArgs& a, int v) {
   if (a.dn_graph) atomicAdd(a.dn_graph + a.gid[v], 1u);
 }
 
+// The rows of a class this sweep: what the majority filter left of it, or its
+// part of the worklist.
+__device__ __forceinline__ const int* class_work(const SweepArgs& a, int cls) {
+  return (a.work2 && cls >= a.ctr->filter_from ? a.work2 : a.work) + a.ctr->cls_start[cls];
+}
+
 __device__ __forceinline__ bool stopped(const SweepArgs& a) { return a.stop && *(volatile const int*)a.stop; }
 
 // Phase of vertex v in the asynchronous sweep with seed `seed` (the sweep

@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(TILE_BLOCK, TILE_MIN_BLOCKS) tile_sweep_kernel
   const Pol pol = make_pol();
   const int rounds = a.probe_cap < SKETCH_ROUNDS ? a.probe_cap : SKETCH_ROUNDS;
   const unsigned cnt = a.ctr->cls_count[cls];
-  const int* __restrict__ work = a.work + a.ctr->cls_start[cls];
+  const int* __restrict__ work = class_work(a, cls);
   const unsigned nwarps = (gridDim.x * blockDim.x) >> 5, warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   // rows per tile: 32 once every warp gets several tiles, fewer for short worklists
   unsigned per = 32;
