@@ -94,6 +94,9 @@ struct gsl_ctx {
   int* fix_dev = nullptr;               // 3 ints
   int* fix_h = nullptr;                 // pinned mirror
 
+  SoloState* solo = nullptr;            // one-launch path of small graphs: device state and pinned mirror
+  SoloState* solo_h = nullptr;
+
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
 
   // host-buffer path: column chunks copied on their own stream
@@ -845,6 +848,80 @@ int run_modularity(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const i
   return GSL_OK;
 }
 
+// Graphs up to these sizes run in one cooperative launch (solo_kernel.cu).
+constexpr long long SOLO_MAX_N = 1ll << 19, SOLO_MAX_ENTRIES = 1ll << 23;
+
+// Synchronous sweeps (lpa) and / or the split of a small graph in one launch.
+// *handled stays false when the call does not qualify: larger graphs, rows
+// past SOLO_ROW_MAX, profiling, or any tuning set by the caller (the class
+// kernels it tunes are then what runs).
+int run_solo(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t* labels_init,
+             const int32_t* labels_in, bool lpa, bool split, double tol, int32_t max_iters, int32_t mode,
+             int32_t* out, gsl_stats* st, long long* pieces, cudaStream_t s, bool* handled) {
+  *handled = false;
+  static const Tuning defaults;
+  if (c->prof || mode != GSL_MODE_SYNC || g->n > SOLO_MAX_N || g->nnz > SOLO_MAX_ENTRIES || max_iters > SOLO_SWEEPS ||
+      !c->di.cooperative || memcmp(&c->tune, &defaults, sizeof(Tuning)) != 0)
+    return GSL_OK;
+  SweepArgs a{};
+  a.off = OFF(g);
+  a.col = g->cols;
+  a.w = weights;
+  a.ctr = &c->solo->ctr;
+  a.probe_cap = c->tune.probe_cap;
+  a.n = g->n;
+  SoloArgs q{};
+  q.state = c->solo;
+  q.nnz = g->nnz;
+  q.labels_init = labels_init;
+  q.labels_in = labels_in;
+  q.lpa = lpa ? 1 : 0;
+  q.split = split ? 1 : 0;
+  q.tol = tol;
+  q.max_iters = max_iters;
+  for (int i = 0; i < 2; ++i) {
+    q.lab[i] = c->lab[i];
+    q.flag[i] = c->flag[i];
+  }
+  if (int r = grow(c, c->scratch, c->cap_scratch, SOLO_LISTS * 3 * SOLO_ROW_MAX)) return r;
+  q.lists = c->scratch;
+  q.longs = c->work;
+  q.parent = c->parent;
+  q.named = c->rank;
+  q.out = out;
+  CK(cudaMemsetAsync(c->solo, 0, sizeof(SoloState), s));
+  if (launch_solo(a, q, weights ? 1 : 0, c->di, s) != cudaSuccess) {   // no cooperative launch of this size here
+    cudaGetLastError();
+    return GSL_OK;
+  }
+  CK(cudaMemcpyAsync(c->solo_h, c->solo, sizeof(SoloState), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  const SoloState& r = *c->solo_h;
+  const int err = r.ctr.err;
+  if (!err && !r.abandoned && r.longest > SOLO_ROW_MAX) return GSL_OK;
+  *handled = true;
+  if (r.abandoned) return fail(c, GSL_ERR_TIMEOUT, "small graph: a grid barrier hit its bound");
+  if (int e = map_err(c, err, lpa ? "lpa" : "split")) return e;
+  if (st) {
+    if (lpa) {
+      st->iterations = r.sweeps;
+      st->converged = r.converged;
+      st->edges_scanned = (int64_t)r.scanned;
+      for (int t = 0; t < r.sweeps && t < GSL_STATS_SWEEPS; ++t) {
+        st->changed[t] = (int64_t)r.changed[t];
+        st->active[t] = (int64_t)r.active[t];
+      }
+      st->ms_lpa = 1e-6f * (float)(r.time_ns[1] - r.time_ns[0]);
+    }
+    if (split) {
+      st->ms_split = 1e-6f * (float)(r.time_ns[2] - r.time_ns[lpa ? 1 : 0]);
+      st->communities = (int64_t)r.pieces;
+    }
+  }
+  if (pieces) *pieces = (long long)r.pieces;
+  return GSL_OK;
+}
+
 struct DeviceGuard {
   int prev = -1;
   explicit DeviceGuard(int dev) {
@@ -982,6 +1059,7 @@ int gsl_ctx_create(gsl_ctx** out, int device) {
   c->device = device;
   DeviceGuard dg(device);
   cudaDeviceGetAttribute(&c->di.sm_count, cudaDevAttrMultiProcessorCount, device);
+  cudaDeviceGetAttribute(&c->di.cooperative, cudaDevAttrCooperativeLaunch, device);
   cudaDeviceGetAttribute(&c->di.max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   bool ok = cudaMalloc(&c->ctr, sizeof(Counters)) == cudaSuccess &&
             cudaMallocHost(&c->ctr_h, sizeof(Counters)) == cudaSuccess &&
@@ -990,7 +1068,9 @@ int gsl_ctx_create(gsl_ctx** out, int device) {
             cudaMalloc(&c->k_dev, sizeof(unsigned long long)) == cudaSuccess &&
             cudaMallocHost(&c->k_h, sizeof(unsigned long long)) == cudaSuccess &&
             cudaMalloc(&c->fix_dev, 3 * sizeof(int)) == cudaSuccess &&
-            cudaMallocHost(&c->fix_h, 3 * sizeof(int)) == cudaSuccess;
+            cudaMallocHost(&c->fix_h, 3 * sizeof(int)) == cudaSuccess &&
+            cudaMalloc(&c->solo, sizeof(SoloState)) == cudaSuccess &&
+            cudaMallocHost(&c->solo_h, sizeof(SoloState)) == cudaSuccess;
   for (int i = 0; ok && i < 4; ++i) ok = cudaEventCreate(&c->ev[i]) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
@@ -1009,13 +1089,14 @@ int gsl_ctx_destroy(gsl_ctx* c) {
                    c->block_sums, c->partials, c->scratch, c->hub_scratch, c->rowbits, c->lg, c->work2, c->gbits, c->fkeys, c->fvals, c->hub_piece_start,
                    c->hub_ustart, c->hub_best, c->hub_own, c->hub_wsum, c->hub_used_cnt, c->hub_clu, c->hub_used, c->hub_tab,
                    c->ctr, c->sums, c->k_dev,
-                   c->st_off, c->st_col, c->st_w, c->st_lab, c->fix_w, c->fix_dev, c->kw};
+                   c->st_off, c->st_col, c->st_w, c->st_lab, c->fix_w, c->fix_dev, c->kw, c->solo};
   for (void* p : dptrs)
     if (p) cudaFree(p);
   if (c->ctr_h) cudaFreeHost(c->ctr_h);
   if (c->sums_h) cudaFreeHost(c->sums_h);
   if (c->k_h) cudaFreeHost(c->k_h);
   if (c->fix_h) cudaFreeHost(c->fix_h);
+  if (c->solo_h) cudaFreeHost(c->solo_h);
   for (auto& e : c->ev)
     if (e) cudaEventDestroy(e);
   for (auto& e : c->evpool) cudaEventDestroy(e);
@@ -1308,6 +1389,11 @@ int gsl_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
   DeviceGuard dg(c->device);
   cudaStream_t s = (cudaStream_t)stream;
   if (int r = ensure_vertex_scratch(c, g->n)) return r;
+  bool handled = false;
+  if (int r = run_solo(c, g, weights, labels_init, nullptr, true, false, tol, max_iters, mode, labels_out, st, nullptr,
+                       s, &handled))
+    return r;
+  if (handled) return GSL_OK;
   CK(cudaEventRecord(c->ev[0], s));
   if (int r = prepare_graph(c, g, s)) return r;
   int* fin = nullptr;
@@ -1424,8 +1510,18 @@ int gsl_split(gsl_ctx* c, const gsl_csr* g, const int32_t* labels_in, int32_t* l
   DeviceGuard dg(c->device);
   cudaStream_t s = (cudaStream_t)stream;
   if (int r = ensure_vertex_scratch(c, g->n)) return r;
-  if (int r = prepare_graph(c, g, s)) return r;
   long long k = 0;
+  if (!renumber) {
+    bool handled = false;
+    if (int r = run_solo(c, g, nullptr, nullptr, labels_in, false, true, 0.0, 0, GSL_MODE_SYNC, labels_out, nullptr,
+                         &k, s, &handled))
+      return r;
+    if (handled) {
+      if (k_out) *k_out = k;
+      return GSL_OK;
+    }
+  }
+  if (int r = prepare_graph(c, g, s)) return r;
   if (int r = run_split(c, g, labels_in, labels_out, renumber, &k, s)) return r;
   if (k_out) *k_out = k;
   return GSL_OK;
@@ -1518,6 +1614,11 @@ int gsl_gsllpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, double tol,
   DeviceGuard dg(c->device);
   cudaStream_t s = (cudaStream_t)stream;
   if (int r = ensure_vertex_scratch(c, g->n)) return r;
+  bool handled = false;
+  if (int r = run_solo(c, g, weights, nullptr, nullptr, true, true, tol, max_iters, mode, labels_out, st, nullptr, s,
+                       &handled))
+    return r;
+  if (handled) return GSL_OK;
   CK(cudaEventRecord(c->ev[0], s));
   if (int r = prepare_graph(c, g, s)) return r;
   int* fin = nullptr;

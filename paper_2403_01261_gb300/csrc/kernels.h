@@ -61,6 +61,7 @@ struct ClassBounds {
 struct DeviceInfo {
   int sm_count = 0;
   int max_smem_optin = 0;
+  int cooperative = 0;
 };
 
 // lpa_kernels.cu
@@ -206,6 +207,38 @@ cudaError_t launch_f32_to_fixed(const float* w, long long nnz, int shift, int* w
 cudaError_t launch_modularity_f32(const long long* off, const int* col, const float* wf, const int* labels,
                                   long long n, double* sigma, double* sums, Counters* ctr, const DeviceInfo& di,
                                   cudaStream_t s);
+
+// solo_kernel.cu: sweeps and split of a small graph in one cooperative launch.
+constexpr int SOLO_SWEEPS = 64;        // sweeps whose counts fit the state
+constexpr long long SOLO_ROW_MAX = 32768;   // longest row it takes
+constexpr int SOLO_LISTS = 32;         // blocks with label lists for rows of more than 4096 entries
+struct SoloState {   // zero before the launch
+  unsigned arrived, released, verdict, abandoned;   // grid barrier
+  unsigned nlong, nhuge;               // rows of more than 256 and of more than 4096 entries
+  int sweeps, converged;
+  long long longest;                   // a row longer than SOLO_ROW_MAX: nothing was done
+  unsigned long long changed[SOLO_SWEEPS], active[SOLO_SWEEPS];
+  unsigned long long scanned, pieces;
+  long long time_ns[3];                // start, end of the sweeps, end of the split
+  Counters ctr;                        // only its error bits are used
+};
+struct SoloArgs {
+  SoloState* state;
+  long long nnz;
+  const int* labels_init;              // sweeps start here (null: identity)
+  const int* labels_in;                // split alone: the labels to split
+  int lpa, split;
+  double tol;
+  int max_iters;                       // <= SOLO_SWEEPS
+  int* lab[2];
+  unsigned char* flag[2];
+  int* lists;                          // SOLO_LISTS label lists of 3 * SOLO_ROW_MAX ints
+  int* longs;                          // scratch, n ints each
+  int* parent;
+  int* named;
+  int* out;
+};
+cudaError_t launch_solo(const SweepArgs& a, const SoloArgs& q, int weights, const DeviceInfo& di, cudaStream_t s);
 
 // split_kernels.cu.  parent and named: n ints of scratch each.
 cudaError_t launch_split(const long long* off, const int* col, long long n, const int* labels,

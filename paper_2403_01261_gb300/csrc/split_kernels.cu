@@ -28,63 +28,11 @@
 // All loops are bounded (parents strictly decrease along a path and a
 // failed CAS strictly lowers the root being linked); the bound is a safety
 // net that raises ERRBIT_TIMEOUT.
-#include "kernels.h"
+#include "uf_device.cuh"
 
 namespace gsl {
 
 namespace {
-
-// Bound of the union-find loops.  The default is a compile-time constant
-// (the loops are measurably faster that way); kernels instantiated with
-// UfCap<0> take a bound lowered at run time (gsl_ctx_set_retry_bounds).
-constexpr int UF_CAP = 1 << 26;
-template <int FIXED>
-struct UfCap {
-  int runtime;
-  __device__ __forceinline__ int get() const { return FIXED > 0 ? FIXED : runtime; }
-};
-
-template <int F>
-__device__ __forceinline__ int uf_find(int* p, int x, int* err, UfCap<F> cap) {
-  const int bound = cap.get();
-  for (int it = 0; it < bound; ++it) {
-    const int px = __ldcg(p + x);
-    if (px == x) return x;
-    const int ppx = __ldcg(p + px);
-    if (ppx != px) __stcg(p + x, ppx);
-    x = ppx;
-  }
-  raise_err(err, ERRBIT_TIMEOUT);
-  return x;
-}
-
-template <int F>
-__device__ __forceinline__ void uf_unite(int* p, int a, int b, int* err, UfCap<F> cap) {
-  const int bound = cap.get();
-  for (int it = 0; it < bound; ++it) {
-    a = uf_find(p, a, err, cap);
-    b = uf_find(p, b, err, cap);
-    if (a == b) return;
-    const int hi = a > b ? a : b, lo = a > b ? b : a;
-    const int old = atomicCAS(p + hi, hi, lo);
-    if (old == hi) return;
-    a = old;   // hi got a parent meanwhile: continue from it
-    b = lo;
-  }
-  raise_err(err, ERRBIT_TIMEOUT);
-}
-
-// Slot of community label c in a table of n entries.
-__device__ __forceinline__ long long comm_slot(int c, long long n) {
-  if (c >= 0 && (long long)c < n) return c;
-  unsigned x = (unsigned)c;
-  x ^= x >> 16;
-  x *= 0x7FEB352Du;
-  x ^= x >> 15;
-  x *= 0x846CA68Bu;
-  x ^= x >> 16;
-  return (long long)(((unsigned long long)x * (unsigned long long)n) >> 32);
-}
 
 constexpr int SPLIT_SAMPLE = 2;   // same-community links per vertex before the named pieces are known
 constexpr int SPLIT_SCAN = 8;     // row entries the sampling pass looks at for them
