@@ -78,6 +78,13 @@ __device__ __forceinline__ void count_graph_change(const SweepArgs& a, int v) {
   if (a.dn_graph) atomicAdd(a.dn_graph + a.gid[v], 1u);
 }
 
+// Batched mode: the changed lanes' graphs, one add per graph present.
+__device__ __forceinline__ void count_tile_changes(const SweepArgs& a, int v, bool changed) {
+  const int g = changed ? a.gid[v] : -1;
+  const unsigned m = __match_any_sync(FULL, g);
+  if (changed && (m & lanemask_lt()) == 0) atomicAdd(a.dn_graph + g, (unsigned)__popc(m));
+}
+
 // The rows of a class this sweep: what the majority filter left of it, or its
 // part of the worklist.
 __device__ __forceinline__ const int* class_work(const SweepArgs& a, int cls) {

@@ -56,13 +56,6 @@ __device__ __forceinline__ void flush_tile(Counters* ctr, unsigned dn, unsigned 
     }
   }
 }
-
-// Batched mode: the changed lanes' graphs, one add per graph present.
-__device__ __forceinline__ void count_tile_changes(const SweepArgs& a, int v, bool changed) {
-  const int g = changed ? a.gid[v] : -1;
-  const unsigned m = __match_any_sync(FULL, g);
-  if (changed && (m & lanemask_lt()) == 0) atomicAdd(a.dn_graph + g, (unsigned)__popc(m));
-}
 }  // namespace
 
 // Classes 0..2 among the vertices [v0, v1): all of them (all_active) or
