@@ -776,15 +776,10 @@ int run_split(gsl_ctx* c, const gsl_csr* g, const int32_t* labels_in, int32_t* l
   const long long n = g->n;
   if (int r = reset_sweep_counters(c, s)) return r;
   int pe = prof_begin(c, s);
-  CK(launch_bin(OFF(g), n, nullptr, 1, c->tune, c->work, c->ctr, c->di, s));
-  prof_end(c, pe, SL_BIN, s, 1);
-  c->profile.slot[SL_BIN].vertices += n;
-  c->profile.slot[SL_BIN].bytes += 20.0 * (double)n;
-  pe = prof_begin(c, s);
   // c->rank is free until the renumbering below: it holds the named pieces
   CK(launch_split(OFF(g), g->cols, n, labels_in, c->work, c->ctr, c->parent, c->rank, labels_out, c->tune, c->di,
                   s));
-  prof_end(c, pe, SL_SPLIT, s, 17);
+  prof_end(c, pe, SL_SPLIT, s, SPLIT_LAUNCHES);
   // per vertex: parent init, own label, offsets, compress read and label
   // write; per entry: the column and, for the half with j < u, the label
   c->profile.slot[SL_SPLIT].vertices += n;

@@ -240,9 +240,11 @@ struct SoloArgs {
 };
 cudaError_t launch_solo(const SweepArgs& a, const SoloArgs& q, int weights, const DeviceInfo& di, cudaStream_t s);
 
-// split_kernels.cu.  parent and named: n ints of scratch each.
+// split_kernels.cu.  list, parent and named: n ints of scratch each;
+// Counters::hook_rows zero.
+constexpr int SPLIT_LAUNCHES = 9;
 cudaError_t launch_split(const long long* off, const int* col, long long n, const int* labels,
-                         const int* work, Counters* ctr, int* parent, int* named, int* out, const Tuning& t,
+                         int* list, Counters* ctr, int* parent, int* named, int* out, const Tuning& t,
                          const DeviceInfo& di, cudaStream_t s);
 cudaError_t launch_renumber(const int* rep, int* out, long long n, int* rank, unsigned long long* block_sums,
                             long long nblocks_cap, unsigned long long* k_dev, const DeviceInfo& di,

@@ -343,7 +343,10 @@ __global__ void __launch_bounds__(SOLO_BLOCK, SOLO_BLOCKS_PER_SM) solo_kernel(Sw
       q.flag[0][v] = 0;
       q.flag[1][v] = 0;
     }
-    if (q.split) __stcg(q.parent + v, (int)v);
+    if (q.split) {
+      __stcg(q.parent + v, (int)v);
+      __stcg(q.named + v, -1);
+    }
   }
   // one atomic per block: thousands on one address would take longer than a sweep
   if (threadIdx.x == 0) sh.sums[0] = 0;
@@ -418,7 +421,7 @@ __global__ void __launch_bounds__(SOLO_BLOCK, SOLO_BLOCKS_PER_SM) solo_kernel(Sw
   if (!grid_sync(st, &a0.ctr->err, gen)) return;
   for (long long v = first; v < n; v += stride) {
     const int r = uf_find(q.parent, (int)v, err, cap);
-    __stcg(q.named + comm_slot(__ldcg(labels + v), n), r);
+    if (r != (int)v) __stcg(q.named + comm_slot(__ldcg(labels + v), n), r);   // as name_pieces_kernel
   }
   if (!grid_sync(st, &a0.ctr->err, gen)) return;
   const long long nwarps = stride >> 5;

@@ -15,16 +15,21 @@
 //     Computation via Subgraph Sampling", IPDPS 2018): first every vertex
 //     links with its first SPLIT_SAMPLE row entries of its own community;
 //     after flattening, every community names one of its pieces (the root
-//     one of its vertices holds, the last write winning; the community of
-//     the most frequent root among sampled vertices names that root), and
-//     only vertices outside their community's named piece offer their
-//     remaining entries.  An edge inside a named piece is redundant, and an
-//     edge between a named piece and another piece of the same community is
-//     offered from the other end, so the components are the same as
-//     offering every edge.  Communities are mapped to a table of n slots
-//     (label c in [0, n) to slot c, others by a hash); a slot shared by two
-//     communities names a piece of one of them, and the other's vertices
+//     one of its vertices below a root holds, the last write winning; the
+//     community of the most frequent root among sampled vertices names that
+//     root), and only vertices outside their community's named piece offer
+//     their remaining entries.  An edge inside a named piece is redundant,
+//     and an edge between a named piece and another piece of the same
+//     community is offered from the other end, so the components are the
+//     same as offering every edge.  Communities are mapped to a table of n
+//     slots (label c in [0, n) to slot c, others by a hash); a slot shared by
+//     two communities names a piece of one of them, and the other's vertices
 //     then all offer their entries, which is slower but still exact.
+// The second phase takes the vertices in natural order, one lane each: a warp
+// per vertex spent four dependent loads on finding out that there was nothing
+// to offer, and stray members, written last, named their own single-vertex
+// pieces, so that most of their communities offered everything (4 M-vertex
+// planted partition: 0.85 ms of hooks, now 0.08).
 // All loops are bounded (parents strictly decrease along a path and a
 // failed CAS strictly lowers the root being linked); the bound is a safety
 // net that raises ERRBIT_TIMEOUT.
@@ -75,7 +80,7 @@ __global__ void init_parent_kernel(int* __restrict__ p, long long n) {
     p[v] = (int)v;
 }
 
-// Phase 1: every vertex links with the first SPLIT_SAMPLE same-community
+// Every vertex links with the first SPLIT_SAMPLE same-community
 // neighbours among its first SPLIT_SCAN row entries.
 // The first two entries' columns and labels are requested together; the
 // rest of the scan (when they are not both links) goes one entry at a time.
@@ -106,14 +111,14 @@ __global__ void sample_link_kernel(const long long* __restrict__ off, const int*
   }
 }
 
-// Phases 2 and 5: every parent becomes the root.
+// Every parent becomes the root.
 template <int F>
 __global__ void flatten_kernel(int* p, int* out, long long n, Counters* ctr, UfCap<F> cap) {   // out may equal p
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x)
     out[v] = uf_find(p, (int)v, &ctr->err, cap);
 }
 
-// Phase 3: the most frequent root among 1024 sampled vertices (one block
+// The most frequent root among 1024 sampled vertices (one block
 // of 1024 threads: sample, bitonic sort in shared memory, longest run).
 __global__ void __launch_bounds__(1024) giant_kernel(const int* p, long long n, Counters* ctr) {
   __shared__ int a[1024];
@@ -148,14 +153,20 @@ __global__ void __launch_bounds__(1024) giant_kernel(const int* p, long long n, 
   }
 }
 
-// Phase 3b: every community names a piece: the root its vertices hold
-// after flattening, the last write winning; then the community of the most
-// frequent sampled root (giant_kernel) names that root.  Every slot read
-// later was written by the vertex reading it, so no initial value is needed.
+// Every community names a piece: the root its vertices hold after flattening,
+// the last write winning; then the community of the most frequent sampled
+// root (giant_kernel) names that root.  Roots do not name themselves: a
+// community's stray members, scattered over the ids and often written last,
+// would name their single-vertex pieces and leave the others to offer their
+// whole rows.  Slots nobody names hold -1, and their pieces all offer.
 __global__ void name_pieces_kernel(const int* __restrict__ p, const int* __restrict__ labels, long long n,
                                    int* __restrict__ named) {
-  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x)
-    named[comm_slot(labels[v], n)] = p[v];
+  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
+    const int r = p[v];
+    if (r == (int)v) continue;
+    int* slot = named + comm_slot(labels[v], n);
+    if (*slot != r) *slot = r;   // one community may hold nearly every vertex: mostly read
+  }
 }
 
 __global__ void name_giant_kernel(const int* __restrict__ labels, long long n, int* __restrict__ named,
@@ -164,49 +175,66 @@ __global__ void name_giant_kernel(const int* __restrict__ labels, long long n, i
   if (g >= 0 && (long long)g < n) named[comm_slot(labels[g], n)] = g;
 }
 
-// Phase 4, classes 0..7: G lanes per vertex; vertices in their community's
-// named piece are skipped, the others offer entries SPLIT_SAMPLE.. of their
-// row (both directions: the other end may be skipped).
-template <int G, int F>
-__global__ void __launch_bounds__(256) hook_group_kernel(const long long* __restrict__ off, const int* __restrict__ col,
-                                                          const int* __restrict__ labels, int* p, long long n,
-                                                          const int* __restrict__ work, Counters* ctr, int cls,
-                                                          UfCap<F> cap, const int* __restrict__ named) {
-  const unsigned cnt = (unsigned)ctr->cls_total[cls];
-  const int* w = work + ctr->cls_start[cls];
-  const int gl = threadIdx.x & (G - 1);
-  const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
-  const long long ng = ((long long)gridDim.x * blockDim.x) / G;
-  for (long long item = gid; item < (long long)cnt; item += ng) {
-    const int u = w[item];
-    const long long s = off[u], e = off[u + 1];
-    if (e - s <= SPLIT_SAMPLE) continue;
-    const int ru = __ldcg(p + u);
-    const int cu = labels[u];
-    if (ru == named[comm_slot(cu, n)]) continue;
-    for (long long k = s + SPLIT_SAMPLE + gl; k < e; k += G) hook_entry_flat(col, labels, p, n, u, cu, ru, k, &ctr->err, cap);
+// Vertices outside their community's named piece offer entries SPLIT_SAMPLE..
+// of their row (both directions: the other end may be skipped): rows of up to
+// HOOK_LANE entries by their lane, up to HOOK_WARP by the warp, longer ones
+// are listed for hook_long_kernel.
+constexpr int HOOK_LANE = 8, HOOK_WARP = 2048;
+
+template <int F>
+__global__ void __launch_bounds__(256) hook_kernel(const long long* __restrict__ off, const int* __restrict__ col,
+                                                    const int* __restrict__ labels, int* p, long long n,
+                                                    int* __restrict__ list, Counters* ctr, UfCap<F> cap,
+                                                    const int* __restrict__ named) {
+  const int lane = threadIdx.x & 31;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long w = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); w < n; w += stride) {   // warp-uniform
+    const long long u = w + lane;
+    long long s = 0, e = 0;
+    int cu = 0, ru = 0;
+    bool offer = false;
+    if (u < n) {
+      s = off[u] + SPLIT_SAMPLE;
+      e = off[u + 1];
+      if (s < e) {
+        ru = __ldcg(p + u);
+        cu = labels[u];
+        offer = ru != named[comm_slot(cu, n)];
+      }
+    }
+    if (offer && e - s > HOOK_WARP) {
+      list[atomicAdd(&ctr->hook_rows, 1u)] = (int)u;
+      offer = false;
+    }
+    if (offer && e - s <= HOOK_LANE) {
+      for (long long k = s; k < e; ++k) hook_entry_flat(col, labels, p, n, (int)u, cu, ru, k, &ctr->err, cap);
+      offer = false;
+    }
+    __syncwarp();
+    unsigned mask = __ballot_sync(FULL, offer);
+    while (mask) {
+      const int r = __ffs((int)mask) - 1;
+      mask &= mask - 1;
+      const long long rs = __shfl_sync(FULL, s, r), re = __shfl_sync(FULL, e, r);
+      const int rc = __shfl_sync(FULL, cu, r), rr = __shfl_sync(FULL, ru, r);
+      for (long long k = rs + lane; k < re; k += 32)
+        hook_entry_flat(col, labels, p, n, (int)w + r, rc, rr, k, &ctr->err, cap);
+      __syncwarp();
+    }
   }
 }
 
-// Phase 4, classes 8..9: one block per vertex.
+// The listed rows, one block each.
 template <int F>
-__global__ void __launch_bounds__(512) hook_block_kernel(const long long* __restrict__ off, const int* __restrict__ col,
-                                                          const int* __restrict__ labels, int* p, long long n,
-                                                          const int* __restrict__ work, Counters* ctr, int cls,
-                                                          UfCap<F> cap, const int* __restrict__ named) {
-  const unsigned cnt = (unsigned)ctr->cls_total[cls];
-  const int* w = work + ctr->cls_start[cls];
-  __shared__ int s_root;
-  for (long long item = blockIdx.x; item < (long long)cnt; item += gridDim.x) {
-    const int u = w[item];
-    const long long s = off[u], e = off[u + 1];
-    if (threadIdx.x == 0) s_root = __ldcg(p + u);
-    __syncthreads();
-    const int ru = s_root;
-    __syncthreads();
-    const int cu = labels[u];
-    if (ru == named[comm_slot(cu, n)]) continue;
-    for (long long k = s + SPLIT_SAMPLE + threadIdx.x; k < e; k += blockDim.x)
+__global__ void __launch_bounds__(512) hook_long_kernel(const long long* __restrict__ off, const int* __restrict__ col,
+                                                         const int* __restrict__ labels, int* p, long long n,
+                                                         const int* __restrict__ list, Counters* ctr, UfCap<F> cap) {
+  const unsigned cnt = ctr->hook_rows;
+  for (unsigned i = blockIdx.x; i < cnt; i += gridDim.x) {
+    const int u = list[i];
+    const int ru = __ldcg(p + u), cu = labels[u];   // any value p[u] has held will do
+    const long long e = off[u + 1];
+    for (long long k = off[u] + SPLIT_SAMPLE + threadIdx.x; k < e; k += blockDim.x)
       hook_entry_flat(col, labels, p, n, u, cu, ru, k, &ctr->err, cap);
   }
 }
@@ -409,38 +437,30 @@ int grid_for(long long items, int block, const DeviceInfo& di, int per_sm = 8) {
 }  // namespace
 
 template <int F>
-void launch_split_t(const long long* off, const int* col, long long n, const int* labels, const int* work,
-                    Counters* ctr, int* parent, int* named, int* out, UfCap<F> cap, const DeviceInfo& di,
-                    cudaStream_t s) {
-  init_parent_kernel<<<grid_for(n, 256, di), 256, 0, s>>>(parent, n);
-  sample_link_kernel<F><<<grid_for(n, 256, di), 256, 0, s>>>(off, col, labels, parent, n, ctr, cap);
-  flatten_kernel<F><<<grid_for(n, 256, di), 256, 0, s>>>(parent, parent, n, ctr, cap);
+void launch_split_t(const long long* off, const int* col, long long n, const int* labels, int* list, Counters* ctr,
+                    int* parent, int* named, int* out, UfCap<F> cap, const DeviceInfo& di, cudaStream_t s) {
+  const int g = grid_for(n, 256, di);
+  init_parent_kernel<<<g, 256, 0, s>>>(parent, n);
+  sample_link_kernel<F><<<g, 256, 0, s>>>(off, col, labels, parent, n, ctr, cap);
+  flatten_kernel<F><<<g, 256, 0, s>>>(parent, parent, n, ctr, cap);
   giant_kernel<<<1, 1024, 0, s>>>(parent, n, ctr);
-  name_pieces_kernel<<<grid_for(n, 256, di), 256, 0, s>>>(parent, labels, n, named);
+  cudaMemsetAsync(named, 0xFF, sizeof(int) * (size_t)n, s);
+  name_pieces_kernel<<<g, 256, 0, s>>>(parent, labels, n, named);
   name_giant_kernel<<<1, 1, 0, s>>>(labels, n, named, ctr);
-  const int g = 8 * di.sm_count;
-  hook_group_kernel<1, F><<<g, 256, 0, s>>>(off, col, labels, parent, n, work, ctr, 0, cap, named);
-  hook_group_kernel<2, F><<<g, 256, 0, s>>>(off, col, labels, parent, n, work, ctr, 1, cap, named);
-  hook_group_kernel<4, F><<<g, 256, 0, s>>>(off, col, labels, parent, n, work, ctr, 2, cap, named);
-  hook_group_kernel<8, F><<<g, 256, 0, s>>>(off, col, labels, parent, n, work, ctr, 3, cap, named);
-  hook_group_kernel<16, F><<<g, 256, 0, s>>>(off, col, labels, parent, n, work, ctr, 4, cap, named);
-  hook_group_kernel<32, F><<<g, 256, 0, s>>>(off, col, labels, parent, n, work, ctr, 5, cap, named);
-  hook_group_kernel<32, F><<<g, 256, 0, s>>>(off, col, labels, parent, n, work, ctr, CLS_WARP_S, cap, named);
-  hook_group_kernel<32, F><<<g, 256, 0, s>>>(off, col, labels, parent, n, work, ctr, CLS_WARP_L, cap, named);
-  hook_block_kernel<F><<<4 * di.sm_count, 512, 0, s>>>(off, col, labels, parent, n, work, ctr, CLS_BLOCK, cap, named);
-  hook_block_kernel<F><<<4 * di.sm_count, 512, 0, s>>>(off, col, labels, parent, n, work, ctr, CLS_HUB, cap, named);
-  flatten_kernel<F><<<grid_for(n, 256, di), 256, 0, s>>>(parent, out, n, ctr, cap);
-  count_launches(17);
+  hook_kernel<F><<<g, 256, 0, s>>>(off, col, labels, parent, n, list, ctr, cap, named);
+  hook_long_kernel<F><<<4 * di.sm_count, 512, 0, s>>>(off, col, labels, parent, n, list, ctr, cap);
+  flatten_kernel<F><<<g, 256, 0, s>>>(parent, out, n, ctr, cap);
+  count_launches(SPLIT_LAUNCHES);
 }
 
-cudaError_t launch_split(const long long* off, const int* col, long long n, const int* labels, const int* work,
+cudaError_t launch_split(const long long* off, const int* col, long long n, const int* labels, int* list,
                          Counters* ctr, int* parent, int* named, int* out, const Tuning& t, const DeviceInfo& di,
                          cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (t.uf_cap == UF_CAP)
-    launch_split_t(off, col, n, labels, work, ctr, parent, named, out, UfCap<UF_CAP>{0}, di, s);
+    launch_split_t(off, col, n, labels, list, ctr, parent, named, out, UfCap<UF_CAP>{0}, di, s);
   else
-    launch_split_t(off, col, n, labels, work, ctr, parent, named, out, UfCap<0>{t.uf_cap}, di, s);
+    launch_split_t(off, col, n, labels, list, ctr, parent, named, out, UfCap<0>{t.uf_cap}, di, s);
   return cudaGetLastError();
 }
 
