@@ -251,14 +251,17 @@ __device__ __forceinline__ void sketch_rounds(Items& items, const int* wp, const
       if (open(l)) {
         const unsigned h = t.slot((unsigned)l, r);
         // every weight is at least 1, so a label of a shared slot has at most the slot's sum less one
-        if (t.lab[h] == EMPTY32 && beats<S>(t.sum[h] - 1, ~(unsigned)l, best)) left = true;
+        if (t.lab[h] == EMPTY32 && t.sum[h] && beats<S>(t.sum[h] - 1, ~(unsigned)l, best)) left = true;
         else l = (int)((unsigned)l | SETTLED);
       }
     });
     if (!team_any<T>(left)) return;
     if (r + 1 - first_round >= rounds) break;
   }
-  if (rounds < SKETCH_ROUNDS) raise_err(err, ERRBIT_TIMEOUT);   // a lowered retry bound
+  if (rounds < SKETCH_ROUNDS) {   // a lowered retry bound
+    raise_err(err, ERRBIT_TIMEOUT);
+    return;
+  }
   // labels that met another one in every round: one by one, the smallest first
   for (;;) {
     unsigned x = EMPTY32;

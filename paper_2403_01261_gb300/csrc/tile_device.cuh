@@ -95,10 +95,13 @@ __device__ __forceinline__ Best<S> group_sketch(GroupSlots<S>& slots, int base, 
     if (act) *sum = 0;
     __syncwarp();
     take_better(best, group_best<G>(act && !shared_slot ? c : (S)0, lbl, gmask));
-    act = act && shared_slot && beats<S>(c - 1, ~(unsigned)lbl, best);
+    act = act && shared_slot && c && beats<S>(c - 1, ~(unsigned)lbl, best);
     if (!__any_sync(FULL, act)) return best;
     if (r + 1 >= rounds) {
-      if (rounds < SKETCH_ROUNDS) raise_err(err, ERRBIT_TIMEOUT);   // a lowered retry bound
+      if (rounds < SKETCH_ROUNDS) {   // a lowered retry bound
+        raise_err(err, ERRBIT_TIMEOUT);
+        return best;
+      }
       const unsigned m = __match_any_sync(FULL, act ? lbl : -1) & gmask;
       S e = 0;
       if (act) e = mask_sum(m, wt);   // m: the lanes of this label, all here
