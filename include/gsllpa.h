@@ -83,35 +83,40 @@ int gsl_ctx_create(gsl_ctx** ctx, int device);
 int gsl_ctx_destroy(gsl_ctx* ctx);
 
 /* Degree-class thresholds of the sweep kernels: vertices of degree
- * 33..warp_max are handled by one warp each, degree warp_max+1..blk_max by
- * one block each, larger degrees (hubs) by one 8-CTA thread-block cluster
- * each (or in 8192-entry pieces spread over blocks: see
- * gsl_ctx_set_hub_cluster).  Label sums use shared-memory hash tables
- * (8 KB per warp, 96 KB per block, 8 x 96 KB per cluster) and spill to
- * context-owned global tables when a vertex has more distinct neighbour
- * labels than fit.  Defaults 1024 and 32768.  Requires 32 <= warp_max <=
- * 2^20 and warp_max <= blk_max.  Results do not depend on these values. */
+ * 33..warp_max (256 at most by one warp, longer ones by 128 threads),
+ * warp_max+1..blk_max by a 256-thread block each.  Larger degrees (hubs) run
+ * beside those while none exceeds 2^20 and blk_max is at least its default;
+ * else they take one 8-CTA thread-block cluster each, or 8192-entry pieces
+ * spread over blocks (gsl_ctx_set_hub_cluster).  Labels are counted in
+ * shared-memory sketches; rows past 4096 entries keep a label list in
+ * context-owned memory.  Defaults 1024 and 131072.  Requires 32 <= warp_max
+ * <= 2^20 and warp_max <= blk_max.  Results do not depend on these values.
+ *
+ * A context on which no tuning differs from its default runs synchronous
+ * calls on small graphs (up to 2^19 vertices, 2^23 entries and 32768 entries
+ * a row, max_iters <= 64) in one cooperative launch. */
 int gsl_ctx_set_tuning(gsl_ctx* ctx, int32_t warp_max, int32_t blk_max);
 
-/* Shape of the block kernel (degree warp_max+1..blk_max and hub pieces):
- * threads per block (128, 256 or 512) and shared-memory table slots per
- * block (8 bytes each; at least 16 * threads, so that the slots warps may
- * still claim after a table is declared full -- up to 128 per warp -- fit
- * in its last quarter, and the table must fit one block's shared memory).  Defaults 512 and 12288.  Hub rows are split into pieces only
- * while a piece always fits the table (at least ~11,600 slots); below that
- * hubs take one block each.  Results do not depend on these values. */
+/* Shape of the hub kernels (clusters and pieces): threads per block of the
+ * piece kernel (128, 256 or 512) and shared-memory table slots per block (8
+ * bytes each; at least 16 * threads, and the table must fit one block's
+ * shared memory).  Defaults 512 and 12288.  Hub rows are split into pieces
+ * only while a piece always fits the table (at least ~11,600 slots); below
+ * that hubs take one block each.  Results do not depend on these values. */
 int gsl_ctx_set_block_config(gsl_ctx* ctx, int32_t threads, int32_t table_slots);
 
-/* Own-label majority filter for rows of the two longest table classes
- * (degree above 256 up to blk_max; the paper has no counterpart), and also
- * for the rows of 33..256 entries from sweep 4 on in single-graph calls and
- * from sweep 6 on in the batched loop.  Before their hash tables are built,
- * one lean warp-per-row pass sums the weight of a row's entries carrying
- * the vertex's own label; when it is more than half of the row's weight
- * (the vertex itself excluded) the own label is Eq. 2's strict argmax and
- * the row is done.  mode 0: never; 1 (default): from sweep 3 on (sweep 2
- * reads the nearly all-distinct labels of sweep 1); 2: every sweep after
- * the first.  Labels and statistics do not depend on the mode. */
+/* Majority filter (the paper has no counterpart).  Before the rows of more
+ * than 32 entries are counted, one lean pass sums the weight of a row's
+ * entries that carry one label; when it is more than half of the row's weight
+ * (the vertex itself excluded) that label is Eq. 2's strict argmax and the row
+ * is done.  In synchronous single-graph sweeps a sample of the entries picks
+ * the label: one that most entries of the graph carry (tested on every row of
+ * more than 32 entries), else the vertex's own (rows above 256 entries, and
+ * those of 33..256 from sweep 4 on), or no label when few neighbours share
+ * any.  The batched loop (33..256 entries from sweep 6 on) and asynchronous
+ * sweeps test the own label.  mode 0: never; 1 (default): from sweep 3 on
+ * (sweep 2 reads the nearly all-distinct labels of sweep 1); 2: every sweep
+ * after the first.  Labels and change counts do not depend on the mode. */
 int gsl_ctx_set_majority(gsl_ctx* ctx, int32_t mode);
 
 /* Two-phase synchronous sweeps (the paper has no counterpart: it is a GPU
@@ -132,19 +137,21 @@ int gsl_ctx_set_pregather(gsl_ctx* ctx, int32_t mode);
  * GSL_ERR_INVALID.  Labels do not depend on it. */
 int gsl_ctx_set_f32_fixed(gsl_ctx* ctx, int32_t mode);
 
-/* Hub rows (synchronous or asynchronous sweeps, integer weights) whose
- * degree is at most max_degree are aggregated by one thread-block cluster
- * of 8 CTAs each: the row's label table is spread over the 8 CTAs' shared
- * memories and filled with distributed-shared-memory atomics.  A row with
- * more distinct labels than those tables hold is redone in a global-memory
- * table.  Longer hubs are cut into pieces of 8192 entries.  0 turns the
- * clusters off; by default every hub row goes to a cluster.  max_degree
- * < 0: GSL_ERR_INVALID.  Labels and statistics do not depend on it. */
+/* Hub rows that the hub kernels take (gsl_ctx_set_tuning; integer weights)
+ * and whose degree is at most max_degree are aggregated by one thread-block
+ * cluster of 8 CTAs each: the row's label table is spread over the 8 CTAs'
+ * shared memories and filled with distributed-shared-memory atomics.  A row
+ * with more distinct labels than those tables hold is redone in a
+ * global-memory table.  Longer hubs are cut into pieces of 8192 entries.  0
+ * turns the clusters off; by default every such row goes to a cluster.
+ * max_degree < 0: GSL_ERR_INVALID.  Labels and statistics do not depend on
+ * it. */
 int gsl_ctx_set_hub_cluster(gsl_ctx* ctx, int64_t max_degree);
 
 /* Bounds of the device-side retry loops (the paper has no counterpart).
- * Every open-addressing insert of the sweep tables stops after probe_bound
- * probes, and every union-find find or union of the split after
+ * Every open-addressing insert of the hub and float64 tables stops after
+ * probe_bound probes, every row's sketch after probe_bound counting rounds
+ * (bounds below 8), and every union-find find or union of the split after
  * unionfind_bound steps; a loop that reaches its bound raises an error bit,
  * the kernel finishes without waiting on anything, and the call returns
  * GSL_ERR_TIMEOUT (labels unspecified).  The defaults (2^24 probes, 2^26
@@ -237,10 +244,11 @@ int gsl_lpa(gsl_ctx* ctx, const gsl_csr* g, const int32_t* weights, const int32_
  * agree to rounding; they are whenever every partial sum is exact in
  * float64 (for instance small integers or multiples of 1/8).  Modularity is
  * formed from float64 sums.  When every weight is a multiple of 2^-S and
- * every row's total times 2^S stays below 2^31 (checked through the largest
- * weight and the largest degree), every float64 sum is exact and the
- * sweeps run on the integer path with weights w * 2^S, which compares the
- * same sums scaled by 2^S: the labels are the float path's
+ * every weight times 2^S below 2^31 and every row's total times 2^S below
+ * 2^53 (checked through the largest weight and the largest degree), every
+ * float64 sum is exact and the sweeps run on the integer path with weights
+ * w * 2^S (32-bit sums below 2^31, else 64-bit), which compares the same
+ * sums scaled by 2^S: the labels are the float path's
  * (gsl_ctx_set_f32_fixed turns this off). */
 int gsl_lpa_f32(gsl_ctx* ctx, const gsl_csr* g, const float* weights, const int32_t* labels_init,
                 double tolerance, int32_t max_iters, int32_t mode, int32_t* labels_out, gsl_stats* stats,

@@ -140,11 +140,12 @@ namespace {
 // int64_t is `long` on LP64 Linux; the kernels take `long long`.
 inline const long long* OFF(const gsl_csr* g) { return reinterpret_cast<const long long*>(g->offsets); }
 
-// Single-graph sweeps: from this sweep on, the own-label majority filter
-// takes the rows of class 6 too, once most of them keep their label (R-MAT
-// 25, ms per step: from sweep 4 51.3 -> 50.6; from sweep 3 no gain, as
-// sweep 3's class-6 rows mostly change and the filter's pass over them is
-// then repeated by the warp kernel).  The batched loop's planted-partition
+// Single-graph sweeps: from this sweep on, the own-label test of the majority
+// filter takes the rows of class 6 too, once most of them keep their label
+// (measured on R-MAT 25 when it was the only test, ms per step: from sweep 4
+// 51.3 -> 50.6; from sweep 3 no gain, as sweep 3's class-6 rows mostly change
+// and the filter's pass over them is then repeated by the warp kernel).  The
+// test for a label that dominates the graph takes them whenever it is on.  The batched loop's planted-partition
 // graphs settle later (4096-graph batch, ms per step: none 459.8, from
 // sweep 4 500.5, from sweep 6 454.1).
 constexpr int FILTER6_FROM = 4;

@@ -8,11 +8,14 @@
 // threads add: the synchronous sweep is deterministic.
 //
 // Work is split by degree class (binning pass below):
-//   d <= 32          one lane, half a warp or a warp per row (tile_kernels.cu).
+//   d <= 32          one lane, half a warp or a warp per row (tile_kernels.cu)
 //   d <= warp_small  one warp per row      (sketch_kernels.cu)
 //   d <= warp_max    128 threads per row   (the same)
 //   d <= blk_max     256 threads per row   (the same)
-//   larger           thread-block clusters or pieces (hub_kernels.cu)
+//   larger           beside those, or in thread-block clusters and pieces
+//                    (hub_kernels.cu)
+// Small graphs run whole in one launch (solo_kernel.cu).  This file holds the
+// classification, the binning and the streamed first sweep.
 //
 // Pruning (lpaMove(): a processed vertex is re-marked when a neighbour
 // changes): a vertex whose label changes sets the next-frontier flag of each
