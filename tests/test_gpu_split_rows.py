@@ -35,3 +35,23 @@ def test_split_with_strays(gpu_lib, name):
             assert np.array_equal(got.cpu().numpy(), want) and k == pieces
             got, k = c.split(off, col, torch.from_numpy(lab).to(DEV), renumber=True)
             assert k == pieces and np.array_equal(got.cpu().numpy(), np.unique(want, return_inverse=True)[1])
+
+
+@pytest.mark.parametrize("n", [622_591, 622_593, 933_889, 1_245_184, 1_245_185, 1_400_003])
+def test_split_of_long_paths(gpu_lib, n):
+    """Communities of 2000 vertices on a path with cuts: runs of vertices a warp
+    links, their last one ragged, and more runs than warps."""
+    rng = np.random.default_rng(n)
+    linked = rng.random(n - 1) < 0.995
+    deg = np.zeros(n, np.int64)
+    deg[:-1] += linked
+    deg[1:] += linked
+    off = np.concatenate(([0], np.cumsum(deg)))
+    u = np.flatnonzero(linked)
+    row, col = np.concatenate((u, u + 1)), np.concatenate((u + 1, u))
+    col = col[np.lexsort((col, row))].astype(np.int32)
+    lab = (np.arange(n) // 2000).astype(np.int32)
+    first = np.concatenate(([True], ~linked | (lab[1:] != lab[:-1])))
+    want = np.maximum.accumulate(np.where(first, np.arange(n), 0))
+    got, k = gpu_lib.split(*(torch.from_numpy(x).to(DEV) for x in (off, col, lab)))
+    assert k == first.sum() and np.array_equal(got.cpu().numpy(), want)
