@@ -176,6 +176,9 @@ int fail(gsl_ctx* c, int code, const char* fmt, ...) {
 template <typename T>
 int grow(gsl_ctx* c, T*& ptr, long long& cap, long long need) {
   if (need <= cap && ptr) return GSL_OK;
+  // the captured batched loop holds the addresses of the buffers it was
+  // captured with, and this call may fail before it captures again
+  c->batch_key.clear();
   if (ptr) cudaFree(ptr);
   ptr = nullptr;
   cap = 0;
