@@ -93,6 +93,9 @@ cudaError_t launch_phase_reset(Counters* ctr, const int* stop, cudaStream_t s);
 // sums (so in the other sweep launchers).
 long long sketch_blocks(const DeviceInfo& di);
 long long sketch_register_row();
+// Blocks of a launch with per_sm resident per SM; with lists no more than
+// sketch_blocks() of the same device, since each uses its own scratch region.
+int sketch_grid(int per_sm, bool lists, const DeviceInfo& di);
 cudaError_t launch_sketch(const SweepArgs& a, int cls, int longest, int weights, bool async_mode,
                           const DeviceInfo& di, cudaStream_t s);
 // Classes 3..8 on the worklist; class 8's launch sweeps class 9 as well when

@@ -248,15 +248,16 @@ cudaError_t launch_sketch_g(const SweepArgs& a, int cls, const DeviceInfo& di, c
   constexpr int block = T == 32 ? 256 : T;
   const size_t smem = (sizeof(unsigned) << team_lg<T>()) * (size_t)(block / T);
   void (*const kernel)(SweepArgs, int) = sketch_kernel_for<T, WT, A, G>();
-  thread_local int grid = 0;
-  if (!grid) {
+  // per host thread and device; the grid itself is formed anew on every launch
+  thread_local int per_sm = 0, per_sm_of = -1;
+  int dev = 0;
+  if (cudaError_t e = cudaGetDevice(&dev)) return e;
+  if (dev != per_sm_of) {
     if (cudaError_t e = raise_smem_limit((const void*)kernel, smem)) return e;
-    int per_sm = 0;
     if (cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem)) return e;
-    grid = (per_sm < 1 ? 1 : per_sm) * di.sm_count;
-    if (T == T_BLOCK && grid > sketch_blocks(di)) grid = (int)sketch_blocks(di);   // one scratch region each
+    per_sm_of = dev;
   }
-  kernel<<<grid, block, smem, s>>>(a, cls);
+  kernel<<<sketch_grid(per_sm, T == T_BLOCK, di), block, smem, s>>>(a, cls);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -281,6 +282,10 @@ cudaError_t launch_sketch_w(const SweepArgs& a, int cls, int longest, bool async
 }  // namespace
 
 long long sketch_blocks(const DeviceInfo& di) { return (long long)BLOCKS_PER_SM * di.sm_count; }
+int sketch_grid(int per_sm, bool lists, const DeviceInfo& di) {
+  const long long grid = (long long)(per_sm < 1 ? 1 : per_sm) * di.sm_count;
+  return (int)(lists && grid > sketch_blocks(di) ? sketch_blocks(di) : grid);
+}
 long long sketch_register_row() { return (long long)T_BLOCK * K_BLOCK; }
 
 cudaError_t launch_sketch(const SweepArgs& a, int cls, int longest, int weights, bool async_mode,
