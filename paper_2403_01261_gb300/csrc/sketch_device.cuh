@@ -164,7 +164,8 @@ __device__ __forceinline__ S team_total(unsigned long long x, TeamShared<T, S>* 
 template <int T, int WT, typename S, typename Items>
 __device__ __forceinline__ bool sketch_top(Items& items, const int* wp, const Sketch& t, Best<unsigned> mine,
                                            Best<S>& best, unsigned& open_items, TeamShared<T, S>* sh) {
-  const Best<unsigned> top = team_best<T>(mine, sh);   // with the barrier that ends the adds
+  if (T == 32) __syncwarp();   // ends the adds; team_best's barrier does so for a block
+  const Best<unsigned> top = team_best<T>(mine, sh);
   open_items = 0;
   // whether a label bounded by counter value c can beat `best`
   auto can_beat = [&](unsigned c, unsigned inv) {
