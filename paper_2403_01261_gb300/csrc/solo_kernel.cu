@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(SOLO_BLOCK, SOLO_BLOCKS_PER_SM) solo_kernel(Sw
       s = a0.off[u] + SOLO_SAMPLE;
       e = a0.off[u + 1];
       cu = __ldcg(labels + u);
-      offer = s < e && uf_find(q.parent, (int)u, err, cap) != __ldcg(q.named + comm_slot(cu, n));
+      offer = s < e && outside_named(q.named + comm_slot(cu, n), uf_find(q.parent, (int)u, err, cap));
     }
     unsigned mask = __ballot_sync(FULL, offer);
     while (mask) {

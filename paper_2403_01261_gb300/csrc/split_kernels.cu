@@ -17,7 +17,8 @@
 //     after flattening, every community names one of its pieces (the root
 //     one of its vertices below a root holds, the last write winning; the
 //     community of the most frequent root among sampled vertices names that
-//     root), and only vertices outside their community's named piece offer
+//     root; a community of roots only names the piece of the first vertex that
+//     asks), and only vertices outside their community's named piece offer
 //     their remaining entries.  An edge inside a named piece is redundant,
 //     and an edge between a named piece and another piece of the same
 //     community is offered from the other end, so the components are the
@@ -181,7 +182,7 @@ __global__ void __launch_bounds__(1024) giant_kernel(const int* p, long long n, 
 // root (giant_kernel) names that root.  Roots do not name themselves: a
 // community's stray members, scattered over the ids and often written last,
 // would name their single-vertex pieces and leave the others to offer their
-// whole rows.  Slots nobody names hold -1, and their pieces all offer.
+// whole rows.  Slots nobody names here hold -1 (outside_named).
 __global__ void name_pieces_kernel(const int* __restrict__ p, const int* __restrict__ labels, long long n,
                                    int* __restrict__ named) {
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
@@ -208,7 +209,7 @@ template <int F>
 __global__ void __launch_bounds__(256) hook_kernel(const long long* __restrict__ off, const int* __restrict__ col,
                                                     const int* __restrict__ labels, int* p, long long n,
                                                     int* __restrict__ list, Counters* ctr, UfCap<F> cap,
-                                                    const int* __restrict__ named) {
+                                                    int* named) {
   const int lane = threadIdx.x & 31;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long w = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); w < n; w += stride) {   // warp-uniform
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(256) hook_kernel(const long long* __restrict__
       if (s < e) {
         ru = __ldcg(p + u);
         cu = labels[u];
-        offer = ru != named[comm_slot(cu, n)];
+        offer = outside_named(named + comm_slot(cu, n), ru);
       }
     }
     if (offer && e - s > HOOK_WARP) {
