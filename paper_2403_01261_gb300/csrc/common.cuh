@@ -42,6 +42,7 @@ struct Counters {
   unsigned int uns_count[NCLASS];          // majority filter: rows left for the table kernels
   unsigned int phase_cls[NCLASS];          // asynchronous sweeps: cls_count of the sweep's first phase
   unsigned int filter_next;                // majority filter: rows its blocks have taken
+  unsigned int filter_long, filter_pieces; // majority filter: long rows listed, and their pieces
   int filter_from;                         // classes from this one on were filtered (SweepArgs::work2 holds their rows)
   int giant_on, giant_label;               // the filter tests for this label instead of the own one
   unsigned int hook_rows;                  // split: long rows with entries left to offer

@@ -17,7 +17,9 @@
 // degree, others against the row total that sweep 1 stored.
 //
 // Classes 6 and 7 take a warp per row; 8 and 9 a block per row from a
-// counter, so that no long row is left to one warp.  Bound by the gathers.
+// counter, so that no long row is left to one warp; rows past FILTER_LONG are
+// only listed there, in pieces of FILTER_PIECE entries that the blocks of a
+// second kernel share.  Bound by the gathers.
 #include "sweep_device.cuh"
 
 namespace gsl {
@@ -168,7 +170,7 @@ template <int WT, bool ASYNC, bool GIANT>
 __device__ __forceinline__ void filter_blocks(const SweepArgs& a, int* __restrict__ out) {
   using S = typename SumOf<WT>::T;
   __shared__ S s_hit, s_all;
-  __shared__ unsigned s_next;
+  __shared__ unsigned s_next, s_slot, s_piece;
   __shared__ int s_changed;
   const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
   const Pol pol = make_pol();
@@ -186,8 +188,21 @@ __device__ __forceinline__ void filter_blocks(const SweepArgs& a, int* __restric
       s_next = gridDim.x + atomicAdd(&a.ctr->filter_next, 1u);
     }
     __syncthreads();
+    const unsigned next = s_next;
     const long long s = a.off[v];
     const int d = (int)(a.off[v + 1] - s);
+    if (d > FILTER_LONG && a.long_rows) {   // block-uniform
+      const int pieces = (d + FILTER_PIECE - 1) / FILTER_PIECE;
+      if (tid == 0) {
+        s_slot = atomicAdd(&a.ctr->filter_long, 1u);
+        s_piece = atomicAdd(&a.ctr->filter_pieces, (unsigned)pieces);
+        a.long_rows[s_slot] = FilterLong{0, 0, 0, v, cls, (unsigned)pieces};
+      }
+      __syncthreads();
+      for (int k = tid; k < pieces; k += T) a.long_pieces[s_piece + k] = make_int2((int)s_slot, k);
+      i = next;
+      continue;
+    }
     const int old = own_label<ASYNC>(a, v);
     const int* cp = a.col + s;
     const int* wp = a.w + s;
@@ -220,7 +235,6 @@ __device__ __forceinline__ void filter_blocks(const SweepArgs& a, int* __restric
     all = warp_total(all);
     if (lane == 0 && all) atomicAdd(&s_all, all);
     __syncthreads();
-    const unsigned next = s_next;
     const unsigned long long h = 2ull * (unsigned long long)s_hit;
     const bool settled = h > bound || h > (unsigned long long)s_all;   // all of the row was read unless h > bound
     if (tid == 0) {
@@ -241,6 +255,93 @@ __device__ __forceinline__ void filter_blocks(const SweepArgs& a, int* __restric
       }
     }
     i = next;
+  }
+  flush_filter(a.ctr, my_dn, my_scan, my_settled);
+}
+
+// One block per listed piece of a long row.  A piece is skipped once the
+// pieces before it have settled the row; the one that ends last decides.
+// One block over the whole row took 0.5 ms per million entries, however idle
+// the rest of the chip (one hub of 8 M entries among 88 M others: 3.85 ms a
+// pass, 0.06 in pieces; of 1 M: 0.51 and 0.05).  From 65,536 entries on, which
+// a block reads in about 30 us, that is longer than what a sweep costs anyway.
+template <int WT, bool ASYNC, bool GIANT>
+__device__ __forceinline__ void filter_pieces(const SweepArgs& a, int* __restrict__ out) {
+  using S = typename SumOf<WT>::T;
+  __shared__ unsigned long long s_hit, s_all;
+  __shared__ int s_skip, s_changed;
+  const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
+  const Pol pol = make_pol();
+  const int giant = a.ctr->giant_label;
+  const unsigned total = a.ctr->filter_pieces;
+  unsigned long long my_dn = 0, my_scan = 0, my_settled = 0;
+  for (unsigned i = blockIdx.x; i < total; i += gridDim.x) {
+    const int2 piece = a.long_pieces[i];
+    FilterLong* row = a.long_rows + piece.x;
+    const int v = row->v;
+    const long long s = a.off[v];
+    const int d = (int)(a.off[v + 1] - s), from = piece.y * FILTER_PIECE, len = min(d - from, FILTER_PIECE);
+    const int old = own_label<ASYNC>(a, v);
+    const unsigned long long bound = row_bound<WT>(a, v, d);
+    if (tid == 0) {
+      s_hit = 0;
+      s_all = 0;
+      s_changed = 0;
+      s_skip = bound != ~0ull && 2ull * __ldcg(&row->hit) > bound;
+    }
+    __syncthreads();
+    const bool skip = s_skip != 0;
+    if (!skip) {
+      const int* cp = a.col + s + from;
+      const int* wp = a.w + s + from;
+      const int* lp = a.lg ? a.lg + s + from : nullptr;
+      S hit = 0, all = 0;
+      int jn[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) jn[u] = later_col(a, cp, len, tid + u * T, pol);
+      for (int r0 = 0; r0 < len; r0 += 4 * T) {
+        int j[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) j[u] = jn[u];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) jn[u] = later_col(a, cp, len, r0 + 4 * T + tid + u * T, pol);
+        filter_entries<WT, ASYNC, GIANT>(a, lp, v, old, wp, r0 + tid, T, j, pol, hit, all);
+      }
+      hit = warp_total(hit);
+      all = warp_total(all);
+      if (lane == 0) {
+        if (hit) atomicAdd(&s_hit, (unsigned long long)hit);
+        if (all) atomicAdd(&s_all, (unsigned long long)all);
+      }
+    }
+    __syncthreads();
+    if (tid == 0) {
+      if (!skip) {
+        atomicAdd(&row->hit, s_hit);
+        atomicAdd(&row->all, s_all);
+        atomicAdd(&row->read, (unsigned long long)len);
+      }
+      __threadfence();
+      if (atomicSub(&row->left, 1u) == 1u) {
+        __threadfence();
+        const unsigned long long h = 2ull * __ldcg(&row->hit);
+        if (h > bound || h > __ldcg(&row->all)) {   // all of the row was read unless h > bound
+          s_changed = settle<ASYNC>(a, v, GIANT ? giant : old, old, my_dn);
+          my_scan += __ldcg(&row->read);
+          my_settled += 1;
+        } else {
+          out[a.ctr->cls_start[row->cls] + atomicAdd(&a.ctr->uns_count[row->cls], 1u)] = v;
+        }
+      }
+    }
+    __syncthreads();
+    if (GIANT && a.mark && s_changed) {
+      for (int e = tid; e < d; e += T) {
+        const int j = ld_stream(a.col + s + e, pol.stream);
+        if ((unsigned)j < (unsigned)a.n) a.fnext[j] = 1;
+      }
+    }
+    __syncthreads();   // s_changed is cleared for the next piece
   }
   flush_filter(a.ctr, my_dn, my_scan, my_settled);
 }
@@ -329,6 +430,13 @@ __global__ void __launch_bounds__(256, 6) filter_block_kernel(SweepArgs a, int* 
   else filter_blocks<WT, ASYNC, false>(a, out);
 }
 
+template <int WT, bool ASYNC>
+__global__ void __launch_bounds__(256, 6) filter_long_kernel(SweepArgs a, int* __restrict__ out) {
+  if (stopped(a)) return;
+  if (!ASYNC && a.ctr->giant_on) filter_pieces<WT, ASYNC, true>(a, out);
+  else filter_pieces<WT, ASYNC, false>(a, out);
+}
+
 // The rows passed on become the class counts.
 __global__ void filter_counts_kernel(Counters* ctr, const int* stop, int first_cls, int last_cls) {
   if (stop && *(volatile const int*)stop) return;
@@ -346,6 +454,7 @@ namespace {
 template <int WT, bool A>
 void launch_filter_t(const SweepArgs& a, int* out, bool warps, bool blocks, const DeviceInfo& di, cudaStream_t s) {
   if (blocks) filter_block_kernel<WT, A><<<6 * di.sm_count, 256, 0, s>>>(a, out);
+  if (blocks && a.long_rows) filter_long_kernel<WT, A><<<6 * di.sm_count, 256, 0, s>>>(a, out);
   if (warps) filter_warp_kernel<WT, A><<<6 * di.sm_count, 256, 0, s>>>(a, out);
 }
 }  // namespace
@@ -355,7 +464,7 @@ cudaError_t launch_majority_filter(const SweepArgs& a, long long nnz, int* out, 
                                    const DeviceInfo& di, cudaStream_t s, int* kernels) {
   sample = sample && !async_mode && nnz > 0;   // in place, the sampled labels may change under the sweep
   filter_plan_kernel<<<1, sample ? 1024 : 32, 0, s>>>(a, nnz, first_cls, sample ? 1 : 0, seed);
-  int launches = 2 + (warps ? 1 : 0) + (blocks ? 1 : 0);
+  int launches = 2 + (warps ? 1 : 0) + (blocks ? (a.long_rows ? 2 : 1) : 0);
   if (sample) {
     long long g = (a.n + 255) / 256;
     const long long cap = 8ll * di.sm_count;

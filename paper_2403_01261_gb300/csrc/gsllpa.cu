@@ -45,6 +45,10 @@ struct gsl_ctx {
   long long cap_fkeys = 0, cap_fvals = 0;
   unsigned* gbits = nullptr;            // majority filter: vertices carrying the giant label
   long long cap_gbits = 0;
+  FilterLong* long_rows = nullptr;      // majority filter: rows read in pieces, and the pieces
+  long long cap_long_rows = 0;
+  int2* long_pieces = nullptr;
+  long long cap_long_pieces = 0;
   int* work2 = nullptr;                 // worklist of the rows the majority filter leaves
   long long cap_work2 = 0;
   int* lg = nullptr;                    // labels gathered per CSR entry (two-phase sweeps)
@@ -347,9 +351,18 @@ int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s) {
 }
 
 
-// Label lists for the rows that one block sweeps.
-int ensure_scratch(gsl_ctx* c, bool hub_kernels, SweepArgs* a) {
+// Label lists for the rows that one block sweeps, and the majority filter's
+// pieces of long rows.
+int ensure_scratch(gsl_ctx* c, long long nnz, bool hub_kernels, SweepArgs* a) {
   const long long maxd = c->ctr_h->max_degree;
+  a->long_rows = nullptr;
+  if (maxd > FILTER_LONG && c->tune.majority) {
+    const long long rows = nnz / FILTER_LONG + 1;
+    if (int r = grow(c, c->long_rows, c->cap_long_rows, rows)) return r;
+    if (int r = grow(c, c->long_pieces, c->cap_long_pieces, nnz / FILTER_PIECE + rows)) return r;
+    a->long_rows = c->long_rows;
+    a->long_pieces = c->long_pieces;
+  }
   const long long longest = maxd < c->tune.blk_max ? maxd : c->tune.blk_max;
   a->scratch_region = longest > sketch_register_row() ? 3 * longest : 0;   // labels, parts, their weights
   if (a->scratch_region)
@@ -411,7 +424,7 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
   a.probe_cap = c->tune.probe_cap;
   a.work = c->work;
   const bool hub_kernels = c->hub_ready && !wide   /* 32-bit sums */;
-  if (int r = ensure_scratch(c, hub_kernels, &a)) return r;
+  if (int r = ensure_scratch(c, g->nnz, hub_kernels, &a)) return r;
   a.n = n;
   if (wt) {   // weighted degrees, written by sweep 1 for the early stops of later sweeps
     if (int r = grow(c, c->kw, c->cap_kw, n)) return r;
@@ -965,7 +978,7 @@ cudaError_t enqueue_batch_sweeps(gsl_ctx* c, const gsl_csr* g, int num_graphs, c
   a.ctr = c->ctr;
   a.probe_cap = c->tune.probe_cap;
   a.work = c->work;
-  ck(ensure_scratch(c, false, &a) == GSL_OK ? cudaSuccess : cudaErrorMemoryAllocation);   // in place since before a capture
+  ck(ensure_scratch(c, g->nnz, false, &a) == GSL_OK ? cudaSuccess : cudaErrorMemoryAllocation);   // in place since before a capture
   a.n = n;
   a.gid = c->gid;
   a.vptr = c->vptr;
@@ -1085,7 +1098,7 @@ int gsl_ctx_destroy(gsl_ctx* c) {
   if (!c) return GSL_OK;
   DeviceGuard dg(c->device);
   void* dptrs[] = {c->lab[0], c->lab[1], c->flag[0], c->flag[1], c->work, c->parent, c->rank, c->sigma,
-                   c->block_sums, c->partials, c->scratch, c->hub_scratch, c->rowbits, c->lg, c->work2, c->gbits, c->fkeys, c->fvals, c->hub_piece_start,
+                   c->block_sums, c->partials, c->scratch, c->hub_scratch, c->rowbits, c->lg, c->work2, c->gbits, c->long_rows, c->long_pieces, c->fkeys, c->fvals, c->hub_piece_start,
                    c->hub_ustart, c->hub_best, c->hub_own, c->hub_wsum, c->hub_used_cnt, c->hub_clu, c->hub_used, c->hub_tab,
                    c->ctr, c->sums, c->k_dev,
                    c->st_off, c->st_col, c->st_w, c->st_lab, c->fix_w, c->fix_dev, c->kw, c->solo};
@@ -1668,7 +1681,7 @@ int gsl_gsllpa_batch(gsl_ctx* c, const gsl_csr* g, int32_t num_graphs, const int
     if (int r = prepare_graph(c, g, s)) return r;
   if (n > 0) {
     SweepArgs lists{};
-    if (int r = ensure_scratch(c, false, &lists)) return r;
+    if (int r = ensure_scratch(c, g->nnz, false, &lists)) return r;
   }
   CK(cudaMemsetAsync(c->done, 0, (size_t)num_graphs, s));
   CK(cudaMemsetAsync(c->iters, 0, sizeof(int) * (size_t)num_graphs, s));
@@ -1864,7 +1877,7 @@ int gsllpa_host_overlapped(gsl_ctx* c, int64_t n, int64_t nnz, const int64_t* of
   a.probe_cap = c->tune.probe_cap;
   a.work = c->work;
   const bool hub_kernels = c->hub_ready;
-  if (int r = ensure_scratch(c, hub_kernels, &a)) return r;
+  if (int r = ensure_scratch(c, nnz, hub_kernels, &a)) return r;
   a.n = n;
   a.prev = c->lab[1];
   a.next = c->lab[0];

@@ -6,6 +6,16 @@
 
 namespace gsl {
 
+// Majority filter: rows of more than FILTER_LONG entries are read in pieces of
+// FILTER_PIECE by any number of blocks.
+constexpr int FILTER_LONG = 65536, FILTER_PIECE = 8192;
+struct FilterLong {   // one such row
+  unsigned long long hit, all;   // weight of the tested label and of the whole row, so far
+  unsigned long long read;       // entries read
+  int v, cls;
+  unsigned left;                 // pieces still to end
+};
+
 // Arguments of one label-propagation sweep.
 struct SweepArgs {
   const long long* off;      // CSR offsets [n+1]
@@ -17,6 +27,8 @@ struct SweepArgs {
   const int* work;           // worklist (class regions at Counters::cls_start)
   const int* work2;          // rows the majority filter left, the same regions (null: no filter this sweep)
   const unsigned* bits;      // majority filter: one bit per vertex carrying the giant label
+  FilterLong* long_rows;     // majority filter: long rows and their pieces as (row, piece); null: the graph has none
+  int2* long_pieces;
   Counters* ctr;
   int* scratch;              // label lists of rows longer than a block's registers, one region per block
   long long scratch_region;  // ints per region (three lists of the longest row)

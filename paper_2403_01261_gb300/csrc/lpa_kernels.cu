@@ -570,6 +570,8 @@ __global__ void phase_reset_kernel(Counters* ctr, const int* stop) {
   ctr->hub_clusters = 0;
   ctr->hub_clu_next = 0;
   ctr->filter_next = 0;
+  ctr->filter_long = 0;
+  ctr->filter_pieces = 0;
 }
 
 cudaError_t launch_phase_reset(Counters* ctr, const int* stop, cudaStream_t s) {
