@@ -299,11 +299,18 @@ long long class_vertices(const gsl_ctx* c, int first, int last) {
   return v;
 }
 
-// Class 9 rows go to the hub kernels (clusters, pieces) when one is longer than
-// a block should be left with, or when the class starts below its default
-// bound; else to the block kernel.  A block takes about 1 ms per million
-// entries; R-MAT 25's rows of 131,073..864,000 entries beside the shorter ones
-// cost less there than in clusters of their own (2.3 ms a call).
+// Class 9 rows go to the hub kernels (clusters, pieces) when one block would
+// hold up the sweep with the longest of them, or when the class starts below its
+// default bound; else to the block kernel.  A block takes about 1 ms per million
+// entries whatever their labels, a whole sweep 0.008 ms per million (R-MAT 25's
+// sweep 2), so a row hides behind the others from 128 times its entries on.
+// Calls in ms, block / hub kernels: a star of 200,000 leaves 5.0 / 2.5, of
+// 1,000,000 21.5 / 6.6, four stars of 300,000 7.5 / 3.3; where the labels read
+// are distinct the two are closer: one hub of 200,000 among 2 M other entries
+// 0.69 / 0.78, of 1 M among 10 M 1.91 / 2.02, four of 1 M among 80 M 3.05 /
+// 2.80.  R-MAT 25's rows of 131,073..864,000 entries cost 2.3 ms more a call in
+// the hub kernels.
+constexpr long long HUB_BLOCK_REST = 128;
 constexpr long long HUB_BLOCK_MAX = 1ll << 20;
 
 // Resets all counters, classifies every vertex by degree (validating the
@@ -323,7 +330,8 @@ int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s) {
   // class 9 (hubs) in pieces: per-hub plan arrays and table regions
   const long long hubs = (long long)c->ctr_h->cls_total[CLS_HUB];
   const long long hub_e = (long long)c->ctr_h->hub_entries;
-  c->hub_ready = hubs > 0 && (maxd > HUB_BLOCK_MAX || c->tune.blk_max < Tuning().blk_max) &&
+  c->hub_ready = hubs > 0 &&
+                 (maxd > HUB_BLOCK_MAX || g->nnz < HUB_BLOCK_REST * maxd || c->tune.blk_max < Tuning().blk_max) &&
                  hub_pieces_fit(c->tune) && 2 * hub_e < (1ll << 32);
   if (c->hub_ready) {
     const long long old_tab = c->cap_hub_tab;
