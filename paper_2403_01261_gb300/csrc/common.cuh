@@ -45,7 +45,7 @@ struct Counters {
   unsigned int filter_long, filter_pieces; // majority filter: long rows listed, and their pieces
   int filter_from;                         // classes from this one on were filtered (SweepArgs::work2 holds their rows)
   int giant_on, giant_label;               // the filter tests for this label instead of the own one
-  unsigned int hook_rows;                  // split: long rows with entries left to offer
+  unsigned int hook_rows, hook_long;       // split: listed rows with entries left to offer, and long ones
   unsigned int row_next[NCLASS];           // rows of a class taken so far by the blocks that share them
   unsigned long long tile_active;          // vertices of classes 0..2 swept
   unsigned long long tile_scanned;         // and their CSR entries

@@ -434,7 +434,10 @@ __global__ void __launch_bounds__(SOLO_BLOCK, SOLO_BLOCKS_PER_SM) solo_kernel(Sw
       s = a0.off[u] + SOLO_SAMPLE;
       e = a0.off[u + 1];
       cu = __ldcg(labels + u);
-      offer = s < e && outside_named(q.named + comm_slot(cu, n), uf_find(q.parent, (int)u, err, cap));
+      if (s < e) {
+        const int root = uf_find(q.parent, (int)u, err, cap);
+        offer = root != community_name(q.named + comm_slot(cu, n), root);
+      }
     }
     unsigned mask = __ballot_sync(FULL, offer);
     while (mask) {

@@ -58,22 +58,6 @@ __device__ __forceinline__ bool hook_entry(const int* col, const int* labels, in
   return true;
 }
 
-// The same after flattening, with ru = u's parent read once per row: when
-// j's parent is ru, u and j already share a tree (trees only merge), so the
-// union is skipped without walking either path.
-template <int F>
-__device__ __forceinline__ void hook_entry_flat(const int* col, const int* labels, int* p, long long n, int u,
-                                                int cu, int ru, long long e, int* err, UfCap<F> cap) {
-  const int j = ld_stream(col + e);
-  if ((unsigned)j >= (unsigned)n) {
-    raise_err(err, ERRBIT_INVALID);
-    return;
-  }
-  if (j == u || ld_label_ro(labels + j) != cu) return;
-  if (__ldcg(p + j) == ru) return;
-  uf_unite(p, u, j, err, cap);
-}
-
 }  // namespace
 
 __global__ void init_parent_kernel(int* __restrict__ p, long long n) {
@@ -182,7 +166,7 @@ __global__ void __launch_bounds__(1024) giant_kernel(const int* p, long long n, 
 // root (giant_kernel) names that root.  Roots do not name themselves: a
 // community's stray members, scattered over the ids and often written last,
 // would name their single-vertex pieces and leave the others to offer their
-// whole rows.  Slots nobody names here hold -1 (outside_named).
+// whole rows.  Slots nobody names here hold -1 (community_name).
 __global__ void name_pieces_kernel(const int* __restrict__ p, const int* __restrict__ labels, long long n,
                                    int* __restrict__ named) {
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
@@ -200,10 +184,37 @@ __global__ void name_giant_kernel(const int* __restrict__ labels, long long n, i
 }
 
 // Vertices outside their community's named piece offer entries SPLIT_SAMPLE..
-// of their row (both directions: the other end may be skipped): rows of up to
-// HOOK_LANE entries by their lane, up to HOOK_WARP by the warp, longer ones
-// are listed for hook_long_kernel.
-constexpr int HOOK_LANE = 8, HOOK_WARP = 2048;
+// of their row (both directions: the other end may be skipped), unless their
+// parent has become the named root by the time their row is reached.  Rows of up
+// to HOOK_LANE entries go by their lane, longer ones by this warp, two at a time,
+// while they are HOOK_STEPS steps of 32 entries in all.  A warp that meets more
+// lists them, for a warp each (hook_rows_kernel) or past HOOK_WARP entries for a
+// block each (hook_long_kernel), which also stop inside a row.  Left where they
+// were met, the dense rows of a small graph, or the heavy ids of one that is
+// sorted by degree, ran on a fraction of the chip: split after LPA of 60,000
+// vertices of 1500 entries 2.43 ms, listed 0.43; 2 million vertices, a few of
+// them heavy, in 1000 communities 1.64 and 0.77.  Asked again, hubs seldom read
+// their rows: R-MAT 24 in 1000 random communities 9.5 and 4.4 ms.  At 32 steps
+// the heavy ids take 1.19 ms, at 128 the split of 30,000 vertices of 900 entries
+// 0.45 instead of 0.35; one row at a time a circulant of 16 neighbours takes 0.49
+// instead of 0.38.
+constexpr int HOOK_LANE = 8, HOOK_STEPS = 64, HOOK_WARP = 2048;
+
+// Offers the entries k, k + step, .. below end of u's row, none when u's parent
+// is the root `name`; EVERY: and no more once it has become that.
+template <bool EVERY, int F>
+__device__ __forceinline__ void hook_row(const int* col, const int* labels, int* p, long long n, int u, int cu,
+                                         int name, long long k, long long end, int step, int* err, UfCap<F> cap) {
+  int ru = __ldcg(p + u);
+  for (; k < end; k += step) {
+    const int j = ld_stream(col + k);
+    if (ru == name) return;
+    const int next = EVERY ? __ldcg(p + u) : ru;
+    if ((unsigned)j >= (unsigned)n) raise_err(err, ERRBIT_INVALID);
+    else if (j != u && ld_label_ro(labels + j) == cu && __ldcg(p + j) != ru) uf_unite(p, u, j, err, cap);
+    ru = next;
+  }
+}
 
 template <int F>
 __global__ void __launch_bounds__(256) hook_kernel(const long long* __restrict__ off, const int* __restrict__ col,
@@ -215,51 +226,86 @@ __global__ void __launch_bounds__(256) hook_kernel(const long long* __restrict__
   for (long long w = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); w < n; w += stride) {   // warp-uniform
     const long long u = w + lane;
     long long s = 0, e = 0;
-    int cu = 0, ru = 0;
-    bool offer = false;
+    int cu = 0, ru = 0, slot = -1, name = 0;
     if (u < n) {
       s = off[u] + SPLIT_SAMPLE;
       e = off[u + 1];
       if (s < e) {
         ru = __ldcg(p + u);
         cu = labels[u];
-        offer = outside_named(named + comm_slot(cu, n), ru);
+        slot = (int)comm_slot(cu, n);
+        name = __ldcg(named + slot);
       }
     }
-    if (offer && e - s > HOOK_WARP) {
-      list[atomicAdd(&ctr->hook_rows, 1u)] = (int)u;
+    if (__any_sync(FULL, name == -1)) {   // one lane asks for all of its community
+      const unsigned same = __match_any_sync(FULL, name == -1 ? slot : -1);
+      const int leader = __ffs((int)same) - 1;
+      int first = 0;
+      if (name == -1 && lane == leader) first = community_name(named + slot, ru);
+      first = __shfl_sync(FULL, first, leader);
+      if (name == -1) name = first;
+    }
+    bool offer = slot >= 0 && ru != name;
+    if (offer && e - s > HOOK_WARP) {   // from the list's end
+      list[n - 1 - (long long)atomicAdd(&ctr->hook_long, 1u)] = (int)u;
       offer = false;
     }
     if (offer && e - s <= HOOK_LANE) {
-      for (long long k = s; k < e; ++k) hook_entry_flat(col, labels, p, n, (int)u, cu, ru, k, &ctr->err, cap);
+      hook_row<false>(col, labels, p, n, (int)u, cu, name, s, e, 1, &ctr->err, cap);
       offer = false;
     }
     __syncwarp();
     unsigned mask = __ballot_sync(FULL, offer);
-    while (mask) {
-      const int r = __ffs((int)mask) - 1;
+    if (!mask) continue;
+    if (__reduce_add_sync(FULL, offer ? (unsigned)((e - s + 31) >> 5) : 0u) > HOOK_STEPS) {
+      unsigned base = 0;
+      if (lane == 0) base = atomicAdd(&ctr->hook_rows, (unsigned)__popc(mask));
+      base = __shfl_sync(FULL, base, 0);
+      if (offer) list[base + __popc(mask & ((1u << lane) - 1u))] = (int)u;
+      continue;
+    }
+    while (mask) {   // two rows at a time, half a warp each
+      const int r0 = __ffs((int)mask) - 1;
       mask &= mask - 1;
+      const int r1 = __ffs((int)mask) - 1;   // -1: none
+      mask &= mask - 1;
+      const int r = lane < 16 ? r0 : (r1 < 0 ? r0 : r1);
       const long long rs = __shfl_sync(FULL, s, r), re = __shfl_sync(FULL, e, r);
-      const int rc = __shfl_sync(FULL, cu, r), rr = __shfl_sync(FULL, ru, r);
-      for (long long k = rs + lane; k < re; k += 32)
-        hook_entry_flat(col, labels, p, n, (int)w + r, rc, rr, k, &ctr->err, cap);
+      const int rc = __shfl_sync(FULL, cu, r), rn = __shfl_sync(FULL, name, r);
+      hook_row<false>(col, labels, p, n, (int)w + r, rc, rn, rs + (r1 < 0 ? lane : (lane & 15)), re, r1 < 0 ? 32 : 16,
+                      &ctr->err, cap);
       __syncwarp();
     }
   }
 }
 
-// The listed rows, one block each.
+// The listed rows, a warp each.  A warp takes a run of the list, so that the
+// rows in flight lie in many communities and their unions seldom compete.
+template <int F>
+__global__ void __launch_bounds__(256) hook_rows_kernel(const long long* __restrict__ off, const int* __restrict__ col,
+                                                         const int* __restrict__ labels, int* p, long long n,
+                                                         const int* __restrict__ list, Counters* ctr, UfCap<F> cap,
+                                                         const int* __restrict__ named) {
+  const unsigned cnt = ctr->hook_rows, nwarps = (gridDim.x * blockDim.x) >> 5;
+  const unsigned part = (cnt + nwarps - 1) / nwarps, w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  for (unsigned i = w * part; i < cnt && i < (w + 1) * part; ++i) {
+    const int u = list[i], cu = labels[u];
+    hook_row<true>(col, labels, p, n, u, cu, named[comm_slot(cu, n)], off[u] + SPLIT_SAMPLE + (threadIdx.x & 31),
+                off[u + 1], 32, &ctr->err, cap);
+  }
+}
+
+// The listed long rows, one block each.
 template <int F>
 __global__ void __launch_bounds__(512) hook_long_kernel(const long long* __restrict__ off, const int* __restrict__ col,
                                                          const int* __restrict__ labels, int* p, long long n,
-                                                         const int* __restrict__ list, Counters* ctr, UfCap<F> cap) {
-  const unsigned cnt = ctr->hook_rows;
+                                                         const int* __restrict__ list, Counters* ctr, UfCap<F> cap,
+                                                         const int* __restrict__ named) {
+  const unsigned cnt = ctr->hook_long;
   for (unsigned i = blockIdx.x; i < cnt; i += gridDim.x) {
-    const int u = list[i];
-    const int ru = __ldcg(p + u), cu = labels[u];   // any value p[u] has held will do
-    const long long e = off[u + 1];
-    for (long long k = off[u] + SPLIT_SAMPLE + threadIdx.x; k < e; k += blockDim.x)
-      hook_entry_flat(col, labels, p, n, u, cu, ru, k, &ctr->err, cap);
+    const int u = list[n - 1 - i], cu = labels[u];
+    hook_row<true>(col, labels, p, n, u, cu, named[comm_slot(cu, n)], off[u] + SPLIT_SAMPLE + threadIdx.x, off[u + 1],
+                (int)blockDim.x, &ctr->err, cap);
   }
 }
 
@@ -472,7 +518,8 @@ void launch_split_t(const long long* off, const int* col, long long n, const int
   name_pieces_kernel<<<g, 256, 0, s>>>(parent, labels, n, named);
   name_giant_kernel<<<1, 1, 0, s>>>(labels, n, named, ctr);
   hook_kernel<F><<<g, 256, 0, s>>>(off, col, labels, parent, n, list, ctr, cap, named);
-  hook_long_kernel<F><<<4 * di.sm_count, 512, 0, s>>>(off, col, labels, parent, n, list, ctr, cap);
+  hook_rows_kernel<F><<<8 * di.sm_count, 256, 0, s>>>(off, col, labels, parent, n, list, ctr, cap, named);
+  hook_long_kernel<F><<<4 * di.sm_count, 512, 0, s>>>(off, col, labels, parent, n, list, ctr, cap, named);
   flatten_kernel<F><<<g, 256, 0, s>>>(parent, out, n, ctr, cap);
   count_launches(SPLIT_LAUNCHES);
 }
