@@ -1,0 +1,39 @@
+"""The one-launch path of small graphs, against the oracle: few rows that hold
+many entries."""
+import numpy as np
+import pytest
+import torch
+
+import inputs as I
+import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+def launched(gpu_lib, call):
+    before = gpu_lib.kernel_launches()
+    out = call()
+    return out, gpu_lib.kernel_launches() - before
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("n", [64, 129, 500, 1200])
+def test_few_dense_rows(gpu_lib, n, weighted):
+    g = I.random_graph(n, 0.97, seed=n)
+    if weighted:
+        g = I.Graph(g.offsets, g.cols, I.symmetric_weights(g, 4, 30))
+    off, col = torch.from_numpy(g.offsets).to(DEV), torch.from_numpy(g.cols).to(DEV)
+    w = torch.from_numpy(g.weights).to(DEV) if weighted else None
+    c = gpu_lib.Context(0)
+    rng = np.random.default_rng(3)
+    for labels in (2, 5, n):
+        prev = rng.integers(0, labels, n).astype(np.int32)
+        got, launches = launched(gpu_lib, lambda: c.lpa(off, col, w, labels_init=torch.from_numpy(prev).to(DEV),
+                                                        tolerance=0.0, max_iters=1))
+        assert launches == 1 and np.array_equal(got.cpu().numpy(), O.sync_sweep(g, prev)[0])
+    (got, st), launches = launched(gpu_lib, lambda: c.gsllpa(off, col, w, tolerance=0.0, max_iters=9, stats=True))
+    want, t, dn = O.gsl_lpa(g, 0.0, 9)
+    assert launches == 1 and st["iterations"] == t and st["changed"] == dn[:t].tolist()
+    assert np.array_equal(got.cpu().numpy(), want)
