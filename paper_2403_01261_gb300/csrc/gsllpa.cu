@@ -23,6 +23,7 @@ struct gsl_ctx {
   int device = 0;
   DeviceInfo di;
   Tuning tune;
+  Tuning run;                      // of the call under way: tune, with the class bound prepare_graph chose
   std::string last_error;
 
   long long cap_n = 0;             // vertex capacity of the per-vertex scratch
@@ -300,39 +301,55 @@ long long class_vertices(const gsl_ctx* c, int first, int last) {
 }
 
 // Class 9 rows go to the hub kernels (clusters, pieces) when one block would
-// hold up the sweep with the longest of them, or when the class starts below its
-// default bound; else to the block kernel.  A block takes about 1 ms per million
+// hold up the sweep with the longest of them, or when the caller has lowered the
+// class's bound; else to the block kernel.  A block takes about 1 ms per million
 // entries whatever their labels, a whole sweep 0.008 ms per million (R-MAT 25's
 // sweep 2), so a row hides behind the others from 128 times its entries on.
+// Where the longest does not, the class starts at HUB_MIN entries.
 // Calls in ms, block / hub kernels: a star of 200,000 leaves 5.0 / 2.5, of
-// 1,000,000 21.5 / 6.6, four stars of 300,000 7.5 / 3.3; where the labels read
-// are distinct the two are closer: one hub of 200,000 among 2 M other entries
-// 0.69 / 0.78, of 1 M among 10 M 1.91 / 2.02, four of 1 M among 80 M 3.05 /
-// 2.80.  R-MAT 25's rows of 131,073..864,000 entries cost 2.3 ms more a call in
-// the hub kernels.
+// 1,000,000 21.5 / 6.6, four stars of 300,000 7.5 / 3.3, 40 rows of 130,000 and
+// little else 5.5 / 3.4;
+// where the labels read are distinct the two are closer: one hub of 200,000
+// among 2 M other entries 0.69 / 0.78, of 1 M among 10 M 1.91 / 2.02, four of
+// 1 M among 80 M 3.05 / 2.80.  R-MAT 25's rows of 131,073..864,000 entries cost
+// 2.3 ms more a call in the hub kernels.
 constexpr long long HUB_BLOCK_REST = 128;
 constexpr long long HUB_BLOCK_MAX = 1ll << 20;
+constexpr int HUB_MIN = 32768;
 
-// Resets all counters, classifies every vertex by degree (validating the
-// offsets) and sizes the hub tables.  Synchronises the stream.
-int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s) {
+// Resets all counters and classifies every vertex by degree (validating the
+// offsets) under c->run.  Synchronises the stream.
+int classify(gsl_ctx* c, const gsl_csr* g, cudaStream_t s) {
   CK(cudaMemsetAsync(c->ctr, 0, sizeof(Counters), s));
   const int pe = prof_begin(c, s);
-  CK(launch_class_histogram(OFF(g), g->n, g->nnz, c->tune, c->ctr, c->di, s));
+  CK(launch_class_histogram(OFF(g), g->n, g->nnz, c->run, c->ctr, c->di, s));
   prof_end(c, pe, SL_CLASSIFY, s, 2);
   c->profile.slot[SL_CLASSIFY].vertices += g->n;
   c->profile.slot[SL_CLASSIFY].bytes += 8.0 * (double)(g->n + 1);
   CK(cudaMemcpyAsync(c->ctr_h, c->ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   prof_resolve(c);
-  if (int r = map_err(c, c->ctr_h->err, "offsets")) return r;
+  return map_err(c, c->ctr_h->err, "offsets");
+}
+
+// Classes of the call under way and, for sweeps that may use them (hubs), the
+// hub kernels' tables.  Synchronises the stream.
+int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s, bool sweeps = false) {
+  c->run = c->tune;
+  if (int r = classify(c, g, s)) return r;
   const long long maxd = c->ctr_h->max_degree;
+  const bool alone = g->nnz < HUB_BLOCK_REST * maxd;   // no rest of a sweep to hide the longest row
+  c->hub_ready = false;
+  if (!sweeps || !hub_pieces_fit(c->run)) return GSL_OK;
+  if (alone && maxd > HUB_MIN && c->tune.blk_max == Tuning().blk_max) {
+    c->run.blk_max = std::max(HUB_MIN, c->run.warp_max);
+    if (int r = classify(c, g, s)) return r;
+  }
   // class 9 (hubs) in pieces: per-hub plan arrays and table regions
   const long long hubs = (long long)c->ctr_h->cls_total[CLS_HUB];
   const long long hub_e = (long long)c->ctr_h->hub_entries;
-  c->hub_ready = hubs > 0 &&
-                 (maxd > HUB_BLOCK_MAX || g->nnz < HUB_BLOCK_REST * maxd || c->tune.blk_max < Tuning().blk_max) &&
-                 hub_pieces_fit(c->tune) && 2 * hub_e < (1ll << 32);
+  c->hub_ready = hubs > 0 && (maxd > HUB_BLOCK_MAX || alone || c->tune.blk_max < Tuning().blk_max) &&
+                 2 * hub_e < (1ll << 32);
   if (c->hub_ready) {
     const long long old_tab = c->cap_hub_tab;
     const unsigned long long* old_ptr = c->hub_tab;
@@ -371,7 +388,7 @@ int ensure_scratch(gsl_ctx* c, long long nnz, bool hub_kernels, SweepArgs* a) {
     a->long_rows = c->long_rows;
     a->long_pieces = c->long_pieces;
   }
-  const long long longest = maxd < c->tune.blk_max ? maxd : c->tune.blk_max;
+  const long long longest = maxd < c->run.blk_max ? maxd : c->run.blk_max;
   a->scratch_region = longest > sketch_register_row() ? 3 * longest : 0;   // labels, parts, their weights
   if (a->scratch_region)
     if (int r = grow(c, c->scratch, c->cap_scratch, sketch_blocks(c->di) * a->scratch_region)) return r;
@@ -520,7 +537,7 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
         if (all_active && binned_all) {
           CK(launch_all_counts(c->ctr, CLS_BINNED, s));
         } else {
-          CK(launch_bin(OFF(g), n, c->flag[t & 1], all_active ? 1 : 0, c->tune, c->work, c->ctr, c->di, s, nullptr,
+          CK(launch_bin(OFF(g), n, c->flag[t & 1], all_active ? 1 : 0, c->run, c->work, c->ctr, c->di, s, nullptr,
                         nullptr, nullptr, async_mode ? ph : -1, (unsigned)t, CLS_BINNED));
           binned_all = all_active && !async_mode;   // the worklist now holds every vertex of these classes
         }
@@ -545,10 +562,10 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
                      c->hub_wsum,        c->hub_used_cnt, c->hub_used, c->hub_tab, c->hub_clu};
           c->hub_dirty = true;   // until this sweep is known to have finished cleanly
           int kernels = 0;
-          CK(launch_hub_pieces(a, hp, wt != 0, async_mode, c->tune, c->di, s, &kernels));
+          CK(launch_hub_pieces(a, hp, wt != 0, async_mode, c->run, c->di, s, &kernels));
           prof_end(c, pe, SL_SWEEP0 + k, s, kernels);
         } else {
-          CK(launch_sweep_class(a, k, wt, async_mode, c->tune, maxd, c->di, s));
+          CK(launch_sweep_class(a, k, wt, async_mode, c->run, maxd, c->di, s));
           prof_end(c, pe, SL_SWEEP0 + k, s, 1);
         }
       }
@@ -688,7 +705,7 @@ int run_lpa_f32(gsl_ctx* c, const gsl_csr* g, const float* wf, const int32_t* la
       if (ph == 1) CK(launch_phase_reset(c->ctr, nullptr, s));
       {
         const int pe = prof_begin(c, s);
-        CK(launch_bin(OFF(g), n, c->flag[t & 1], all_active ? 1 : 0, c->tune, c->work, c->ctr, c->di, s, nullptr,
+        CK(launch_bin(OFF(g), n, c->flag[t & 1], all_active ? 1 : 0, c->run, c->work, c->ctr, c->di, s, nullptr,
                       nullptr, nullptr, async_mode ? ph : -1, (unsigned)t));
         prof_end(c, pe, SL_BIN, s, 1);
       }
@@ -841,7 +858,7 @@ int run_modularity(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const i
   CK(cudaMemsetAsync(c->sums, 0, sizeof(ModSums), s));
   if (int r = reset_sweep_counters(c, s)) return r;
   if (class_vertices(c, CLS_BINNED, NCLASS - 1) > 0)
-    CK(launch_bin(OFF(g), n, nullptr, 1, c->tune, c->work, c->ctr, c->di, s, nullptr, nullptr, nullptr, -1, 0u,
+    CK(launch_bin(OFF(g), n, nullptr, 1, c->run, c->work, c->ctr, c->di, s, nullptr, nullptr, nullptr, -1, 0u,
                   CLS_BINNED));
   const int pe = prof_begin(c, s);
   CK(launch_modularity(OFF(g), g->cols, weights, n, labels, c->work, c->ctr, c->ctr_h->cls_total, c->sigma,
@@ -1012,7 +1029,7 @@ cudaError_t enqueue_batch_sweeps(gsl_ctx* c, const gsl_csr* g, int num_graphs, c
       if (ph == 1) ck(launch_phase_reset(c->ctr, c->stop, cs));
       if (class_vertices(c, CLS_BINNED, NCLASS - 1) > 0) {
         pe = prof ? prof_begin(c, cs) : -1;
-        ck(launch_bin(OFF(g), n, c->flag[t & 1], t <= 2 ? 1 : 0, c->tune, c->work, c->ctr, c->di, cs, c->gid, c->done,
+        ck(launch_bin(OFF(g), n, c->flag[t & 1], t <= 2 ? 1 : 0, c->run, c->work, c->ctr, c->di, cs, c->gid, c->done,
                       c->stop, async_mode ? ph : -1, (unsigned)t, CLS_BINNED));
         if (prof) prof_end(c, pe, SL_BIN, cs, 1);
       }
@@ -1030,7 +1047,7 @@ cudaError_t enqueue_batch_sweeps(gsl_ctx* c, const gsl_csr* g, int num_graphs, c
       for (int k = CLS_BINNED; k < CLS_HUB; ++k) {
         if (class_vertices(c, k, k) == 0 && !(k == CLS_BLOCK && a.hub_blocks)) continue;
         pe = prof ? prof_begin(c, cs) : -1;
-        ck(launch_sweep_class(a, k, weights ? 1 : 0, async_mode, c->tune, (int)c->ctr_h->max_degree, c->di, cs));
+        ck(launch_sweep_class(a, k, weights ? 1 : 0, async_mode, c->run, (int)c->ctr_h->max_degree, c->di, cs));
         if (prof) prof_end(c, pe, SL_SWEEP0 + k, cs, 1);
       }
       if (class_vertices(c, 0, CLS_BINNED - 1) > 0) {
@@ -1275,7 +1292,7 @@ int gsl_autotune(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, int32_t m
   const std::vector<Tuning> cand = tune_candidates(deg, c->tune, TuneSpace{true}, c->di.max_smem_optin);
   return tune_loop(c, cand, out, [&](const Tuning& t, float* ms) -> int {
     c->tune = t;
-    if (int r = prepare_graph(c, g, s)) return r;
+    if (int r = prepare_graph(c, g, s, true)) return r;
     int* fin = nullptr;
     CK(cudaEventRecord(c->ev[0], s));
     if (int r = run_lpa(c, g, weights, nullptr, 0.0, sweeps, mode, nullptr, s, &fin)) return r;
@@ -1415,7 +1432,7 @@ int gsl_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
     return r;
   if (handled) return GSL_OK;
   CK(cudaEventRecord(c->ev[0], s));
-  if (int r = prepare_graph(c, g, s)) return r;
+  if (int r = prepare_graph(c, g, s, true)) return r;
   int* fin = nullptr;
   if (int r = run_lpa(c, g, weights, labels_init, tol, max_iters, mode, st, s, &fin)) return r;
   CK(cudaMemcpyAsync(labels_out, fin, sizeof(int32_t) * (size_t)g->n, cudaMemcpyDeviceToDevice, s));
@@ -1437,7 +1454,7 @@ int gsl_lpa_f32(gsl_ctx* c, const gsl_csr* g, const float* weights, const int32_
   cudaStream_t s = (cudaStream_t)stream;
   if (int r = ensure_vertex_scratch(c, g->n)) return r;
   CK(cudaEventRecord(c->ev[0], s));
-  if (int r = prepare_graph(c, g, s)) return r;
+  if (int r = prepare_graph(c, g, s, true)) return r;
   int* wi = nullptr;
   bool wide = false;
   if (int r = f32_fixed_point(c, g, weights, s, &wi, &wide)) return r;
@@ -1466,7 +1483,7 @@ int gsl_gsllpa_f32(gsl_ctx* c, const gsl_csr* g, const float* weights, double to
   cudaStream_t s = (cudaStream_t)stream;
   if (int r = ensure_vertex_scratch(c, g->n)) return r;
   CK(cudaEventRecord(c->ev[0], s));
-  if (int r = prepare_graph(c, g, s)) return r;
+  if (int r = prepare_graph(c, g, s, true)) return r;
   int* wi = nullptr;
   bool wide = false;
   if (int r = f32_fixed_point(c, g, weights, s, &wi, &wide)) return r;
@@ -1640,7 +1657,7 @@ int gsl_gsllpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, double tol,
     return r;
   if (handled) return GSL_OK;
   CK(cudaEventRecord(c->ev[0], s));
-  if (int r = prepare_graph(c, g, s)) return r;
+  if (int r = prepare_graph(c, g, s, true)) return r;
   int* fin = nullptr;
   if (int r = run_lpa(c, g, weights, nullptr, tol, max_iters, mode, st, s, &fin)) return r;
   CK(cudaEventRecord(c->ev[1], s));
@@ -1706,7 +1723,7 @@ int gsl_gsllpa_batch(gsl_ctx* c, const gsl_csr* g, int32_t num_graphs, const int
                                       num_graphs, max_iters, mode, (long long)(tol * 1e12), c->ctr_h->max_degree,
                                       (long long)c->lab[0], (long long)c->scratch, (long long)c->hub_scratch,
                                       (long long)c->ctr_h->cls_total[CLS_HUB],
-                                      c->tune.warp_max, c->tune.blk_max, (long long)c->work2,
+                                      c->run.warp_max, c->run.blk_max, (long long)c->work2,
                                       c->tune.majority, c->tune.blk_block, c->tune.blk_slots, c->tune.probe_cap,
                                       c->tune.uf_cap};
   long long graph_launches = 0;
@@ -1862,7 +1879,7 @@ int gsllpa_host_overlapped(gsl_ctx* c, int64_t n, int64_t nnz, const int64_t* of
     CK(cudaEventRecord(c->chunk_ev[(size_t)k], c->copy_stream));
   }
   // offsets: validated and classified (synchronises s; the copies go on)
-  if (int r = prepare_graph(c, &g, s)) return r;
+  if (int r = prepare_graph(c, &g, s, true)) return r;
   CK(cudaMemsetAsync(c->flag[0], 0, (size_t)n, s));
   CK(cudaMemsetAsync(c->flag[1], 0, (size_t)n, s));
   CK(launch_init_labels(nullptr, c->lab[0], c->lab[1], n, c->ctr, c->di, s));
@@ -1905,7 +1922,7 @@ int gsllpa_host_overlapped(gsl_ctx* c, int64_t n, int64_t nnz, const int64_t* of
     if (k > 0) CK(launch_phase_reset(c->ctr, nullptr, s));
     CK(launch_sweep_lanes(a, 0, false, vb[k], vb[k + 1], nullptr, 1, nullptr, 0, 2u, c->di, s));
     if (class_vertices(c, CLS_BINNED, NCLASS - 1) == 0) continue;
-    CK(launch_bin_range(OFF(&g), vb[k], vb[k + 1], c->tune, c->work, c->ctr, c->di, s, CLS_BINNED));
+    CK(launch_bin_range(OFF(&g), vb[k], vb[k + 1], c->run, c->work, c->ctr, c->di, s, CLS_BINNED));
     a.work2 = nullptr;
     if (filter && class_vertices(c, CLS_WARP_L, CLS_HUB) > 0) {
       CK(launch_majority_filter(a, nnz, c->work2, nullptr, 0, false, CLS_WARP_L, false, 0u,
@@ -1920,9 +1937,9 @@ int gsllpa_host_overlapped(gsl_ctx* c, int64_t n, int64_t nnz, const int64_t* of
         HubPlan hp{c->hub_piece_start, c->hub_ustart, c->hub_best, c->hub_own,
                    c->hub_wsum,        c->hub_used_cnt, c->hub_used, c->hub_tab, c->hub_clu};
         int kernels = 0;
-        CK(launch_hub_pieces(a, hp, false, false, c->tune, c->di, s, &kernels));
+        CK(launch_hub_pieces(a, hp, false, false, c->run, c->di, s, &kernels));
       } else {
-        CK(launch_sweep_class(a, cls, 0, false, c->tune, (int)c->ctr_h->max_degree, c->di, s));
+        CK(launch_sweep_class(a, cls, 0, false, c->run, (int)c->ctr_h->max_degree, c->di, s));
       }
     }
   }

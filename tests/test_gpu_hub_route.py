@@ -10,27 +10,29 @@ import oracle as O
 pytestmark = pytest.mark.gpu
 
 DEV = "cuda:0"
-LENGTH = 131_100   # of the class above 131,072
 
 
-def hubs_among(others, seed):
-    """Two rows of LENGTH entries and about `others` entries of random pairs."""
+def hubs_among(length, others, seed):
+    """Two rows of `length` entries and about `others` entries of random pairs."""
     rng = np.random.default_rng(seed)
     n = 140_000
-    u = [rng.integers(0, n, others // 2)] + [np.full(LENGTH, n + k) for k in range(2)]
-    v = [rng.integers(0, n, others // 2)] + [rng.choice(n, LENGTH, replace=False) for _ in range(2)]
+    u = [rng.integers(0, n, others // 2)] + [np.full(length, n + k) for k in range(2)]
+    v = [rng.integers(0, n, others // 2)] + [rng.choice(n, length, replace=False) for _ in range(2)]
     u, v = np.concatenate(u), np.concatenate(v)
     keep = u != v
     return I.csr_from_pairs(n + 2, u[keep], v[keep], perm=rng.permutation(n + 2), name="hubs-among")
 
 
 @pytest.mark.parametrize("weighted", [False, True])
-@pytest.mark.parametrize("others, slot, idle", [(0, "sweep_hub", "sweep_block"), (1_000_000, "sweep_hub", "sweep_block"),
-                                                (17_000_000, "sweep_block", "sweep_hub")])
-def test_route_and_labels(gpu_lib, others, slot, idle, weighted):
-    g = hubs_among(others, seed=others + 1)
+@pytest.mark.parametrize("length, others, slot, idle", [
+    (131_100, 0, "sweep_hub", "sweep_block"), (131_100, 1_000_000, "sweep_hub", "sweep_block"),
+    (131_100, 17_000_000, "sweep_block", "sweep_hub"),
+    (32_769, 0, "sweep_hub", "sweep_block"), (40_000, 1_000_000, "sweep_hub", "sweep_block"),
+    (40_000, 5_300_000, "sweep_block", "sweep_hub")])
+def test_route_and_labels(gpu_lib, length, others, slot, idle, weighted):
+    g = hubs_among(length, others, seed=others + length)
     d = np.diff(g.offsets)
-    assert (d >= LENGTH).sum() == 2 and (g.nnz < 128 * d.max()) == (slot == "sweep_hub")
+    assert (d >= length).sum() == 2 and (g.nnz < 128 * d.max()) == (slot == "sweep_hub")
     if weighted:
         g = I.Graph(g.offsets, g.cols, I.symmetric_weights(g, 4, 9))
     off, col = torch.from_numpy(g.offsets).to(DEV), torch.from_numpy(g.cols).to(DEV)
