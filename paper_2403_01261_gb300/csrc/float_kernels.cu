@@ -153,8 +153,11 @@ __global__ void __launch_bounds__(256) sweep_f_group_kernel(SweepArgs a, const f
   flush_counters(a.ctr, cls, my_dn, my_scan);
 }
 
-// One block per row of classes 6..9; `tb` table slots in shared memory,
-// global regions of 2 * (largest degree) slots per block otherwise.
+// One block per row of classes 7..9; `tb` table slots in shared memory,
+// global regions of 2 * (largest degree) slots per block otherwise.  Blocks take
+// rows from a counter: class 8 spans 1025 to 131,072 entries, and in fixed
+// strides a block with two long ones held up the sweep (R-MAT 22, 20 sweeps:
+// 431 ms a call, 383 so; R-MAT 20 80.8 and 70.2).
 template <bool ASYNC>
 __global__ void __launch_bounds__(F_BLOCK) sweep_f_block_kernel(SweepArgs a, const float* __restrict__ wf, int cls,
                                                                unsigned tb, unsigned* gkeys, double* gvals,
@@ -171,7 +174,12 @@ __global__ void __launch_bounds__(F_BLOCK) sweep_f_block_kernel(SweepArgs a, con
   const Pol pol = make_pol();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   unsigned long long my_dn = 0, my_scan = 0;
-  for (long long item = blockIdx.x; item < (long long)cnt; item += gridDim.x) {
+  __shared__ unsigned s_item;
+  for (;;) {
+    if (threadIdx.x == 0) s_item = atomicAdd(&a.ctr->row_next[cls], 1u);
+    __syncthreads();
+    const unsigned item = s_item;
+    if (item >= cnt) break;
     const int v = work[item];
     const long long s = a.off[v];
     const int d = (int)(a.off[v + 1] - s);
