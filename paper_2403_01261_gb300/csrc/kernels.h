@@ -227,11 +227,17 @@ cudaError_t launch_modularity_f32(const long long* off, const int* col, const fl
 constexpr int SOLO_SWEEPS = 64;        // sweeps whose counts fit the state
 constexpr long long SOLO_ROW_MAX = 32768;   // longest row it takes
 constexpr int SOLO_LISTS = 32;         // blocks with label lists for rows of more than 4096 entries
+// Entries of such rows from which the class kernels, which have a list per
+// block, are faster (ms a call, one launch / class kernels): 1.0 M in rows of
+// 8000 0.40 / 0.57, 2.0 M 0.61 / 0.54, 3.2 M 0.89 / 0.55; 1.15 M in rows of 4500
+// 0.47 / 0.58, 3.6 M 1.07 / 0.54; 1.9 M in rows of 30,000 0.44 / 0.47, 3 M 0.74 / 0.47.
+constexpr unsigned long long SOLO_HUGE_ENTRIES = 3ull << 19;
 struct SoloState {   // zero before the launch
   unsigned arrived, released, verdict, abandoned;   // grid barrier
   unsigned nlong, nhuge;               // rows of more than 256 and of more than 4096 entries
   int sweeps, converged;
-  long long longest;                   // a row longer than SOLO_ROW_MAX: nothing was done
+  unsigned long long huge_entries;     // entries of the rows of more than 4096
+  long long longest;                   // more than SOLO_ROW_MAX (a longer row, or too many huge entries): nothing was done
   unsigned long long changed[SOLO_SWEEPS], active[SOLO_SWEEPS];
   unsigned long long scanned, pieces;
   long long time_ns[3];                // start, end of the sweeps, end of the split

@@ -330,7 +330,11 @@ __global__ void __launch_bounds__(SOLO_BLOCK, SOLO_BLOCKS_PER_SM) solo_kernel(Sw
     const long long s = a0.off[v], e = a0.off[v + 1];
     if (s < 0 || e < s || e > q.nnz || (v == 0 && s != 0) || (v == n - 1 && e != q.nnz)) bad = ERRBIT_INVALID;
     else if (e - s > longest) longest = e - s;
-    if (!bad && e - s > SOLO_REG_ROW) q.longs[n - 1 - (long long)atomicAdd(&st->nhuge, 1u)] = (int)v;
+    if (!bad && e - s > SOLO_REG_ROW) {
+      q.longs[n - 1 - (long long)atomicAdd(&st->nhuge, 1u)] = (int)v;
+      const unsigned long long all = atomicAdd(&st->huge_entries, (unsigned long long)(e - s)) + (unsigned long long)(e - s);
+      if (all > SOLO_HUGE_ENTRIES) longest = SOLO_ROW_MAX + 1;   // left to the class kernels
+    }
     else if (!bad && e - s > SOLO_WARP_ROW) q.longs[atomicAdd(&st->nlong, 1u)] = (int)v;
     if (q.lpa) {
       int x = (int)v;

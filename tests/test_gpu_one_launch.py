@@ -1,11 +1,13 @@
 """The one-launch path of small graphs, against the oracle: few rows that hold
-many entries."""
+many entries, and what it leaves to the class kernels."""
 import numpy as np
 import pytest
 import torch
 
 import inputs as I
 import oracle as O
+
+from test_gpu_split_hooks import rows_of
 
 pytestmark = pytest.mark.gpu
 
@@ -37,3 +39,21 @@ def test_few_dense_rows(gpu_lib, n, weighted):
     want, t, dn = O.gsl_lpa(g, 0.0, 9)
     assert launches == 1 and st["iterations"] == t and st["changed"] == dn[:t].tolist()
     assert np.array_equal(got.cpu().numpy(), want)
+
+
+# rows of more than 4096 entries with 3 * 2^19 entries in all are the most it takes
+@pytest.mark.parametrize("rows, one", [([8000] * 196 + [4864], True), ([8000] * 196 + [4865], False),
+                                       ([4097] * 383, True), ([4097] * 384, False), ([32768] * 3, True),
+                                       ([32769] + [5000] * 3, False)])
+def test_many_huge_rows(gpu_lib, rows, one):
+    g = rows_of(rows, 33_000, len(rows))
+    off, col = torch.from_numpy(g.offsets).to(DEV), torch.from_numpy(g.cols).to(DEV)
+    c = gpu_lib.Context(0)
+    (got, st), launches = launched(gpu_lib, lambda: c.gsllpa(off, col, tolerance=0.0, max_iters=4, stats=True))
+    want, t, dn = O.gsl_lpa(g, 0.0, 4)
+    assert (launches == 1) == one and st["iterations"] == t and st["changed"] == dn[:t].tolist()
+    assert np.array_equal(got.cpu().numpy(), want)
+    lab = (np.arange(g.n) % 3).astype(np.int32)
+    (got, k), launches = launched(gpu_lib, lambda: c.split(off, col, torch.from_numpy(lab).to(DEV)))
+    want = O.split_bfs(g, lab)
+    assert (launches == 1) == one and np.array_equal(got.cpu().numpy(), want)
