@@ -85,16 +85,21 @@ int gsl_ctx_destroy(gsl_ctx* ctx);
 /* Degree-class thresholds of the sweep kernels: vertices of degree
  * 33..warp_max (256 at most by one warp, longer ones by 128 threads),
  * warp_max+1..blk_max by a 256-thread block each.  Larger degrees (hubs) run
- * beside those while none exceeds 2^20 and blk_max is at least its default;
- * else they take one 8-CTA thread-block cluster each, or 8192-entry pieces
- * spread over blocks (gsl_ctx_set_hub_cluster).  Labels are counted in
- * shared-memory sketches; rows past 4096 entries keep a label list in
- * context-owned memory.  Defaults 1024 and 131072.  Requires 32 <= warp_max
+ * beside those while none exceeds 2^20 or 1/128 of the graph's entries and
+ * blk_max is at least its default; else they take one 8-CTA thread-block
+ * cluster each, or 8192-entry pieces spread over blocks
+ * (gsl_ctx_set_hub_cluster).  Where the longest row exceeds that 1/128 and
+ * blk_max is the default, rows from 32769 entries on count as hubs.  Labels are
+ * counted in shared-memory sketches; rows past 4096 entries keep a label list
+ * in context-owned memory.  Defaults 1024 and 131072.  Requires 32 <= warp_max
  * <= 2^20 and warp_max <= blk_max.  Results do not depend on these values.
  *
- * A context on which no tuning differs from its default runs synchronous
- * calls on small graphs (up to 2^19 vertices, 2^23 entries and 32768 entries
- * a row, max_iters <= 64) in one cooperative launch. */
+ * Synchronous calls on small graphs (up to 2^19 vertices, 2^23 entries, 32768
+ * entries a row and 3 * 2^19 in rows of more than 4096, max_iters <= 64) run
+ * in one cooperative launch, unless the caller has set the block shape, the
+ * majority or two-phase mode, the hub cluster degree or these thresholds to
+ * other than their defaults, a retry bound is lowered, profiling is on, or
+ * gsl_autotune measured the separate kernels faster. */
 int gsl_ctx_set_tuning(gsl_ctx* ctx, int32_t warp_max, int32_t blk_max);
 
 /* Shape of the hub kernels (clusters and pieces): threads per block of the
@@ -185,13 +190,16 @@ typedef struct {
  * blk_max >= warp_max, x block shape (threads, table slots) in {(512,
  * 12288), (256, 6144)}, x majority mode in {0, 1, 2}, x two-phase mode in
  * {0, 1}; settings that run the same kernels on g (the same binning of
- * g's degrees, and a block shape or majority mode only where g has rows
- * that use it) are timed once.  The fastest setting is set on the context
- * (the setting the context had on entry wins ties).  1 <= sweeps <= 64.
- * Labels do not depend on any of these settings, so tuning changes only
- * speed.  The context's scratch is used; the graph is only read.
- * Synchronises `stream`.  Errors as gsl_lpa; on error the entry setting
- * is restored. */
+ * g's degrees, a block shape only where g has rows for the hub kernels, a
+ * majority mode only where it has rows of more than 32 entries) are timed
+ * once.  Where g is small enough for the one-launch path (gsl_ctx_set_tuning)
+ * that path is a candidate too; when it is the fastest the entry setting
+ * stays and small graphs take it, otherwise they take the separate kernels.
+ * The fastest setting is set on the context (the setting the context had on
+ * entry wins ties).  1 <= sweeps <= 64.  Labels do not depend on any of these
+ * settings, so tuning changes only speed.  The context's scratch is used; the
+ * graph is only read.  Synchronises `stream`.  Errors as gsl_lpa; on error
+ * the entry setting is restored. */
 int gsl_autotune(gsl_ctx* ctx, const gsl_csr* g, const int32_t* weights, int32_t mode, int32_t sweeps,
                  gsl_tune_result* out, void* stream);
 

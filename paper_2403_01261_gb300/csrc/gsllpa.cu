@@ -23,6 +23,7 @@ struct gsl_ctx {
   int device = 0;
   DeviceInfo di;
   Tuning tune;
+  bool class_kernels = false;      // for small graphs too: the caller's tuning, or the autotuner measured them faster
   Tuning run;                      // of the call under way: tune, with the class bound prepare_graph chose
   std::string last_error;
 
@@ -890,15 +891,15 @@ constexpr long long SOLO_MAX_N = 1ll << 19, SOLO_MAX_ENTRIES = 1ll << 23;
 
 // Synchronous sweeps (lpa) and / or the split of a small graph in one launch.
 // *handled stays false when the call does not qualify: larger graphs, rows
-// past SOLO_ROW_MAX, profiling, or any tuning set by the caller (the class
-// kernels it tunes are then what runs).
+// past SOLO_ROW_MAX, profiling, lowered retry bounds, or c->class_kernels.
 int run_solo(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t* labels_init,
              const int32_t* labels_in, bool lpa, bool split, double tol, int32_t max_iters, int32_t mode,
              int32_t* out, gsl_stats* st, long long* pieces, cudaStream_t s, bool* handled) {
   *handled = false;
-  static const Tuning defaults;
-  if (c->prof || mode != GSL_MODE_SYNC || g->n > SOLO_MAX_N || g->nnz > SOLO_MAX_ENTRIES || max_iters > SOLO_SWEEPS ||
-      !c->di.cooperative || memcmp(&c->tune, &defaults, sizeof(Tuning)) != 0)
+  const Tuning d;
+  if (c->prof || c->class_kernels || c->tune.probe_cap != d.probe_cap || c->tune.uf_cap != d.uf_cap ||
+      mode != GSL_MODE_SYNC || g->n > SOLO_MAX_N || g->nnz > SOLO_MAX_ENTRIES || max_iters > SOLO_SWEEPS ||
+      !c->di.cooperative)
     return GSL_OK;
   SweepArgs a{};
   a.off = OFF(g);
@@ -956,6 +957,14 @@ int run_solo(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t
     }
   }
   if (pieces) *pieces = (long long)r.pieces;
+  return GSL_OK;
+}
+
+// After a setting of the class kernels: a caller who changes one wants them to
+// run, on small graphs too.
+int tuned_by_caller(gsl_ctx* c) {
+  const Tuning d;
+  c->class_kernels = memcmp(&c->tune, &d, sizeof(Tuning)) != 0;
   return GSL_OK;
 }
 
@@ -1154,37 +1163,39 @@ int gsl_ctx_set_tuning(gsl_ctx* c, int32_t warp_max, int32_t blk_max) {
     return fail(c, GSL_ERR_INVALID, "need 32 <= warp_max <= 2^20 and blk_max >= warp_max");
   c->tune.warp_max = warp_max;
   c->tune.blk_max = blk_max;
-  return GSL_OK;
+  return tuned_by_caller(c);
 }
 
 }  // extern "C"
 
 // Candidate settings of the autotuners, for a graph with the given sorted
 // degrees.  Two settings are the same run when they bin every vertex alike
-// and agree on every knob that acts on the classes the graph populates:
-// the block shape only matters with rows above warp_max, the majority
-// filter only with rows in classes 7-8 (warp_small+1 .. blk_max).
+// and agree on every knob that acts on the rows the graph has: the block shape
+// on those of the hub kernels (never in the batched loop), the majority filter
+// on those of more than 32 entries.
 namespace {
 struct TuneSpace {
-  bool pregather;   // also try two-phase sweeps
+  bool pregather;   // two-phase sweeps
+  bool hubs;        // the hub kernels take part
 };
 
 long long count_le(const std::vector<long long>& deg_sorted, long long x) {
   return (long long)(std::upper_bound(deg_sorted.begin(), deg_sorted.end(), x) - deg_sorted.begin());
 }
 
-bool same_run(const std::vector<long long>& deg_sorted, const gsl::Tuning& a, const gsl::Tuning& b) {
+bool same_run(const std::vector<long long>& deg_sorted, const gsl::Tuning& a, const gsl::Tuning& b,
+              const TuneSpace& sp) {
   const gsl::ClassBounds ca = gsl::class_bounds(a), cb = gsl::class_bounds(b);
   const long long n = (long long)deg_sorted.size();
   if (count_le(deg_sorted, ca.warp_small) != count_le(deg_sorted, cb.warp_small) ||
       count_le(deg_sorted, ca.warp_max) != count_le(deg_sorted, cb.warp_max) ||
       count_le(deg_sorted, ca.blk_max) != count_le(deg_sorted, cb.blk_max))
     return false;
-  if (a.pregather != b.pregather) return false;
-  const bool block_rows = count_le(deg_sorted, ca.warp_max) < n;
-  if (block_rows && (a.blk_block != b.blk_block || a.blk_slots != b.blk_slots)) return false;
-  const bool filter_rows = count_le(deg_sorted, ca.blk_max) > count_le(deg_sorted, ca.warp_small);
-  if (filter_rows && a.majority != b.majority) return false;
+  if (sp.pregather && a.pregather != b.pregather) return false;
+  if (sp.hubs && count_le(deg_sorted, std::min(ca.blk_max, HUB_MIN)) < n &&
+      (a.blk_block != b.blk_block || a.blk_slots != b.blk_slots))
+    return false;
+  if (count_le(deg_sorted, 32) < n && a.majority != b.majority) return false;
   return true;
 }
 
@@ -1208,7 +1219,7 @@ std::vector<gsl::Tuning> tune_candidates(const std::vector<long long>& deg_sorte
             t.blk_block = sh[0];
             t.blk_slots = sh[1];
             bool dup = false;
-            for (const gsl::Tuning& u : cand) dup = dup || same_run(deg_sorted, t, u);
+            for (const gsl::Tuning& u : cand) dup = dup || same_run(deg_sorted, t, u, sp);
             if (!dup) cand.push_back(t);
           }
       }
@@ -1289,18 +1300,49 @@ int gsl_autotune(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, int32_t m
   if (int r = ensure_vertex_scratch(c, g->n)) return r;
   std::vector<long long> deg;
   if (int r = sorted_degrees(c, g, s, &deg)) return r;
-  const std::vector<Tuning> cand = tune_candidates(deg, c->tune, TuneSpace{true}, c->di.max_smem_optin);
-  return tune_loop(c, cand, out, [&](const Tuning& t, float* ms) -> int {
-    c->tune = t;
-    if (int r = prepare_graph(c, g, s, true)) return r;
-    int* fin = nullptr;
+  const std::vector<Tuning> cand = tune_candidates(deg, c->tune, TuneSpace{true, true}, c->di.max_smem_optin);
+  const Tuning entry = c->tune;
+  const bool entry_class = c->class_kernels;
+  if (int r = tune_loop(c, cand, out, [&](const Tuning& t, float* ms) -> int {
+        c->tune = t;
+        if (int r = prepare_graph(c, g, s, true)) return r;
+        int* fin = nullptr;
+        CK(cudaEventRecord(c->ev[0], s));
+        if (int r = run_lpa(c, g, weights, nullptr, 0.0, sweeps, mode, nullptr, s, &fin)) return r;
+        CK(cudaEventRecord(c->ev[1], s));
+        CK(cudaEventSynchronize(c->ev[1]));
+        CK(cudaEventElapsedTime(ms, c->ev[0], c->ev[1]));
+        return GSL_OK;
+      }))
+    return r;
+  // a small graph's calls take the one-launch path, which none of these
+  // settings acts on: it is a candidate of its own
+  c->class_kernels = false;
+  float ms = 0.f;
+  bool handled = false;
+  for (int rep = 0; rep < 2; ++rep) {   // the first untimed
     CK(cudaEventRecord(c->ev[0], s));
-    if (int r = run_lpa(c, g, weights, nullptr, 0.0, sweeps, mode, nullptr, s, &fin)) return r;
+    const int r = run_solo(c, g, weights, nullptr, nullptr, true, false, 0.0, sweeps, mode, c->parent, nullptr, nullptr,
+                           s, &handled);
+    if (r || !handled) {
+      if (r) c->tune = entry;
+      c->class_kernels = entry_class;
+      return r;
+    }
     CK(cudaEventRecord(c->ev[1], s));
     CK(cudaEventSynchronize(c->ev[1]));
-    CK(cudaEventElapsedTime(ms, c->ev[0], c->ev[1]));
-    return GSL_OK;
-  });
+    CK(cudaEventElapsedTime(&ms, c->ev[0], c->ev[1]));
+  }
+  out->candidates += 1;
+  if (!entry_class) out->entry_ms = ms;
+  if (ms <= out->best_ms) {
+    c->tune = entry;
+    fill_result(entry, out);
+    out->best_ms = ms;
+  } else {
+    c->class_kernels = true;
+  }
+  return GSL_OK;
 }
 
 int gsl_autotune_batch(gsl_ctx* c, const gsl_csr* g, int32_t num_graphs, const int64_t* vptr_host,
@@ -1320,7 +1362,7 @@ int gsl_autotune_batch(gsl_ctx* c, const gsl_csr* g, int32_t num_graphs, const i
   std::vector<long long> deg;
   if (int r = sorted_degrees(c, g, s, &deg)) return r;
   // the batched loop has no two-phase mode
-  const std::vector<Tuning> cand = tune_candidates(deg, c->tune, TuneSpace{false}, c->di.max_smem_optin);
+  const std::vector<Tuning> cand = tune_candidates(deg, c->tune, TuneSpace{false, false}, c->di.max_smem_optin);
   return tune_loop(c, cand, out, [&](const Tuning& t, float* ms) -> int {
     c->tune = t;
     c->batch_key.clear();
@@ -1346,7 +1388,7 @@ int gsl_ctx_set_block_config(gsl_ctx* c, int32_t threads, int32_t table_slots) {
   c->tune.blk_block = threads;
   c->tune.blk_slots = table_slots;
   c->batch_key.clear();   // the captured batched loop used the old shape
-  return GSL_OK;
+  return tuned_by_caller(c);
 }
 
 int gsl_ctx_set_majority(gsl_ctx* c, int32_t mode) {
@@ -1354,7 +1396,7 @@ int gsl_ctx_set_majority(gsl_ctx* c, int32_t mode) {
   if (mode < 0 || mode > 2) return fail(c, GSL_ERR_INVALID, "majority mode must be 0, 1 or 2");
   c->tune.majority = mode;
   c->batch_key.clear();
-  return GSL_OK;
+  return tuned_by_caller(c);
 }
 
 int gsl_ctx_set_f32_fixed(gsl_ctx* c, int32_t mode) {
@@ -1368,7 +1410,7 @@ int gsl_ctx_set_hub_cluster(gsl_ctx* c, int64_t max_degree) {
   if (!c) return GSL_ERR_INVALID;
   if (max_degree < 0) return fail(c, GSL_ERR_INVALID, "hub cluster degree must be >= 0");
   c->tune.hub_cluster_max = max_degree > (1ll << 30) ? (1 << 30) : (int)max_degree;
-  return GSL_OK;
+  return tuned_by_caller(c);
 }
 
 int gsl_ctx_set_retry_bounds(gsl_ctx* c, int32_t probe_bound, int32_t unionfind_bound) {
@@ -1385,7 +1427,7 @@ int gsl_ctx_set_pregather(gsl_ctx* c, int32_t mode) {
   if (!c) return GSL_ERR_INVALID;
   if (mode < 0 || mode > 2) return fail(c, GSL_ERR_INVALID, "pregather mode must be 0, 1 or 2");
   c->tune.pregather = mode;
-  return GSL_OK;
+  return tuned_by_caller(c);
 }
 
 int gsl_ctx_set_batch_mode(gsl_ctx* c, int32_t use_cuda_graph) {
