@@ -5,6 +5,7 @@
 // when dN/N <= tolerance or after max_iters sweeps.  The split of Algorithm
 // 2 and the modularity of Eq. 1 follow as separate kernel sequences.  The
 // context owns all scratch memory and grows it on demand.
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstddef>
@@ -886,20 +887,45 @@ int run_modularity(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const i
   return GSL_OK;
 }
 
+// Calls of gsl_lpa and gsl_gsllpa that threads of this process have under way
+// on a device.  It decides between two paths of the same result only.
+class CallUnderWay {
+ public:
+  explicit CallUnderWay(int device) : count_(counts()[device & 63]) { with_ = count_.fetch_add(1) + 1; }
+  ~CallUnderWay() { count_.fetch_sub(1); }
+  CallUnderWay(const CallUnderWay&) = delete;
+  int with() const { return with_; }   // this one included, at its start
+
+ private:
+  static std::atomic<int>* counts() {
+    static std::atomic<int> c[64];
+    return c;
+  }
+  std::atomic<int>& count_;
+  int with_;
+};
+
 // Graphs up to these sizes run in one cooperative launch (solo_kernel.cu).
-constexpr long long SOLO_MAX_N = 1ll << 19, SOLO_MAX_ENTRIES = 1ll << 23;
+// From about 19,000 vertices on the launch fills the chip, so those of several
+// threads take turns; the class kernels of several calls share it.  Past
+// SOLO_SHARED_N vertices under way they are faster (ms a call, one launch /
+// class kernels, planted partitions of degree 20): 4 threads with 100,000
+// vertices 0.32 / 0.36, 200,000 0.60 / 0.47, 300,000 0.70 / 0.57; 8 threads with
+// 50,000 0.23 / 0.24, 100,000 0.34 / 0.28, 300,000 0.68 / 0.51; 2 threads with
+// 300,000 0.64 / 0.75, 400,000 0.87 / 0.84.
+constexpr long long SOLO_MAX_N = 1ll << 19, SOLO_MAX_ENTRIES = 1ll << 23, SOLO_SHARED_N = 3ll << 18;
 
 // Synchronous sweeps (lpa) and / or the split of a small graph in one launch.
 // *handled stays false when the call does not qualify: larger graphs, rows
 // past SOLO_ROW_MAX, profiling, lowered retry bounds, or c->class_kernels.
 int run_solo(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t* labels_init,
              const int32_t* labels_in, bool lpa, bool split, double tol, int32_t max_iters, int32_t mode,
-             int32_t* out, gsl_stats* st, long long* pieces, cudaStream_t s, bool* handled) {
+             int32_t* out, gsl_stats* st, long long* pieces, cudaStream_t s, bool* handled, int calls = 1) {
   *handled = false;
   const Tuning d;
   if (c->prof || c->class_kernels || c->tune.probe_cap != d.probe_cap || c->tune.uf_cap != d.uf_cap ||
       mode != GSL_MODE_SYNC || g->n > SOLO_MAX_N || g->nnz > SOLO_MAX_ENTRIES || max_iters > SOLO_SWEEPS ||
-      !c->di.cooperative)
+      !c->di.cooperative || (calls > 1 && calls * g->n > SOLO_SHARED_N))
     return GSL_OK;
   SweepArgs a{};
   a.off = OFF(g);
@@ -1471,9 +1497,10 @@ int gsl_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
   DeviceGuard dg(c->device);
   cudaStream_t s = (cudaStream_t)stream;
   if (int r = ensure_vertex_scratch(c, g->n)) return r;
+  const CallUnderWay call(c->device);
   bool handled = false;
   if (int r = run_solo(c, g, weights, labels_init, nullptr, true, false, tol, max_iters, mode, labels_out, st, nullptr,
-                       s, &handled))
+                       s, &handled, call.with()))
     return r;
   if (handled) return GSL_OK;
   CK(cudaEventRecord(c->ev[0], s));
@@ -1696,9 +1723,10 @@ int gsl_gsllpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, double tol,
   DeviceGuard dg(c->device);
   cudaStream_t s = (cudaStream_t)stream;
   if (int r = ensure_vertex_scratch(c, g->n)) return r;
+  const CallUnderWay call(c->device);
   bool handled = false;
   if (int r = run_solo(c, g, weights, nullptr, nullptr, true, true, tol, max_iters, mode, labels_out, st, nullptr, s,
-                       &handled))
+                       &handled, call.with()))
     return r;
   if (handled) return GSL_OK;
   CK(cudaEventRecord(c->ev[0], s));
