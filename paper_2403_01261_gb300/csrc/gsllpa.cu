@@ -590,7 +590,8 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
       const double per_e = 4.0 + (a.ident ? 0.0 : 4.0) + (weights ? 4.0 : 0.0);
       long long act_all = 0;
       for (int k = 0; k < NCLASS; ++k) {
-        auto& sl = c->profile.slot[SL_SWEEP0 + k];
+        // the block kernel's launch has swept class 9 where the hub kernels do not
+        auto& sl = c->profile.slot[SL_SWEEP0 + (k == CLS_HUB && !hub_kernels ? CLS_BLOCK : k)];
         const long long v = (long long)(c->ctr_h->cls_count[k] + c->ctr_h->phase_cls[k]);
         const long long e = (long long)c->ctr_h->cls_scanned[k];
         sl.vertices += v;
@@ -615,7 +616,11 @@ int run_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
         auto& sf = c->profile.slot[SL_FILTER];
         sf.vertices += rows;
         sf.entries += fe;
-        sf.bytes += per_v * (double)rows + per_e * (double)fe;
+        // testing for a label that dominates the graph reads a bit per
+        // neighbour, from a bitmap made of every vertex's label
+        const bool bits = c->ctr_h->giant_on != 0;
+        sf.bytes += per_v * (double)rows + (bits ? per_e - 4.0 + 0.125 : per_e) * (double)fe +
+                    (bits ? 4.125 * (double)n : 0.0);
       }
       auto& sb = c->profile.slot[SL_BIN];
       sb.vertices += all_active ? n : act_all;
@@ -859,13 +864,19 @@ int run_modularity(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const i
   CK(cudaMemsetAsync(c->sigma, 0, sizeof(unsigned long long) * (size_t)n, s));
   CK(cudaMemsetAsync(c->sums, 0, sizeof(ModSums), s));
   if (int r = reset_sweep_counters(c, s)) return r;
-  if (class_vertices(c, CLS_BINNED, NCLASS - 1) > 0)
+  if (class_vertices(c, CLS_BINNED, NCLASS - 1) > 0) {
+    const int pe = prof_begin(c, s);
     CK(launch_bin(OFF(g), n, nullptr, 1, c->run, c->work, c->ctr, c->di, s, nullptr, nullptr, nullptr, -1, 0u,
                   CLS_BINNED));
+    prof_end(c, pe, SL_BIN, s, 1);
+    c->profile.slot[SL_BIN].vertices += n;
+    c->profile.slot[SL_BIN].bytes += 20.0 * (double)n;
+  }
   const int pe = prof_begin(c, s);
+  int kernels = 0;
   CK(launch_modularity(OFF(g), g->cols, weights, n, labels, c->work, c->ctr, c->ctr_h->cls_total, c->sigma,
-                       c->partials, np, c->sums, c->di, s));
-  prof_end(c, pe, SL_MOD, s, 13);
+                       c->partials, np, c->sums, c->di, s, &kernels));
+  prof_end(c, pe, SL_MOD, s, kernels);
   // per vertex: offsets, label, Sigma update (read+write) and square pass;
   // per entry: column, neighbour label and weight
   c->profile.slot[SL_MOD].vertices += n;

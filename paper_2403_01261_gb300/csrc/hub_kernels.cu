@@ -452,7 +452,7 @@ namespace {
 // (0: such clusters cannot run); cached per size.
 template <bool W, bool A>
 int cluster_slots(size_t smem) {
-  thread_local size_t cached_smem = 0;   // per host thread (see block_grid_size)
+  thread_local size_t cached_smem = 0;   // per host thread and table size
   thread_local int cached = 0;
   if (cached_smem == smem) return cached;
   cached_smem = smem;

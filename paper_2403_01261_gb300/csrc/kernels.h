@@ -47,7 +47,7 @@ struct SweepArgs {
   const int* lg;             // sync mode: labels gathered per entry, lg[e] = prev[col[e]] (null: gather)
   int spread;                // labels read are nearly all distinct (sweep 2 from the identity labelling)
   unsigned* kw;              // weighted degree per vertex of classes 6-9: written in sweep 1 (check), then read by
-                             // the early stops of the majority filter and the hub clusters (null: none)
+                             // the majority filter and class 6's own-label test (null: none)
   int probe_cap;             // bound on the probes of one hash-table insert (past it: ERRBIT_TIMEOUT)
 };
 
@@ -290,11 +290,11 @@ struct ModSums {
   unsigned long long s2_lo, s2_hi;
 };
 // `work` holds the binning of classes CLS_BINNED.. of every vertex, totals
-// the host's copy of the class totals.
+// the host's copy of the class totals.  *kernels = launches made.
 cudaError_t launch_modularity(const long long* off, const int* col, const int* w, long long n,
                               const int* labels, const int* work, Counters* ctr, const unsigned long long* totals,
                               unsigned long long* sigma, unsigned long long* partials, long long nparts,
-                              ModSums* out, const DeviceInfo& di, cudaStream_t s);
+                              ModSums* out, const DeviceInfo& di, cudaStream_t s, int* kernels);
 long long modularity_partials(const DeviceInfo& di);
 
 }  // namespace gsl

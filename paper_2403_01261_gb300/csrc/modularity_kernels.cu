@@ -315,7 +315,8 @@ long long modularity_partials(const DeviceInfo& di) { return 4ll * di.sm_count; 
 cudaError_t launch_modularity(const long long* off, const int* col, const int* w, long long n, const int* labels,
                               const int* work, Counters* ctr, const unsigned long long* totals,
                               unsigned long long* sigma, unsigned long long* partials, long long nparts, ModSums* out,
-                              const DeviceInfo& di, cudaStream_t s) {
+                              const DeviceInfo& di, cudaStream_t s, int* kernels) {
+  *kernels = 0;
   if (n <= 0) return cudaSuccess;
   static_assert(CLS_BINNED == 3 && MOD_LANE_ROW == 4, "classes 0..2 are the rows of one lane");
   int launches = w ? launch_mod_rows<true>(off, col, w, n, labels, work, ctr, totals, sigma, out, di, s)
@@ -324,7 +325,8 @@ cudaError_t launch_modularity(const long long* off, const int* col, const int* w
   if (np > (n + 255) / 256) np = (n + 255) / 256;
   mod_square_kernel<<<(int)np, 256, 0, s>>>(sigma, n, partials);
   mod_final_kernel<<<1, 256, 0, s>>>(partials, np, out);
-  count_launches(launches + 2);
+  *kernels = launches + 2;
+  count_launches(*kernels);
   return cudaGetLastError();
 }
 
