@@ -57,3 +57,30 @@ def test_many_huge_rows(gpu_lib, rows, one):
     (got, k), launches = launched(gpu_lib, lambda: c.split(off, col, torch.from_numpy(lab).to(DEV)))
     want = O.split_bfs(g, lab)
     assert (launches == 1) == one and np.array_equal(got.cpu().numpy(), want)
+
+
+def ring(n):
+    u = np.arange(n)
+    return I.csr_from_pairs(n, u, (u + 1) % n, name="ring")
+
+
+def circulant(n, half, extra=0):
+    u = np.repeat(np.arange(n), half)
+    v = (u + np.tile(np.arange(1, half + 1), n)) % n
+    more = np.arange(extra)
+    return I.csr_from_pairs(n, np.concatenate((u, more)), np.concatenate((v, more + n // 2)), name="circulant")
+
+
+# 2^19 vertices, 2^23 entries and 64 sweeps are the most it takes
+@pytest.mark.parametrize("graph, sweeps, one", [
+    (lambda: ring(1 << 19), 5, True), (lambda: ring((1 << 19) + 1), 5, False),
+    (lambda: circulant(1 << 17, 32), 3, True), (lambda: circulant(1 << 17, 32, extra=1), 3, False),
+    (lambda: ring(1000), 64, True), (lambda: ring(1000), 65, False)])
+def test_limits(gpu_lib, graph, sweeps, one):
+    g = graph()
+    off, col = torch.from_numpy(g.offsets).to(DEV), torch.from_numpy(g.cols).to(DEV)
+    c = gpu_lib.Context(0)
+    (got, st), launches = launched(gpu_lib, lambda: c.gsllpa(off, col, tolerance=0.0, max_iters=sweeps, stats=True))
+    want, t, dn = O.gsl_lpa(g, 0.0, sweeps)
+    assert (launches == 1) == one and st["iterations"] == t and st["changed"] == dn[:len(st["changed"])].tolist()
+    assert np.array_equal(got.cpu().numpy(), want)
