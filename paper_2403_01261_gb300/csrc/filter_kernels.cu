@@ -27,7 +27,11 @@ namespace gsl {
 namespace {
 
 constexpr int KW_SHIFT = 22;   // 64-bit sums: row totals are stored as (total >> 22) + 1
-// Sampled shares of neighbours from which the tests pay.
+// Sampled shares of neighbours from which the tests are made.  Neither line is
+// sharp (ms a call).  Giant label from 45 / 55 / 68 %: R-MAT 25 29.6 / 29.9 /
+// 29.7, R-MAT 22 with int32 weights 11.6 / 11.5 / 12.1, heavy-tailed 2 M vertices
+// 2.50 / 2.39 / 2.37; own label from 25 / 40 / 55 %: R-MAT 22 with int32 weights
+// 11.5 / 11.5 / 11.3, 700,000-vertex planted partition 1.92 / 1.90 / 1.89.
 constexpr int GIANT_PERCENT = 55, OWN_PERCENT = 40;
 
 // Weight the tested label must exceed half of: an upper bound of the row's
@@ -262,9 +266,10 @@ __device__ __forceinline__ void filter_blocks(const SweepArgs& a, int* __restric
 // One block per listed piece of a long row.  A piece is skipped once the
 // pieces before it have settled the row; the one that ends last decides.
 // One block over the whole row took 0.5 ms per million entries, however idle
-// the rest of the chip (one hub of 8 M entries among 88 M others: 3.85 ms a
-// pass, 0.06 in pieces; of 1 M: 0.51 and 0.05).  From 65,536 entries on, which
-// a block reads in about 30 us, that is longer than what a sweep costs anyway.
+// the rest of the chip: one hub of 8 M entries among 80 M others 3.85 ms a pass,
+// 0.06 in pieces; of 2 M among 60 M 1.04 and 0.10; of 1 M among 10 M 0.51 and less
+// than 0.05.  From 65,536 entries on, which a block reads in about 30 us, that is
+// longer than what a small graph's sweep takes.
 template <int WT, bool ASYNC, bool GIANT>
 __device__ __forceinline__ void filter_pieces(const SweepArgs& a, int* __restrict__ out) {
   using S = typename SumOf<WT>::T;
@@ -416,6 +421,9 @@ __global__ void __launch_bounds__(256) giant_bits_kernel(const int* __restrict__
   }
 }
 
+// Six blocks per SM: 40 registers, of which the synchronous forms of the warp
+// kernel, which hold both tests, spill 104 to 180 bytes.  R-MAT 25 at 4 / 5 / 6 /
+// 8 blocks: 30.6 / 29.7 / 29.9 / 30.4 ms a call, the filter 9.3 / 8.5 / 8.5 / 9.2.
 template <int WT, bool ASYNC>
 __global__ void __launch_bounds__(256, 6) filter_warp_kernel(SweepArgs a, int* __restrict__ out) {
   if (stopped(a)) return;

@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(SOLO_BLOCK, SOLO_BLOCKS_PER_SM) solo_kernel(Sw
   const unsigned nlong = ld_acquire(&st->nlong), nhuge = ld_acquire(&st->nhuge);
   const int rounds = a0.probe_cap < SKETCH_ROUNDS ? a0.probe_cap : SKETCH_ROUNDS;
   const int* labels = q.labels_in;
-  int tsh = 0;   // vertices per warp and step: one while there are warps enough
+  int tsh = 0;   // log2 of the vertices a warp takes in one step: the most that leave no warp without a full step
   while (tsh < 5 && (n >> (tsh + 1)) >= (long long)gridDim.x * SOLO_WARPS) ++tsh;
   if (q.lpa) {
     int t = 0, converged = 0;
@@ -474,8 +474,9 @@ __global__ void __launch_bounds__(SOLO_BLOCK, SOLO_BLOCKS_PER_SM) solo_kernel(Sw
 
 cudaError_t launch_solo(const SweepArgs& a, const SoloArgs& q, int weights, const DeviceInfo& di, cudaStream_t s) {
   const void* fn = weights ? (const void*)solo_kernel<1> : (const void*)solo_kernel<0>;
-  // four vertices per warp until the grid is full: four rows' loads are in
-  // flight together, and the barrier is cheaper with fewer blocks; a block per
+  // four vertices per warp until the grid is full (in steps of one to four,
+  // tsh): several rows' loads are in flight together, and the barrier is cheaper
+  // with fewer blocks; a block per
   // SOLO_BLOCK_ENTRIES entries where few rows hold many (the complete graph of
   // 1000 vertices: 0.10 ms a call instead of 0.25 with its 32 blocks, of 2000
   // 0.12 instead of 0.35)
