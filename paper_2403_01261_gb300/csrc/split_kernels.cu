@@ -234,16 +234,19 @@ __global__ void __launch_bounds__(256) hook_kernel(const long long* __restrict__
         ru = __ldcg(p + u);
         cu = labels[u];
         slot = (int)comm_slot(cu, n);
-        name = __ldcg(named + slot);
+        name = named[slot];   // through L1: a name stays, and -1 is looked at again
       }
     }
-    if (__any_sync(FULL, name == -1)) {   // one lane asks for all of its community
-      const unsigned same = __match_any_sync(FULL, name == -1 ? slot : -1);
+    // one lane asks for all of its community; a row that the sampling pass has
+    // scanned is offered for less
+    const bool ask = name == -1 && e - s > SPLIT_SCAN - SPLIT_SAMPLE;
+    if (__any_sync(FULL, ask)) {
+      const unsigned same = __match_any_sync(FULL, ask ? slot : -1);
       const int leader = __ffs((int)same) - 1;
       int first = 0;
-      if (name == -1 && lane == leader) first = community_name(named + slot, ru);
+      if (ask && lane == leader) first = community_name(named + slot, ru);
       first = __shfl_sync(FULL, first, leader);
-      if (name == -1) name = first;
+      if (ask) name = first;
     }
     bool offer = slot >= 0 && ru != name;
     if (offer && e - s > HOOK_WARP) {   // from the list's end
