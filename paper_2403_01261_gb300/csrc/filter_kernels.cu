@@ -17,7 +17,8 @@
 // degree, others against the row total that sweep 1 stored.
 //
 // Classes 6 and 7 take a warp per row; 8 and 9 a block per row from a
-// counter, so that no long row is left to one warp; rows past FILTER_LONG are
+// counter, so that no long row is left to one warp; where the rest of the graph
+// does not hide its longest row (SweepArgs::long_rows), rows past FILTER_LONG are
 // only listed there, in pieces of FILTER_PIECE entries that the blocks of a
 // second kernel share.  Bound by the gathers.
 #include "sweep_device.cuh"
@@ -269,7 +270,8 @@ __device__ __forceinline__ void filter_blocks(const SweepArgs& a, int* __restric
 // the rest of the chip: one hub of 8 M entries among 80 M others 3.85 ms a pass,
 // 0.06 in pieces; of 2 M among 60 M 1.04 and 0.10; of 1 M among 10 M 0.51 and less
 // than 0.05.  From 65,536 entries on, which a block reads in about 30 us, that is
-// longer than what a small graph's sweep takes.
+// longer than what a small graph's sweep takes.  R-MAT 25 has no use for it (8.4
+// ms a call by blocks, 8.5 in pieces).
 template <int WT, bool ASYNC, bool GIANT>
 __device__ __forceinline__ void filter_pieces(const SweepArgs& a, int* __restrict__ out) {
   using S = typename SumOf<WT>::T;

@@ -319,6 +319,12 @@ constexpr long long HUB_BLOCK_REST = 128;
 constexpr long long HUB_BLOCK_MAX = 1ll << 20;
 constexpr int HUB_MIN = 32768;
 
+// Whether the longest of the prepared graph's rows stands out like that.
+bool longest_alone(const gsl_ctx* c, long long nnz) {
+  const long long maxd = c->ctr_h->max_degree;
+  return maxd > HUB_BLOCK_MAX || nnz < HUB_BLOCK_REST * maxd;
+}
+
 // Resets all counters and classifies every vertex by degree (validating the
 // offsets) under c->run.  Synchronises the stream.
 int classify(gsl_ctx* c, const gsl_csr* g, cudaStream_t s) {
@@ -340,17 +346,17 @@ int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s, bool sweeps = fa
   c->run = c->tune;
   if (int r = classify(c, g, s)) return r;
   const long long maxd = c->ctr_h->max_degree;
-  const bool alone = g->nnz < HUB_BLOCK_REST * maxd;   // no rest of a sweep to hide the longest row
+  const bool alone = longest_alone(c, g->nnz);
   c->hub_ready = false;
   if (!sweeps || !hub_pieces_fit(c->run)) return GSL_OK;
-  if (alone && maxd > HUB_MIN && c->tune.blk_max == Tuning().blk_max) {
+  if (g->nnz < HUB_BLOCK_REST * maxd && maxd > HUB_MIN && c->tune.blk_max == Tuning().blk_max) {
     c->run.blk_max = std::max(HUB_MIN, c->run.warp_max);
     if (int r = classify(c, g, s)) return r;
   }
   // class 9 (hubs) in pieces: per-hub plan arrays and table regions
   const long long hubs = (long long)c->ctr_h->cls_total[CLS_HUB];
   const long long hub_e = (long long)c->ctr_h->hub_entries;
-  c->hub_ready = hubs > 0 && (maxd > HUB_BLOCK_MAX || alone || c->tune.blk_max < Tuning().blk_max) &&
+  c->hub_ready = hubs > 0 && (alone || c->tune.blk_max < Tuning().blk_max) &&
                  2 * hub_e < (1ll << 32);
   if (c->hub_ready) {
     const long long old_tab = c->cap_hub_tab;
@@ -383,7 +389,7 @@ int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s, bool sweeps = fa
 int ensure_scratch(gsl_ctx* c, long long nnz, bool hub_kernels, SweepArgs* a) {
   const long long maxd = c->ctr_h->max_degree;
   a->long_rows = nullptr;
-  if (maxd > FILTER_LONG && c->tune.majority) {
+  if (maxd > FILTER_LONG && c->tune.majority && longest_alone(c, nnz)) {
     const long long rows = nnz / FILTER_LONG + 1;
     if (int r = grow(c, c->long_rows, c->cap_long_rows, rows)) return r;
     if (int r = grow(c, c->long_pieces, c->cap_long_pieces, nnz / FILTER_PIECE + rows)) return r;

@@ -6,8 +6,8 @@
 
 namespace gsl {
 
-// Majority filter: rows of more than FILTER_LONG entries are read in pieces of
-// FILTER_PIECE by any number of blocks.
+// Majority filter: where nothing hides the longest row, rows of more than
+// FILTER_LONG entries are read in pieces of FILTER_PIECE by any number of blocks.
 constexpr int FILTER_LONG = 65536, FILTER_PIECE = 8192;
 struct FilterLong {   // one such row
   unsigned long long hit, all;   // weight of the tested label and of the whole row, so far
