@@ -84,3 +84,18 @@ def test_limits(gpu_lib, graph, sweeps, one):
     want, t, dn = O.gsl_lpa(g, 0.0, sweeps)
     assert (launches == 1) == one and st["iterations"] == t and st["changed"] == dn[:len(st["changed"])].tolist()
     assert np.array_equal(got.cpu().numpy(), want)
+
+
+def test_split_of_long_rows_side_by_side(gpu_lib):
+    """Rows around the border between a warp and a block, and up to the longest
+    the launch takes, in communities that their sampled entries leave apart."""
+    g = rows_of([255, 256, 257, 258] * 40 + [300, 4096, 4097, 20_000, 32_768], 33_000, 9)
+    off, col = torch.from_numpy(g.offsets).to(DEV), torch.from_numpy(g.cols).to(DEV)
+    c = gpu_lib.Context(0)
+    ids, rng = np.arange(g.n), np.random.default_rng(5)
+    for lab in (ids, ids % 2, rng.integers(0, 40, g.n), rng.integers(0, 2000, g.n), ids // 700, np.zeros(g.n)):
+        lab = lab.astype(np.int32)
+        want = O.split_bfs(g, lab)
+        for _ in range(3):   # the order of the unions differs from call to call
+            (got, k), launches = launched(gpu_lib, lambda: c.split(off, col, torch.from_numpy(lab).to(DEV)))
+            assert launches == 1 and np.array_equal(got.cpu().numpy(), want) and k == (want == ids).sum()
