@@ -174,12 +174,8 @@ __global__ void __launch_bounds__(F_BLOCK) sweep_f_block_kernel(SweepArgs a, con
   const Pol pol = make_pol();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   unsigned long long my_dn = 0, my_scan = 0;
-  __shared__ unsigned s_item;
-  for (;;) {
-    if (threadIdx.x == 0) s_item = atomicAdd(&a.ctr->row_next[cls], 1u);
-    __syncthreads();
-    const unsigned item = s_item;
-    if (item >= cnt) break;
+  __shared__ unsigned s_next;
+  for (unsigned item = blockIdx.x; item < cnt; item = s_next) {   // the first on SMs of their own
     const int v = work[item];
     const long long s = a.off[v];
     const int d = (int)(a.off[v + 1] - s);
@@ -191,7 +187,10 @@ __global__ void __launch_bounds__(F_BLOCK) sweep_f_block_kernel(SweepArgs a, con
       keys[k] = EMPTY32;
       vals[k] = 0.0;
     }
-    if (threadIdx.x == 0) s_own = 0.0;
+    if (threadIdx.x == 0) {
+      s_own = 0.0;
+      s_next = gridDim.x + atomicAdd(&a.ctr->row_next[cls], 1u);
+    }
     const int old = own_label<ASYNC>(a, v);
     __syncthreads();
     const int* cp = a.col + s;
