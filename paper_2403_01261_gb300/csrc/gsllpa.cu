@@ -319,11 +319,17 @@ constexpr long long HUB_BLOCK_REST = 128;
 constexpr long long HUB_BLOCK_MAX = 1ll << 20;
 constexpr int HUB_MIN = 32768;
 
-// Whether the longest of the prepared graph's rows stands out like that.
-bool longest_alone(const gsl_ctx* c, long long nnz) {
+// Whether the longest of the prepared graph's rows stands out like that, with
+// less than `rest` times its entries in the graph.
+bool longest_alone(const gsl_ctx* c, long long nnz, long long rest) {
   const long long maxd = c->ctr_h->max_degree;
-  return maxd > HUB_BLOCK_MAX || nnz < HUB_BLOCK_REST * maxd;
+  return maxd > HUB_BLOCK_MAX || nnz < rest * maxd;
 }
+
+// The majority filter reads rows in pieces from a little earlier: asynchronous
+// sweeps, two passes each, over 32 M entries of which one row has 127,000 take
+// 4.5 ms for five by blocks, 3.9 in pieces.
+constexpr long long FILTER_REST = 512;
 
 // Resets all counters and classifies every vertex by degree (validating the
 // offsets) under c->run.  Synchronises the stream.
@@ -346,7 +352,7 @@ int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s, bool sweeps = fa
   c->run = c->tune;
   if (int r = classify(c, g, s)) return r;
   const long long maxd = c->ctr_h->max_degree;
-  const bool alone = longest_alone(c, g->nnz);
+  const bool alone = longest_alone(c, g->nnz, HUB_BLOCK_REST);
   c->hub_ready = false;
   if (!sweeps || !hub_pieces_fit(c->run)) return GSL_OK;
   if (g->nnz < HUB_BLOCK_REST * maxd && maxd > HUB_MIN && c->tune.blk_max == Tuning().blk_max) {
@@ -389,7 +395,7 @@ int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s, bool sweeps = fa
 int ensure_scratch(gsl_ctx* c, long long nnz, bool hub_kernels, SweepArgs* a) {
   const long long maxd = c->ctr_h->max_degree;
   a->long_rows = nullptr;
-  if (maxd > FILTER_LONG && c->tune.majority && longest_alone(c, nnz)) {
+  if (maxd > FILTER_LONG && c->tune.majority && longest_alone(c, nnz, FILTER_REST)) {
     const long long rows = nnz / FILTER_LONG + 1;
     if (int r = grow(c, c->long_rows, c->cap_long_rows, rows)) return r;
     if (int r = grow(c, c->long_pieces, c->cap_long_pieces, nnz / FILTER_PIECE + rows)) return r;
@@ -923,6 +929,10 @@ class CallUnderWay {
 };
 
 // Graphs up to these sizes run in one cooperative launch (solo_kernel.cu).
+// At the limits it is still the faster alone (ms a call, one launch / class
+// kernels): planted partitions of 500,000 vertices and degree 10 1.15 / 1.27, of
+// 400,000 and 20 0.80 / 1.29, of 300,000 and 26 (7.8 M entries) 0.80 / 1.44, of
+// 20,000 and 328 (6.6 M) 0.68 / 0.74, a lattice of 500,000 0.42 / 0.80.
 // From about 19,000 vertices on the launch fills the chip, so those of several
 // threads take turns; the class kernels of several calls share it.  Past
 // SOLO_SHARED_N vertices under way they are faster (ms a call, one launch /
