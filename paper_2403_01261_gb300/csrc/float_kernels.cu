@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(256) sweep_f_group_kernel(SweepArgs a, const f
 // global regions of 2 * (largest degree) slots per block otherwise.  Blocks take
 // rows from a counter: class 8 spans 1025 to 131,072 entries, and in fixed
 // strides a block with two long ones held up the sweep (R-MAT 22, 20 sweeps:
-// 431 ms a call, 383 so; R-MAT 20 80.8 and 70.2).
+// 431 ms a call, 377 so; R-MAT 20 80.8 and 70.2).
 template <bool ASYNC>
 __global__ void __launch_bounds__(F_BLOCK) sweep_f_block_kernel(SweepArgs a, const float* __restrict__ wf, int cls,
                                                                unsigned tb, unsigned* gkeys, double* gvals,
