@@ -390,17 +390,24 @@ int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s, bool sweeps = fa
 }
 
 
+// Room for the pieces of rows past FILTER_LONG; without it a block takes each.
+bool piece_room(gsl_ctx* c, long long nnz) {
+  const bool ok = grow(c, c->long_pieces, c->cap_long_pieces, nnz / FILTER_PIECE + nnz / FILTER_LONG + 1) == GSL_OK &&
+                  grow(c, c->long_rows, c->cap_long_rows, nnz / FILTER_LONG + 1) == GSL_OK;
+  if (!ok) c->last_error.clear();
+  return ok;
+}
+
 // Label lists for the rows that one block sweeps, and the majority filter's
 // pieces of long rows.
 int ensure_scratch(gsl_ctx* c, long long nnz, bool hub_kernels, SweepArgs* a) {
   const long long maxd = c->ctr_h->max_degree;
   a->long_rows = nullptr;
   if (maxd > FILTER_LONG && c->tune.majority && longest_alone(c, nnz, FILTER_REST)) {
-    const long long rows = nnz / FILTER_LONG + 1;
-    if (int r = grow(c, c->long_rows, c->cap_long_rows, rows)) return r;
-    if (int r = grow(c, c->long_pieces, c->cap_long_pieces, nnz / FILTER_PIECE + rows)) return r;
-    a->long_rows = c->long_rows;
-    a->long_pieces = c->long_pieces;
+    if (piece_room(c, nnz)) {
+      a->long_rows = c->long_rows;
+      a->long_pieces = c->long_pieces;
+    }
   }
   const long long longest = maxd < c->run.blk_max ? maxd : c->run.blk_max;
   a->scratch_region = longest > sketch_register_row() ? 3 * longest : 0;   // labels, parts, their weights
@@ -873,6 +880,8 @@ int run_modularity(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const i
   if (int r = grow(c, c->sigma, c->cap_sigma, n)) return r;
   const long long np = modularity_partials(c->di);
   if (int r = grow(c, c->partials, c->cap_partials, 2 * np)) return r;
+  // one block takes 1.5 ns per entry of a row, the whole chip 0.007
+  const bool shared = c->ctr_h->max_degree > FILTER_LONG && longest_alone(c, g->nnz, 256) && piece_room(c, g->nnz);
   CK(cudaMemsetAsync(c->sigma, 0, sizeof(unsigned long long) * (size_t)n, s));
   CK(cudaMemsetAsync(c->sums, 0, sizeof(ModSums), s));
   if (int r = reset_sweep_counters(c, s)) return r;
@@ -887,7 +896,7 @@ int run_modularity(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const i
   const int pe = prof_begin(c, s);
   int kernels = 0;
   CK(launch_modularity(OFF(g), g->cols, weights, n, labels, c->work, c->ctr, c->ctr_h->cls_total, c->sigma,
-                       c->partials, np, c->sums, c->di, s, &kernels));
+                       c->partials, np, shared ? c->long_pieces : nullptr, c->sums, c->di, s, &kernels));
   prof_end(c, pe, SL_MOD, s, kernels);
   // per vertex: offsets, label, Sigma update (read+write) and square pass;
   // per entry: column, neighbour label and weight

@@ -290,11 +290,13 @@ struct ModSums {
   unsigned long long s2_lo, s2_hi;
 };
 // `work` holds the binning of classes CLS_BINNED.. of every vertex, totals
-// the host's copy of the class totals.  *kernels = launches made.
+// the host's copy of the class totals, pieces (null: rows are not shared) room
+// for those of the rows past FILTER_LONG, Counters::filter_pieces zero.
+// *kernels = launches made.
 cudaError_t launch_modularity(const long long* off, const int* col, const int* w, long long n,
                               const int* labels, const int* work, Counters* ctr, const unsigned long long* totals,
                               unsigned long long* sigma, unsigned long long* partials, long long nparts,
-                              ModSums* out, const DeviceInfo& di, cudaStream_t s, int* kernels);
+                              int2* pieces, ModSums* out, const DeviceInfo& di, cudaStream_t s, int* kernels);
 long long modularity_partials(const DeviceInfo& di);
 
 }  // namespace gsl
