@@ -310,12 +310,18 @@ long long class_vertices(const gsl_ctx* c, int first, int last) {
 // Where the longest does not, the class starts at HUB_MIN entries.
 // Calls in ms, block / hub kernels: a star of 200,000 leaves 5.0 / 2.5, of
 // 1,000,000 21.5 / 6.6, four stars of 300,000 7.5 / 3.3, 40 rows of 130,000 and
-// little else 5.5 / 3.4;
-// where the labels read are distinct the two are closer: one hub of 200,000
-// among 2 M other entries 0.69 / 0.78, of 1 M among 10 M 1.91 / 2.02, four of
-// 1 M among 80 M 3.05 / 2.80.  R-MAT 25's rows of 131,073..864,000 entries cost
-// 2.3 ms more a call in the hub kernels.
-constexpr long long HUB_BLOCK_REST = 128;
+// little else 5.5 / 3.4; where the labels read are distinct the two are closer:
+// one hub of 200,000 among 2 M other entries 0.69 / 0.78, of 1 M among 10 M 1.91 /
+// 2.02, four of 1 M among 80 M 3.05 / 2.80.  R-MAT 25's rows of 131,073..864,000
+// entries cost 2.3 ms more a call in the hub kernels.
+// Sweeps that settle soon hide less.  Rows past 131,072 entries take the hub
+// kernels up to 512 times (three of 700,000 among 180 M, int32 weights 19.7 / 17.7,
+// from random labels 12.8 / 9.9; R-MAT 22, at 878 times, 4.5 / 4.7), shorter ones
+// do not (R-MAT 20, 64,000 at 487 times: 1.31 / 1.39).  Asynchronous sweeps are two
+// passes over half of the rows each: up to 768 times (five sweeps over a hub of
+// 300,000 at 668 times 6.4 / 4.4, over 100 of 50,000 at 296 2.0 / 1.4; R-MAT 22 5.9
+// / 6.5).
+constexpr long long HUB_BLOCK_REST = 128, HUB_LONG_REST = 512, HUB_ASYNC_REST = 768;
 constexpr long long HUB_BLOCK_MAX = 1ll << 20;
 constexpr int HUB_MIN = 32768;
 
@@ -346,16 +352,19 @@ int classify(gsl_ctx* c, const gsl_csr* g, cudaStream_t s) {
   return map_err(c, c->ctr_h->err, "offsets");
 }
 
-// Classes of the call under way and, for sweeps that may use them (hubs), the
-// hub kernels' tables.  Synchronises the stream.
-int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s, bool sweeps = false) {
+// Classes of the call under way and, for sweeps of one graph (mode: GSL_MODE_*),
+// the hub kernels' tables.  Synchronises the stream.
+int prepare_graph(gsl_ctx* c, const gsl_csr* g, cudaStream_t s, int mode = -1) {
   c->run = c->tune;
   if (int r = classify(c, g, s)) return r;
-  const long long maxd = c->ctr_h->max_degree;
-  const bool alone = longest_alone(c, g->nnz, HUB_BLOCK_REST);
   c->hub_ready = false;
-  if (!sweeps || !hub_pieces_fit(c->run)) return GSL_OK;
-  if (g->nnz < HUB_BLOCK_REST * maxd && maxd > HUB_MIN && c->tune.blk_max == Tuning().blk_max) {
+  if (mode < 0 || !hub_pieces_fit(c->run)) return GSL_OK;
+  const long long maxd = c->ctr_h->max_degree;
+  const bool by_default = c->tune.blk_max == Tuning().blk_max;
+  const long long rest = mode == GSL_MODE_ASYNC ? HUB_ASYNC_REST
+                                                : (maxd > Tuning().blk_max ? HUB_LONG_REST : HUB_BLOCK_REST);
+  const bool alone = longest_alone(c, g->nnz, rest);
+  if (g->nnz < rest * maxd && maxd > HUB_MIN && by_default) {
     c->run.blk_max = std::max(HUB_MIN, c->run.warp_max);
     if (int r = classify(c, g, s)) return r;
   }
@@ -1370,7 +1379,7 @@ int gsl_autotune(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, int32_t m
   const bool entry_class = c->class_kernels;
   if (int r = tune_loop(c, cand, out, [&](const Tuning& t, float* ms) -> int {
         c->tune = t;
-        if (int r = prepare_graph(c, g, s, true)) return r;
+        if (int r = prepare_graph(c, g, s, mode)) return r;
         int* fin = nullptr;
         CK(cudaEventRecord(c->ev[0], s));
         if (int r = run_lpa(c, g, weights, nullptr, 0.0, sweeps, mode, nullptr, s, &fin)) return r;
@@ -1540,7 +1549,7 @@ int gsl_lpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, const int32_t*
     return r;
   if (handled) return GSL_OK;
   CK(cudaEventRecord(c->ev[0], s));
-  if (int r = prepare_graph(c, g, s, true)) return r;
+  if (int r = prepare_graph(c, g, s, mode)) return r;
   int* fin = nullptr;
   if (int r = run_lpa(c, g, weights, labels_init, tol, max_iters, mode, st, s, &fin)) return r;
   CK(cudaMemcpyAsync(labels_out, fin, sizeof(int32_t) * (size_t)g->n, cudaMemcpyDeviceToDevice, s));
@@ -1562,7 +1571,7 @@ int gsl_lpa_f32(gsl_ctx* c, const gsl_csr* g, const float* weights, const int32_
   cudaStream_t s = (cudaStream_t)stream;
   if (int r = ensure_vertex_scratch(c, g->n)) return r;
   CK(cudaEventRecord(c->ev[0], s));
-  if (int r = prepare_graph(c, g, s, true)) return r;
+  if (int r = prepare_graph(c, g, s, mode)) return r;
   int* wi = nullptr;
   bool wide = false;
   if (int r = f32_fixed_point(c, g, weights, s, &wi, &wide)) return r;
@@ -1591,7 +1600,7 @@ int gsl_gsllpa_f32(gsl_ctx* c, const gsl_csr* g, const float* weights, double to
   cudaStream_t s = (cudaStream_t)stream;
   if (int r = ensure_vertex_scratch(c, g->n)) return r;
   CK(cudaEventRecord(c->ev[0], s));
-  if (int r = prepare_graph(c, g, s, true)) return r;
+  if (int r = prepare_graph(c, g, s, mode)) return r;
   int* wi = nullptr;
   bool wide = false;
   if (int r = f32_fixed_point(c, g, weights, s, &wi, &wide)) return r;
@@ -1766,7 +1775,7 @@ int gsl_gsllpa(gsl_ctx* c, const gsl_csr* g, const int32_t* weights, double tol,
     return r;
   if (handled) return GSL_OK;
   CK(cudaEventRecord(c->ev[0], s));
-  if (int r = prepare_graph(c, g, s, true)) return r;
+  if (int r = prepare_graph(c, g, s, mode)) return r;
   int* fin = nullptr;
   if (int r = run_lpa(c, g, weights, nullptr, tol, max_iters, mode, st, s, &fin)) return r;
   CK(cudaEventRecord(c->ev[1], s));
@@ -1988,7 +1997,7 @@ int gsllpa_host_overlapped(gsl_ctx* c, int64_t n, int64_t nnz, const int64_t* of
     CK(cudaEventRecord(c->chunk_ev[(size_t)k], c->copy_stream));
   }
   // offsets: validated and classified (synchronises s; the copies go on)
-  if (int r = prepare_graph(c, &g, s, true)) return r;
+  if (int r = prepare_graph(c, &g, s, GSL_MODE_SYNC)) return r;
   CK(cudaMemsetAsync(c->flag[0], 0, (size_t)n, s));
   CK(cudaMemsetAsync(c->flag[1], 0, (size_t)n, s));
   CK(launch_init_labels(nullptr, c->lab[0], c->lab[1], n, c->ctr, c->di, s));

@@ -24,15 +24,17 @@ def hubs_among(length, others, seed):
 
 
 @pytest.mark.parametrize("weighted", [False, True])
+# hidden by 512 times the longest row's entries, up to 131,072 by 128 times
 @pytest.mark.parametrize("length, others, slot, idle", [
-    (131_100, 0, "sweep_hub", "sweep_block"), (131_100, 1_000_000, "sweep_hub", "sweep_block"),
-    (131_100, 17_000_000, "sweep_block", "sweep_hub"),
+    (131_100, 0, "sweep_hub", "sweep_block"), (131_100, 17_000_000, "sweep_hub", "sweep_block"),
+    (131_100, 68_000_000, "sweep_block", "sweep_hub"),
     (32_769, 0, "sweep_hub", "sweep_block"), (40_000, 1_000_000, "sweep_hub", "sweep_block"),
     (40_000, 5_300_000, "sweep_block", "sweep_hub")])
 def test_route_and_labels(gpu_lib, length, others, slot, idle, weighted):
     g = hubs_among(length, others, seed=others + length)
     d = np.diff(g.offsets)
-    assert (d >= length).sum() == 2 and (g.nnz < 128 * d.max()) == (slot == "sweep_hub")
+    rest = 512 if length > 131_072 else 128
+    assert (d >= length).sum() == 2 and (g.nnz < rest * d.max()) == (slot == "sweep_hub")
     if weighted:
         g = I.Graph(g.offsets, g.cols, I.symmetric_weights(g, 4, 9))
     off, col = torch.from_numpy(g.offsets).to(DEV), torch.from_numpy(g.cols).to(DEV)
@@ -45,3 +47,19 @@ def test_route_and_labels(gpu_lib, length, others, slot, idle, weighted):
     assert np.array_equal(got.cpu().numpy(), want)
     launches = {p["name"]: p["launches"] for p in c.profile()}
     assert launches[slot] > 0 and launches[idle] == 0
+
+
+# in place, up to 768 times
+@pytest.mark.parametrize("others, slot", [(5_300_000, "sweep_hub"), (32_000_000, "sweep_block")])
+def test_route_in_place(gpu_lib, others, slot):
+    g = hubs_among(40_000, others, seed=others)
+    assert (g.nnz < 768 * np.diff(g.offsets).max()) == (slot == "sweep_hub")
+    off, col = torch.from_numpy(g.offsets).to(DEV), torch.from_numpy(g.cols).to(DEV)
+    c = gpu_lib.Context(0)
+    c.set_profiling(True)
+    got, st = c.lpa(off, col, mode=1, tolerance=0.0, max_iters=40, stats=True)
+    lab = got.cpu().numpy()
+    if st["changed"][-1] == 0:   # settled: every vertex holds its Eq. 2 label
+        assert (O.sync_sweep(g, lab)[0] == lab).all()
+    launches = {p["name"]: p["launches"] for p in c.profile()}
+    assert ((lab >= 0) & (lab < g.n)).all() and launches[slot] > 0

@@ -58,6 +58,6 @@ def test_filter_bytes(gpu_lib):
 
 def test_block_kernel_books_the_hubs_it_sweeps(gpu_lib):
     from test_gpu_hub_route import hubs_among
-    g = hubs_among(131_100, 17_000_000, 5)   # two rows of class 9, hidden by the rest
+    g = hubs_among(131_100, 68_000_000, 5)   # two rows of class 9, hidden by the rest
     _, _, prof = profiled(gpu_lib, g, lambda c, off, col: c.lpa(off, col, tolerance=0.0, max_iters=2))
     assert prof["sweep_hub"]["entries"] == 0 and prof["sweep_block"]["entries"] >= 2 * 131_100
