@@ -85,11 +85,12 @@ int gsl_ctx_destroy(gsl_ctx* ctx);
 /* Degree-class thresholds of the sweep kernels: vertices of degree
  * 33..warp_max (256 at most by one warp, longer ones by 128 threads),
  * warp_max+1..blk_max by a 256-thread block each.  Larger degrees (hubs) run
- * beside those while none exceeds 2^20 or 1/128 of the graph's entries and
- * blk_max is at least its default; else they take one 8-CTA thread-block
- * cluster each, or 8192-entry pieces spread over blocks
- * (gsl_ctx_set_hub_cluster).  Where the longest row exceeds that 1/128 and
- * blk_max is the default, rows from 32769 entries on count as hubs.  Labels are
+ * beside those while none exceeds 2^20 or stands out of the graph and blk_max
+ * is at least its default; else they take one 8-CTA thread-block cluster each,
+ * or 8192-entry pieces spread over blocks (gsl_ctx_set_hub_cluster).  The
+ * longest row stands out when the graph has less than 128 times its entries
+ * (512 times past 131072 entries; 768 times in asynchronous sweeps); rows from
+ * 32769 entries on then count as hubs if blk_max is the default.  Labels are
  * counted in shared-memory sketches; rows past 4096 entries keep a label list
  * in context-owned memory.  Defaults 1024 and 131072.  Requires 32 <= warp_max
  * <= 2^20 and warp_max <= blk_max.  Results do not depend on these values.
