@@ -263,7 +263,7 @@ cudaError_t launch_solo(const SweepArgs& a, const SoloArgs& q, int weights, cons
 
 // split_kernels.cu.  list, parent and named: n ints of scratch each;
 // Counters::hook_rows and hook_long zero.
-constexpr int SPLIT_LAUNCHES = 10;
+constexpr int SPLIT_LAUNCHES = 9;
 cudaError_t launch_split(const long long* off, const int* col, long long n, const int* labels,
                          int* list, Counters* ctr, int* parent, int* named, int* out, const Tuning& t,
                          const DeviceInfo& di, cudaStream_t s);

@@ -188,8 +188,8 @@ __global__ void name_giant_kernel(const int* __restrict__ labels, long long n, i
 // parent has become the named root by the time their row is reached.  Rows of up
 // to HOOK_LANE entries go by their lane, longer ones by this warp, two at a time,
 // while they are HOOK_STEPS steps of 32 entries in all.  A warp that meets more
-// lists them, for a warp each (hook_rows_kernel) or past HOOK_WARP entries for a
-// block each (hook_long_kernel), which also stop inside a row.  Left where they
+// lists them, for a warp each or past HOOK_WARP entries for a block each
+// (hook_listed_kernel), which also stop inside a row.  Left where they
 // were met, the dense rows of a small graph, or the heavy ids of one that is
 // sorted by degree, ran on a fraction of the chip: split after LPA of 60,000
 // vertices of 1500 entries 2.43 ms, listed 0.43; 2 million vertices, a few of
@@ -282,33 +282,26 @@ __global__ void __launch_bounds__(256) hook_kernel(const long long* __restrict__
   }
 }
 
-// The listed rows, a warp each.  A warp takes a run of the list, so that the
-// rows in flight lie in many communities and their unions seldom compete.
+// The listed rows: the long ones a block each, then the others a warp each.  A
+// warp takes a run of the list, so that the rows in flight lie in many communities
+// and their unions seldom compete.
 template <int F>
-__global__ void __launch_bounds__(256) hook_rows_kernel(const long long* __restrict__ off, const int* __restrict__ col,
-                                                         const int* __restrict__ labels, int* p, long long n,
-                                                         const int* __restrict__ list, Counters* ctr, UfCap<F> cap,
-                                                         const int* __restrict__ named) {
-  const unsigned cnt = ctr->hook_rows, nwarps = (gridDim.x * blockDim.x) >> 5;
-  const unsigned part = (cnt + nwarps - 1) / nwarps, w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+__global__ void __launch_bounds__(512) hook_listed_kernel(const long long* __restrict__ off, const int* __restrict__ col,
+                                                           const int* __restrict__ labels, int* p, long long n,
+                                                           const int* __restrict__ list, Counters* ctr, UfCap<F> cap,
+                                                           const int* __restrict__ named) {
+  const unsigned longs = ctr->hook_long, cnt = ctr->hook_rows;
+  for (unsigned i = blockIdx.x; i < longs; i += gridDim.x) {
+    const int u = list[n - 1 - i], cu = labels[u];
+    hook_row<true>(col, labels, p, n, u, cu, named[comm_slot(cu, n)], off[u] + SPLIT_SAMPLE + threadIdx.x, off[u + 1],
+                   (int)blockDim.x, &ctr->err, cap);
+  }
+  const unsigned nwarps = (gridDim.x * blockDim.x) >> 5, part = (cnt + nwarps - 1) / nwarps;
+  const unsigned w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   for (unsigned i = w * part; i < cnt && i < (w + 1) * part; ++i) {
     const int u = list[i], cu = labels[u];
     hook_row<true>(col, labels, p, n, u, cu, named[comm_slot(cu, n)], off[u] + SPLIT_SAMPLE + (threadIdx.x & 31),
-                off[u + 1], 32, &ctr->err, cap);
-  }
-}
-
-// The listed long rows, one block each.
-template <int F>
-__global__ void __launch_bounds__(512) hook_long_kernel(const long long* __restrict__ off, const int* __restrict__ col,
-                                                         const int* __restrict__ labels, int* p, long long n,
-                                                         const int* __restrict__ list, Counters* ctr, UfCap<F> cap,
-                                                         const int* __restrict__ named) {
-  const unsigned cnt = ctr->hook_long;
-  for (unsigned i = blockIdx.x; i < cnt; i += gridDim.x) {
-    const int u = list[n - 1 - i], cu = labels[u];
-    hook_row<true>(col, labels, p, n, u, cu, named[comm_slot(cu, n)], off[u] + SPLIT_SAMPLE + threadIdx.x, off[u + 1],
-                (int)blockDim.x, &ctr->err, cap);
+                   off[u + 1], 32, &ctr->err, cap);
   }
 }
 
@@ -521,8 +514,7 @@ void launch_split_t(const long long* off, const int* col, long long n, const int
   name_pieces_kernel<<<g, 256, 0, s>>>(parent, labels, n, named);
   name_giant_kernel<<<1, 1, 0, s>>>(labels, n, named, ctr);
   hook_kernel<F><<<g, 256, 0, s>>>(off, col, labels, parent, n, list, ctr, cap, named);
-  hook_rows_kernel<F><<<8 * di.sm_count, 256, 0, s>>>(off, col, labels, parent, n, list, ctr, cap, named);
-  hook_long_kernel<F><<<4 * di.sm_count, 512, 0, s>>>(off, col, labels, parent, n, list, ctr, cap, named);
+  hook_listed_kernel<F><<<4 * di.sm_count, 512, 0, s>>>(off, col, labels, parent, n, list, ctr, cap, named);
   flatten_kernel<F><<<g, 256, 0, s>>>(parent, out, n, ctr, cap);
   count_launches(SPLIT_LAUNCHES);
 }
